@@ -1,0 +1,654 @@
+// rbf.cu -- interface interpolation of stage two in three dimensions (Sec.
+// 2.1, Fig. 2.2; pdd_interface_interp): per plane, a radial basis function
+// interpolant with the cubic kernel |r|^3 and a linear polynomial term through
+// the plane's nodes and n_bnd points per edge of the plane's perimeter, where
+// the boundary data g are known.  The saddle-point system
+//   [Phi P; P^T 0] [w; c] = [v; 0],  Phi_ij = |x_i - x_j|^3,  P_i = (1, s_i, t_i)
+// is solved in FP64 by Gaussian elimination with partial pivoting, then
+// evaluated at the query points.
+//
+// What bounds it: the FP64 pipe (1/64 rate: 2 lanes per clock and SM).  On the
+// 9 planes of the 4096-node workload (M about 590) the elimination needs
+// 6.0e8 multiply-adds (1.0 ms on all 152 SMs) and the evaluation at 9 x 129^2
+// points 8.7e7 kernel values (1.4 ms at ten FP64 instructions each).
+//
+// Elimination.  Right-looking in panels of NB columns over the list of rows
+// that have not been a pivot yet (rows are not moved).  Two launches per panel:
+//   1. rbf_step_kernel<..., kNext>: the columns of the next panel are updated
+//      by the current one;
+//   2. rbf_step_kernel<..., kRest>: one block per plane factors the next panel
+//      (pivot search, multipliers) while the other blocks update all the
+//      columns behind it by the current panel.
+// So the serial pivot chain of a panel runs beside the update, which spreads
+// over the whole GPU.  Every matrix element sees the same multiply-adds in
+// the same order as in the plain row-by-row elimination (one FMA per step in
+// step order, l = a / pivot), whatever the panel width.  Factored rows go to U
+// in pivot order.
+//
+// Measured on the 9 planes (device time): elimination and back substitution
+// 11.75 ms by one 8-block cluster per plane with a cluster barrier per step
+// (20 us a step) -> 2.9 ms; evaluation 2.28 -> 1.56 ms.
+#include <cmath>
+#include <cstring>
+#include <vector>
+
+#include "ctx.hpp"
+#include "models.cuh"
+
+namespace pdd {
+
+constexpr int64_t kRbfMaxSystem = 6144;  // unknowns per plane (weights + 3)
+constexpr int kRbfThreads = 512;
+constexpr int kRbfTileR = 64;            // rows of an update tile
+constexpr size_t kRbfPanelBytes = 200 * 1024;  // panel in shared memory (rows x NB doubles)
+
+struct RbfPlane {
+  int64_t node0, m;      // this plane's nodes: [node0, node0 + m) of the call's list
+  int64_t sys0;          // offset of its system A (M rows of M + 1: the matrix, then the right-hand side)
+  int64_t row0;          // offset of its rows in the per-row arrays (M of them)
+  int64_t pts0;          // offset of its 2-D points (M - 3 of them) and values
+  int64_t q0, q;         // its query points
+  int32_t axis, M;       // plane normal axis; system size
+  double pos;
+};
+
+// Scratch of the elimination (device pointers, all planes).
+struct RbfWork {
+  const RbfPlane *planes;
+  int32_t n_planes;
+  double *A;             // systems, row-major, M x (M + 1) each
+  double *U;             // factored rows in pivot order, same layout
+  double *x;             // solutions [row0 + k]
+  double *L[2];          // multipliers of the active rows, by panel parity: [row0 + pos][NB]
+  int32_t *act[2];       // active rows (not yet a pivot) after a panel, by parity: [row0 + pos]
+  double *L11[2];        // per plane: multipliers of the panel's pivot rows [NB][NB]
+  int32_t *piv[2];       // per plane: the panel's pivot rows [NB]
+  int *singular;
+};
+
+// sqrt of r2 >= 0 in FP64 by Heron's iteration from a binary32 seed: the
+// hardware reciprocal square root y of r2 cut to a float gives s0 = r2 y and
+// h = y / 2 (20 bits kept, in the high words), and two corrections
+// s <- s + (r2 - s^2) h (the residual exact by FMA) reach the last bit: the
+// relative error goes 2^-20 -> 2^-39 -> below 2^-58 before the final rounding.
+// Four FP64 instructions, where the library's square root takes several times
+// that on this 1/64-rate pipe.  Outside [2^-100, 2^100) (a query on a point,
+// far-away points) the library function.
+__device__ __forceinline__ double sqrt_r2(double r2) {
+  const int hi = __double2hiint(r2);
+  if (static_cast<unsigned>(hi - (923 << 20)) >= (200u << 20)) return sqrt(r2);
+  // the high word's 11-bit exponent rebiased to 8 bits, 20 mantissa bits kept
+  const float f = __int_as_float((hi - (896 << 20)) << 3);
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
+  const double s0 = __hiloint2double((__float_as_int(f * y) >> 3) + (896 << 20), 0);
+  const double h = __hiloint2double((__float_as_int(0.5f * y) >> 3) + (896 << 20), 0);
+  const double s1 = fma(fma(-s0, s0, r2), h, s0);
+  return fma(fma(-s1, s1, r2), h, s1);
+}
+
+// The plane's two in-plane coordinates of a 3-D point.
+__device__ __forceinline__ void plane_coords(int axis, const double *x, double &s, double &t) {
+  s = x[axis == 0 ? 1 : 0];
+  t = x[axis == 2 ? 1 : 2];
+}
+
+// Interpolation points of every plane: its nodes, then n_bnd points per edge
+// of its perimeter (corners once) with the boundary data g.
+template <class Model>
+__global__ void rbf_points_kernel(const RbfPlane *planes, int32_t n_planes, const double *nodes,
+                                  const double *vals, int32_t n_bnd, ModelConst mc, double *pts,
+                                  double *pv) {
+  const int p = blockIdx.y;
+  if (p >= n_planes) return;
+  const RbfPlane P = planes[p];
+  const int64_t npt = P.M - 3;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < npt;
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    double s, t, v;
+    if (i < P.m) {
+      plane_coords(P.axis, nodes + 3 * (P.node0 + i), s, t);
+      v = vals[P.node0 + i];
+    } else {
+      // perimeter of the unit square in (s, t): edge e, point k of n_bnd
+      const int64_t b = i - P.m;
+      const int e = static_cast<int>(b / n_bnd);
+      const double u = static_cast<double>(b % n_bnd) / n_bnd;
+      s = e == 0 ? u : (e == 1 ? 1.0 : (e == 2 ? 1.0 - u : 0.0));
+      t = e == 0 ? 0.0 : (e == 1 ? u : (e == 2 ? 1.0 : 1.0 - u));
+      double x[3];
+      x[P.axis] = P.pos;
+      x[P.axis == 0 ? 1 : 0] = s;
+      x[P.axis == 2 ? 1 : 2] = t;
+      v = Model::template g<double>(mc, x);
+    }
+    pts[2 * (P.pts0 + i)] = s;
+    pts[2 * (P.pts0 + i) + 1] = t;
+    pv[P.pts0 + i] = v;
+  }
+}
+
+// The systems (matrix and right-hand side in one row), the first list of
+// active rows: all of them.
+__global__ void rbf_assemble_kernel(RbfWork W, const double *pts, const double *pv) {
+  const RbfPlane P = W.planes[blockIdx.y];
+  const int M = P.M, ld = M + 1, npt = M - 3;
+  double *A = W.A + P.sys0;
+  const double *xy = pts + 2 * P.pts0;
+  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+       e < static_cast<int64_t>(M) * ld; e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const int i = static_cast<int>(static_cast<uint32_t>(e) / static_cast<uint32_t>(ld));
+    const int j = static_cast<int>(e) - i * ld;
+    double a;
+    if (j == M) {
+      a = i < npt ? pv[P.pts0 + i] : 0.0;
+      W.act[1][P.row0 + i] = i;
+    } else if (i < npt && j < npt) {
+      const double ds = xy[2 * i] - xy[2 * j], dt = xy[2 * i + 1] - xy[2 * j + 1];
+      const double r2 = ds * ds + dt * dt;
+      a = r2 * sqrt_r2(r2);
+    } else if (i < npt) {
+      a = j == npt ? 1.0 : xy[2 * i + (j - npt - 1)];
+    } else if (j < npt) {
+      a = i == npt ? 1.0 : xy[2 * j + (i - npt - 1)];
+    } else {
+      a = 0.0;
+    }
+    A[e] = a;
+  }
+}
+
+// a / b for the pivot b with r = 1 / b correctly rounded (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000", 1990): q = a r, then one
+// correction by the exact remainder gives the correctly rounded quotient while
+// nothing underflows: three FP64 instructions per row instead of a division.
+__device__ __forceinline__ double markstein_div(double a, double b, double r) {
+  const double q = a * r;
+  return fma(fma(-q, b, a), r, q);
+}
+
+// Factor panel `panel` of a plane (columns [k0, k0 + nb)): one block.  The
+// active rows' panel entries sit in shared memory, column by column; thread t
+// owns the list positions t, t + 512, ...  Each step takes the unused row of
+// largest |entry| (lowest row index on ties), forms the multipliers of the
+// other unused rows and updates their remaining panel entries; the update of
+// the next column comes first and yields the next step's candidates in the
+// same pass.  On return the list of rows still active, their multipliers, the
+// pivot rows and their own multipliers are stored for the update, and U has
+// the panel's columns of the pivot rows.
+template <int NB>
+__device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel, double *smem) {
+  const int k0 = panel * NB;
+  const int M = P.M, ld = M + 1;
+  if (k0 >= M) return;
+  const int nb = min(NB, M - k0);
+  const int R = M - k0;  // active rows before this panel
+  const int par = panel & 1;
+  const int32_t *act = W.act[par ^ 1] + P.row0;
+  const double *A = W.A + P.sys0;
+  double *U = W.U + P.sys0;
+  double *S = smem;  // S[c * R + pos]
+  __shared__ uint32_t c_hi[2][kRbfThreads / 32], c_lo[2][kRbfThreads / 32];
+  __shared__ int32_t c_pos[2][kRbfThreads / 32];
+  __shared__ double s_r;
+  __shared__ int32_t s_piv[NB];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int nw = kRbfThreads / 32;
+  for (int e = tid; e < R * NB; e += kRbfThreads) {
+    const int pos = e / NB, c = e % NB;
+    if (c < nb) S[c * R + pos] = A[static_cast<int64_t>(act[pos]) * ld + k0 + c];
+  }
+  __syncthreads();
+  uint32_t used = 0;  // bit i: own position tid + 512 i has been a pivot
+  // candidate of this thread: bits of |entry| plus one (0: none, and for NaN)
+  // and its position (the list keeps rows in increasing order, so the lowest
+  // position is the lowest row)
+  unsigned long long key = 0;
+  int32_t kpos = 0x7fffffff;
+  auto consider = [&](double v, int pos) {
+    const unsigned long long b =
+        v == v ? (static_cast<unsigned long long>(__double_as_longlong(v)) & 0x7fffffffffffffffull) + 1
+               : 0ull;
+    if (b > key) {
+      key = b;
+      kpos = pos;
+    }
+  };
+  for (int pos = tid; pos < R; pos += kRbfThreads) consider(S[pos], pos);
+  for (int kk = 0; kk < nb; ++kk) {
+    const int sl = kk & 1;
+    // warp candidate: largest key, then lowest position
+    {
+      const uint32_t hi = static_cast<uint32_t>(key >> 32);
+      const uint32_t mh = __reduce_max_sync(kFull, hi);
+      const uint32_t lo = hi == mh ? static_cast<uint32_t>(key) : 0u;
+      const uint32_t ml = __reduce_max_sync(kFull, lo);
+      const int32_t mp = __reduce_min_sync(kFull, hi == mh && lo == ml ? kpos : 0x7fffffff);
+      if (lane == 0) {
+        c_hi[sl][warp] = mh;
+        c_lo[sl][warp] = ml;
+        c_pos[sl][warp] = mp;
+      }
+    }
+    __syncthreads();
+    // every warp finds the block's pivot from the warp candidates
+    const uint32_t hi = lane < nw ? c_hi[sl][lane] : 0u;
+    const uint32_t mh = __reduce_max_sync(kFull, hi);
+    const uint32_t lo = lane < nw && hi == mh ? c_lo[sl][lane] : 0u;
+    const uint32_t ml = __reduce_max_sync(kFull, lo);
+    const bool top = lane < nw && hi == mh && lo == ml;
+    const int32_t mp = __reduce_min_sync(kFull, top ? c_pos[sl][lane] : 0x7fffffff);
+    // NaN in every unused row: no pivot (flagged; the solution is not used)
+    const bool none = (mh | ml) == 0u;
+    const int pr = none ? 0 : mp;
+    const double akk = S[kk * R + pr];
+    if (tid == 0) {
+      if (none || !(fabs(akk) > 0.0)) *W.singular = 1;
+      s_r = 1.0 / akk;
+      s_piv[kk] = pr;
+    }
+    if (pr % kRbfThreads == tid) used |= 1u << (pr / kRbfThreads);
+    __syncthreads();
+    const double r = s_r;
+    // far from overflow and underflow the corrected quotient is the division
+    const bool plain = !(fabs(akk) > 0x1p-500 && fabs(akk) < 0x1p500);
+    key = 0;
+    kpos = 0x7fffffff;
+    const int c1 = kk + 1;
+    for (int i = 0, pos = tid; pos < R; ++i, pos += kRbfThreads) {
+      if ((used >> i) & 1u) continue;
+      const double a = S[kk * R + pos];
+      const double l = plain ? a / akk : markstein_div(a, akk, r);
+      S[kk * R + pos] = l;
+      if (c1 < nb) {
+        const double v = fma(-l, S[c1 * R + pr], S[c1 * R + pos]);
+        S[c1 * R + pos] = v;
+        consider(v, pos);
+      }
+      // (the pivot row's entries are read by every thread and written by none)
+#pragma unroll 4
+      for (int c = kk + 2; c < nb; ++c)
+        S[c * R + pos] = fma(-l, S[c * R + pr], S[c * R + pos]);
+    }
+  }
+  __syncthreads();
+  // the panel's columns of U, the pivot rows, their multipliers
+  double *L11 = W.L11[par] + (blockIdx.x * NB) * NB;
+  for (int e = tid; e < nb * nb; e += kRbfThreads) {
+    const int i = e / nb, c = e % nb;
+    const double v = S[c * R + s_piv[i]];
+    if (c >= i) U[static_cast<int64_t>(k0 + i) * ld + k0 + c] = v;
+    else L11[i * NB + c] = v;
+  }
+  if (tid < nb) W.piv[par][blockIdx.x * NB + tid] = act[s_piv[tid]];
+  // rows still active keep their order: the new position is the old one less
+  // the pivots before it
+  int32_t *act2 = W.act[par] + P.row0;
+  double *L = W.L[par] + P.row0 * NB;
+  for (int i = 0, pos = tid; pos < R; ++i, pos += kRbfThreads) {
+    if ((used >> i) & 1u) continue;
+    int np = pos;
+    for (int c = 0; c < nb; ++c) np -= s_piv[c] < pos ? 1 : 0;
+    act2[np] = act[pos];
+    for (int c = 0; c < nb; ++c) L[static_cast<int64_t>(np) * NB + c] = S[c * R + pos];
+  }
+}
+
+// Update by panel `panel` (already factored) of a tile of TC columns from
+// column c0 (below c1) and kRbfTileR active rows from position r0.  The block
+// first solves for the pivot rows' entries of its columns (unit lower
+// triangle, one thread per column; the tiles of the first row store them in
+// U), then updates its rows: one FMA per element and pivot, in pivot order.
+template <int NB, int TC>
+__device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int plane, int panel, int r0,
+                                int c0, int c1, double *smem) {
+  const int k0 = panel * NB, M = P.M, ld = M + 1;
+  const int nb = min(NB, M - k0);
+  const int R = M - k0 - nb;
+  const int par = panel & 1;
+  double *A = W.A + P.sys0;
+  double *Us = smem;                 // [NB][TC]
+  double *Ls = smem + NB * TC;       // [kRbfTileR][NB + 1]
+  const int tid = threadIdx.x;
+  const int rows = min(kRbfTileR, R - r0);
+  const double *L = W.L[par] + (P.row0 + r0) * NB;
+  if (tid < TC) {
+    const int j = c0 + tid;
+    if (j < c1) {
+      const double *L11 = W.L11[par] + plane * NB * NB;
+      const int32_t *piv = W.piv[par] + plane * NB;
+      double u[NB];
+#pragma unroll
+      for (int i = 0; i < NB; ++i) u[i] = i < nb ? A[static_cast<int64_t>(piv[i]) * ld + j] : 0.0;
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+#pragma unroll
+        for (int i = k + 1; i < NB; ++i)
+          if (i < nb) u[i] = fma(-L11[i * NB + k], u[k], u[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        Us[i * TC + tid] = u[i];
+        if (r0 == 0 && i < nb) W.U[P.sys0 + static_cast<int64_t>(k0 + i) * ld + j] = u[i];
+      }
+    }
+  } else {
+    for (int e = tid - TC; e < rows * NB; e += kRbfThreads - TC) {
+      const int pos = e / NB, c = e % NB;
+      Ls[pos * (NB + 1) + c] = c < nb ? L[e] : 0.0;
+    }
+  }
+  __syncthreads();
+  const int tx = tid % TC, ty = tid / TC;
+  const int j = c0 + tx;
+  if (j < c1) {
+    const int32_t *act = W.act[par] + P.row0 + r0;
+    double u[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) u[k] = Us[k * TC + tx];
+    for (int q = ty; q < rows; q += kRbfThreads / TC) {
+      double *pa = A + static_cast<int64_t>(act[q]) * ld + j;
+      double a = *pa;
+#pragma unroll
+      for (int k = 0; k < NB; ++k)
+        if (k < nb) a = fma(-Ls[q * (NB + 1) + k], u[k], a);
+      *pa = a;
+    }
+  }
+  __syncthreads();
+}
+
+// kFirst: panel 0 of every plane is factored (blockIdx.x = plane).
+// kNext: the columns of panel + 1 are updated by `panel` (blockIdx = row
+// tile, plane).
+// kRest: blocks [0, n_planes) factor panel + 1; the others update the columns
+// behind it by `panel` (blockIdx.x - n_planes = (plane, row tile, column
+// tile), column tiles fastest).
+enum { kFirst = 0, kNext = 1, kRest = 2 };
+template <int NB, int kRole>
+__global__ void __launch_bounds__(kRbfThreads)
+rbf_step_kernel(const __grid_constant__ RbfWork W, int panel, int row_tiles, int col_tiles) {
+  extern __shared__ __align__(16) double rbf_smem[];
+  constexpr int TC = 32;
+  if constexpr (kRole == kFirst) {
+    rbf_factor_panel<NB>(W, W.planes[blockIdx.x], 0, rbf_smem);
+  } else if constexpr (kRole == kNext) {
+    const RbfPlane P = W.planes[blockIdx.y];
+    const int k0 = panel * NB;
+    const int r0 = blockIdx.x * kRbfTileR;
+    const int R = P.M - k0 - NB;
+    if (R <= 0 || r0 >= R) return;  // no next panel, or no such rows
+    rbf_update_tile<NB, NB>(W, P, blockIdx.y, panel, r0, k0 + NB, min(k0 + 2 * NB, P.M), rbf_smem);
+  } else {
+    if (static_cast<int>(blockIdx.x) < W.n_planes) {
+      rbf_factor_panel<NB>(W, W.planes[blockIdx.x], panel + 1, rbf_smem);
+      return;
+    }
+    int t = blockIdx.x - W.n_planes;
+    const int ct = t % col_tiles;
+    t /= col_tiles;
+    const int rt = t % row_tiles, p = t / row_tiles;
+    const RbfPlane P = W.planes[p];
+    const int k0 = panel * NB;
+    if (k0 >= P.M) return;
+    const int R = P.M - k0 - min(NB, P.M - k0);
+    const int r0 = rt * kRbfTileR, c0 = min(k0 + 2 * NB, P.M) + ct * TC;
+    // (the first row tile also runs without active rows: it stores U)
+    if ((r0 >= R && rt > 0) || c0 > P.M) return;
+    rbf_update_tile<NB, TC>(W, P, p, panel, r0, c0, P.M + 1, rbf_smem);
+  }
+}
+
+// Back substitution, one block per plane, from the last rows up in blocks of
+// 32: one warp solves the 32 x 32 triangle (a lane per row, quotients by
+// markstein_div with the 32 reciprocals formed together), then every row above
+// subtracts the block's 32 columns, one thread per row.
+__global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_constant__ RbfWork W) {
+  extern __shared__ __align__(16) double rbf_smem[];
+  const RbfPlane P = W.planes[blockIdx.x];
+  const int M = P.M, ld = M + 1;
+  const double *U = W.U + P.sys0;
+  double *y = rbf_smem;        // M
+  __shared__ double T[32][33];
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int k = tid; k < M; k += kRbfThreads) y[k] = U[static_cast<int64_t>(k) * ld + M];
+  for (int b1 = M; b1 > 0;) {
+    const int b0 = max(0, b1 - 32), nb = b1 - b0;
+    __syncthreads();
+    for (int e = tid; e < nb * nb; e += kRbfThreads) {
+      const int i = e / nb, c = e % nb;
+      T[i][c] = U[static_cast<int64_t>(b0 + i) * ld + b0 + c];
+    }
+    __syncthreads();
+    if (tid < 32) {
+      const double d = lane < nb ? T[lane][lane] : 1.0;
+      const double r = 1.0 / d;
+      const bool plain = !(fabs(d) > 0x1p-500 && fabs(d) < 0x1p500);
+      double v = lane < nb ? y[b0 + lane] : 0.0;
+      for (int i = nb - 1; i >= 0; --i) {
+        const double q = plain ? v / d : markstein_div(v, d, r);
+        const double xi = __shfl_sync(kFull, q, i);
+        if (lane == i) v = xi;
+        else if (lane < i) v = fma(-T[lane][i], xi, v);
+      }
+      if (lane < nb) y[b0 + lane] = v;
+    }
+    __syncthreads();
+    for (int k = tid; k < b0; k += kRbfThreads) {
+      const double *row = U + static_cast<int64_t>(k) * ld + b0;
+      double v = y[k];
+#pragma unroll 8
+      for (int c = 0; c < nb; ++c) v = fma(-row[c], y[b0 + c], v);
+      y[k] = v;
+    }
+    b1 = b0;
+  }
+  __syncthreads();
+  for (int k = tid; k < M; k += kRbfThreads) W.x[P.row0 + k] = y[k];
+}
+
+// The interpolant at the query points, kRbfQ of them per thread, points and
+// weights staged through shared memory.  Ten FP64 instructions per (query,
+// point) pair (the squared distance 4, its square root 4, two products): the
+// FP64 pipe is the bound.
+constexpr int kRbfQ = 2;
+constexpr int kRbfEvalBlock = 128, kRbfEvalPts = 256;
+__global__ void __launch_bounds__(kRbfEvalBlock)
+rbf_eval_kernel(const __grid_constant__ RbfWork W, const double *__restrict__ pts,
+                const double *__restrict__ query, double *__restrict__ out) {
+  __shared__ double2 sxy[kRbfEvalPts];
+  __shared__ double sw[kRbfEvalPts];
+  const RbfPlane P = W.planes[blockIdx.y];
+  const int npt = P.M - 3;
+  const double *w = W.x + P.row0;
+  const double2 *xy = reinterpret_cast<const double2 *>(pts) + P.pts0;
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * (kRbfEvalBlock * kRbfQ); base < P.q;
+       base += static_cast<int64_t>(gridDim.x) * (kRbfEvalBlock * kRbfQ)) {
+    double s[kRbfQ], t[kRbfQ], acc[kRbfQ];
+#pragma unroll
+    for (int u = 0; u < kRbfQ; ++u) {
+      const int64_t j = min(base + u * kRbfEvalBlock + threadIdx.x, P.q - 1);
+      plane_coords(P.axis, query + 3 * (P.q0 + j), s[u], t[u]);
+      acc[u] = w[npt] + w[npt + 1] * s[u] + w[npt + 2] * t[u];
+    }
+    for (int i0 = 0; i0 < npt; i0 += kRbfEvalPts) {
+      const int n = min(kRbfEvalPts, npt - i0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < n; i += kRbfEvalBlock) {
+        sxy[i] = xy[i0 + i];
+        sw[i] = w[i0 + i];
+      }
+      __syncthreads();
+#pragma unroll 2
+      for (int i = 0; i < n; ++i) {
+        const double2 p = sxy[i];
+        const double wi = sw[i];
+#pragma unroll
+        for (int u = 0; u < kRbfQ; ++u) {
+          const double ds = s[u] - p.x, dt = t[u] - p.y;
+          const double r2 = ds * ds + dt * dt;
+          acc[u] = fma(wi, r2 * sqrt_r2(r2), acc[u]);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kRbfQ; ++u) {
+      const int64_t j = base + u * kRbfEvalBlock + threadIdx.x;
+      if (j < P.q) out[P.q0 + j] = acc[u];
+    }
+  }
+}
+
+// The launches of the elimination for panel width NB.
+template <int NB>
+static pdd_status rbf_launch(pdd_ctx *ctx, const RbfWork &W, int Mmax) {
+  // a panel of Mmax rows, or an update tile's pivot columns and multipliers
+  const size_t tile = (static_cast<size_t>(NB) * 32 + kRbfTileR * (NB + 1)) * sizeof(double);
+  const size_t panel_smem = std::max(tile, static_cast<size_t>(Mmax) * NB * sizeof(double));
+  auto *first = rbf_step_kernel<NB, kFirst>;
+  auto *next = rbf_step_kernel<NB, kNext>;
+  auto *rest = rbf_step_kernel<NB, kRest>;
+  const int attr = static_cast<int>(panel_smem);
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, attr));
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, attr));
+  const int panels = (Mmax + NB - 1) / NB;
+  const unsigned np = static_cast<unsigned>(W.n_planes);
+  first<<<np, kRbfThreads, panel_smem, ctx->stream>>>(W, 0, 0, 0);
+  for (int p = 0; p < panels; ++p) {
+    const int left = Mmax - (p + 1) * NB;  // active rows of the largest plane after this panel
+    const int rt = std::max(1, (left + kRbfTileR - 1) / kRbfTileR);
+    if (left > 0) next<<<dim3(static_cast<unsigned>(rt), np), kRbfThreads, tile, ctx->stream>>>(W, p, 0, 0);
+    // columns behind the next panel, the right-hand side included (planes with
+    // smaller systems have fewer)
+    const int ct = (std::max(0, left - NB) + 1 + 31) / 32;
+    // the block's shared memory: the next panel of the largest plane
+    const size_t sm = std::max(tile, static_cast<size_t>(std::max(left, 0)) * NB * sizeof(double));
+    rest<<<np * (1u + static_cast<unsigned>(rt * ct)), kRbfThreads, sm, ctx->stream>>>(W, p, rt, ct);
+    PDD_CUDA_TRY(ctx, cudaGetLastError());
+  }
+  return PDD_OK;
+}
+
+pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *h_axis,
+                                 const double *h_pos, const int64_t *h_node_count,
+                                 const double *d_nodes, const double *d_vals, int32_t n_bnd,
+                                 const int64_t *h_query_count, const double *d_query,
+                                 double *d_out) {
+  if (ctx->prob.dim != 3 || ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED)
+    return fail(ctx, PDD_EINVAL, "interface interpolation on planes covers the 3-D family");
+  if (n_planes < 1 || n_planes > 64) return fail(ctx, PDD_EINVAL, "n_planes must be in [1, 64]");
+  if (!h_axis || !h_pos || !h_node_count || !h_query_count)
+    return fail(ctx, PDD_EINVAL, "null host array");
+  if (n_bnd < 1 || n_bnd > 1024) return fail(ctx, PDD_EINVAL, "n_bnd must be in [1, 1024]");
+  std::vector<RbfPlane> pl(static_cast<size_t>(n_planes));
+  int64_t node0 = 0, sys0 = 0, row0 = 0, pts0 = 0, q0 = 0;
+  int32_t Mmax = 0;
+  for (int p = 0; p < n_planes; ++p) {
+    if (h_axis[p] < 0 || h_axis[p] > 2) return fail(ctx, PDD_EINVAL, "axis must be 0, 1 or 2");
+    if (!(h_pos[p] > 0.0 && h_pos[p] < 1.0)) return fail(ctx, PDD_EINVAL, "plane outside (0, 1)");
+    if (h_node_count[p] < 0 || h_query_count[p] < 0) return fail(ctx, PDD_EINVAL, "negative count");
+    const int64_t M = h_node_count[p] + 4LL * n_bnd + 3;
+    if (M > kRbfMaxSystem) return fail(ctx, PDD_EINVAL, "plane %d: system of %lld unknowns above %lld",
+                                       p, static_cast<long long>(M), static_cast<long long>(kRbfMaxSystem));
+    RbfPlane &P = pl[p];
+    P.node0 = node0;
+    P.m = h_node_count[p];
+    P.sys0 = sys0;
+    P.row0 = row0;
+    P.pts0 = pts0;
+    P.q0 = q0;
+    P.q = h_query_count[p];
+    P.axis = h_axis[p];
+    P.M = static_cast<int32_t>(M);
+    P.pos = h_pos[p];
+    node0 += P.m;
+    sys0 += M * (M + 1);
+    row0 += M;
+    pts0 += M - 3;
+    q0 += P.q;
+    Mmax = std::max(Mmax, P.M);
+  }
+  if ((node0 > 0 && (!d_nodes || !d_vals)) || (q0 > 0 && (!d_query || !d_out)))
+    return fail(ctx, PDD_EINVAL, "null buffer");
+  if (q0 == 0) return PDD_OK;
+  PDD_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  // the widest panel whose rows fit in one block's shared memory (16 columns
+  // up to 1600 unknowns, 8 up to 3200, 4 up to the largest system)
+  const int NB = static_cast<size_t>(Mmax) * 16 * sizeof(double) <= kRbfPanelBytes ? 16
+               : static_cast<size_t>(Mmax) * 8 * sizeof(double) <= kRbfPanelBytes ? 8 : 4;
+  static_assert(kRbfMaxSystem * 4 * sizeof(double) <= kRbfPanelBytes, "panel of the largest system");
+  const size_t NP = static_cast<size_t>(n_planes);
+  size_t o = 256;  // the singular flag
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = align_up(o + bytes, 256);
+    return at;
+  };
+  const size_t off_pl = take(pl.size() * sizeof(RbfPlane));
+  const size_t off_pts = take(static_cast<size_t>(pts0) * 2 * sizeof(double));
+  const size_t off_pv = take(static_cast<size_t>(pts0) * sizeof(double));
+  const size_t off_A = take(static_cast<size_t>(sys0) * sizeof(double));
+  const size_t off_U = take(static_cast<size_t>(sys0) * sizeof(double));
+  const size_t off_x = take(static_cast<size_t>(row0) * sizeof(double));
+  size_t off_L[2], off_act[2], off_L11[2], off_piv[2];
+  for (int h = 0; h < 2; ++h) {
+    off_L[h] = take(static_cast<size_t>(row0) * NB * sizeof(double));
+    off_act[h] = take(static_cast<size_t>(row0) * sizeof(int32_t));
+    off_L11[h] = take(NP * NB * NB * sizeof(double));
+    off_piv[h] = take(NP * NB * sizeof(int32_t));
+  }
+  pdd_status st = ensure_scratch(ctx, o);
+  if (st != PDD_OK) return st;
+  char *base = static_cast<char *>(ctx->scratch);
+  auto *d_pl = reinterpret_cast<RbfPlane *>(base + off_pl);
+  double *pts = reinterpret_cast<double *>(base + off_pts);
+  double *pv = reinterpret_cast<double *>(base + off_pv);
+  RbfWork W;
+  W.planes = d_pl;
+  W.n_planes = n_planes;
+  W.A = reinterpret_cast<double *>(base + off_A);
+  W.U = reinterpret_cast<double *>(base + off_U);
+  W.x = reinterpret_cast<double *>(base + off_x);
+  for (int h = 0; h < 2; ++h) {
+    W.L[h] = reinterpret_cast<double *>(base + off_L[h]);
+    W.act[h] = reinterpret_cast<int32_t *>(base + off_act[h]);
+    W.L11[h] = reinterpret_cast<double *>(base + off_L11[h]);
+    W.piv[h] = reinterpret_cast<int32_t *>(base + off_piv[h]);
+  }
+  W.singular = reinterpret_cast<int *>(base);
+  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, 256, ctx->stream));
+  PDD_CUDA_TRY(ctx, cudaMemcpyAsync(d_pl, pl.data(), pl.size() * sizeof(RbfPlane),
+                                    cudaMemcpyHostToDevice, ctx->stream));
+  const dim3 g1(static_cast<unsigned>(std::min<int64_t>((Mmax + 255) / 256, 64)),
+                static_cast<unsigned>(n_planes));
+  rbf_points_kernel<EllipticManufactured><<<g1, 256, 0, ctx->stream>>>(
+      d_pl, n_planes, d_nodes, d_vals, n_bnd, ctx->mc, pts, pv);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  const dim3 g2(static_cast<unsigned>(std::min<int64_t>((int64_t(Mmax) * Mmax + 255) / 256, 4096)),
+                static_cast<unsigned>(n_planes));
+  rbf_assemble_kernel<<<g2, 256, 0, ctx->stream>>>(W, pts, pv);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  st = NB == 16 ? rbf_launch<16>(ctx, W, Mmax)
+     : NB == 8 ? rbf_launch<8>(ctx, W, Mmax)
+               : rbf_launch<4>(ctx, W, Mmax);
+  if (st != PDD_OK) return st;
+  const size_t bsm = static_cast<size_t>(Mmax) * sizeof(double);
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rbf_backsub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(bsm)));
+  rbf_backsub_kernel<<<static_cast<unsigned>(n_planes), kRbfThreads, bsm, ctx->stream>>>(W);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  int64_t qmax = 0;
+  for (const auto &P : pl) qmax = std::max(qmax, P.q);
+  constexpr int64_t kPer = kRbfEvalBlock * kRbfQ;
+  const dim3 g3(static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((qmax + kPer - 1) / kPer, 65535))),
+                static_cast<unsigned>(n_planes));
+  rbf_eval_kernel<<<g3, kRbfEvalBlock, 0, ctx->stream>>>(W, pts, d_query, d_out);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  int hs = 0;
+  PDD_CUDA_TRY(ctx, cudaMemcpyAsync(&hs, W.singular, sizeof hs, cudaMemcpyDeviceToHost, ctx->stream));
+  PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  if (hs) return fail(ctx, PDD_EINVAL, "singular interpolation system (coincident nodes?)");
+  return PDD_OK;
+}
+
+}  // namespace pdd

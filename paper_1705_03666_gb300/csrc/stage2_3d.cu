@@ -1,18 +1,8 @@
 // stage2_3d.cu -- stage two of PDD in three dimensions (Sec. 2.1, Fig. 2.2):
-// the interface interpolation that turns Monte Carlo node values on the
-// internal planes of the cube into Dirichlet data, and the independent
-// subdomain solves of the elliptic problem
+// the independent subdomain solves of the elliptic problem
 //   (1/2) sigma^2 Lap u + b . grad u + c u + f = 0   (Eq. 2.3 without time)
-// by 7-point second differences and central first differences.
-//
-// Interpolation (pdd_interface_interp): per plane, a radial basis function
-// interpolant with the cubic kernel |r|^3 and a linear polynomial term through
-// the plane's nodes and n_bnd points per edge of the plane's perimeter, where
-// the boundary data g are known.  The saddle-point system
-//   [Phi P; P^T 0] [w; c] = [v; 0],  Phi_ij = |x_i - x_j|^3,  P_i = (1, s_i, t_i)
-// is solved in FP64 by Gaussian elimination with partial pivoting, one block
-// per plane (the planes of one call in one launch), then evaluated at the
-// query points, one thread per point.
+// by 7-point second differences and central first differences (the interface
+// interpolation that feeds them is in rbf.cu).
 //
 // Subdomain solve (pdd_subdomain_solve with a 3-D grid): defect correction
 //   u <- u + P^{-1} (rhs - A u)
@@ -24,8 +14,6 @@
 // a subdomain (|b| / |grad| against the Laplacian's scale), so the error
 // contracts by roughly ten per iteration, down to the FP64 residual
 // tolerance.  A plain Jacobi sweep is kept as the reference method.
-#include <cooperative_groups.h>
-
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -34,337 +22,6 @@
 #include "models.cuh"
 
 namespace pdd {
-
-// ---------------------------------------------------------------------------
-// Interface interpolation on planes
-// ---------------------------------------------------------------------------
-constexpr int kRbfBlock = 1024;
-constexpr int64_t kRbfMaxSystem = 6144;  // unknowns per plane (weights + 3)
-
-struct RbfPlane {
-  int64_t node0, m;      // this plane's nodes: [node0, node0 + m) of the call's list
-  int64_t sys0;          // offset of its system (M x M matrix, then M right-hand side)
-  int64_t pts0;          // offset of its 2-D points (M - 3 of them) and values
-  int64_t q0, q;         // its query points
-  int32_t axis, M;       // plane normal axis; system size
-  double pos;
-};
-
-// The plane's two in-plane coordinates of a 3-D point.
-__device__ __forceinline__ void plane_coords(int axis, const double *x, double &s, double &t) {
-  s = x[axis == 0 ? 1 : 0];
-  t = x[axis == 2 ? 1 : 2];
-}
-
-// Interpolation points of every plane: its nodes, then n_bnd points per edge
-// of its perimeter (corners once) with the boundary data g.
-template <class Model>
-__global__ void rbf_points_kernel(const RbfPlane *planes, int32_t n_planes, const double *nodes,
-                                  const double *vals, int32_t n_bnd, ModelConst mc, double *pts,
-                                  double *pv) {
-  const int p = blockIdx.y;
-  if (p >= n_planes) return;
-  const RbfPlane P = planes[p];
-  const int64_t npt = P.M - 3;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < npt;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    double s, t, v;
-    if (i < P.m) {
-      plane_coords(P.axis, nodes + 3 * (P.node0 + i), s, t);
-      v = vals[P.node0 + i];
-    } else {
-      // perimeter of the unit square in (s, t): edge e, point k of n_bnd
-      const int64_t b = i - P.m;
-      const int e = static_cast<int>(b / n_bnd);
-      const double u = static_cast<double>(b % n_bnd) / n_bnd;
-      s = e == 0 ? u : (e == 1 ? 1.0 : (e == 2 ? 1.0 - u : 0.0));
-      t = e == 0 ? 0.0 : (e == 1 ? u : (e == 2 ? 1.0 : 1.0 - u));
-      double x[3];
-      x[P.axis] = P.pos;
-      x[P.axis == 0 ? 1 : 0] = s;
-      x[P.axis == 2 ? 1 : 2] = t;
-      v = Model::template g<double>(mc, x);
-    }
-    pts[2 * (P.pts0 + i)] = s;
-    pts[2 * (P.pts0 + i) + 1] = t;
-    pv[P.pts0 + i] = v;
-  }
-}
-
-__global__ void rbf_assemble_kernel(const RbfPlane *planes, int32_t n_planes, const double *pts,
-                                    const double *pv, double *sys) {
-  const int p = blockIdx.y;
-  if (p >= n_planes) return;
-  const RbfPlane P = planes[p];
-  const int64_t M = P.M, npt = M - 3;
-  double *A = sys + P.sys0, *rhs = sys + P.sys0 + M * M;
-  const double *xy = pts + 2 * P.pts0;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < M * M;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t i = e / M, j = e % M;
-    double a;
-    if (i < npt && j < npt) {
-      const double ds = xy[2 * i] - xy[2 * j], dt = xy[2 * i + 1] - xy[2 * j + 1];
-      const double r2 = ds * ds + dt * dt;
-      a = r2 * sqrt(r2);
-    } else if (i < npt) {
-      a = j == npt ? 1.0 : xy[2 * i + (j - npt - 1)];
-    } else if (j < npt) {
-      a = i == npt ? 1.0 : xy[2 * j + (i - npt - 1)];
-    } else {
-      a = 0.0;
-    }
-    A[e] = a;
-    if (j == 0) rhs[i] = i < npt ? pv[P.pts0 + i] : 0.0;
-  }
-}
-
-// Gaussian elimination with partial pivoting and back substitution, one
-// thread-block cluster of kRbfCluster blocks per plane (the systems are
-// dense FP64 and GB300's FP64 rate is per SM, so a plane's elimination is
-// spread over several SMs).  Rows are not moved: block r of the cluster owns
-// rows i = r (mod kRbfCluster) and keeps its rows' "already a pivot" flags;
-// step k takes as pivot the unused row with the largest |A[i][k]| (lowest
-// index on ties), every block reads that row, and each block eliminates
-// column k from its own unused rows.  One cluster barrier per step: the
-// blocks' pivot candidates sit in double-buffered shared slots read across
-// the cluster, and a block only writes its own rows, which no other block
-// reads before the next barrier (the pivot row is read after it).  Then the
-// first block back-substitutes in pivot order.  On return rhs holds [w; c].
-// A zero pivot sets *singular.
-constexpr int kRbfCluster = 8;
-
-__global__ void __cluster_dims__(kRbfCluster, 1, 1) __launch_bounds__(kRbfBlock)
-rbf_solve_kernel(const RbfPlane *planes, int32_t n_planes, double *sys, int *singular) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int p = blockIdx.x / kRbfCluster;
-  const int r = static_cast<int>(cluster.block_rank());
-  if (p >= n_planes) return;  // whole clusters: every block of it returns
-  const int64_t M = planes[p].M;
-  double *A = sys + planes[p].sys0, *b = A + M * M;
-  // dynamic shared memory: the pivot row (M doubles, with its right-hand
-  // side last), then (first block) the solution and the pivot order, then
-  // the used flags of this block's rows
-  extern __shared__ double dsm[];
-  double *rowk = dsm;                                   // M + 1
-  double *x = rowk + M + 1;                             // M (block 0)
-  int32_t *perm = reinterpret_cast<int32_t *>(x + M);  // M (block 0)
-  unsigned char *used = reinterpret_cast<unsigned char *>(perm + M);  // M / kRbfCluster + 1
-  __shared__ double cand_v[2];
-  __shared__ int64_t cand_i[2];
-  __shared__ double red_v[kRbfBlock / 32];
-  __shared__ int64_t red_i[kRbfBlock / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int64_t nrow = (M - r + kRbfCluster - 1) / kRbfCluster;  // rows r, r + C, ...
-  __shared__ int64_t steps;  // elimination steps completed (M unless a pivot was missing)
-  for (int64_t t = tid; t < nrow; t += blockDim.x) used[t] = 0;
-  if (tid == 0) steps = M;
-  __syncthreads();
-  for (int64_t k = 0; k < M; ++k) {
-    const int slot = static_cast<int>(k & 1);
-    // this block's candidate: the largest |A[i][k]| over its unused rows
-    double best = -1.0;
-    int64_t bi = M;
-    for (int64_t t = tid; t < nrow; t += blockDim.x) {
-      if (used[t]) continue;
-      const int64_t i = r + t * kRbfCluster;
-      const double v = fabs(A[i * M + k]);
-      if (v > best || (v == best && i < bi)) { best = v; bi = i; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(kFull, best, o);
-      const int64_t oi = __shfl_xor_sync(kFull, bi, o);
-      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-    }
-    if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      double bv = red_v[0];
-      int64_t bj = red_i[0];
-      for (int w = 1; w < nw; ++w)
-        if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bj)) { bv = red_v[w]; bj = red_i[w]; }
-      cand_v[slot] = bv;
-      cand_i[slot] = bj;
-    }
-    // the candidates of step k, and every block's rows as updated in step
-    // k - 1, are visible across the cluster after this barrier
-    cluster.sync();
-    __shared__ int64_t piv;
-    if (tid == 0) {
-      double bv = -1.0;
-      int64_t bj = M;
-      for (int q = 0; q < kRbfCluster; ++q) {
-        const double v = *cluster.map_shared_rank(&cand_v[slot], q);
-        const int64_t ii = *cluster.map_shared_rank(&cand_i[slot], q);
-        if (v > bv || (v == bv && ii < bj)) { bv = v; bj = ii; }
-      }
-      piv = bj;
-      if (r == 0) {
-        perm[k] = static_cast<int32_t>(bj);
-        if (!(bv > 0.0)) *singular = 1;
-      }
-      if (bj < M && bj % kRbfCluster == r) used[bj / kRbfCluster] = 1;
-    }
-    __syncthreads();
-    const int64_t pr = piv;
-    if (pr >= M) {  // no unused row left (singular; flagged above)
-      if (tid == 0) steps = k;
-      break;
-    }
-    // the pivot row (columns k .. M - 1) and its right-hand side, read
-    // through L2: its owner wrote it in an earlier step
-    for (int64_t j = k + tid; j < M; j += blockDim.x) rowk[j] = __ldcg(A + pr * M + j);
-    if (tid == 0) rowk[M] = __ldcg(b + pr);
-    __syncthreads();
-    const double akk = rowk[k], bk = rowk[M];
-    // this block's unused rows: multiplier, then the row update (a warp per row)
-    for (int64_t t = warp; t < nrow; t += nw) {
-      if (used[t]) continue;
-      const int64_t i = r + t * kRbfCluster;
-      const double l = A[i * M + k] / akk;
-      __syncwarp();  // every lane has read A[i][k] before lane 0 clears it
-      for (int64_t j = k + 1 + lane; j < M; j += 32) A[i * M + j] = fma(-l, rowk[j], A[i * M + j]);
-      if (lane == 0) {
-        A[i * M + k] = 0.0;
-        b[i] = fma(-l, bk, b[i]);
-      }
-    }
-  }
-  // every row's final state is written before the first block reads it
-  cluster.sync();
-  if (r != 0) return;
-  if (steps < M) {  // incomplete elimination: no solution
-    for (int64_t k = tid; k < M; k += blockDim.x) b[k] = static_cast<double>(NAN);
-    return;
-  }
-  // back substitution in pivot order: x_k = (b_pk - sum_{j>k} A_pk,j x_j) / A_pk,k
-  for (int64_t k = M - 1; k >= 0; --k) {
-    const int64_t pk = perm[k];
-    double acc = 0.0;
-    for (int64_t j = k + 1 + tid; j < M; j += blockDim.x) acc = fma(__ldcg(A + pk * M + j), x[j], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-    if (lane == 0) red_v[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-      for (int w = 0; w < nw; ++w) s += red_v[w];
-      x[k] = (__ldcg(b + pk) - s) / __ldcg(A + pk * M + k);
-    }
-    __syncthreads();
-  }
-  for (int64_t k = tid; k < M; k += blockDim.x) b[k] = x[k];
-}
-
-__global__ void rbf_eval_kernel(const RbfPlane *planes, int32_t n_planes, const double *pts,
-                                const double *sys, const double *query, double *out) {
-  const int p = blockIdx.y;
-  if (p >= n_planes) return;
-  const RbfPlane P = planes[p];
-  const int64_t M = P.M, npt = M - 3;
-  const double *w = sys + P.sys0 + M * M;
-  const double *xy = pts + 2 * P.pts0;
-  for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < P.q;
-       j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    double s, t;
-    plane_coords(P.axis, query + 3 * (P.q0 + j), s, t);
-    double acc = w[npt] + w[npt + 1] * s + w[npt + 2] * t;
-    for (int64_t i = 0; i < npt; ++i) {
-      const double ds = s - xy[2 * i], dt = t - xy[2 * i + 1];
-      const double r2 = ds * ds + dt * dt;
-      acc = fma(w[i], r2 * sqrt(r2), acc);
-    }
-    out[P.q0 + j] = acc;
-  }
-}
-
-pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *h_axis,
-                                 const double *h_pos, const int64_t *h_node_count,
-                                 const double *d_nodes, const double *d_vals, int32_t n_bnd,
-                                 const int64_t *h_query_count, const double *d_query,
-                                 double *d_out) {
-  if (ctx->prob.dim != 3 || ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED)
-    return fail(ctx, PDD_EINVAL, "interface interpolation on planes covers the 3-D family");
-  if (n_planes < 1 || n_planes > 64) return fail(ctx, PDD_EINVAL, "n_planes must be in [1, 64]");
-  if (!h_axis || !h_pos || !h_node_count || !h_query_count)
-    return fail(ctx, PDD_EINVAL, "null host array");
-  if (n_bnd < 1 || n_bnd > 1024) return fail(ctx, PDD_EINVAL, "n_bnd must be in [1, 1024]");
-  std::vector<RbfPlane> pl(static_cast<size_t>(n_planes));
-  int64_t node0 = 0, sys0 = 0, pts0 = 0, q0 = 0;
-  int32_t Mmax = 0;
-  for (int p = 0; p < n_planes; ++p) {
-    if (h_axis[p] < 0 || h_axis[p] > 2) return fail(ctx, PDD_EINVAL, "axis must be 0, 1 or 2");
-    if (!(h_pos[p] > 0.0 && h_pos[p] < 1.0)) return fail(ctx, PDD_EINVAL, "plane outside (0, 1)");
-    if (h_node_count[p] < 0 || h_query_count[p] < 0) return fail(ctx, PDD_EINVAL, "negative count");
-    const int64_t M = h_node_count[p] + 4LL * n_bnd + 3;
-    if (M > kRbfMaxSystem) return fail(ctx, PDD_EINVAL, "plane %d: system of %lld unknowns above %lld",
-                                       p, static_cast<long long>(M), static_cast<long long>(kRbfMaxSystem));
-    RbfPlane &P = pl[p];
-    P.node0 = node0;
-    P.m = h_node_count[p];
-    P.sys0 = sys0;
-    P.pts0 = pts0;
-    P.q0 = q0;
-    P.q = h_query_count[p];
-    P.axis = h_axis[p];
-    P.M = static_cast<int32_t>(M);
-    P.pos = h_pos[p];
-    node0 += P.m;
-    sys0 += M * M + M;
-    pts0 += M - 3;
-    q0 += P.q;
-    Mmax = std::max(Mmax, P.M);
-  }
-  if ((node0 > 0 && (!d_nodes || !d_vals)) || (q0 > 0 && (!d_query || !d_out)))
-    return fail(ctx, PDD_EINVAL, "null buffer");
-  if (q0 == 0) return PDD_OK;
-  PDD_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  const size_t off_pl = 256;
-  const size_t off_pts = align_up(off_pl + pl.size() * sizeof(RbfPlane), 256);
-  const size_t off_pv = align_up(off_pts + static_cast<size_t>(pts0) * 2 * sizeof(double), 256);
-  const size_t off_sys = align_up(off_pv + static_cast<size_t>(pts0) * sizeof(double), 256);
-  const size_t bytes = align_up(off_sys + static_cast<size_t>(sys0) * sizeof(double), 256);
-  pdd_status st = ensure_scratch(ctx, bytes);
-  if (st != PDD_OK) return st;
-  char *base = static_cast<char *>(ctx->scratch);
-  int *singular = reinterpret_cast<int *>(base);
-  auto *d_pl = reinterpret_cast<RbfPlane *>(base + off_pl);
-  double *pts = reinterpret_cast<double *>(base + off_pts);
-  double *pv = reinterpret_cast<double *>(base + off_pv);
-  double *sys = reinterpret_cast<double *>(base + off_sys);
-  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, 256, ctx->stream));
-  PDD_CUDA_TRY(ctx, cudaMemcpyAsync(d_pl, pl.data(), pl.size() * sizeof(RbfPlane),
-                                    cudaMemcpyHostToDevice, ctx->stream));
-  const dim3 g1(static_cast<unsigned>(std::min<int64_t>((Mmax + 255) / 256, 64)),
-                static_cast<unsigned>(n_planes));
-  rbf_points_kernel<EllipticManufactured><<<g1, 256, 0, ctx->stream>>>(
-      d_pl, n_planes, d_nodes, d_vals, n_bnd, ctx->mc, pts, pv);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
-  const dim3 g2(static_cast<unsigned>(std::min<int64_t>((int64_t(Mmax) * Mmax + 255) / 256, 4096)),
-                static_cast<unsigned>(n_planes));
-  rbf_assemble_kernel<<<g2, 256, 0, ctx->stream>>>(d_pl, n_planes, pts, pv, sys);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
-  // pivot row + solution (doubles), pivot order (int32), used flags (bytes)
-  const size_t smem = static_cast<size_t>(2 * Mmax + 1) * sizeof(double) +
-                      static_cast<size_t>(Mmax) * sizeof(int32_t) +
-                      static_cast<size_t>(Mmax / kRbfCluster + 8);
-  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rbf_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
-  rbf_solve_kernel<<<static_cast<unsigned>(n_planes) * kRbfCluster, kRbfBlock, smem, ctx->stream>>>(
-      d_pl, n_planes, sys, singular);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
-  int64_t qmax = 0;
-  for (const auto &P : pl) qmax = std::max(qmax, P.q);
-  const dim3 g3(static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((qmax + 127) / 128, 4096))),
-                static_cast<unsigned>(n_planes));
-  rbf_eval_kernel<<<g3, 128, 0, ctx->stream>>>(d_pl, n_planes, pts, sys, d_query, d_out);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
-  int hs = 0;
-  PDD_CUDA_TRY(ctx, cudaMemcpyAsync(&hs, singular, sizeof hs, cudaMemcpyDeviceToHost, ctx->stream));
-  PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-  if (hs) return fail(ctx, PDD_EINVAL, "singular interpolation system (coincident nodes?)");
-  return PDD_OK;
-}
 
 // ---------------------------------------------------------------------------
 // Subdomain solves on 3-D boxes.  The subdomains of stage two are independent

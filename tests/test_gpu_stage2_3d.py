@@ -224,3 +224,44 @@ def test_batch_rejections(api):
                                                    ctypes.byref(it), ctypes.byref(res), None,
                                                    None)
             assert st == _lib.PDD_EINVAL
+
+
+@pytest.mark.parametrize("sizes", [(7,), (16, 17), (31, 33, 48), (1600, 40), (1601,), (3201, 8)])
+def test_interface_interp_panel_edges(api, sizes):
+    """Systems at the edges of the elimination's panels (16, 8 and 4 columns
+    wide by size; remainders, planes of different sizes in one call): the
+    interpolant reproduces every node value to the residual of a backward
+    stable solve, 16 M 2^-53 max_i sum_j |A_ij| |w_j| with w from torch."""
+    prob = W.elliptic_manufactured()
+    rng = np.random.default_rng(sum(sizes))
+    planes, data = [], []
+    for p, M in enumerate(sizes):
+        m = M - 7                                  # 4 perimeter points (n_bnd = 1) and 3 terms
+        x = np.full((m, 3), 0.5)
+        o = [b for b in range(3) if b != p % 3]
+        x[:, o] = rng.uniform(0.01, 0.99, (m, 2))
+        v = rng.standard_normal(m)
+        planes.append((p % 3, 0.5, x, v))
+        data.append((x[:, o], v))
+    corners = np.array([[0, 0], [1, 0], [1, 1], [0, 1]], dtype=float)
+    queries = []
+    for (axis, pos, x, v) in planes:
+        q = np.full((len(x) + 4, 3), pos)
+        o = [b for b in range(3) if b != axis]
+        q[:, o] = np.concatenate([x[:, o], corners])
+        queries.append(q)
+    with api.Context(prob) as ctx:
+        out = ctx.interface_interp(planes, queries, n_bnd=1)
+    for (axis, pos, _, _), (xy, v), q, got in zip(planes, data, queries, out):
+        pts = torch.from_numpy(np.concatenate([xy, corners])).cuda()
+        # (sin(pi x) sin(pi y) e^z is exactly 0 at these corners)
+        val = torch.from_numpy(np.concatenate([v, np.zeros(4)])).cuda()
+        n = len(pts)
+        A = torch.zeros(n + 3, n + 3, dtype=torch.float64, device="cuda")
+        A[:n, :n] = torch.cdist(pts, pts, compute_mode="donot_use_mm_for_euclid_dist") ** 3
+        A[:n, n], A[:n, n + 1:], A[n, :n], A[n + 1:, :n] = 1.0, pts, 1.0, pts.T
+        w = torch.linalg.solve(A, torch.cat([val, val.new_zeros(3)]))
+        bound = 16 * (n + 3) * 2.0 ** -53 * float((A.abs() @ w.abs()).max())
+        err = float((got - val).abs().max())
+        print(f"M = {n + 3}: node residual {err:.1e}, bound {bound:.1e}")
+        assert err <= bound
