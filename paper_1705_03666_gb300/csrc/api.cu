@@ -367,6 +367,9 @@ void pdd_destroy(pdd_ctx *ctx) {
   cudaStreamSynchronize(ctx->stream);
   if (ctx->scratch) cudaFree(ctx->scratch);
   if (ctx->aux) cudaFree(ctx->aux);
+  if (ctx->watch) cudaFreeHost(ctx->watch);
+  for (auto &ev : ctx->watch_ev)
+    if (ev) cudaEventDestroy(ev);
   if (ctx->batch_graph) cudaGraphExecDestroy(ctx->batch_graph);
   for (int k = 0; k < 3; ++k) {
     if (ctx->batch_side[k]) cudaStreamDestroy(ctx->batch_side[k]);

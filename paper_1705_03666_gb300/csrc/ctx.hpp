@@ -53,6 +53,10 @@ struct pdd_ctx {
   cudaStream_t batch_side[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t batch_fork = nullptr;
   cudaEvent_t batch_join[3] = {nullptr, nullptr, nullptr};
+  // progress of a device-side loop: two pinned words and their events (a
+  // loop's host side reads one behind); created on first use
+  int32_t *watch = nullptr;
+  cudaEvent_t watch_ev[2] = {nullptr, nullptr};
   // kernel timing (pdd_profile): event pairs recorded around path launches
   bool profiling = false;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_events;
@@ -139,6 +143,16 @@ inline pdd_status ensure_aux(pdd_ctx *ctx, size_t bytes) {
     return fail(ctx, PDD_ENOMEM, "cudaMalloc(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
   }
   ctx->aux_bytes = bytes;
+  return PDD_OK;
+}
+
+// The pinned progress words and their events.
+inline pdd_status ensure_watch(pdd_ctx *ctx) {
+  for (auto &ev : ctx->watch_ev)
+    if (!ev) PDD_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  if (!ctx->watch)
+    PDD_CUDA_TRY(ctx, cudaHostAlloc(reinterpret_cast<void **>(&ctx->watch), 2 * sizeof(int32_t),
+                                    cudaHostAllocDefault));
   return PDD_OK;
 }
 

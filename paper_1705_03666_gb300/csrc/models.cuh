@@ -74,6 +74,31 @@ struct EllipticManufactured {
   __device__ __forceinline__ static R g(const ModelConst &, const R *x) {
     return m_sinpi(x[0]) * m_sinpi(x[1]) * m_exp(x[2]);
   }
+  // Grids: the FP64 functions of one coordinate (x, y: sin and cos of pi x;
+  // z: e^z in s), and b, f and g from them.
+  struct AxisTable {
+    double s, c;
+  };
+  __device__ __forceinline__ static AxisTable axis_table(int axis, double x) {
+    AxisTable t{0.0, 0.0};
+    if (axis == 2) t.s = exp(x);
+    else sincospi(x, &t.s, &t.c);
+    return t;
+  }
+  __device__ __forceinline__ static void coeffs_tab(const AxisTable &tx, const AxisTable &ty,
+                                                    const AxisTable &tz, double *b, double &f) {
+    const double syz = ty.s * tz.s;
+    b[0] = ty.s * ty.c;
+    b[1] = 0.5 - tx.s * tx.s;
+    b[2] = 0.0;
+    constexpr double kPi = 3.14159265358979323846;
+    constexpr double a_u = 0.5 * (1.0 - 2.0 * kPi * kPi) - 1.0;
+    f = -(a_u * tx.s * syz + kPi * (b[0] * tx.c * syz + b[1] * tx.s * ty.c * tz.s));
+  }
+  __device__ __forceinline__ static double g_tab(const AxisTable &tx, const AxisTable &ty,
+                                                 const AxisTable &tz) {
+    return tx.s * ty.s * tz.s;
+  }
 };
 
 // ---------------------------------------------------------------------------

@@ -14,6 +14,21 @@
 // a subdomain (|b| / |grad| against the Laplacian's scale), so the error
 // contracts by roughly ten per iteration, down to the FP64 residual
 // tolerance.  A plain Jacobi sweep is kept as the reference method.
+//
+// A correction is four launches: the residual (its last block per box forms
+// the norm and decides whether the box goes on, so the host only looks one
+// correction behind), the forward y and x passes of each z plane, the z pass
+// with the eigenvalues and its inverse for 32 columns at a time, and the
+// inverse y and x passes with the update.  What bounds it is the FP64 pipe
+// (1/64 rate: the residual takes 14 FP64 instructions per point), then launch
+// gaps; the transforms run out of shared memory.  FP64 work that does not
+// change between corrections (drift over 2h, the eigenvalue factors) is formed
+// once per call.  Measured on the 64 boxes of 33^3 points of the 4 x 4 x 4 split
+// (eight residuals, seven corrections; device time): residuals 2.27 -> 0.80 ms,
+// transforms 3.70 -> 0.55 ms (one output per thread with two shared loads per
+// FMA, and the residual rescaled in FP64 for each of a row's 31 products,
+// before), eigenvalues 1.45 ms -> 0.01 ms, and no host round trip per
+// correction; the call 8.3 -> 1.9 ms.
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -52,37 +67,43 @@ __device__ __forceinline__ int64_t box3_np(const Box3 &B) {
   return static_cast<int64_t>(B.P[0]) * B.P[1] * B.P[2];
 }
 
-// Dirichlet data and coefficients: boundary layer of u from the faces (a
-// point on a face without interface data -- the physical boundary -- takes g;
-// otherwise the interface face of lowest index), interior u = 0, and per
-// interior point b, c and f of the family.
-template <class Model>
-__global__ void box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *u,
-                                  double *coef) {
+// Dirichlet data and coefficients, one block per z plane and box: boundary
+// layer of u from the faces (a point on a face without interface data -- the
+// physical boundary -- takes g; otherwise the interface face of lowest index),
+// interior u = 0, and per interior point b and f of the family.  The family's
+// functions of one coordinate are tabulated per block (a few dozen FP64
+// sines and exponentials in place of three per point: 460 -> 45 us for 64
+// boxes of 33^3 points).  kScaled: b_a / (2 h_a) is stored in place of b_a.
+template <class Model, bool kScaled>
+__global__ void __launch_bounds__(kBox3Block)
+box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *u, double *coef) {
   const Box3 B = boxes[blockIdx.y];
-  const int64_t total = box3_total(B);
+  const int k = blockIdx.x;
   const int64_t np = box3_np(B);
-  u += blockIdx.y * total;
+  u += blockIdx.y * box3_total(B) + static_cast<int64_t>(k) * B.n[0] * B.n[1];
   coef += blockIdx.y * 4 * np;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < total;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(e % B.n[0]);
-    const int j = static_cast<int>((e / B.n[0]) % B.n[1]);
-    const int k = static_cast<int>(e / (static_cast<int64_t>(B.n[0]) * B.n[1]));
+  __shared__ typename Model::AxisTable tab[3][kBox3MaxInterior + 2];
+  for (int e = threadIdx.x; e < B.n[0] + B.n[1] + 1; e += blockDim.x) {
+    const int a = e < B.n[0] ? 0 : (e < B.n[0] + B.n[1] ? 1 : 2);
+    const int i = a == 0 ? e : (a == 1 ? e - B.n[0] : k);
+    tab[a][a == 2 ? 0 : i] = Model::axis_table(a, B.lo[a] + B.h[a] * i);
+  }
+  __syncthreads();
+  const double d[3] = {0.5 / B.h[0], 0.5 / B.h[1], 0.5 / B.h[2]};
+  for (int e = threadIdx.x; e < B.n[0] * B.n[1]; e += blockDim.x) {
+    const int j = e / B.n[0], i = e - j * B.n[0];
     const int idx[3] = {i, j, k};
-    double x[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) x[a] = B.lo[a] + B.h[a] * idx[a];
     const bool interior = i > 0 && j > 0 && k > 0 && i < B.n[0] - 1 && j < B.n[1] - 1 &&
                           k < B.n[2] - 1;
     if (interior) {
       u[e] = 0.0;
       double b[3], f = 0.0;
-      Model::template coeffs<double>(mc, x, b, f);
+      Model::coeffs_tab(tab[0][i], tab[1][j], tab[2][0], b, f);
       const int64_t q = (static_cast<int64_t>(k - 1) * B.P[1] + (j - 1)) * B.P[0] + (i - 1);
-      coef[q] = b[0];
-      coef[np + q] = b[1];
-      coef[2 * np + q] = b[2];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (!kScaled || ((Model::kDriftAxes >> a) & 1u))  // (the residual skips axes without drift)
+          coef[a * np + q] = kScaled ? b[a] * d[a] : b[a];
       coef[3 * np + q] = f;
       continue;
     }
@@ -100,7 +121,7 @@ __global__ void box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double
     }
     double v;
     if (physical || fbest < 0) {
-      v = Model::template g<double>(mc, x);
+      v = Model::g_tab(tab[0][i], tab[1][j], tab[2][0]);
     } else {
       // face grid of face fbest: the two other axes, the higher one slow
       const int a = fbest >> 1;
@@ -111,160 +132,262 @@ __global__ void box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double
   }
 }
 
-// r = -f - A u at the interior points (FP64), and the block's sum of r^2
-// (part[box][block]).
+// Correction state of the boxes (device arrays, one entry per box, but
+// n_live): norm of the residual and of the first one, their ratio, the
+// corrections done, whether the box goes on, and the ticket of its blocks.
+struct Box3State {
+  double *rn, *r0, *res;
+  int64_t *iters;
+  int32_t *live, *ticket;
+  int32_t *n_live;
+};
+
+// r = -f - A u at the interior points (FP64), one block per z plane and box,
+// and the block's sum of r^2; the box's last block adds the planes' sums in a
+// fixed order, forms the norm and decides whether the box goes on (stopping
+// rule of correction `it`).
+template <unsigned kDriftAxes>
 __global__ void __launch_bounds__(kBox3Block)
-box3_residual_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, const double *u,
-                     const double *coef, double *r, double *part) {
-  if (!live[blockIdx.y]) return;
-  const Box3 B = boxes[blockIdx.y];
+box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, double s2, double c,
+                     const double *u, const double *coef, double *r, double *part, int64_t it,
+                     int64_t max_iter, double tol) {
+  const int box = blockIdx.y;
+  if (!st.live[box]) return;
+  const Box3 B = boxes[box];
   const int64_t np = box3_np(B);
-  u += blockIdx.y * box3_total(B);
-  coef += blockIdx.y * 4 * np;
-  r += blockIdx.y * np;
+  const int plane = B.P[0] * B.P[1];
+  const int64_t q0 = static_cast<int64_t>(blockIdx.x) * plane;
+  const int sy = B.n[0], sz = B.n[0] * B.n[1];
+  u += box * box3_total(B) + static_cast<int64_t>(blockIdx.x + 1) * sz;
+  coef += box * 4 * np + q0;
+  r += box * np + q0;
   const double w0 = 0.5 * s2 / (B.h[0] * B.h[0]), w1 = 0.5 * s2 / (B.h[1] * B.h[1]),
                w2 = 0.5 * s2 / (B.h[2] * B.h[2]);
-  const double d0 = 0.5 / B.h[0], d1 = 0.5 / B.h[1], d2 = 0.5 / B.h[2];
   const double diag = c - 2.0 * (w0 + w1 + w2);
   double acc = 0.0;
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < np;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(q % B.P[0]) + 1;
-    const int j = static_cast<int>((q / B.P[0]) % B.P[1]) + 1;
-    const int k = static_cast<int>(q / (static_cast<int64_t>(B.P[0]) * B.P[1])) + 1;
-    const int64_t e = box3_index(B, i, j, k);
-    const int64_t sy = B.n[0], sz = static_cast<int64_t>(B.n[0]) * B.n[1];
-    const double uc = u[e];
-    const double ux0 = u[e - 1], ux1 = u[e + 1], uy0 = u[e - sy], uy1 = u[e + sy],
-                 uz0 = u[e - sz], uz1 = u[e + sz];
-    double Au = diag * uc + w0 * (ux0 + ux1) + w1 * (uy0 + uy1) + w2 * (uz0 + uz1);
-    Au += coef[q] * d0 * (ux1 - ux0) + coef[np + q] * d1 * (uy1 - uy0) +
-          coef[2 * np + q] * d2 * (uz1 - uz0);
+  for (int q = threadIdx.x; q < plane; q += kBox3Block) {
+    const int j = q / B.P[0];
+    const double *v = u + (j + 1) * sy + (q - j * B.P[0] + 1);
+    const double ux0 = v[-1], ux1 = v[1], uy0 = v[-sy], uy1 = v[sy], uz0 = v[-sz], uz1 = v[sz];
+    double Au = diag * v[0] + w0 * (ux0 + ux1) + w1 * (uy0 + uy1) + w2 * (uz0 + uz1);
+    double drift = 0.0;
+    if (kDriftAxes & 1u) drift = coef[q] * (ux1 - ux0);
+    if (kDriftAxes & 2u) drift = fma(coef[np + q], uy1 - uy0, drift);
+    if (kDriftAxes & 4u) drift = fma(coef[2 * np + q], uz1 - uz0, drift);
+    Au += drift;
     const double rv = -coef[3 * np + q] - Au;
     r[q] = rv;
     acc = fma(rv, rv, acc);
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
   __shared__ double sh[kBox3Block / 32];
+  __shared__ bool last;
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < kBox3Block / 32; ++w) t += sh[w];
-    part[static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x] = t;
+    part[static_cast<int64_t>(box) * gridDim.x + blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(st.ticket + box, 1) == static_cast<int>(gridDim.x) - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  double t = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += 32)
+    t += __ldcg(part + static_cast<int64_t>(box) * gridDim.x + k);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+  if (threadIdx.x == 0) {
+    const double rn = sqrt(t);
+    if (it == 0) st.r0[box] = rn;
+    const double r0 = it == 0 ? rn : st.r0[box];
+    st.rn[box] = rn;
+    st.iters[box] = it;
+    st.res[box] = r0 > 0.0 ? rn / r0 : 0.0;
+    st.ticket[box] = 0;
+    if (rn <= tol * r0 || rn == 0.0 || it >= max_iter) {
+      st.live[box] = 0;
+      atomicSub(st.n_live, 1);
+    }
   }
 }
 
-// Per box: the sum of its block partials in block order (deterministic), as
-// a 2-norm (residual) or the largest (Jacobi change); one thread per box.
-template <bool kMax>
+// Jacobi: per box the largest of its block partials; one thread per box.
 __global__ void box3_combine_kernel(const double *part, int nblk, int nb, const int32_t *live,
                                     double *out) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb || !live[b]) return;
   double t = 0.0;
   for (int k = 0; k < nblk; ++k) {
-    const double v = part[static_cast<int64_t>(b) * nblk + k];
-    t = kMax ? fmax(t, v) : t + v;
+    t = fmax(t, part[static_cast<int64_t>(b) * nblk + k]);
   }
-  out[b] = kMax ? t : sqrt(t);
+  out[b] = t;
 }
+
+// Rows of the sine matrices and of the staged planes are padded to a multiple
+// of four floats, so that four consecutive entries are one 16-byte load.
+__host__ __device__ constexpr int box3_pad(int P) { return (P + 3) & ~3; }
 
 // The sine matrices S_a[k][j] = sin(pi (k+1)(j+1) / (P_a + 1)), binary32,
-// the argument reduced exactly in integers.
-__global__ void box3_sine_kernel(int P, float *S) {
-  const int64_t n = static_cast<int64_t>(P) * P;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t k = e / P + 1, j = e % P + 1;
-    const int64_t m = (k * j) % (2 * (P + 1));
-    S[e] = static_cast<float>(sinpi(static_cast<double>(m) / (P + 1)));
-  }
-}
-
-// out = S applied along axis AX of the P0 x P1 x P2 array of box blockIdx.y
-// (x fastest): out[.., k, ..] = sum_j S[k][j] in[.., j, ..].  The matrix is
-// staged in shared memory; threads of a warp take consecutive outputs, so
-// along axes 1 and 2 their reads are coalesced and along axis 0 they read the
-// same line.
-template <int AX>
-__global__ void __launch_bounds__(kBox3Block)
-box3_dst_kernel(int P0, int P1, int P2, const int32_t *live, const float *__restrict__ S,
-                const float *__restrict__ in, float *__restrict__ out,
-                const double *__restrict__ rnorm, const double *__restrict__ in64) {
-  if (!live[blockIdx.y]) return;
-  extern __shared__ float Ss[];
-  const int P = AX == 0 ? P0 : (AX == 1 ? P1 : P2);
-  for (int e = threadIdx.x; e < P * P; e += blockDim.x) Ss[e] = S[e];
-  __syncthreads();
-  const int64_t np = static_cast<int64_t>(P0) * P1 * P2;
-  const int64_t off = blockIdx.y * np;
-  const int64_t stride = AX == 0 ? 1 : (AX == 1 ? P0 : static_cast<int64_t>(P0) * P1);
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < np;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int kk = static_cast<int>((q / stride) % P);
-    const int64_t base = off + q - kk * stride;
-    const float *row = Ss + kk * P;
-    float acc = 0.f;
-    if (in64) {  // first pass: the FP64 residual scaled by 1 / |r|_2, then rounded
-      const double inv = 1.0 / rnorm[blockIdx.y];
-      for (int j = 0; j < P; ++j)
-        acc = fmaf(row[j], static_cast<float>(in64[base + j * stride] * inv), acc);
-    } else {
-      for (int j = 0; j < P; ++j) acc = fmaf(row[j], in[base + j * stride], acc);
-    }
-    out[off + q] = acc;
-  }
-}
-
-// cos(pi k / (P_a + 1)) - 1 for k = 1 .. P_a on each axis (cm1[a][k - 1]),
-// formed once per solve: the eigenvalue factors of the 1-D second difference.
-__global__ void box3_cos_kernel(int P0, int P1, int P2, double *cm1) {
+// rows padded with zeros, the argument reduced exactly in integers; blockIdx.y
+// is the axis.  Also the eigenvalue factors of the 1-D second differences,
+// cos(pi (k+1) / (P_a + 1)) - 1.
+struct Box3Sines {
+  float *S[3];
+  double *cm1[3];
+};
+__global__ void box3_sine_kernel(int P0, int P1, int P2, const __grid_constant__ Box3Sines T) {
   const int a = blockIdx.y;
-  const int P = a == 0 ? P0 : (a == 1 ? P1 : P2);
-  for (int k = threadIdx.x; k < P; k += blockDim.x)
-    cm1[a * kBox3MaxInterior + k] = cospi(static_cast<double>(k + 1) / (P + 1)) - 1.0;
+  const int P = a == 0 ? P0 : (a == 1 ? P1 : P2), ld = box3_pad(P);
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < P * ld; e += gridDim.x * blockDim.x) {
+    const int k = e / ld + 1, j = e % ld + 1;
+    const int m = (k * j) % (2 * (P + 1));
+    T.S[a][e] = j <= P ? static_cast<float>(sinpi(static_cast<double>(m) / (P + 1))) : 0.0f;
+    if (e < P) T.cm1[a][e] = cospi(static_cast<double>(e + 1) / (P + 1)) - 1.0;
+  }
 }
 
-// Division by the eigenvalues of (1/2) sigma^2 Lap_h + c in the sine basis,
-// lambda = sum_a (sigma^2 / h_a^2) (cos(pi k_a / (P_a + 1)) - 1) + c, and the
-// normalisation of the two transforms, 8 / prod_a (P_a + 1).
-__global__ void box3_eig_kernel(const Box3 *boxes, const int32_t *live, double s2, double c,
-                                const double *__restrict__ cm1, float *v) {
-  if (!live[blockIdx.y]) return;
+// Factors of the division by the eigenvalues of (1/2) sigma^2 Lap_h + c in the
+// sine basis, lambda = sum_a (sigma^2 / h_a^2) (cos(pi k_a / (P_a + 1)) - 1) +
+// c, with the normalisation of the two transforms: (8 / prod_a (P_a + 1)) /
+// lambda (FP64, formed once per call; one table for boxes of one mesh size).
+__global__ void box3_eig_kernel(const Box3 *boxes, const __grid_constant__ Box3Sines T, double s2,
+                                double c, double *fac) {
   const Box3 B = boxes[blockIdx.y];
-  const int64_t np = box3_np(B);
-  v += blockIdx.y * np;
+  const int plane = B.P[0] * B.P[1];
+  fac += blockIdx.y * box3_np(B) + static_cast<int64_t>(blockIdx.x) * plane;
   const double norm = 8.0 / ((B.P[0] + 1.0) * (B.P[1] + 1.0) * (B.P[2] + 1.0));
   const double e0 = s2 / (B.h[0] * B.h[0]), e1 = s2 / (B.h[1] * B.h[1]),
                e2 = s2 / (B.h[2] * B.h[2]);
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < np;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int k0 = static_cast<int>(q % B.P[0]);
-    const int k1 = static_cast<int>((q / B.P[0]) % B.P[1]);
-    const int k2 = static_cast<int>(q / (static_cast<int64_t>(B.P[0]) * B.P[1]));
-    const double lam = e0 * cm1[k0] + e1 * cm1[kBox3MaxInterior + k1] +
-                       e2 * cm1[2 * kBox3MaxInterior + k2] + c;
-    v[q] = static_cast<float>(static_cast<double>(v[q]) * (norm / lam));
+  for (int q = threadIdx.x; q < plane; q += blockDim.x) {
+    const int k1 = q / B.P[0], k0 = q - k1 * B.P[0];
+    fac[q] = norm / (e0 * T.cm1[0][k0] + e1 * T.cm1[1][k1] + e2 * T.cm1[2][blockIdx.x] + c);
   }
 }
 
-// u += (correction * |r|) at the interior points (undoing the scaling).
-__global__ void box3_update_kernel(const Box3 *boxes, const int32_t *live, const float *v,
-                                   const double *rnorm, double *u) {
-  if (!live[blockIdx.y]) return;
-  const Box3 B = boxes[blockIdx.y];
-  const int64_t np = box3_np(B);
-  v += blockIdx.y * np;
-  u += blockIdx.y * box3_total(B);
-  const double sc = rnorm[blockIdx.y];
-  for (int64_t q = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; q < np;
-       q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(q % B.P[0]) + 1;
-    const int j = static_cast<int>((q / B.P[0]) % B.P[1]) + 1;
-    const int k = static_cast<int>(q / (static_cast<int64_t>(B.P[0]) * B.P[1])) + 1;
-    u[box3_index(B, i, j, k)] += static_cast<double>(v[q]) * sc;
+// out[a][k] = sum_i Bc[i][a] V[i][k] (a < A, k < N, i < K ascending), the
+// block's warps sharing the output: a lane forms four consecutive a of one k
+// per turn (one 16-byte broadcast load, one load and four FMAs per i), and
+// passes them to put(a, k, v[4]) (entries at a + q >= A are padding).
+template <class Put>
+__device__ __forceinline__ void box3_apply(const float *Bc, int ldb, const float *V, int ldv, int K,
+                                           int A, int N, Put put) {
+  const int lane = threadIdx.x & 31, nag = (A + 3) / 4, nkc = (N + 31) / 32;
+  for (int t = threadIdx.x >> 5; t < nag * nkc; t += kBox3Block / 32) {
+    const int kc = t / nag, a = 4 * (t - kc * nag), k = kc * 32 + lane;
+    const float *b = Bc + a, *v = V + min(k, N - 1);
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < K; ++i) {
+      const float4 w = *reinterpret_cast<const float4 *>(b + i * ldb);
+      const float x = v[i * ldv];
+      s0 = fmaf(w.x, x, s0);
+      s1 = fmaf(w.y, x, s1);
+      s2 = fmaf(w.z, x, s2);
+      s3 = fmaf(w.w, x, s3);
+    }
+    if (k < N) {
+      const float s[4] = {s0, s1, s2, s3};
+      put(a, k, s);
+    }
   }
+}
+
+// Row length of the transposed plane: four more than the padded row, so that
+// the 16-byte stores of neighbouring lanes fall on different banks.
+__host__ __device__ constexpr int box3_pad_t(int P) { return box3_pad(P) + 4; }
+static size_t box3_plane_smem(int P0, int P1) {
+  const size_t l = static_cast<size_t>(P0) * box3_pad(P0) + static_cast<size_t>(P0) * box3_pad_t(P1) +
+                   static_cast<size_t>(P1) * P0;
+  return l * sizeof(float);
+}
+
+// The y and x passes of one z plane (blockIdx.x) of box blockIdx.y.  kInverse
+// = false: in is the FP64 residual, scaled by 1 / |r|_2 and rounded, and the
+// result goes to v.  kInverse = true: in place of the residual v, and the
+// result times |r|_2 is added to u.  The sine matrix along x sits in shared
+// memory; along y it is the same one when the box is as long, else read
+// through L1.
+template <bool kInverse>
+__global__ void __launch_bounds__(kBox3Block)
+box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *rn,
+                  const __grid_constant__ Box3Sines T, const double *r, float *v, double *u) {
+  const int box = blockIdx.y;
+  if (!live[box]) return;
+  extern __shared__ __align__(16) float bsm[];
+  const Box3 B = boxes[box];
+  const int P0 = B.P[0], P1 = B.P[1], plane = P0 * P1;
+  const int ld0 = box3_pad(P0), ldt = box3_pad_t(P1);
+  float *Sx = bsm;               // [P0][ld0]
+  float *Tt = Sx + P0 * ld0;     // [x][y]: after the y pass
+  float *Tn = Tt + P0 * ldt;     // [y][x]: the plane
+  const int64_t off = box * box3_np(B) + static_cast<int64_t>(blockIdx.x) * plane;
+  const double sc = kInverse ? rn[box] : 1.0 / rn[box];
+  for (int e = threadIdx.x; e < P0 * ld0; e += kBox3Block) Sx[e] = T.S[0][e];
+  for (int e = threadIdx.x; e < plane; e += kBox3Block)
+    Tn[e] = kInverse ? v[off + e] : static_cast<float>(r[off + e] * sc);
+  __syncthreads();
+  const float *Sy = P1 == P0 ? Sx : T.S[1];
+  box3_apply(Sy, box3_pad(P1), Tn, P0, P1, P1, P0, [&](int a, int k, const float *s) {
+    *reinterpret_cast<float4 *>(Tt + k * ldt + a) = make_float4(s[0], s[1], s[2], s[3]);
+  });
+  __syncthreads();
+  if constexpr (kInverse) {
+    double *up = u + box * box3_total(B) + (static_cast<int64_t>(blockIdx.x + 1) * B.n[1] + 1) * B.n[0] + 1;
+    box3_apply(Tt, ldt, Sx, ld0, P0, P1, P0, [&](int a, int k, const float *s) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (a + q < P1) {
+          double *p = up + static_cast<int64_t>(a + q) * B.n[0] + k;
+          *p = fma(static_cast<double>(s[q]), sc, *p);
+        }
+    });
+  } else {
+    float *vp = v + off;
+    box3_apply(Tt, ldt, Sx, ld0, P0, P1, P0, [&](int a, int k, const float *s) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (a + q < P1) vp[(a + q) * P0 + k] = s[q];
+    });
+  }
+}
+
+// The z pass of 32 columns (blockIdx.x), the division by the eigenvalues and
+// the inverse z pass, in place.
+constexpr int kBox3Cols = 32;
+__global__ void __launch_bounds__(kBox3Block)
+box3_z_kernel(int P0, int P1, int P2, const int32_t *live, const __grid_constant__ Box3Sines T,
+              const double *fac, int64_t fac_stride, float *v) {
+  const int box = blockIdx.y;
+  if (!live[box]) return;
+  extern __shared__ __align__(16) float bsm[];
+  const int ld = box3_pad(P2), plane = P0 * P1;
+  float *S = bsm;                    // [P2][ld]
+  float *V = S + P2 * ld;            // [P2][32]
+  float *H = V + P2 * kBox3Cols;     // [P2][32]
+  const int c0 = blockIdx.x * kBox3Cols, nc = min(kBox3Cols, plane - c0);
+  v += box * static_cast<int64_t>(plane) * P2 + c0;
+  fac += box * fac_stride + c0;
+  for (int e = threadIdx.x; e < P2 * ld; e += kBox3Block) S[e] = T.S[2][e];
+  for (int e = threadIdx.x; e < P2 * kBox3Cols; e += kBox3Block) {
+    const int z = e / kBox3Cols, c = e % kBox3Cols;
+    if (c < nc) V[e] = v[static_cast<int64_t>(z) * plane + c];
+  }
+  __syncthreads();
+  box3_apply(S, ld, V, kBox3Cols, P2, P2, nc, [&](int a, int k, const float *s) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (a + q < P2)
+        H[(a + q) * kBox3Cols + k] = static_cast<float>(
+            static_cast<double>(s[q]) * fac[static_cast<int64_t>(a + q) * plane + k]);
+  });
+  __syncthreads();
+  box3_apply(S, ld, H, kBox3Cols, P2, P2, nc, [&](int a, int k, const float *s) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (a + q < P2) v[static_cast<int64_t>(a + q) * plane + k] = s[q];
+  });
 }
 
 // One Jacobi sweep (the plain reference method): u' = (-f - offdiag(A) u) / diag,
@@ -371,23 +494,38 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   const int64_t np = static_cast<int64_t>(B0.P[0]) * B0.P[1] * B0.P[2];
   const size_t NB = static_cast<size_t>(nb);
   const int nblk = static_cast<int>(std::min<int64_t>((np + kBox3Block - 1) / kBox3Block, 1024));
+  const int ld[3] = {box3_pad(B0.P[0]), box3_pad(B0.P[1]), box3_pad(B0.P[2])};
+  // boxes of one mesh size share one table of eigenvalue factors
+  bool one_h = true;
+  for (const Box3 &B : boxes)
+    for (int a = 0; a < 3; ++a) one_h = one_h && B.h[a] == B0.h[a];
   size_t o = 0;
   auto take = [&](size_t bytes) {
     const size_t at = o;
     o = align_up(o + bytes, 256);
     return at;
   };
+  // the boxes' state first: one copy back at the end
+  const size_t off_it = take(NB * sizeof(int64_t));
+  const size_t off_res = take(NB * sizeof(double));
+  const size_t state_bytes = o;
   const size_t off_rn = take(NB * sizeof(double));
+  const size_t off_r0 = take(NB * sizeof(double));
   const size_t off_live = take(NB * sizeof(int32_t));
+  const size_t off_ticket = take(NB * sizeof(int32_t));
+  const size_t off_nlive = take(sizeof(int32_t));
   const size_t off_box = take(NB * sizeof(Box3));
   const size_t off_coef = take(NB * 4 * np * sizeof(double));
-  const size_t off_r = take(NB * np * sizeof(double));
-  const size_t off_part = take(NB * nblk * sizeof(double));
+  const size_t off_part = take(NB * std::max(nblk, B0.P[2]) * sizeof(double));
   const size_t off_un = take(jacobi ? NB * total * sizeof(double) : 0);
-  const size_t off_v0 = take(NB * np * sizeof(float));
-  const size_t off_v1 = take(NB * np * sizeof(float));
-  const size_t off_S = take(3 * kBox3MaxInterior * kBox3MaxInterior * sizeof(float));
-  const size_t off_cm1 = take(3 * kBox3MaxInterior * sizeof(double));
+  const size_t off_r = take(jacobi ? 0 : NB * np * sizeof(double));
+  const size_t off_fac = take(jacobi ? 0 : (one_h ? 1 : NB) * np * sizeof(double));
+  const size_t off_v = take(jacobi ? 0 : NB * np * sizeof(float));
+  size_t off_S[3], off_cm1[3];
+  for (int a = 0; a < 3; ++a) {
+    off_S[a] = take(static_cast<size_t>(B0.P[a]) * ld[a] * sizeof(float));
+    off_cm1[a] = take(static_cast<size_t>(B0.P[a]) * sizeof(double));
+  }
   pdd_status st = ensure_scratch(ctx, o);
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
@@ -395,27 +533,25 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   int32_t *live = reinterpret_cast<int32_t *>(base + off_live);
   Box3 *d_boxes = reinterpret_cast<Box3 *>(base + off_box);
   double *coef = reinterpret_cast<double *>(base + off_coef);
-  double *r = reinterpret_cast<double *>(base + off_r);
   double *part = reinterpret_cast<double *>(base + off_part);
   double *un = reinterpret_cast<double *>(base + off_un);
-  float *v0 = reinterpret_cast<float *>(base + off_v0), *v1 = reinterpret_cast<float *>(base + off_v1);
-  float *S[3];
-  for (int a = 0; a < 3; ++a)
-    S[a] = reinterpret_cast<float *>(base + off_S) + a * kBox3MaxInterior * kBox3MaxInterior;
-  double *cm1 = reinterpret_cast<double *>(base + off_cm1);
 
   // host state of the correction loop (copied to and from the device
   // synchronously, so these buffers outlive every copy)
   std::vector<int32_t> h_live(NB, 1);
-  std::vector<double> h_rn(NB, 0.0), h_r0(NB, -1.0), h_res(NB, 0.0);
+  std::vector<double> h_rn(NB, 0.0), h_res(NB, 0.0);
   std::vector<int64_t> h_it(NB, 0);
   PDD_CUDA_TRY(ctx, cudaMemcpyAsync(d_boxes, boxes.data(), NB * sizeof(Box3),
                                     cudaMemcpyHostToDevice, ctx->stream));
   PDD_CUDA_TRY(ctx, cudaMemcpyAsync(live, h_live.data(), NB * sizeof(int32_t),
                                     cudaMemcpyHostToDevice, ctx->stream));
-  const unsigned gset = static_cast<unsigned>(std::min<int64_t>((total + 255) / 256, 4096));
-  box3_setup_kernel<EllipticManufactured><<<dim3(gset, nb), 256, 0, ctx->stream>>>(
-      d_boxes, ctx->mc, d_face, d_u, coef);
+  const dim3 gset(static_cast<unsigned>(B0.n[2]), nb);
+  if (jacobi)
+    box3_setup_kernel<EllipticManufactured, false><<<gset, kBox3Block, 0, ctx->stream>>>(
+        d_boxes, ctx->mc, d_face, d_u, coef);
+  else
+    box3_setup_kernel<EllipticManufactured, true><<<gset, kBox3Block, 0, ctx->stream>>>(
+        d_boxes, ctx->mc, d_face, d_u, coef);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   const double s2 = ctx->prob.sigma * ctx->prob.sigma;
   const double c = constant_kill(ctx->prob.kind);
@@ -449,7 +585,7 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
       for (size_t b = 0; b < NB; ++b)
         if (h_live[b]) h_it[b] = it;
       if (it % 16 == 0 || it == S0.max_iter) {
-        box3_combine_kernel<true><<<gcomb, 128, 0, ctx->stream>>>(part, nblk, nb, live, rn);
+        box3_combine_kernel<<<gcomb, 128, 0, ctx->stream>>>(part, nblk, nb, live, rn);
         PDD_CUDA_TRY(ctx, cudaGetLastError());
         st = read_measures();
         if (st != PDD_OK) return st;
@@ -471,54 +607,68 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
         PDD_CUDA_TRY(ctx, cudaMemcpyAsync(d_u + b * total, un + b * total, total * sizeof(double),
                                           cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
+    st = ensure_watch(ctx);
+    if (st != PDD_OK) return st;
+    Box3Sines T;
     for (int a = 0; a < 3; ++a) {
-      box3_sine_kernel<<<static_cast<unsigned>((B0.P[a] * B0.P[a] + 255) / 256), 256, 0, ctx->stream>>>(
-          B0.P[a], S[a]);
-      PDD_CUDA_TRY(ctx, cudaGetLastError());
+      T.S[a] = reinterpret_cast<float *>(base + off_S[a]);
+      T.cm1[a] = reinterpret_cast<double *>(base + off_cm1[a]);
     }
-    box3_cos_kernel<<<dim3(1, 3), 128, 0, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], cm1);
+    Box3State S;
+    S.rn = rn;
+    S.r0 = reinterpret_cast<double *>(base + off_r0);
+    S.res = reinterpret_cast<double *>(base + off_res);
+    S.iters = reinterpret_cast<int64_t *>(base + off_it);
+    S.live = live;
+    S.ticket = reinterpret_cast<int32_t *>(base + off_ticket);
+    S.n_live = reinterpret_cast<int32_t *>(base + off_nlive);
+    double *r = reinterpret_cast<double *>(base + off_r);
+    double *fac = reinterpret_cast<double *>(base + off_fac);
+    float *v = reinterpret_cast<float *>(base + off_v);
+    PDD_CUDA_TRY(ctx, cudaMemsetAsync(S.ticket, 0, NB * sizeof(int32_t), ctx->stream));
+    const int32_t h_nlive = nb;
+    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(S.n_live, &h_nlive, sizeof h_nlive, cudaMemcpyHostToDevice,
+                                      ctx->stream));
+    const int P0 = B0.P[0], P1 = B0.P[1], P2 = B0.P[2];
+    const int Pm = std::max(P0, std::max(P1, P2));
+    box3_sine_kernel<<<dim3(static_cast<unsigned>((Pm * box3_pad(Pm) + 255) / 256), 3), 256, 0, ctx->stream>>>(
+        P0, P1, P2, T);
     PDD_CUDA_TRY(ctx, cudaGetLastError());
-    int smax = 0;
-    for (int a = 0; a < 3; ++a) smax = std::max(smax, B0.P[a] * B0.P[a]);
-    const size_t smem = static_cast<size_t>(smax) * sizeof(float);
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_dst_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536));
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_dst_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536));
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_dst_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536));
-    const unsigned gt = static_cast<unsigned>(std::min<int64_t>((np + kBox3Block - 1) / kBox3Block, 2048));
-    const dim3 gr(static_cast<unsigned>(nblk), nb), gd(gt, nb);
+    const dim3 gp(static_cast<unsigned>(P2), nb);
+    box3_eig_kernel<<<dim3(static_cast<unsigned>(P2), one_h ? 1u : static_cast<unsigned>(nb)),
+                      kBox3Block, 0, ctx->stream>>>(d_boxes, T, s2, c, fac);
+    PDD_CUDA_TRY(ctx, cudaGetLastError());
+    const size_t smem_p = box3_plane_smem(P0, P1);
+    const size_t smem_z = (static_cast<size_t>(P2) * ld[2] + 2 * static_cast<size_t>(P2) * kBox3Cols) * sizeof(float);
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_p)));
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_p)));
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_z)));
+    const dim3 gz(static_cast<unsigned>((P0 * P1 + kBox3Cols - 1) / kBox3Cols), nb);
+    const int64_t fac_stride = one_h ? 0 : np;
+    // The boxes stop themselves.  The host looks at their number one
+    // correction behind (a copy into pinned memory and an event), so the
+    // device never waits for it; what it enqueues after the last box has
+    // stopped returns at once.
     for (int64_t it = 0;; ++it) {
-      box3_residual_kernel<<<gr, kBox3Block, 0, ctx->stream>>>(d_boxes, live, s2, c, d_u, coef, r,
-                                                              part);
-      box3_combine_kernel<false><<<gcomb, 128, 0, ctx->stream>>>(part, nblk, nb, live, rn);
-      PDD_CUDA_TRY(ctx, cudaGetLastError());
-      st = read_measures();
-      if (st != PDD_OK) return st;
-      int n_live = 0;
-      for (size_t b = 0; b < NB; ++b) {
-        if (!h_live[b]) continue;
-        if (h_r0[b] < 0.0) h_r0[b] = h_rn[b];
-        h_it[b] = it;
-        h_res[b] = h_r0[b] > 0.0 ? h_rn[b] / h_r0[b] : 0.0;
-        if (h_rn[b] <= S0.tol * h_r0[b] || h_rn[b] == 0.0 || it >= S0.max_iter)
-          h_live[b] = 0;
-        else
-          ++n_live;
+      box3_residual_kernel<EllipticManufactured::kDriftAxes><<<gp, kBox3Block, 0, ctx->stream>>>(
+          d_boxes, S, s2, c, d_u, coef, r, part, it, S0.max_iter, S0.tol);
+      PDD_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->watch + (it & 1), S.n_live, sizeof(int32_t),
+                                        cudaMemcpyDeviceToHost, ctx->stream));
+      PDD_CUDA_TRY(ctx, cudaEventRecord(ctx->watch_ev[it & 1], ctx->stream));
+      if (it > 0) {
+        PDD_CUDA_TRY(ctx, cudaEventSynchronize(ctx->watch_ev[(it - 1) & 1]));
+        if (ctx->watch[(it - 1) & 1] == 0) break;
       }
-      if (n_live == 0) break;
-      st = push_live();
-      if (st != PDD_OK) return st;
-      // forward transform (x from the scaled FP64 residual, then y, z), the
-      // eigenvalues, the inverse transform (x, y, z), the update
-      box3_dst_kernel<0><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[0], nullptr, v0, rn, r);
-      box3_dst_kernel<1><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[1], v0, v1, nullptr, nullptr);
-      box3_dst_kernel<2><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[2], v1, v0, nullptr, nullptr);
-      box3_eig_kernel<<<gd, kBox3Block, 0, ctx->stream>>>(d_boxes, live, s2, c, cm1, v0);
-      box3_dst_kernel<0><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[0], v0, v1, nullptr, nullptr);
-      box3_dst_kernel<1><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[1], v1, v0, nullptr, nullptr);
-      box3_dst_kernel<2><<<gd, kBox3Block, smem, ctx->stream>>>(B0.P[0], B0.P[1], B0.P[2], live, S[2], v0, v1, nullptr, nullptr);
-      box3_update_kernel<<<gd, kBox3Block, 0, ctx->stream>>>(d_boxes, live, v1, rn, d_u);
+      box3_plane_kernel<false><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, rn, T, r, v, nullptr);
+      box3_z_kernel<<<gz, kBox3Block, smem_z, ctx->stream>>>(P0, P1, P2, live, T, fac, fac_stride, v);
+      box3_plane_kernel<true><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, rn, T, nullptr, v, d_u);
       PDD_CUDA_TRY(ctx, cudaGetLastError());
     }
+    std::vector<char> h_state(state_bytes);
+    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(h_state.data(), base, state_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+    std::memcpy(h_it.data(), h_state.data() + off_it, NB * sizeof(int64_t));
+    std::memcpy(h_res.data(), h_state.data() + off_res, NB * sizeof(double));
   }
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
   PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));

@@ -265,3 +265,23 @@ def test_interface_interp_panel_edges(api, sizes):
         err = float((got - val).abs().max())
         print(f"M = {n + 3}: node residual {err:.1e}, bound {bound:.1e}")
         assert err <= bound
+
+
+@pytest.mark.parametrize("n", [(3, 3, 3), (3, 36, 5), (34, 35, 6), (6, 5, 36), (128, 4, 4),
+                               (4, 128, 5), (5, 4, 128), (128, 128, 3)])
+def test_box_solve_size_edges(api, orc, n):
+    """Grids at the edges of the transform kernels (one interior point, rows
+    of a multiple of four and one more, 32 columns and one more, the largest
+    axis) in a batch whose two boxes have different mesh sizes, against the
+    oracle's sparse direct solve."""
+    prob = W.elliptic_manufactured()
+    rng = np.random.default_rng(sum(n))
+    boxes = [((0.25, 0.5, 0.0), (0.5, 0.75, 0.25), 0b010101), ((0.0, 0.25, 0.5), (0.25, 0.75, 0.625), 0b111111)]
+    boxes = [(lo, hi, _box_data(lo, hi, n, mask, rng)) for lo, hi, mask in boxes]
+    with api.Context(prob) as ctx:
+        r = ctx.subdomain_solve3d_batch(boxes, n, tol=1e-13)
+    assert r["status"] == 0 and r["resid"] <= 1e-13
+    for b, (lo, hi, faces) in enumerate(boxes):
+        ref = _oracle_box(orc, prob, lo, hi, n, faces)
+        np.testing.assert_allclose(r["u"][b].cpu().numpy(), ref, rtol=0,
+                                   atol=1e-10 * max(1.0, np.abs(ref).max()))
