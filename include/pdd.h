@@ -533,6 +533,31 @@ PDD_API pdd_status pdd_subdomain_solve_batch(pdd_ctx *ctx, const pdd_subdomain *
                                              double *resid, int64_t *iters_each,
                                              double *resid_each);
 
+/* Stage two on the cube split into split^3 subdomains (Sec. 2.1, Fig. 2.2):
+ * the node estimates d_values [n] at d_nodes [n][3] (FP64) are interpolated on
+ * the 3 (split - 1) internal planes x_a = k / split (pdd_interface_interp with
+ * n_bnd points per edge, evaluated on the plane's grid x grid points), and
+ * the subdomains are solved as pdd_subdomain_solve_batch solves them, with the
+ * interpolated values on their interface faces and g on the cube's boundary.
+ * A node belongs to the planes whose coordinate it has exactly and, with
+ * d_axis (int32 [n], may be NULL), whose axis is d_axis[i].  d_planes
+ * [3 (split - 1)][grid][grid] (axis-major, then k; higher axis slow) and d_u
+ * [grid][grid][grid] ([z][y][x]) are written in full; *iters and *resid (host,
+ * may be NULL) get the largest count and residual over the subdomains.
+ * grid - 1 must be a multiple of split, split in [2, 22].  PDD_EINVAL and
+ * PDD_ETIMEOUT as for the two calls it combines.  Synchronises. */
+typedef struct {
+  int32_t grid, split, n_bnd, method;
+  int64_t max_iter;
+  double tol;
+} pdd_stage2_params;
+
+PDD_API pdd_status pdd_elliptic3d_stage2(pdd_ctx *ctx, const double *d_nodes,
+                                         const double *d_values, const int32_t *d_axis,
+                                         int64_t n, const pdd_stage2_params *params,
+                                         double *d_planes, double *d_u, int64_t *iters,
+                                         double *resid);
+
 /* The plain GPU form of pdd_interface_solve, kept as a comparison baseline:
  * one kernel launch per node, one thread per path, block sums added to FP64
  * node accumulators with atomics (so the last bits depend on scheduling), no

@@ -61,6 +61,11 @@ class Subdomain(ctypes.Structure):
                 ("max_iter", ctypes.c_int64), ("tol", ctypes.c_double)]
 
 
+class Stage2Params(ctypes.Structure):
+    _fields_ = [("grid", ctypes.c_int32), ("split", ctypes.c_int32), ("n_bnd", ctypes.c_int32),
+                ("method", ctypes.c_int32), ("max_iter", ctypes.c_int64), ("tol", ctypes.c_double)]
+
+
 class BatchNodes(ctypes.Structure):
     _fields_ = [("d_nodes", ctypes.c_void_p), ("d_problem", ctypes.c_void_p),
                 ("d_dt", ctypes.c_void_p), ("n", ctypes.c_int64)]
@@ -116,6 +121,10 @@ _SIGS = {
                                                  ctypes.POINTER(ctypes.c_double),
                                                  ctypes.POINTER(ctypes.c_int64),
                                                  ctypes.POINTER(ctypes.c_double)]),
+    "pdd_elliptic3d_stage2": (ctypes.c_int, [_VP, _VP, _VP, _VP, _I64,
+                                             ctypes.POINTER(Stage2Params), _VP, _VP,
+                                             ctypes.POINTER(ctypes.c_int64),
+                                             ctypes.POINTER(ctypes.c_double)]),
     "pdd_interface_grad": (ctypes.c_int, [_VP, _VP, _I64, ctypes.POINTER(MCParams), _VP, _VP,
                                           _VP, _VP, _VP, ctypes.POINTER(Diag)]),
     "pdd_set_params": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_double), ctypes.c_int32]),

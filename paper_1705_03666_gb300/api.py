@@ -643,13 +643,12 @@ def elliptic3d_pdd_solve(ctx: Context, nodes, values, node_axis=None, *, grid: i
     """Stage two of PDD for the 3-D problem on the unit cube split into
     split^3 subdomains (Sec. 2.1, Fig. 2.2): the node estimates `values` at
     `nodes` (every node on one of the internal planes x_a = k / split) are
-    interpolated on each plane (pdd_interface_interp, evaluated on the
-    plane's grid of `grid` x `grid` points; node_axis, if given, names the
-    plane axis each node belongs to, so that a node on two planes' line of
-    intersection is used by its own plane only), and the subdomains are
-    solved independently, all in one batched call (pdd_subdomain_solve_batch),
+    interpolated on each plane (evaluated on the plane's grid of `grid` x
+    `grid` points; node_axis, if given, names the plane axis each node belongs
+    to, so that a node on two planes' line of intersection is used by its own
+    plane only), and the subdomains are solved independently, all together,
     with the interpolated values on their interface faces and g on the cube's
-    boundary.  Returns the global solution
+    boundary: one library call (pdd_elliptic3d_stage2).  Returns the global solution
     u [grid, grid, grid] ([z][y][x]), the largest iteration count and
     residual, and the time of each part is left to the caller."""
     if ctx.prob["problem"] != "elliptic_manufactured":
@@ -659,49 +658,29 @@ def elliptic3d_pdd_solve(ctx: Context, nodes, values, node_axis=None, *, grid: i
     dev = ctx.device
     nodes = _dev_f64(nodes, dev).reshape(-1, 3)
     values = _dev_f64(values, dev).reshape(-1)
+    if values.numel() != nodes.shape[0]:
+        raise ValueError("values must have one entry per node")
     if node_axis is not None:
         node_axis = torch.as_tensor(node_axis, device=dev).reshape(-1)
-    t = torch.linspace(0.0, 1.0, grid, dtype=_F64, device=dev)
-    planes, queries = [], []
-    for a in range(3):
-        for k in range(1, split):
-            pos = k / split
-            sel = nodes[:, a] == pos
-            if node_axis is not None:
-                sel &= node_axis == a
-            planes.append((a, pos, nodes[sel], values[sel]))
-            o = [b for b in range(3) if b != a]
-            g2, g1 = torch.meshgrid(t, t, indexing="ij")      # [slow = o[1]][fast = o[0]]
-            q = torch.empty((grid * grid, 3), dtype=_F64, device=dev)
-            q[:, a] = pos
-            q[:, o[0]] = g1.reshape(-1)
-            q[:, o[1]] = g2.reshape(-1)
-            queries.append(q)
-    vals = ctx.interface_interp(planes, queries, n_bnd=n_bnd)
-    plane_grid = {(a, k): vals[a * (split - 1) + k - 1].reshape(grid, grid)
-                  for a in range(3) for k in range(1, split)}
-    m = (grid - 1) // split + 1
+        if node_axis.is_floating_point():   # a value that is no axis names none
+            node_axis = torch.where(node_axis == node_axis.floor(), node_axis, -1.0)
+        node_axis = node_axis.clamp(-1, 3).to(_I32)
+        node_axis = node_axis.expand(nodes.shape[0]) if node_axis.numel() == 1 else node_axis
+        node_axis = node_axis.contiguous()
+        if node_axis.numel() != nodes.shape[0]:
+            raise ValueError("node_axis must have one entry per node")
+    planes = torch.empty((3 * (split - 1), grid, grid), dtype=_F64, device=dev)
     u = torch.empty((grid, grid, grid), dtype=_F64, device=dev)
-    boxes, slices = [], []
-    for kz in range(split):
-        for ky in range(split):
-            for kx in range(split):
-                kk = (kx, ky, kz)
-                lo = [kk[a] / split for a in range(3)]
-                hi = [(kk[a] + 1) / split for a in range(3)]
-                sl = [slice(kk[a] * (m - 1), kk[a] * (m - 1) + m) for a in range(3)]
-                faces = {}
-                for a in range(3):
-                    o = [b for b in range(3) if b != a]
-                    for side in (0, 1):
-                        plane = kk[a] + side
-                        if 0 < plane < split:
-                            pg = plane_grid[(a, plane)]
-                            faces[2 * a + side] = pg[sl[o[1]], sl[o[0]]].contiguous()
-                boxes.append((lo, hi, faces))
-                slices.append(sl)
-    # the split^3 subdomains are independent: one batched solve
-    r = ctx.subdomain_solve3d_batch(boxes, (m, m, m), method=method, tol=tol, max_iter=max_iter)
-    for b, sl in enumerate(slices):
-        u[sl[2], sl[1], sl[0]] = r["u"][b]
-    return {"u": u, "iters": r["iters"], "resid": r["resid"], "plane_values": plane_grid}
+    sp = _lib.Stage2Params(int(grid), int(split), int(n_bnd), _lib.STENCIL[method], int(max_iter),
+                           float(tol))
+    it, res = ctypes.c_int64(0), ctypes.c_double(0.0)
+    with torch.cuda.device(dev):
+        ctx._bind_stream()
+        st = ctx.lib.pdd_elliptic3d_stage2(
+            ctx.handle, nodes.data_ptr(), values.data_ptr(),
+            node_axis.data_ptr() if node_axis is not None else None, nodes.shape[0],
+            ctypes.byref(sp), planes.data_ptr(), u.data_ptr(), ctypes.byref(it), ctypes.byref(res))
+    _lib.check(st, ctx.handle, allow=(_lib.PDD_OK, _lib.PDD_ETIMEOUT))
+    return {"u": u, "iters": it.value, "resid": res.value,
+            "plane_values": {(a, k): planes[a * (split - 1) + k - 1]
+                             for a in range(3) for k in range(1, split)}}

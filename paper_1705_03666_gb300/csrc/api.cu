@@ -199,6 +199,16 @@ pdd_status pdd_subdomain_solve_batch(pdd_ctx *ctx, const pdd_subdomain *sds, int
                                            iters_each, resid_each);
 }
 
+pdd_status pdd_elliptic3d_stage2(pdd_ctx *ctx, const double *d_nodes, const double *d_values,
+                                 const int32_t *d_axis, int64_t n, const pdd_stage2_params *params,
+                                 double *d_planes, double *d_u, int64_t *iters, double *resid) {
+  if (!ctx) return PDD_EINVAL;
+  ctx->last_error.clear();
+  const TraceRange trace(__func__);
+  return pdd::elliptic3d_stage2_impl(ctx, d_nodes, d_values, d_axis, n, params, d_planes, d_u, iters,
+                                     resid);
+}
+
 pdd_status pdd_interface_grad(pdd_ctx *ctx, const double *d_nodes, int64_t n,
                               const pdd_mc_params *mc, const double *d_grad_out, double *d_jac,
                               double *d_jac_se, double *d_dtheta, double *d_dphi,

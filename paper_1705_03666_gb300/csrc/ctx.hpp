@@ -222,7 +222,10 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
                                  const double *h_pos, const int64_t *h_node_count,
                                  const double *d_nodes, const double *d_vals, int32_t n_bnd,
                                  const int64_t *h_query_count, const double *d_query,
-                                 double *d_out);
+                                 double *d_out, const int64_t *h_node_off = nullptr);
+pdd_status elliptic3d_stage2_impl(pdd_ctx *ctx, const double *d_nodes, const double *d_values,
+                                  const int32_t *d_axis, int64_t n, const pdd_stage2_params *sp,
+                                  double *d_planes, double *d_u, int64_t *iters, double *resid);
 pdd_status subdomain_solve3d_impl(pdd_ctx *ctx, const pdd_subdomain *sd, const double *d_face,
                                   int64_t m, double *d_u, int64_t *iters, double *resid);
 pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, int32_t nb,

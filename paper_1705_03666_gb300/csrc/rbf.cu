@@ -533,7 +533,7 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
                                  const double *h_pos, const int64_t *h_node_count,
                                  const double *d_nodes, const double *d_vals, int32_t n_bnd,
                                  const int64_t *h_query_count, const double *d_query,
-                                 double *d_out) {
+                                 double *d_out, const int64_t *h_node_off) {
   if (ctx->prob.dim != 3 || ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED)
     return fail(ctx, PDD_EINVAL, "interface interpolation on planes covers the 3-D family");
   if (n_planes < 1 || n_planes > 64) return fail(ctx, PDD_EINVAL, "n_planes must be in [1, 64]");
@@ -551,7 +551,7 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
     if (M > kRbfMaxSystem) return fail(ctx, PDD_EINVAL, "plane %d: system of %lld unknowns above %lld",
                                        p, static_cast<long long>(M), static_cast<long long>(kRbfMaxSystem));
     RbfPlane &P = pl[p];
-    P.node0 = node0;
+    P.node0 = h_node_off ? h_node_off[p] : node0;
     P.m = h_node_count[p];
     P.sys0 = sys0;
     P.row0 = row0;

@@ -54,14 +54,17 @@ struct Box3 {
   int n[3];           // grid points per axis, boundary included
   int P[3];           // interior points per axis
   int mask;           // bit 2a + side: that face carries interface data
+  int face_ld[6];       // row length of each face's data (its slow axis)
   int64_t face_off[6];  // offset of each face's data in the caller's array
+  // the box's grid in the caller's array: point (i, j, k) is at u_off + k u_sz
+  // + j u_sy + i (a box of its own, or a block of one global grid: boxes that
+  // share a face then write the same values on it)
+  int64_t u_off, u_sz;
+  int u_sy;
 };
 
 __device__ __forceinline__ int64_t box3_index(const Box3 &B, int i, int j, int k) {
-  return (static_cast<int64_t>(k) * B.n[1] + j) * B.n[0] + i;
-}
-__device__ __forceinline__ int64_t box3_total(const Box3 &B) {
-  return static_cast<int64_t>(B.n[0]) * B.n[1] * B.n[2];
+  return B.u_off + k * B.u_sz + static_cast<int64_t>(j) * B.u_sy + i;
 }
 __device__ __forceinline__ int64_t box3_np(const Box3 &B) {
   return static_cast<int64_t>(B.P[0]) * B.P[1] * B.P[2];
@@ -80,7 +83,7 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
   const Box3 B = boxes[blockIdx.y];
   const int k = blockIdx.x;
   const int64_t np = box3_np(B);
-  u += blockIdx.y * box3_total(B) + static_cast<int64_t>(k) * B.n[0] * B.n[1];
+  u += B.u_off + k * B.u_sz;
   coef += blockIdx.y * 4 * np;
   __shared__ typename Model::AxisTable tab[3][kBox3MaxInterior + 2];
   for (int e = threadIdx.x; e < B.n[0] + B.n[1] + 1; e += blockDim.x) {
@@ -93,10 +96,11 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
   for (int e = threadIdx.x; e < B.n[0] * B.n[1]; e += blockDim.x) {
     const int j = e / B.n[0], i = e - j * B.n[0];
     const int idx[3] = {i, j, k};
+    double *ue = u + static_cast<int64_t>(j) * B.u_sy + i;
     const bool interior = i > 0 && j > 0 && k > 0 && i < B.n[0] - 1 && j < B.n[1] - 1 &&
                           k < B.n[2] - 1;
     if (interior) {
-      u[e] = 0.0;
+      *ue = 0.0;
       double b[3], f = 0.0;
       Model::coeffs_tab(tab[0][i], tab[1][j], tab[2][0], b, f);
       const int64_t q = (static_cast<int64_t>(k - 1) * B.P[1] + (j - 1)) * B.P[0] + (i - 1);
@@ -126,9 +130,9 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
       // face grid of face fbest: the two other axes, the higher one slow
       const int a = fbest >> 1;
       const int a1 = a == 0 ? 1 : 0, a2 = a == 2 ? 1 : 2;
-      v = face[B.face_off[fbest] + static_cast<int64_t>(idx[a2]) * B.n[a1] + idx[a1]];
+      v = face[B.face_off[fbest] + static_cast<int64_t>(idx[a2]) * B.face_ld[fbest] + idx[a1]];
     }
-    u[e] = v;
+    *ue = v;
   }
 }
 
@@ -157,8 +161,8 @@ box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, do
   const int64_t np = box3_np(B);
   const int plane = B.P[0] * B.P[1];
   const int64_t q0 = static_cast<int64_t>(blockIdx.x) * plane;
-  const int sy = B.n[0], sz = B.n[0] * B.n[1];
-  u += box * box3_total(B) + static_cast<int64_t>(blockIdx.x + 1) * sz;
+  const int64_t sy = B.u_sy, sz = B.u_sz;
+  u += box3_index(B, 1, 1, static_cast<int>(blockIdx.x) + 1);
   coef += box * 4 * np + q0;
   r += box * np + q0;
   const double w0 = 0.5 * s2 / (B.h[0] * B.h[0]), w1 = 0.5 * s2 / (B.h[1] * B.h[1]),
@@ -167,7 +171,7 @@ box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, do
   double acc = 0.0;
   for (int q = threadIdx.x; q < plane; q += kBox3Block) {
     const int j = q / B.P[0];
-    const double *v = u + (j + 1) * sy + (q - j * B.P[0] + 1);
+    const double *v = u + j * sy + (q - j * B.P[0]);
     const double ux0 = v[-1], ux1 = v[1], uy0 = v[-sy], uy1 = v[sy], uz0 = v[-sz], uz1 = v[sz];
     double Au = diag * v[0] + w0 * (ux0 + ux1) + w1 * (uy0 + uy1) + w2 * (uz0 + uz1);
     double drift = 0.0;
@@ -334,12 +338,12 @@ box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *rn,
   });
   __syncthreads();
   if constexpr (kInverse) {
-    double *up = u + box * box3_total(B) + (static_cast<int64_t>(blockIdx.x + 1) * B.n[1] + 1) * B.n[0] + 1;
+    double *up = u + box3_index(B, 1, 1, static_cast<int>(blockIdx.x) + 1);
     box3_apply(Tt, ldt, Sx, ld0, P0, P1, P0, [&](int a, int k, const float *s) {
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (a + q < P1) {
-          double *p = up + static_cast<int64_t>(a + q) * B.n[0] + k;
+          double *p = up + static_cast<int64_t>(a + q) * B.u_sy + k;
           *p = fma(static_cast<double>(s[q]), sc, *p);
         }
     });
@@ -398,8 +402,6 @@ box3_jacobi_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, 
   if (!live[blockIdx.y]) return;
   const Box3 B = boxes[blockIdx.y];
   const int64_t np = box3_np(B);
-  u += blockIdx.y * box3_total(B);
-  un += blockIdx.y * box3_total(B);
   coef += blockIdx.y * 4 * np;
   const double w0 = 0.5 * s2 / (B.h[0] * B.h[0]), w1 = 0.5 * s2 / (B.h[1] * B.h[1]),
                w2 = 0.5 * s2 / (B.h[2] * B.h[2]);
@@ -412,7 +414,7 @@ box3_jacobi_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, 
     const int j = static_cast<int>((q / B.P[0]) % B.P[1]) + 1;
     const int k = static_cast<int>(q / (static_cast<int64_t>(B.P[0]) * B.P[1])) + 1;
     const int64_t e = box3_index(B, i, j, k);
-    const int64_t sy = B.n[0], sz = static_cast<int64_t>(B.n[0]) * B.n[1];
+    const int64_t sy = B.u_sy, sz = B.u_sz;
     const double ux0 = u[e - 1], ux1 = u[e + 1], uy0 = u[e - sy], uy1 = u[e + sy],
                  uz0 = u[e - sz], uz1 = u[e + sz];
     const double off = (w0 - coef[q] * d0) * ux0 + (w0 + coef[q] * d0) * ux1 +
@@ -433,64 +435,17 @@ box3_jacobi_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, 
   }
 }
 
-// A batch of nb boxes with the same grid size and method: the faces of box b
-// follow those of box b - 1 in d_face, and d_u is [nb][n2][n1][n0].  *iters
-// and *resid (if non-null) get the largest count and relative residual over
-// the boxes; iters_each / resid_each (host, nb entries, may be null) get each
-// box's own.
-pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, int32_t nb,
-                                        const double *d_face, int64_t m, double *d_u,
-                                        int64_t *iters, double *resid, int64_t *iters_each,
-                                        double *resid_each) {
-  if (!sds || nb < 1 || nb > 65535) return fail(ctx, PDD_EINVAL, "batch of 1 .. 65535 boxes");
-  if (ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED || ctx->prob.dim != 3)
-    return fail(ctx, PDD_EINVAL, "the 3-D subdomain solver covers the 3-D family");
-  if (reflect_mask(ctx) != 0)
-    return fail(ctx, PDD_EINVAL, "the 3-D subdomain solver takes Dirichlet data only");
-  const pdd_subdomain &S0 = sds[0];
-  std::vector<Box3> boxes(static_cast<size_t>(nb));
-  int64_t off = 0;
-  for (int32_t b = 0; b < nb; ++b) {
-    const pdd_subdomain *sd = sds + b;
-    Box3 &B = boxes[static_cast<size_t>(b)];
-    for (int a = 0; a < 3; ++a) {
-      if (sd->n[a] < 3 || sd->n[a] - 2 > kBox3MaxInterior)
-        return fail(ctx, PDD_EINVAL, "3-D grids take 3 .. %d points per axis", kBox3MaxInterior + 2);
-      if (sd->n[a] != S0.n[a])
-        return fail(ctx, PDD_EINVAL, "the boxes of a batch share one grid size");
-      if (!(sd->hi[a] > sd->lo[a]) || sd->lo[a] < 0.0 || sd->hi[a] > 1.0)
-        return fail(ctx, PDD_EINVAL, "box must be non-empty and inside the unit cube");
-      B.lo[a] = sd->lo[a];
-      B.n[a] = sd->n[a];
-      B.P[a] = sd->n[a] - 2;
-      B.h[a] = (sd->hi[a] - sd->lo[a]) / (sd->n[a] - 1);
-    }
-    if (sd->iface_axis < 0 || sd->iface_axis > 63 || sd->iface_side != 0)
-      return fail(ctx, PDD_EINVAL, "3-D: iface_axis is a mask of interface faces (0..63), "
-                                   "iface_side must be 0");
-    if (sd->method != PDD_STENCIL_DST && sd->method != PDD_STENCIL_JACOBI)
-      return fail(ctx, PDD_EINVAL, "3-D methods: PDD_STENCIL_DST or PDD_STENCIL_JACOBI");
-    if (sd->method != S0.method || sd->max_iter != S0.max_iter || !(sd->tol == S0.tol))
-      return fail(ctx, PDD_EINVAL, "the boxes of a batch share one method and stopping rule");
-    if (sd->max_iter < 1 || !(sd->tol >= 0.0)) return fail(ctx, PDD_EINVAL, "bad stopping rule");
-    B.mask = sd->iface_axis;
-    for (int fc = 0; fc < 6; ++fc) {
-      B.face_off[fc] = off;
-      if ((B.mask >> fc) & 1) {
-        const int a = fc >> 1;
-        off += static_cast<int64_t>(B.n[a == 0 ? 1 : 0]) * B.n[a == 2 ? 1 : 2];
-      }
-    }
-  }
-  if (m != off) return fail(ctx, PDD_EINVAL, "expected %lld face values, got %lld",
-                            static_cast<long long>(off), static_cast<long long>(m));
-  if (off > 0 && !d_face) return fail(ctx, PDD_EINVAL, "null face data");
-  if (!d_u) return fail(ctx, PDD_EINVAL, "null output");
-  PDD_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-
+// The boxes' solves (one grid size and method; faces and grids where the boxes
+// say, u_span values of d_u in all).  *iters and *resid (if non-null) get the
+// largest count and relative residual over the boxes; iters_each / resid_each
+// (host, one entry per box, may be null) get each box's own.
+static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int32_t method,
+                              int64_t max_iter, double tol, const double *d_face, double *d_u,
+                              int64_t u_span, int64_t *iters, double *resid, int64_t *iters_each,
+                              double *resid_each) {
+  const int32_t nb = static_cast<int32_t>(boxes.size());
   const Box3 &B0 = boxes[0];
-  const bool jacobi = S0.method == PDD_STENCIL_JACOBI;
-  const int64_t total = static_cast<int64_t>(B0.n[0]) * B0.n[1] * B0.n[2];
+  const bool jacobi = method == PDD_STENCIL_JACOBI;
   const int64_t np = static_cast<int64_t>(B0.P[0]) * B0.P[1] * B0.P[2];
   const size_t NB = static_cast<size_t>(nb);
   const int nblk = static_cast<int>(std::min<int64_t>((np + kBox3Block - 1) / kBox3Block, 1024));
@@ -517,7 +472,7 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   const size_t off_box = take(NB * sizeof(Box3));
   const size_t off_coef = take(NB * 4 * np * sizeof(double));
   const size_t off_part = take(NB * std::max(nblk, B0.P[2]) * sizeof(double));
-  const size_t off_un = take(jacobi ? NB * total * sizeof(double) : 0);
+  const size_t off_un = take(jacobi ? u_span * sizeof(double) : 0);
   const size_t off_r = take(jacobi ? 0 : NB * np * sizeof(double));
   const size_t off_fac = take(jacobi ? 0 : (one_h ? 1 : NB) * np * sizeof(double));
   const size_t off_v = take(jacobi ? 0 : NB * np * sizeof(float));
@@ -573,18 +528,18 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   if (jacobi) {
     // each box sweeps between its own two buffers; a box that stops keeps its
     // latest iterate where its own step count left it
-    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(un, d_u, NB * total * sizeof(double),
+    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(un, d_u, u_span * sizeof(double),
                                       cudaMemcpyDeviceToDevice, ctx->stream));
     const unsigned gj = static_cast<unsigned>(nblk);
     int n_live = nb;
-    for (int64_t it = 1; it <= S0.max_iter && n_live > 0; ++it) {
+    for (int64_t it = 1; it <= max_iter && n_live > 0; ++it) {
       const bool odd = (it & 1) != 0;
       box3_jacobi_kernel<<<dim3(gj, nb), kBox3Block, 0, ctx->stream>>>(
           d_boxes, live, s2, c, odd ? d_u : un, odd ? un : d_u, coef, part);
       PDD_CUDA_TRY(ctx, cudaGetLastError());
       for (size_t b = 0; b < NB; ++b)
         if (h_live[b]) h_it[b] = it;
-      if (it % 16 == 0 || it == S0.max_iter) {
+      if (it % 16 == 0 || it == max_iter) {
         box3_combine_kernel<<<gcomb, 128, 0, ctx->stream>>>(part, nblk, nb, live, rn);
         PDD_CUDA_TRY(ctx, cudaGetLastError());
         st = read_measures();
@@ -592,7 +547,7 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
         for (size_t b = 0; b < NB; ++b) {
           if (!h_live[b]) continue;
           h_res[b] = h_rn[b];
-          if (h_rn[b] < S0.tol || it == S0.max_iter) {
+          if (h_rn[b] < tol || it == max_iter) {
             h_live[b] = 0;
             --n_live;
           }
@@ -602,10 +557,15 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
       }
     }
     // a box whose last sweep was odd holds its iterate in un
-    for (size_t b = 0; b < NB; ++b)
-      if (h_it[b] & 1)
-        PDD_CUDA_TRY(ctx, cudaMemcpyAsync(d_u + b * total, un + b * total, total * sizeof(double),
-                                          cudaMemcpyDeviceToDevice, ctx->stream));
+    for (size_t b = 0; b < NB; ++b) {
+      if (!(h_it[b] & 1)) continue;
+      const Box3 &B = boxes[b];
+      for (int k = 0; k < B.n[2]; ++k)
+        PDD_CUDA_TRY(ctx, cudaMemcpy2DAsync(d_u + B.u_off + k * B.u_sz, B.u_sy * sizeof(double),
+                                            un + B.u_off + k * B.u_sz, B.u_sy * sizeof(double),
+                                            B.n[0] * sizeof(double), static_cast<size_t>(B.n[1]),
+                                            cudaMemcpyDeviceToDevice, ctx->stream));
+    }
   } else {
     st = ensure_watch(ctx);
     if (st != PDD_OK) return st;
@@ -651,7 +611,7 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
     // stopped returns at once.
     for (int64_t it = 0;; ++it) {
       box3_residual_kernel<EllipticManufactured::kDriftAxes><<<gp, kBox3Block, 0, ctx->stream>>>(
-          d_boxes, S, s2, c, d_u, coef, r, part, it, S0.max_iter, S0.tol);
+          d_boxes, S, s2, c, d_u, coef, r, part, it, max_iter, tol);
       PDD_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->watch + (it & 1), S.n_live, sizeof(int32_t),
                                         cudaMemcpyDeviceToHost, ctx->stream));
       PDD_CUDA_TRY(ctx, cudaEventRecord(ctx->watch_ev[it & 1], ctx->stream));
@@ -678,7 +638,7 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   for (size_t b = 0; b < NB; ++b) {
     it_max = std::max(it_max, h_it[b]);
     res_max = std::max(res_max, h_res[b]);
-    unmet |= jacobi ? h_res[b] >= S0.tol : h_res[b] > S0.tol;
+    unmet |= jacobi ? h_res[b] >= tol : h_res[b] > tol;
     if (iters_each) iters_each[b] = h_it[b];
     if (resid_each) resid_each[b] = h_res[b];
   }
@@ -688,9 +648,215 @@ pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, 
   return PDD_OK;
 }
 
+// A batch of nb boxes with the same grid size and method: the faces of box b
+// follow those of box b - 1 in d_face, and d_u is [nb][n2][n1][n0].  *iters
+// and *resid (if non-null) get the largest count and relative residual over
+// the boxes; iters_each / resid_each (host, nb entries, may be null) get each
+// box's own.
+pdd_status subdomain_solve3d_batch_impl(pdd_ctx *ctx, const pdd_subdomain *sds, int32_t nb,
+                                        const double *d_face, int64_t m, double *d_u,
+                                        int64_t *iters, double *resid, int64_t *iters_each,
+                                        double *resid_each) {
+  if (!sds || nb < 1 || nb > 65535) return fail(ctx, PDD_EINVAL, "batch of 1 .. 65535 boxes");
+  if (ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED || ctx->prob.dim != 3)
+    return fail(ctx, PDD_EINVAL, "the 3-D subdomain solver covers the 3-D family");
+  if (reflect_mask(ctx) != 0)
+    return fail(ctx, PDD_EINVAL, "the 3-D subdomain solver takes Dirichlet data only");
+  const pdd_subdomain &S0 = sds[0];
+  std::vector<Box3> boxes(static_cast<size_t>(nb));
+  int64_t off = 0;
+  for (int32_t b = 0; b < nb; ++b) {
+    const pdd_subdomain *sd = sds + b;
+    Box3 &B = boxes[static_cast<size_t>(b)];
+    for (int a = 0; a < 3; ++a) {
+      if (sd->n[a] < 3 || sd->n[a] - 2 > kBox3MaxInterior)
+        return fail(ctx, PDD_EINVAL, "3-D grids take 3 .. %d points per axis", kBox3MaxInterior + 2);
+      if (sd->n[a] != S0.n[a])
+        return fail(ctx, PDD_EINVAL, "the boxes of a batch share one grid size");
+      if (!(sd->hi[a] > sd->lo[a]) || sd->lo[a] < 0.0 || sd->hi[a] > 1.0)
+        return fail(ctx, PDD_EINVAL, "box must be non-empty and inside the unit cube");
+      B.lo[a] = sd->lo[a];
+      B.n[a] = sd->n[a];
+      B.P[a] = sd->n[a] - 2;
+      B.h[a] = (sd->hi[a] - sd->lo[a]) / (sd->n[a] - 1);
+    }
+    if (sd->iface_axis < 0 || sd->iface_axis > 63 || sd->iface_side != 0)
+      return fail(ctx, PDD_EINVAL, "3-D: iface_axis is a mask of interface faces (0..63), "
+                                   "iface_side must be 0");
+    if (sd->method != PDD_STENCIL_DST && sd->method != PDD_STENCIL_JACOBI)
+      return fail(ctx, PDD_EINVAL, "3-D methods: PDD_STENCIL_DST or PDD_STENCIL_JACOBI");
+    if (sd->method != S0.method || sd->max_iter != S0.max_iter || !(sd->tol == S0.tol))
+      return fail(ctx, PDD_EINVAL, "the boxes of a batch share one method and stopping rule");
+    if (sd->max_iter < 1 || !(sd->tol >= 0.0)) return fail(ctx, PDD_EINVAL, "bad stopping rule");
+    B.mask = sd->iface_axis;
+    for (int fc = 0; fc < 6; ++fc) {
+      B.face_off[fc] = off;
+      if ((B.mask >> fc) & 1) {
+        const int a = fc >> 1;
+        B.face_ld[fc] = B.n[a == 0 ? 1 : 0];
+        off += static_cast<int64_t>(B.face_ld[fc]) * B.n[a == 2 ? 1 : 2];
+      }
+    }
+    B.u_sy = B.n[0];
+    B.u_sz = static_cast<int64_t>(B.n[0]) * B.n[1];
+    B.u_off = b * B.u_sz * B.n[2];
+  }
+  if (m != off) return fail(ctx, PDD_EINVAL, "expected %lld face values, got %lld",
+                            static_cast<long long>(off), static_cast<long long>(m));
+  if (off > 0 && !d_face) return fail(ctx, PDD_EINVAL, "null face data");
+  if (!d_u) return fail(ctx, PDD_EINVAL, "null output");
+  PDD_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+
+  return solve_boxes(ctx, boxes, S0.method, S0.max_iter, S0.tol, d_face, d_u,
+                     nb * boxes[0].u_sz * boxes[0].n[2], iters, resid, iters_each, resid_each);
+}
+
 pdd_status subdomain_solve3d_impl(pdd_ctx *ctx, const pdd_subdomain *sd, const double *d_face,
                                   int64_t m, double *d_u, int64_t *iters, double *resid) {
   return subdomain_solve3d_batch_impl(ctx, sd, 1, d_face, m, d_u, iters, resid, nullptr, nullptr);
+}
+
+// ---------------------------------------------------------------------------
+// Stage two on the split cube (pdd_elliptic3d_stage2): nodes sorted to their
+// planes, the planes' interpolants on their grids, and the boxes solved in
+// place in the global grid, their faces read from the plane grids (no packing
+// and no scatter of the solution).
+// ---------------------------------------------------------------------------
+constexpr int kPickBlock = 1024;
+
+// Nodes of plane blockIdx.x (axis a = p / (split - 1), x_a = (p mod (split -
+// 1) + 1) / split; with axis, only the nodes that name a) and their values,
+// in node order, at most cap of them; count[p] is how many there are.
+__global__ void __launch_bounds__(kPickBlock)
+stage2_pick_kernel(const double *nodes, const double *values, const int32_t *axis, int64_t n,
+                   int split, int64_t cap, double *pn, double *pv, int64_t *count) {
+  const int a = blockIdx.x / (split - 1);
+  const double pos = static_cast<double>(blockIdx.x % (split - 1) + 1) / split;
+  pn += blockIdx.x * cap * 3;
+  pv += blockIdx.x * cap;
+  __shared__ int warp_sum[kPickBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t base = 0;
+  for (int64_t i0 = 0; i0 < n; i0 += kPickBlock) {
+    const int64_t i = i0 + threadIdx.x;
+    const bool on = i < n && nodes[3 * i + a] == pos && (!axis || axis[i] == a);
+    const unsigned m = __ballot_sync(kFull, on);
+    if (lane == 0) warp_sum[warp] = __popc(m);
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < kPickBlock / 32; ++w) {
+      before += w < warp ? warp_sum[w] : 0;
+      all += warp_sum[w];
+    }
+    const int64_t e = base + before + __popc(m & ((1u << lane) - 1u));
+    if (on && e < cap) {
+      for (int d = 0; d < 3; ++d) pn[3 * e + d] = nodes[3 * i + d];
+      pv[e] = values[i];
+    }
+    base += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) count[blockIdx.x] = base;
+}
+
+// The grid points of every plane ([slow = higher axis][fast = lower axis]).
+__global__ void stage2_grid_kernel(int split, int grid, double *q) {
+  const int p = blockIdx.y, a = p / (split - 1);
+  const int a1 = a == 0 ? 1 : 0, a2 = a == 2 ? 1 : 2;
+  q += 3 * static_cast<int64_t>(p) * grid * grid;
+  const double step = 1.0 / (grid - 1);
+  // (from both ends, so that the last point is 1 exactly)
+  auto t = [&](int i) { return i < grid / 2 ? i * step : 1.0 - (grid - 1 - i) * step; };
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < grid * grid; e += gridDim.x * blockDim.x) {
+    const int j = e / grid, i = e - j * grid;
+    q[3 * static_cast<int64_t>(e) + a] = static_cast<double>(p % (split - 1) + 1) / split;
+    q[3 * static_cast<int64_t>(e) + a1] = t(i);
+    q[3 * static_cast<int64_t>(e) + a2] = t(j);
+  }
+}
+
+pdd_status elliptic3d_stage2_impl(pdd_ctx *ctx, const double *d_nodes, const double *d_values,
+                                  const int32_t *d_axis, int64_t n, const pdd_stage2_params *sp,
+                                  double *d_planes, double *d_u, int64_t *iters, double *resid) {
+  if (!sp || !d_planes || !d_u) return fail(ctx, PDD_EINVAL, "null argument");
+  if (ctx->prob.kind != PDD_PROB_ELLIPTIC_MANUFACTURED || ctx->prob.dim != 3)
+    return fail(ctx, PDD_EINVAL, "the 3-D stage two covers the 3-D family");
+  if (reflect_mask(ctx) != 0)
+    return fail(ctx, PDD_EINVAL, "the 3-D subdomain solver takes Dirichlet data only");
+  const int split = sp->split, grid = sp->grid;
+  if (split < 2 || split > 22) return fail(ctx, PDD_EINVAL, "split must be in [2, 22]");
+  if (grid < 3 || (grid - 1) % split) return fail(ctx, PDD_EINVAL, "grid - 1 must be a multiple of split");
+  const int m = (grid - 1) / split + 1;
+  if (m < 3 || m - 2 > kBox3MaxInterior)
+    return fail(ctx, PDD_EINVAL, "3-D grids take 3 .. %d points per axis", kBox3MaxInterior + 2);
+  if (sp->method != PDD_STENCIL_DST && sp->method != PDD_STENCIL_JACOBI)
+    return fail(ctx, PDD_EINVAL, "3-D methods: PDD_STENCIL_DST or PDD_STENCIL_JACOBI");
+  if (sp->max_iter < 1 || !(sp->tol >= 0.0)) return fail(ctx, PDD_EINVAL, "bad stopping rule");
+  if (n < 0 || (n > 0 && (!d_nodes || !d_values))) return fail(ctx, PDD_EINVAL, "null buffer");
+  PDD_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  const int np = 3 * (split - 1);
+  const int64_t g2 = static_cast<int64_t>(grid) * grid;
+  // (a plane with more nodes than any system may hold is refused below)
+  const int64_t cap = std::min<int64_t>(n, 8192);
+  const size_t off_cnt = 0, off_n = 512;
+  const size_t off_v = align_up(off_n + static_cast<size_t>(np) * cap * 3 * sizeof(double), 256);
+  const size_t off_q = align_up(off_v + static_cast<size_t>(np) * cap * sizeof(double), 256);
+  // the auxiliary buffer: the interpolation and the boxes use the scratch
+  pdd_status st = ensure_aux(ctx, off_q + static_cast<size_t>(np) * g2 * 3 * sizeof(double));
+  if (st != PDD_OK) return st;
+  char *base = static_cast<char *>(ctx->aux);
+  auto *cnt = reinterpret_cast<int64_t *>(base + off_cnt);
+  auto *pn = reinterpret_cast<double *>(base + off_n);
+  auto *pv = reinterpret_cast<double *>(base + off_v);
+  auto *q = reinterpret_cast<double *>(base + off_q);
+  stage2_pick_kernel<<<np, kPickBlock, 0, ctx->stream>>>(d_nodes, d_values, d_axis, n, split, cap,
+                                                         pn, pv, cnt);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  stage2_grid_kernel<<<dim3(static_cast<unsigned>(std::min<int64_t>((g2 + 255) / 256, 1024)),
+                            static_cast<unsigned>(np)), 256, 0, ctx->stream>>>(split, grid, q);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  int64_t h_cnt[64], h_off[64], h_q[64];
+  int32_t h_axis[64];
+  double h_pos[64];
+  PDD_CUDA_TRY(ctx, cudaMemcpyAsync(h_cnt, cnt, np * sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
+  PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  for (int p = 0; p < np; ++p) {
+    h_axis[p] = p / (split - 1);
+    h_pos[p] = static_cast<double>(p % (split - 1) + 1) / split;
+    h_off[p] = p * cap;
+    h_q[p] = g2;
+  }
+  st = interface_interp_impl(ctx, np, h_axis, h_pos, h_cnt, pn, pv, sp->n_bnd, h_q, q, d_planes, h_off);
+  if (st != PDD_OK) return st;
+  std::vector<Box3> boxes;
+  for (int kz = 0; kz < split; ++kz)
+    for (int ky = 0; ky < split; ++ky)
+      for (int kx = 0; kx < split; ++kx) {
+        const int kk[3] = {kx, ky, kz};
+        Box3 B;
+        std::memset(&B, 0, sizeof B);
+        for (int a = 0; a < 3; ++a) {
+          B.lo[a] = static_cast<double>(kk[a]) / split;
+          B.n[a] = m;
+          B.P[a] = m - 2;
+          B.h[a] = (static_cast<double>(kk[a] + 1) / split - B.lo[a]) / (m - 1);
+        }
+        for (int fc = 0; fc < 6; ++fc) {
+          const int a = fc >> 1, plane = kk[a] + (fc & 1);
+          if (plane == 0 || plane == split) continue;
+          const int a1 = a == 0 ? 1 : 0, a2 = a == 2 ? 1 : 2;
+          B.mask |= 1 << fc;
+          B.face_ld[fc] = grid;
+          B.face_off[fc] = (a * (split - 1) + plane - 1) * g2 +
+                           static_cast<int64_t>(kk[a2] * (m - 1)) * grid + kk[a1] * (m - 1);
+        }
+        B.u_sy = grid;
+        B.u_sz = g2;
+        B.u_off = (kz * g2 + static_cast<int64_t>(ky) * grid + kx) * (m - 1);
+        boxes.push_back(B);
+      }
+  return solve_boxes(ctx, boxes, sp->method, sp->max_iter, sp->tol, d_planes, d_u, g2 * grid, iters,
+                     resid, nullptr, nullptr);
 }
 
 }  // namespace pdd

@@ -285,3 +285,56 @@ def test_box_solve_size_edges(api, orc, n):
         ref = _oracle_box(orc, prob, lo, hi, n, faces)
         np.testing.assert_allclose(r["u"][b].cpu().numpy(), ref, rtol=0,
                                    atol=1e-10 * max(1.0, np.abs(ref).max()))
+
+
+@pytest.mark.parametrize("split,with_axis,method", [(2, True, "dst"), (4, True, "dst"),
+                                                    (4, False, "dst"), (2, True, "jacobi")])
+def test_stage_two_call_equals_its_parts(api, split, with_axis, method):
+    """elliptic3d_pdd_solve (one library call, boxes in place in the global
+    grid) gives the bits of interface_interp and subdomain_solve3d_batch
+    called one after the other; grid - 1 is a power of two, so the grid points
+    are exact on both sides."""
+    prob = W.elliptic_manufactured()
+    rng = np.random.default_rng(split)
+    grid, n = 17, 150
+    axis = rng.integers(0, 3, n)
+    nodes = rng.uniform(0.02, 0.98, (n, 3))
+    nodes[np.arange(n), axis] = rng.integers(1, split, n) / split
+    vals = _exact(nodes) + 1e-3 * rng.standard_normal(n)
+    t = np.linspace(0, 1, grid)
+    G2, G1 = np.meshgrid(t, t, indexing="ij")
+    planes, queries, keys = [], [], []
+    for a in range(3):
+        for k in range(1, split):
+            sel = (nodes[:, a] == k / split) & ((axis == a) if with_axis else True)
+            o = [b for b in range(3) if b != a]
+            q = np.full((grid * grid, 3), k / split)
+            q[:, o[0]], q[:, o[1]] = G1.ravel(), G2.ravel()
+            planes.append((a, k / split, nodes[sel], vals[sel]))
+            queries.append(q)
+            keys.append((a, k))
+    m = (grid - 1) // split + 1
+    with api.Context(prob) as ctx:
+        r = api.elliptic3d_pdd_solve(ctx, nodes, vals, axis if with_axis else None, grid=grid,
+                                     split=split, n_bnd=8, method=method, tol=1e-11,
+                                     max_iter=5000)
+        pv = ctx.interface_interp(planes, queries, n_bnd=8)
+        pv = {k: v.reshape(grid, grid) for k, v in zip(keys, pv)}
+        boxes, slices = [], []
+        for kk in np.ndindex(split, split, split):
+            kk = kk[::-1]
+            sl = [slice(c * (m - 1), c * (m - 1) + m) for c in kk]
+            faces = {}
+            for a in range(3):
+                o = [b for b in range(3) if b != a]
+                for side in (0, 1):
+                    if 0 < kk[a] + side < split:
+                        faces[2 * a + side] = pv[(a, kk[a] + side)][sl[o[1]], sl[o[0]]].contiguous()
+            boxes.append(([c / split for c in kk], [(c + 1) / split for c in kk], faces))
+            slices.append(sl)
+        rb = ctx.subdomain_solve3d_batch(boxes, (m, m, m), method=method, tol=1e-11, max_iter=5000)
+    for k in keys:
+        assert torch.equal(r["plane_values"][k], pv[k]), k
+    for b, sl in enumerate(slices):
+        assert torch.equal(r["u"][sl[2], sl[1], sl[0]], rb["u"][b]), b
+    assert r["iters"] == rb["iters"] and r["resid"] == rb["resid"]
