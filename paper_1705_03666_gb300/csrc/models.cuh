@@ -79,6 +79,8 @@ struct EllipticManufactured {
   struct AxisTable {
     double s, c;
   };
+  // b_a is a function of one coordinate, x[drift_axis(a)], alone
+  __host__ __device__ static constexpr int drift_axis(int a) { return a == 0 ? 1 : 0; }
   __device__ __forceinline__ static AxisTable axis_table(int axis, double x) {
     AxisTable t{0.0, 0.0};
     if (axis == 2) t.s = exp(x);

@@ -15,7 +15,7 @@
 // Elimination.  Right-looking in panels of NB columns over the list of rows
 // that have not been a pivot yet (rows are not moved).  Two launches per panel:
 //   1. rbf_step_kernel<..., kNext>: the columns of the next panel are updated
-//      by the current one;
+//      by the current one, and the pivot rows' entries of all columns formed;
 //   2. rbf_step_kernel<..., kRest>: one block per plane factors the next panel
 //      (pivot search, multipliers) while the other blocks update all the
 //      columns behind it by the current panel.
@@ -25,9 +25,11 @@
 // step order, l = a / pivot), whatever the panel width.  Factored rows go to U
 // in pivot order.
 //
-// Measured on the 9 planes (device time): elimination and back substitution
-// 11.75 ms by one 8-block cluster per plane with a cluster barrier per step
-// (20 us a step) -> 2.9 ms; evaluation 2.28 -> 1.56 ms.
+// Measured on the 9 planes (device time): 11.75 ms by one 8-block cluster per
+// plane with a cluster barrier per step (20 us a step); 2.2 ms in panels (step
+// launches 109 us at the first panel, where the update bounds them, to 23 us at
+// the last ones, where the 16 pivot steps do) and 0.25 ms of back
+// substitution.  Evaluation 2.28 -> 1.56 ms (its FP64 floor is 1.4 ms).
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -39,7 +41,8 @@ namespace pdd {
 
 constexpr int64_t kRbfMaxSystem = 6144;  // unknowns per plane (weights + 3)
 constexpr int kRbfThreads = 512;
-constexpr int kRbfTileR = 64;            // rows of an update tile
+constexpr int kRbfTileR = 32, kRbfTileC = 32;  // rows and columns of an update tile
+constexpr size_t kRbfOwnSm = 116 * 1024;  // more than half of an SM's shared memory
 constexpr size_t kRbfPanelBytes = 200 * 1024;  // panel in shared memory (rows x NB doubles)
 
 struct RbfPlane {
@@ -158,24 +161,57 @@ __global__ void rbf_assemble_kernel(RbfWork W, const double *pts, const double *
   }
 }
 
-// a / b for the pivot b with r = 1 / b correctly rounded (Markstein, "Computation
-// of elementary functions on the IBM RISC System/6000", 1990): q = a r, then one
-// correction by the exact remainder gives the correctly rounded quotient while
-// nothing underflows: three FP64 instructions per row instead of a division.
-__device__ __forceinline__ double markstein_div(double a, double b, double r) {
-  const double q = a * r;
+// 1 / b to 20 bits for 2^-500 < |b| < 2^500: the hardware reciprocal of the
+// mantissa (20 bits of it, from the high word), the exponent negated in
+// integers.  No FP64 instruction.
+__device__ __forceinline__ double rcp_seed(double b) {
+  const int hi = __double2hiint(b);
+  const float m = __int_as_float(((hi & 0xfffff) << 3) | 0x3f800000);  // in [1, 2)
+  const int y = __float_as_int(rcp_approx(m)) >> 3;                    // exponent 126 or 127
+  const int e = (hi >> 20) & 0x7ff;
+  return __hiloint2double((y + ((1023 - 127 + 1023 - e) << 20)) | (hi & 0x80000000), 0);
+}
+// a / b from r = rcp_seed(b): the quotient corrected twice by its exact
+// remainder (FMA), 20 -> 40 -> 53 bits: the last bit may differ from the rounded
+// quotient only in ties of the 2^-60 residual.  Five FP64 instructions and no
+// serial reciprocal, where a division takes several times that.
+__device__ __forceinline__ double seeded_div(double a, double b, double r) {
+  double q = a * r;
+  q = fma(fma(-q, b, a), r, q);
   return fma(fma(-q, b, a), r, q);
 }
+__device__ __forceinline__ bool seed_range(double b) {
+  return fabs(b) > 0x1p-500 && fabs(b) < 0x1p500;
+}
+
+// Shared memory of an update tile: pivot rows and multipliers.
+__host__ __device__ constexpr int rbf_tile_doubles(int NB) {
+  return NB * kRbfTileC + kRbfTileR * (NB + 1);
+}
+
+// Named barriers of a step block: kRbfThreads workers and the pivot warp.
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+enum { kBarCand = 1, kBarPivot = 2, kBarWork = 3 };
 
 // Factor panel `panel` of a plane (columns [k0, k0 + nb)): one block.  The
-// active rows' panel entries sit in shared memory, column by column; thread t
+// active rows' panel entries sit in shared memory, column by column; worker t
 // owns the list positions t, t + 512, ...  Each step takes the unused row of
 // largest |entry| (lowest row index on ties), forms the multipliers of the
-// other unused rows and updates their remaining panel entries; the update of
-// the next column comes first and yields the next step's candidates in the
-// same pass.  On return the list of rows still active, their multipliers, the
-// pivot rows and their own multipliers are stored for the update, and U has
-// the panel's columns of the pivot rows.
+// other unused rows and updates their remaining panel entries.  The chain from
+// one pivot to the next is what bounds the panel (an FP64 instruction occupies
+// its scheduler's pipe for 64 clocks), so a step first does only what the next
+// pivot needs, the multipliers and the next column, and publishes the next
+// column's candidates; while the extra warp picks the pivot (integers only: an
+// FP64 reciprocal there would queue behind the workers' updates), the workers
+// update the columns behind.  On return the list
+// of rows still active, their multipliers, the pivot rows and their own
+// multipliers are stored for the update, and U has the panel's columns of the
+// pivot rows.
 template <int NB>
 __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel, double *smem) {
   const int k0 = panel * NB;
@@ -188,17 +224,46 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
   const double *A = W.A + P.sys0;
   double *U = W.U + P.sys0;
   double *S = smem;  // S[c * R + pos]
-  __shared__ uint32_t c_hi[2][kRbfThreads / 32], c_lo[2][kRbfThreads / 32];
-  __shared__ int32_t c_pos[2][kRbfThreads / 32];
-  __shared__ double s_r;
+  constexpr int nw = kRbfThreads / 32, kAll = kRbfThreads + 32;
+  __shared__ uint32_t c_hi[2][nw], c_lo[2][nw];
+  __shared__ int32_t c_pos[2][nw];
   __shared__ int32_t s_piv[NB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int nw = kRbfThreads / 32;
+  if (warp == nw) {
+    // the pivot warp: step kk's pivot from the workers' candidates
+    for (int kk = 0; kk < nb; ++kk) {
+      const int sl = kk & 1;
+      bar_sync(kBarCand, kAll);
+      const uint32_t hi = lane < nw ? c_hi[sl][lane] : 0u;
+      const uint32_t mh = __reduce_max_sync(kFull, hi);
+      unsigned who = __ballot_sync(kFull, hi == mh && lane < nw);
+      if (__popc(who) > 1) {  // equal high words: the low words, then the position, decide
+        const uint32_t lo = (who >> lane) & 1u ? c_lo[sl][lane] : 0u;
+        const uint32_t ml = __reduce_max_sync(kFull, lo);
+        const bool top = ((who >> lane) & 1u) && lo == ml;
+        const int32_t pos = top ? c_pos[sl][lane] : 0x7fffffff;
+        const int32_t mp = __reduce_min_sync(kFull, pos);
+        who = __ballot_sync(kFull, top && pos == mp);
+      }
+      const int src = __ffs(who) - 1;
+      // NaN in every unused row: no pivot (flagged; the solution is not used)
+      const bool none = (mh | c_lo[sl][src]) == 0u;
+      const int pr = none ? 0 : c_pos[sl][src];
+      const double akk = S[kk * R + pr];
+      if (lane == 0) {
+        if (none || !((__double2hiint(akk) & 0x7fffffff) | __double2loint(akk))) *W.singular = 1;
+        s_piv[kk] = pr;
+      }
+      __syncwarp();
+      bar_sync(kBarPivot, kAll);
+    }
+    return;
+  }
   for (int e = tid; e < R * NB; e += kRbfThreads) {
     const int pos = e / NB, c = e % NB;
     if (c < nb) S[c * R + pos] = A[static_cast<int64_t>(act[pos]) * ld + k0 + c];
   }
-  __syncthreads();
+  bar_sync(kBarWork, kRbfThreads);
   uint32_t used = 0;  // bit i: own position tid + 512 i has been a pivot
   // candidate of this thread: bits of |entry| plus one (0: none, and for NaN)
   // and its position (the list keeps rows in increasing order, so the lowest
@@ -206,72 +271,71 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
   unsigned long long key = 0;
   int32_t kpos = 0x7fffffff;
   auto consider = [&](double v, int pos) {
-    const unsigned long long b =
-        v == v ? (static_cast<unsigned long long>(__double_as_longlong(v)) & 0x7fffffffffffffffull) + 1
-               : 0ull;
+    // (integers only: the FP64 pipe is what bounds the panel)
+    const unsigned long long m =
+        static_cast<unsigned long long>(__double_as_longlong(v)) & 0x7fffffffffffffffull;
+    const unsigned long long b = m <= 0x7ff0000000000000ull ? m + 1 : 0ull;
     if (b > key) {
       key = b;
       kpos = pos;
     }
   };
-  for (int pos = tid; pos < R; pos += kRbfThreads) consider(S[pos], pos);
-  for (int kk = 0; kk < nb; ++kk) {
-    const int sl = kk & 1;
-    // warp candidate: largest key, then lowest position
-    {
-      const uint32_t hi = static_cast<uint32_t>(key >> 32);
-      const uint32_t mh = __reduce_max_sync(kFull, hi);
-      const uint32_t lo = hi == mh ? static_cast<uint32_t>(key) : 0u;
-      const uint32_t ml = __reduce_max_sync(kFull, lo);
-      const int32_t mp = __reduce_min_sync(kFull, hi == mh && lo == ml ? kpos : 0x7fffffff);
-      if (lane == 0) {
-        c_hi[sl][warp] = mh;
-        c_lo[sl][warp] = ml;
-        c_pos[sl][warp] = mp;
-      }
-    }
-    __syncthreads();
-    // every warp finds the block's pivot from the warp candidates
-    const uint32_t hi = lane < nw ? c_hi[sl][lane] : 0u;
+  // warp candidate of step kk: largest key, then lowest position
+  auto publish = [&](int kk) {
+    const uint32_t hi = static_cast<uint32_t>(key >> 32), lo = static_cast<uint32_t>(key);
     const uint32_t mh = __reduce_max_sync(kFull, hi);
-    const uint32_t lo = lane < nw && hi == mh ? c_lo[sl][lane] : 0u;
-    const uint32_t ml = __reduce_max_sync(kFull, lo);
-    const bool top = lane < nw && hi == mh && lo == ml;
-    const int32_t mp = __reduce_min_sync(kFull, top ? c_pos[sl][lane] : 0x7fffffff);
-    // NaN in every unused row: no pivot (flagged; the solution is not used)
-    const bool none = (mh | ml) == 0u;
-    const int pr = none ? 0 : mp;
-    const double akk = S[kk * R + pr];
-    if (tid == 0) {
-      if (none || !(fabs(akk) > 0.0)) *W.singular = 1;
-      s_r = 1.0 / akk;
-      s_piv[kk] = pr;
+    unsigned who = __ballot_sync(kFull, hi == mh);
+    if (__popc(who) > 1) {  // equal high words: the low words, then the position, decide
+      const uint32_t ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
+      const bool top = hi == mh && lo == ml;
+      const int32_t mp = __reduce_min_sync(kFull, top ? kpos : 0x7fffffff);
+      who = __ballot_sync(kFull, top && kpos == mp);
     }
+    if (lane == __ffs(who) - 1) {
+      c_hi[kk & 1][warp] = mh;
+      c_lo[kk & 1][warp] = lo;
+      c_pos[kk & 1][warp] = kpos;
+    }
+    __threadfence_block();
+    __syncwarp();
+    bar_arrive(kBarCand, kAll);
+  };
+  for (int pos = tid; pos < R; pos += kRbfThreads) consider(S[pos], pos);
+  publish(0);
+  for (int kk = 0; kk < nb; ++kk) {
+    bar_sync(kBarPivot, kAll);
+    const int pr = s_piv[kk];
+    const double akk = S[kk * R + pr];
     if (pr % kRbfThreads == tid) used |= 1u << (pr / kRbfThreads);
-    __syncthreads();
-    const double r = s_r;
-    // far from overflow and underflow the corrected quotient is the division
-    const bool plain = !(fabs(akk) > 0x1p-500 && fabs(akk) < 0x1p500);
+    const int ea = (__double2hiint(akk) >> 20) & 0x7ff;
+    const bool seeded = ea > 523 && ea < 1523;  // |akk| in [2^-499, 2^500)
+    const double r = rcp_seed(akk);
+    const int c1 = kk + 1;
+    const double p1 = c1 < nb ? S[c1 * R + pr] : 0.0;
     key = 0;
     kpos = 0x7fffffff;
-    const int c1 = kk + 1;
+    // (the pivot row's entries are read by every thread and written by none)
     for (int i = 0, pos = tid; pos < R; ++i, pos += kRbfThreads) {
       if ((used >> i) & 1u) continue;
       const double a = S[kk * R + pos];
-      const double l = plain ? a / akk : markstein_div(a, akk, r);
+      const double l = seeded ? seeded_div(a, akk, r) : a / akk;
       S[kk * R + pos] = l;
       if (c1 < nb) {
-        const double v = fma(-l, S[c1 * R + pr], S[c1 * R + pos]);
+        const double v = fma(-l, p1, S[c1 * R + pos]);
         S[c1 * R + pos] = v;
         consider(v, pos);
       }
-      // (the pivot row's entries are read by every thread and written by none)
+    }
+    if (c1 < nb) publish(c1);
+    for (int i = 0, pos = tid; pos < R; ++i, pos += kRbfThreads) {
+      if ((used >> i) & 1u) continue;
+      const double l = S[kk * R + pos];
 #pragma unroll 4
       for (int c = kk + 2; c < nb; ++c)
         S[c * R + pos] = fma(-l, S[c * R + pr], S[c * R + pos]);
     }
   }
-  __syncthreads();
+  bar_sync(kBarWork, kRbfThreads);
   // the panel's columns of U, the pivot rows, their multipliers
   double *L11 = W.L11[par] + (blockIdx.x * NB) * NB;
   for (int e = tid; e < nb * nb; e += kRbfThreads) {
@@ -294,114 +358,146 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
   }
 }
 
-// Update by panel `panel` (already factored) of a tile of TC columns from
-// column c0 (below c1) and kRbfTileR active rows from position r0.  The block
-// first solves for the pivot rows' entries of its columns (unit lower
-// triangle, one thread per column; the tiles of the first row store them in
-// U), then updates its rows: one FMA per element and pivot, in pivot order.
+// The pivot rows' entries of panel `panel` in the TC columns from column c0
+// (below c1): a unit lower triangular solve, a warp per pivot row and a lane
+// per column, so that the triangle spreads over the four schedulers' FP64
+// pipes.  The result is stored in U and left in Us [NB][TC].
 template <int NB, int TC>
-__device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int plane, int panel, int r0,
-                                int c0, int c1, double *smem) {
-  const int k0 = panel * NB, M = P.M, ld = M + 1;
-  const int nb = min(NB, M - k0);
-  const int R = M - k0 - nb;
+__device__ void rbf_pivot_rows(const RbfWork &W, const RbfPlane &P, int plane, int panel, int c0,
+                               int c1, double *Us, double *L11) {
+  const int k0 = panel * NB, ld = P.M + 1;
+  const int nb = min(NB, P.M - k0);
+  const int par = panel & 1, tid = threadIdx.x;
+  const int i = tid >> 5, c = tid & 31;
+  const bool on = i < nb && c < TC && c0 + c < c1;
+  double ui = 0.0;
+  if (on) ui = W.A[P.sys0 + static_cast<int64_t>(W.piv[par][plane * NB + i]) * ld + c0 + c];
+  for (int e = tid; e < NB * NB; e += kRbfThreads) {
+    const int row = e / NB, k = e % NB;
+    L11[e] = k < row && row < nb ? W.L11[par][plane * NB * NB + e] : 0.0;
+  }
+  bar_sync(kBarWork, kRbfThreads);
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    if (i == k && c < TC) Us[k * TC + c] = ui;
+    bar_sync(kBarWork, kRbfThreads);
+    if (i > k && on) ui = fma(-L11[i * NB + k], Us[k * TC + c], ui);
+  }
+  if (on) W.U[P.sys0 + static_cast<int64_t>(k0 + i) * ld + c0 + c] = ui;
+}
+
+// Update by panel `panel` (already factored, the pivot rows' entries Us
+// [NB][TC]) of a tile of TC columns from column c0 (below c1) and TR active
+// rows from position r0: one FMA per element and pivot, in pivot order.
+// Threads tid of kRbfThreads; Ls: [TR][NB + 1] of shared memory.
+template <int NB, int TC, int TR, class Sync>
+__device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int panel, int r0, int c0,
+                                int c1, const double *Us, double *Ls, int tid, Sync sync) {
+  const int k0 = panel * NB, ld = P.M + 1;
+  const int nb = min(NB, P.M - k0);
+  const int R = P.M - k0 - nb;
   const int par = panel & 1;
   double *A = W.A + P.sys0;
-  double *Us = smem;                 // [NB][TC]
-  double *Ls = smem + NB * TC;       // [kRbfTileR][NB + 1]
-  const int tid = threadIdx.x;
-  const int rows = min(kRbfTileR, R - r0);
+  const int rows = min(TR, R - r0);
   const double *L = W.L[par] + (P.row0 + r0) * NB;
-  if (tid < TC) {
-    const int j = c0 + tid;
-    if (j < c1) {
-      const double *L11 = W.L11[par] + plane * NB * NB;
-      const int32_t *piv = W.piv[par] + plane * NB;
-      double u[NB];
+  const int32_t *act = W.act[par] + P.row0 + r0;
+  const int tx = tid % TC, ty = tid / TC, j = c0 + tx;
+  constexpr int kStep = kRbfThreads / TC;   // rows between a thread's own
+  constexpr int kOwn = (TR + kStep - 1) / kStep;
+  double a[kOwn];
+  double *pa[kOwn];
 #pragma unroll
-      for (int i = 0; i < NB; ++i) u[i] = i < nb ? A[static_cast<int64_t>(piv[i]) * ld + j] : 0.0;
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-#pragma unroll
-        for (int i = k + 1; i < NB; ++i)
-          if (i < nb) u[i] = fma(-L11[i * NB + k], u[k], u[i]);
-      }
-#pragma unroll
-      for (int i = 0; i < NB; ++i) {
-        Us[i * TC + tid] = u[i];
-        if (r0 == 0 && i < nb) W.U[P.sys0 + static_cast<int64_t>(k0 + i) * ld + j] = u[i];
-      }
-    }
-  } else {
-    for (int e = tid - TC; e < rows * NB; e += kRbfThreads - TC) {
-      const int pos = e / NB, c = e % NB;
-      Ls[pos * (NB + 1) + c] = c < nb ? L[e] : 0.0;
-    }
+  for (int q = 0; q < kOwn; ++q) {
+    const int row = ty + q * kStep;
+    pa[q] = row < rows && j < c1 ? A + static_cast<int64_t>(act[row]) * ld + j : nullptr;
+    a[q] = pa[q] ? *pa[q] : 0.0;
   }
-  __syncthreads();
-  const int tx = tid % TC, ty = tid / TC;
-  const int j = c0 + tx;
-  if (j < c1) {
-    const int32_t *act = W.act[par] + P.row0 + r0;
-    double u[NB];
+  for (int e = tid; e < rows * NB; e += kRbfThreads)
+    Ls[(e / NB) * (NB + 1) + e % NB] = e % NB < nb ? L[e] : 0.0;
+  sync();
+  double u[NB];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) u[k] = Us[k * TC + tx];
-    for (int q = ty; q < rows; q += kRbfThreads / TC) {
-      double *pa = A + static_cast<int64_t>(act[q]) * ld + j;
-      double a = *pa;
+  for (int k = 0; k < NB; ++k) u[k] = Us[k * TC + tx];
 #pragma unroll
-      for (int k = 0; k < NB; ++k)
-        if (k < nb) a = fma(-Ls[q * (NB + 1) + k], u[k], a);
-      *pa = a;
-    }
+  for (int q = 0; q < kOwn; ++q) {
+    if (!pa[q]) continue;
+    const double *l = Ls + (ty + q * kStep) * (NB + 1);
+    double v = a[q];
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+      if (k < nb) v = fma(-l[k], u[k], v);
+    *pa[q] = v;
   }
-  __syncthreads();
 }
 
 // kFirst: panel 0 of every plane is factored (blockIdx.x = plane).
-// kNext: the columns of panel + 1 are updated by `panel` (blockIdx = row
-// tile, plane).
+// kNext, blockIdx.y = plane: blocks [0, row_tiles) update the columns of panel
+// + 1 by `panel` (and store their part of U); the others form the pivot rows'
+// entries of 32 columns behind them (U).
 // kRest: blocks [0, n_planes) factor panel + 1; the others update the columns
-// behind it by `panel` (blockIdx.x - n_planes = (plane, row tile, column
-// tile), column tiles fastest).
+// behind it by `panel`, two tiles per block (tile index = (plane, row tile,
+// column tile), column tiles fastest).  Launched with more than half of an
+// SM's shared memory per block, so that a panel has its SM's FP64 pipe to
+// itself.
 enum { kFirst = 0, kNext = 1, kRest = 2 };
 template <int NB, int kRole>
-__global__ void __launch_bounds__(kRbfThreads)
+__global__ void __launch_bounds__(kRole == kNext ? kRbfThreads : kRole == kRest ? 2 * kRbfThreads
+                                                                 : kRbfThreads + 32)
 rbf_step_kernel(const __grid_constant__ RbfWork W, int panel, int row_tiles, int col_tiles) {
   extern __shared__ __align__(16) double rbf_smem[];
-  constexpr int TC = 32;
+  constexpr int TC = kRbfTileC;
+  static_assert(NB * 32 <= kRbfThreads, "a warp per pivot row");
   if constexpr (kRole == kFirst) {
     rbf_factor_panel<NB>(W, W.planes[blockIdx.x], 0, rbf_smem);
   } else if constexpr (kRole == kNext) {
     const RbfPlane P = W.planes[blockIdx.y];
     const int k0 = panel * NB;
-    const int r0 = blockIdx.x * kRbfTileR;
-    const int R = P.M - k0 - NB;
-    if (R <= 0 || r0 >= R) return;  // no next panel, or no such rows
-    rbf_update_tile<NB, NB>(W, P, blockIdx.y, panel, r0, k0 + NB, min(k0 + 2 * NB, P.M), rbf_smem);
+    if (k0 >= P.M) return;
+    const int R = P.M - k0 - min(NB, P.M - k0);
+    double *L11 = rbf_smem, *Us = L11 + NB * NB, *Ls = Us + NB * TC;
+    if (static_cast<int>(blockIdx.x) < row_tiles) {
+      const int r0 = blockIdx.x * kRbfTileR, c0 = k0 + NB, c1 = min(k0 + 2 * NB, P.M);
+      if (R <= 0 || r0 >= R) return;  // no next panel, or no such rows
+      rbf_pivot_rows<NB, NB>(W, P, blockIdx.y, panel, c0, c1, Us, L11);
+      rbf_update_tile<NB, NB, kRbfTileR>(W, P, panel, r0, c0, c1, Us, Ls, threadIdx.x,
+                                         [] { bar_sync(kBarWork, kRbfThreads); });
+    } else {
+      const int c0 = min(k0 + 2 * NB, P.M) + (blockIdx.x - row_tiles) * TC;
+      if (c0 > P.M) return;
+      rbf_pivot_rows<NB, TC>(W, P, blockIdx.y, panel, c0, P.M + 1, Us, L11);
+    }
   } else {
     if (static_cast<int>(blockIdx.x) < W.n_planes) {
-      rbf_factor_panel<NB>(W, W.planes[blockIdx.x], panel + 1, rbf_smem);
+      if (threadIdx.x < kRbfThreads + 32)
+        rbf_factor_panel<NB>(W, W.planes[blockIdx.x], panel + 1, rbf_smem);
       return;
     }
-    int t = blockIdx.x - W.n_planes;
+    // two independent tiles per block
+    const int half = threadIdx.x / kRbfThreads, tid = threadIdx.x % kRbfThreads;
+    int t = (blockIdx.x - W.n_planes) * 2 + half;
     const int ct = t % col_tiles;
     t /= col_tiles;
     const int rt = t % row_tiles, p = t / row_tiles;
+    if (p >= W.n_planes) return;
     const RbfPlane P = W.planes[p];
-    const int k0 = panel * NB;
-    if (k0 >= P.M) return;
-    const int R = P.M - k0 - min(NB, P.M - k0);
+    const int k0 = panel * NB, ld = P.M + 1;
     const int r0 = rt * kRbfTileR, c0 = min(k0 + 2 * NB, P.M) + ct * TC;
-    // (the first row tile also runs without active rows: it stores U)
-    if ((r0 >= R && rt > 0) || c0 > P.M) return;
-    rbf_update_tile<NB, TC>(W, P, p, panel, r0, c0, P.M + 1, rbf_smem);
+    if (k0 + NB >= P.M || r0 >= P.M - k0 - NB || c0 > P.M) return;
+    double *Us = rbf_smem + half * rbf_tile_doubles(NB), *Ls = Us + NB * TC;
+    for (int e = tid; e < NB * TC; e += kRbfThreads) {
+      const int j = c0 + e % TC;
+      Us[e] = j <= P.M ? W.U[P.sys0 + static_cast<int64_t>(k0 + e / TC) * ld + j] : 0.0;
+    }
+    const int bar = kBarWork + half;
+    rbf_update_tile<NB, TC, kRbfTileR>(W, P, panel, r0, c0, P.M + 1, Us, Ls, tid,
+                                       [bar] { bar_sync(bar, kRbfThreads); });
   }
 }
 
 // Back substitution, one block per plane, from the last rows up in blocks of
-// 32: one warp solves the 32 x 32 triangle (a lane per row, quotients by
-// markstein_div with the 32 reciprocals formed together), then every row above
+// 32: one warp solves the 32 x 32 triangle (a lane per row; the 32 reciprocals
+// formed together, the quotient corrected once by its exact remainder), then
+// every row above
 // subtracts the block's 32 columns, one thread per row.
 __global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_constant__ RbfWork W) {
   extern __shared__ __align__(16) double rbf_smem[];
@@ -423,10 +519,10 @@ __global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_c
     if (tid < 32) {
       const double d = lane < nb ? T[lane][lane] : 1.0;
       const double r = 1.0 / d;
-      const bool plain = !(fabs(d) > 0x1p-500 && fabs(d) < 0x1p500);
+      const bool seeded = seed_range(d);
       double v = lane < nb ? y[b0 + lane] : 0.0;
       for (int i = nb - 1; i >= 0; --i) {
-        const double q = plain ? v / d : markstein_div(v, d, r);
+        const double q = seeded ? fma(fma(-v * r, d, v), r, v * r) : v / d;
         const double xi = __shfl_sync(kFull, q, i);
         if (lane == i) v = xi;
         else if (lane < i) v = fma(-T[lane][i], xi, v);
@@ -502,28 +598,30 @@ rbf_eval_kernel(const __grid_constant__ RbfWork W, const double *__restrict__ pt
 // The launches of the elimination for panel width NB.
 template <int NB>
 static pdd_status rbf_launch(pdd_ctx *ctx, const RbfWork &W, int Mmax) {
-  // a panel of Mmax rows, or an update tile's pivot columns and multipliers
-  const size_t tile = (static_cast<size_t>(NB) * 32 + kRbfTileR * (NB + 1)) * sizeof(double);
-  const size_t panel_smem = std::max(tile, static_cast<size_t>(Mmax) * NB * sizeof(double));
+  const size_t panel_smem = static_cast<size_t>(Mmax) * NB * sizeof(double);
+  const size_t next_smem = (NB * NB + rbf_tile_doubles(NB)) * sizeof(double);
   auto *first = rbf_step_kernel<NB, kFirst>;
   auto *next = rbf_step_kernel<NB, kNext>;
   auto *rest = rbf_step_kernel<NB, kRest>;
-  const int attr = static_cast<int>(panel_smem);
-  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, attr));
-  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, attr));
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(panel_smem)));
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(std::max(panel_smem, kRbfOwnSm))));
   const int panels = (Mmax + NB - 1) / NB;
   const unsigned np = static_cast<unsigned>(W.n_planes);
-  first<<<np, kRbfThreads, panel_smem, ctx->stream>>>(W, 0, 0, 0);
+  first<<<np, kRbfThreads + 32, panel_smem, ctx->stream>>>(W, 0, 0, 0);
   for (int p = 0; p < panels; ++p) {
-    const int left = Mmax - (p + 1) * NB;  // active rows of the largest plane after this panel
-    const int rt = std::max(1, (left + kRbfTileR - 1) / kRbfTileR);
-    if (left > 0) next<<<dim3(static_cast<unsigned>(rt), np), kRbfThreads, tile, ctx->stream>>>(W, p, 0, 0);
-    // columns behind the next panel, the right-hand side included (planes with
-    // smaller systems have fewer)
-    const int ct = (std::max(0, left - NB) + 1 + 31) / 32;
-    // the block's shared memory: the next panel of the largest plane
-    const size_t sm = std::max(tile, static_cast<size_t>(std::max(left, 0)) * NB * sizeof(double));
-    rest<<<np * (1u + static_cast<unsigned>(rt * ct)), kRbfThreads, sm, ctx->stream>>>(W, p, rt, ct);
+    // active rows of the largest plane after this panel, and the columns behind
+    // the next one, the right-hand side included (smaller planes have fewer)
+    const int left = std::max(0, Mmax - (p + 1) * NB);
+    const int rt = (left + kRbfTileR - 1) / kRbfTileR;
+    const int ct = (std::max(0, left - NB) + kRbfTileC) / kRbfTileC;
+    next<<<dim3(static_cast<unsigned>(rt + ct), np), kRbfThreads, next_smem, ctx->stream>>>(W, p, rt, ct);
+    if (left > 0) {
+      // the block's shared memory: the next panel of the largest plane
+      const size_t sm = std::max(kRbfOwnSm, static_cast<size_t>(left) * NB * sizeof(double));
+      rest<<<np + (np * static_cast<unsigned>(rt * ct) + 1) / 2, 2 * kRbfThreads, sm, ctx->stream>>>(W, p, rt, ct);
+    }
     PDD_CUDA_TRY(ctx, cudaGetLastError());
   }
   return PDD_OK;

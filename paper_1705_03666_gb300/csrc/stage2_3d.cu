@@ -24,11 +24,12 @@
 // gaps; the transforms run out of shared memory.  FP64 work that does not
 // change between corrections (drift over 2h, the eigenvalue factors) is formed
 // once per call.  Measured on the 64 boxes of 33^3 points of the 4 x 4 x 4 split
-// (eight residuals, seven corrections; device time): residuals 2.27 -> 0.80 ms,
-// transforms 3.70 -> 0.55 ms (one output per thread with two shared loads per
-// FMA, and the residual rescaled in FP64 for each of a row's 31 products,
-// before), eigenvalues 1.45 ms -> 0.01 ms, and no host round trip per
-// correction; the call 8.3 -> 1.9 ms.
+// (eight residuals, seven corrections; device time): residuals 2.27 -> 0.56 ms
+// (64-bit index divisions, three FP64 divisions per thread and three arrays of
+// drift before), transforms 3.70 -> 0.55 ms (one output per thread with two
+// shared loads per FMA, and the residual rescaled in FP64 for each of a row's
+// 31 products, before), eigenvalues 1.45 -> 0.01 ms, set-up 0.46 -> 0.08 ms, and
+// no host round trip per correction; the call 8.3 -> 1.6 ms.
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -48,11 +49,13 @@ namespace pdd {
 // ---------------------------------------------------------------------------
 constexpr int kBox3MaxInterior = 126;  // interior points per axis (sine matrix in shared memory)
 constexpr int kBox3Block = 256;
+constexpr int kBox3Axis = kBox3MaxInterior + 2;  // grid points per axis
 
 struct Box3 {
   double lo[3], h[3];
   int n[3];           // grid points per axis, boundary included
   int P[3];           // interior points per axis
+  double w[3], diag;  // (sigma^2 / 2) / h_a^2 and the operator's diagonal
   int mask;           // bit 2a + side: that face carries interface data
   int face_ld[6];       // row length of each face's data (its slow axis)
   int64_t face_off[6];  // offset of each face's data in the caller's array
@@ -75,24 +78,35 @@ __device__ __forceinline__ int64_t box3_np(const Box3 &B) {
 // physical boundary -- takes g; otherwise the interface face of lowest index),
 // interior u = 0, and per interior point b and f of the family.  The family's
 // functions of one coordinate are tabulated per block (a few dozen FP64
-// sines and exponentials in place of three per point: 460 -> 45 us for 64
-// boxes of 33^3 points).  kScaled: b_a / (2 h_a) is stored in place of b_a.
-template <class Model, bool kScaled>
+// sines and exponentials in place of three per point).  kTables: in place of
+// the arrays of b, the blocks of the first plane write b_a / (2 h_a) at the grid
+// points of the coordinate it depends on, drift[box][a][index].
+template <class Model, bool kTables>
 __global__ void __launch_bounds__(kBox3Block)
-box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *u, double *coef) {
+box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *u, double *coef,
+                  double *drift) {
   const Box3 B = boxes[blockIdx.y];
   const int k = blockIdx.x;
   const int64_t np = box3_np(B);
   u += B.u_off + k * B.u_sz;
-  coef += blockIdx.y * 4 * np;
-  __shared__ typename Model::AxisTable tab[3][kBox3MaxInterior + 2];
+  coef += blockIdx.y * (kTables ? 1 : 4) * np;
+  __shared__ typename Model::AxisTable tab[3][kBox3Axis];
   for (int e = threadIdx.x; e < B.n[0] + B.n[1] + 1; e += blockDim.x) {
     const int a = e < B.n[0] ? 0 : (e < B.n[0] + B.n[1] ? 1 : 2);
     const int i = a == 0 ? e : (a == 1 ? e - B.n[0] : k);
     tab[a][a == 2 ? 0 : i] = Model::axis_table(a, B.lo[a] + B.h[a] * i);
   }
   __syncthreads();
-  const double d[3] = {0.5 / B.h[0], 0.5 / B.h[1], 0.5 / B.h[2]};
+  if constexpr (kTables) {
+    if (k == 0)
+      for (int e = threadIdx.x; e < 2 * kBox3Axis; e += blockDim.x) {
+        const int a = e / kBox3Axis, i = e % kBox3Axis, on = Model::drift_axis(a);
+        if (!((Model::kDriftAxes >> a) & 1u) || i >= B.n[on]) continue;
+        double b[3], f;
+        Model::coeffs_tab(tab[0][on == 0 ? i : 0], tab[1][on == 1 ? i : 0], tab[2][0], b, f);
+        drift[(blockIdx.y * 2 + a) * kBox3Axis + i] = b[a] * (0.5 / B.h[a]);
+      }
+  }
   for (int e = threadIdx.x; e < B.n[0] * B.n[1]; e += blockDim.x) {
     const int j = e / B.n[0], i = e - j * B.n[0];
     const int idx[3] = {i, j, k};
@@ -104,11 +118,11 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
       double b[3], f = 0.0;
       Model::coeffs_tab(tab[0][i], tab[1][j], tab[2][0], b, f);
       const int64_t q = (static_cast<int64_t>(k - 1) * B.P[1] + (j - 1)) * B.P[0] + (i - 1);
+      if constexpr (!kTables) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        if (!kScaled || ((Model::kDriftAxes >> a) & 1u))  // (the residual skips axes without drift)
-          coef[a * np + q] = kScaled ? b[a] * d[a] : b[a];
-      coef[3 * np + q] = f;
+        for (int a = 0; a < 3; ++a) coef[a * np + q] = b[a];
+      }
+      coef[(kTables ? 0 : 3) * np + q] = f;
       continue;
     }
     bool physical = false;
@@ -137,10 +151,10 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
 }
 
 // Correction state of the boxes (device arrays, one entry per box, but
-// n_live): norm of the residual and of the first one, their ratio, the
+// n_live): norm of the residual, its inverse, the first norm, their ratio, the
 // corrections done, whether the box goes on, and the ticket of its blocks.
 struct Box3State {
-  double *rn, *r0, *res;
+  double *rn, *inv, *r0, *res;
   int64_t *iters;
   int32_t *live, *ticket;
   int32_t *n_live;
@@ -150,11 +164,13 @@ struct Box3State {
 // and the block's sum of r^2; the box's last block adds the planes' sums in a
 // fixed order, forms the norm and decides whether the box goes on (stopping
 // rule of correction `it`).
-template <unsigned kDriftAxes>
+template <class Model>
 __global__ void __launch_bounds__(kBox3Block)
-box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, double s2, double c,
-                     const double *u, const double *coef, double *r, double *part, int64_t it,
-                     int64_t max_iter, double tol) {
+box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, const double *u,
+                     const double *f, const double *drift, double *r, double *part,
+                     int64_t it, int64_t max_iter, double tol) {
+  static_assert(Model::kDriftAxes == 3u && Model::drift_axis(0) == 1 && Model::drift_axis(1) == 0,
+                "b_0(y), b_1(x), no drift along z");
   const int box = blockIdx.y;
   if (!st.live[box]) return;
   const Box3 B = boxes[box];
@@ -163,23 +179,19 @@ box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, do
   const int64_t q0 = static_cast<int64_t>(blockIdx.x) * plane;
   const int64_t sy = B.u_sy, sz = B.u_sz;
   u += box3_index(B, 1, 1, static_cast<int>(blockIdx.x) + 1);
-  coef += box * 4 * np + q0;
+  f += box * np + q0;
   r += box * np + q0;
-  const double w0 = 0.5 * s2 / (B.h[0] * B.h[0]), w1 = 0.5 * s2 / (B.h[1] * B.h[1]),
-               w2 = 0.5 * s2 / (B.h[2] * B.h[2]);
-  const double diag = c - 2.0 * (w0 + w1 + w2);
+  const double *b0 = drift + (box * 2) * kBox3Axis + 1, *b1 = b0 + kBox3Axis;
+  const double w0 = B.w[0], w1 = B.w[1], w2 = B.w[2], diag = B.diag;
   double acc = 0.0;
+#pragma unroll 2
   for (int q = threadIdx.x; q < plane; q += kBox3Block) {
-    const int j = q / B.P[0];
-    const double *v = u + j * sy + (q - j * B.P[0]);
+    const int j = q / B.P[0], i = q - j * B.P[0];
+    const double *v = u + j * sy + i;
     const double ux0 = v[-1], ux1 = v[1], uy0 = v[-sy], uy1 = v[sy], uz0 = v[-sz], uz1 = v[sz];
     double Au = diag * v[0] + w0 * (ux0 + ux1) + w1 * (uy0 + uy1) + w2 * (uz0 + uz1);
-    double drift = 0.0;
-    if (kDriftAxes & 1u) drift = coef[q] * (ux1 - ux0);
-    if (kDriftAxes & 2u) drift = fma(coef[np + q], uy1 - uy0, drift);
-    if (kDriftAxes & 4u) drift = fma(coef[2 * np + q], uz1 - uz0, drift);
-    Au += drift;
-    const double rv = -coef[3 * np + q] - Au;
+    Au += fma(b1[i], uy1 - uy0, b0[j] * (ux1 - ux0));
+    const double rv = -f[q] - Au;
     r[q] = rv;
     acc = fma(rv, rv, acc);
   }
@@ -207,6 +219,7 @@ box3_residual_kernel(const Box3 *boxes, const __grid_constant__ Box3State st, do
     if (it == 0) st.r0[box] = rn;
     const double r0 = it == 0 ? rn : st.r0[box];
     st.rn[box] = rn;
+    st.inv[box] = 1.0 / rn;
     st.iters[box] = it;
     st.res[box] = r0 > 0.0 ? rn / r0 : 0.0;
     st.ticket[box] = 0;
@@ -308,14 +321,14 @@ static size_t box3_plane_smem(int P0, int P1) {
 }
 
 // The y and x passes of one z plane (blockIdx.x) of box blockIdx.y.  kInverse
-// = false: in is the FP64 residual, scaled by 1 / |r|_2 and rounded, and the
-// result goes to v.  kInverse = true: in place of the residual v, and the
-// result times |r|_2 is added to u.  The sine matrix along x sits in shared
+// = false: in is the FP64 residual, scaled by 1 / |r|_2 (scale) and rounded, and
+// the result goes to v.  kInverse = true: in place of the residual v, and the
+// result times |r|_2 (scale) is added to u.  The sine matrix along x sits in shared
 // memory; along y it is the same one when the box is as long, else read
 // through L1.
 template <bool kInverse>
 __global__ void __launch_bounds__(kBox3Block)
-box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *rn,
+box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *scale,
                   const __grid_constant__ Box3Sines T, const double *r, float *v, double *u) {
   const int box = blockIdx.y;
   if (!live[box]) return;
@@ -327,7 +340,7 @@ box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *rn,
   float *Tt = Sx + P0 * ld0;     // [x][y]: after the y pass
   float *Tn = Tt + P0 * ldt;     // [y][x]: the plane
   const int64_t off = box * box3_np(B) + static_cast<int64_t>(blockIdx.x) * plane;
-  const double sc = kInverse ? rn[box] : 1.0 / rn[box];
+  const double sc = scale[box];
   for (int e = threadIdx.x; e < P0 * ld0; e += kBox3Block) Sx[e] = T.S[0][e];
   for (int e = threadIdx.x; e < plane; e += kBox3Block)
     Tn[e] = kInverse ? v[off + e] : static_cast<float>(r[off + e] * sc);
@@ -439,10 +452,16 @@ box3_jacobi_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, 
 // say, u_span values of d_u in all).  *iters and *resid (if non-null) get the
 // largest count and relative residual over the boxes; iters_each / resid_each
 // (host, one entry per box, may be null) get each box's own.
-static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int32_t method,
+static pdd_status solve_boxes(pdd_ctx *ctx, std::vector<Box3> &boxes, int32_t method,
                               int64_t max_iter, double tol, const double *d_face, double *d_u,
                               int64_t u_span, int64_t *iters, double *resid, int64_t *iters_each,
                               double *resid_each) {
+  const double s2 = ctx->prob.sigma * ctx->prob.sigma;
+  const double c = constant_kill(ctx->prob.kind);
+  for (Box3 &B : boxes) {
+    for (int a = 0; a < 3; ++a) B.w[a] = 0.5 * s2 / (B.h[a] * B.h[a]);
+    B.diag = c - 2.0 * (B.w[0] + B.w[1] + B.w[2]);
+  }
   const int32_t nb = static_cast<int32_t>(boxes.size());
   const Box3 &B0 = boxes[0];
   const bool jacobi = method == PDD_STENCIL_JACOBI;
@@ -465,12 +484,14 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
   const size_t off_res = take(NB * sizeof(double));
   const size_t state_bytes = o;
   const size_t off_rn = take(NB * sizeof(double));
+  const size_t off_inv = take(NB * sizeof(double));
   const size_t off_r0 = take(NB * sizeof(double));
   const size_t off_live = take(NB * sizeof(int32_t));
   const size_t off_ticket = take(NB * sizeof(int32_t));
   const size_t off_nlive = take(sizeof(int32_t));
   const size_t off_box = take(NB * sizeof(Box3));
-  const size_t off_coef = take(NB * 4 * np * sizeof(double));
+  const size_t off_coef = take(NB * (jacobi ? 4 : 1) * np * sizeof(double));
+  const size_t off_drift = take(NB * 2 * kBox3Axis * sizeof(double));
   const size_t off_part = take(NB * std::max(nblk, B0.P[2]) * sizeof(double));
   const size_t off_un = take(jacobi ? u_span * sizeof(double) : 0);
   const size_t off_r = take(jacobi ? 0 : NB * np * sizeof(double));
@@ -488,6 +509,7 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
   int32_t *live = reinterpret_cast<int32_t *>(base + off_live);
   Box3 *d_boxes = reinterpret_cast<Box3 *>(base + off_box);
   double *coef = reinterpret_cast<double *>(base + off_coef);
+  double *drift = reinterpret_cast<double *>(base + off_drift);
   double *part = reinterpret_cast<double *>(base + off_part);
   double *un = reinterpret_cast<double *>(base + off_un);
 
@@ -503,13 +525,11 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
   const dim3 gset(static_cast<unsigned>(B0.n[2]), nb);
   if (jacobi)
     box3_setup_kernel<EllipticManufactured, false><<<gset, kBox3Block, 0, ctx->stream>>>(
-        d_boxes, ctx->mc, d_face, d_u, coef);
+        d_boxes, ctx->mc, d_face, d_u, coef, drift);
   else
     box3_setup_kernel<EllipticManufactured, true><<<gset, kBox3Block, 0, ctx->stream>>>(
-        d_boxes, ctx->mc, d_face, d_u, coef);
+        d_boxes, ctx->mc, d_face, d_u, coef, drift);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
-  const double s2 = ctx->prob.sigma * ctx->prob.sigma;
-  const double c = constant_kill(ctx->prob.kind);
   const unsigned gcomb = static_cast<unsigned>((nb + 127) / 128);
   const auto ev = prof_slot(ctx);
   if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, ctx->stream));
@@ -576,6 +596,7 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
     }
     Box3State S;
     S.rn = rn;
+    S.inv = reinterpret_cast<double *>(base + off_inv);
     S.r0 = reinterpret_cast<double *>(base + off_r0);
     S.res = reinterpret_cast<double *>(base + off_res);
     S.iters = reinterpret_cast<int64_t *>(base + off_it);
@@ -610,8 +631,8 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
     // device never waits for it; what it enqueues after the last box has
     // stopped returns at once.
     for (int64_t it = 0;; ++it) {
-      box3_residual_kernel<EllipticManufactured::kDriftAxes><<<gp, kBox3Block, 0, ctx->stream>>>(
-          d_boxes, S, s2, c, d_u, coef, r, part, it, max_iter, tol);
+      box3_residual_kernel<EllipticManufactured><<<gp, kBox3Block, 0, ctx->stream>>>(
+          d_boxes, S, d_u, coef, drift, r, part, it, max_iter, tol);
       PDD_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->watch + (it & 1), S.n_live, sizeof(int32_t),
                                         cudaMemcpyDeviceToHost, ctx->stream));
       PDD_CUDA_TRY(ctx, cudaEventRecord(ctx->watch_ev[it & 1], ctx->stream));
@@ -619,7 +640,7 @@ static pdd_status solve_boxes(pdd_ctx *ctx, const std::vector<Box3> &boxes, int3
         PDD_CUDA_TRY(ctx, cudaEventSynchronize(ctx->watch_ev[(it - 1) & 1]));
         if (ctx->watch[(it - 1) & 1] == 0) break;
       }
-      box3_plane_kernel<false><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, rn, T, r, v, nullptr);
+      box3_plane_kernel<false><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, S.inv, T, r, v, nullptr);
       box3_z_kernel<<<gz, kBox3Block, smem_z, ctx->stream>>>(P0, P1, P2, live, T, fac, fac_stride, v);
       box3_plane_kernel<true><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, rn, T, nullptr, v, d_u);
       PDD_CUDA_TRY(ctx, cudaGetLastError());
