@@ -17,7 +17,7 @@
 #include <cstring>
 
 #include "ctx.hpp"
-#include "path_kernel.cuh"
+#include "grad_kernel.cuh"
 #include "reduce.cuh"
 
 namespace pdd {
@@ -286,21 +286,12 @@ pdd_status interface_grad_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   a.score = rec;
   a.rk = make_round_keys(mc->seed);
   const double sig = ctx->prob.sigma, dt = mc->dt;
-  a.inv_s2dt = 1.0 / (sig * sig * dt);
-  a.dt_d = dt;
-  a.sdt_d = sig * std::sqrt(dt);
-  a.thr_d = 9.0 * sig * sig * dt;
-  a.ecdt_d = 1.0;
-  a.dt_f = static_cast<float>(dt);
-  a.sdt_f = static_cast<float>(a.sdt_d);
-  a.thr_f = static_cast<float>(a.thr_d);
-  a.l2cdt_f = 0.0f;
+  path_step_args(a, sig, dt, 0.0, mc->bridge != 0, 2);
   a.lr_scale = static_cast<float>(std::sqrt(dt) / sig);
   a.max_steps = static_cast<int32_t>(mc->max_steps);
-  a.bridge = mc->bridge ? 1 : 0;
   a.mc = ctx->mc;
 
-  auto kern = path_kernel<PoissonFourier, Box<2>, float, true>;
+  auto kern = path_lr_kernel<PoissonFourier, Box<2>, float>;
   int bps = 0;
   PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPathBlockOf<float>, 0));
   if (bps < 1) bps = 1;

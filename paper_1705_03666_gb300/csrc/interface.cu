@@ -93,17 +93,8 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   a.rk = make_round_keys(mc->seed);
   const double sig = ctx->prob.sigma, dt = mc->dt;
   const double c_kill = constant_kill(ctx->prob.kind);
-  a.inv_s2dt = 1.0 / (sig * sig * dt);
-  a.dt_d = dt;
-  a.sdt_d = sig * std::sqrt(dt);
-  a.thr_d = 9.0 * sig * sig * dt;
-  a.ecdt_d = std::exp(c_kill * dt);
-  a.dt_f = static_cast<float>(a.dt_d);
-  a.sdt_f = static_cast<float>(a.sdt_d);
-  a.thr_f = static_cast<float>(a.thr_d);
-  a.l2cdt_f = static_cast<float>(c_kill * dt * 1.4426950408889634);
+  path_step_args(a, sig, dt, c_kill, mc->bridge != 0, Geom::reach(sig * std::sqrt(dt)));
   a.max_steps = static_cast<int32_t>(mc->max_steps);
-  a.bridge = mc->bridge ? 1 : 0;
   a.mc = ctx->mc;
   if (diag) {
     a.dump_score = diag->d_path_score;
@@ -113,15 +104,15 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
 
   auto kern = path_kernel<Model, Geom, R>;
   int bps = 0;
-  PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPathBlockOf<R>, 0));
+  PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kForwardBlock, 0));
   if (bps < 1) bps = 1;
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
-  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kPathBlockOf<R> - 1) / kPathBlockOf<R>));
+  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kForwardBlock - 1) / kForwardBlock));
 
   const auto ev = prof_slot(ctx);
   if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, ctx->stream));
-  kern<<<static_cast<unsigned>(grid), kPathBlockOf<R>, 0, ctx->stream>>>(a);
+  kern<<<static_cast<unsigned>(grid), kForwardBlock, 0, ctx->stream>>>(a);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
   fix_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(

@@ -212,6 +212,18 @@ struct Box {
     for (int k = 0; k < D; ++k) in = in && (x[k] > R(0)) && (x[k] < R(1));
     return in;
   }
+  // Lower bound on the distance to every face, 1/2 - max_k |x_k - 1/2| (exact
+  // up to rounding); <= 0 unless the point is strictly inside (x_k - 1/2 rounds
+  // monotonically, so a coordinate outside (0, 1) cannot give less than 1/2).
+  __device__ __forceinline__ static float edge(const float *x) {
+    float m = fabsf(x[0] - 0.5f);
+    if constexpr (D == 2) m = fmaxf(m, fabsf(x[1] - 0.5f));
+    if constexpr (D == 3) m = max3_abs(m, x[1] - 0.5f, x[2] - 0.5f);
+    return 0.5f - m;
+  }
+  // The most faces within bridge reach of one step (opposite ones cannot both
+  // be while sigma^2 dt <= 1/36).
+  static int reach(double) { return D; }
   // Distance to the plane of face j, positive on the domain side.
   template <typename R>
   __device__ __forceinline__ static R face_dist(int j, const R *x) {
@@ -333,6 +345,19 @@ struct LShape {
     return x[0] > R(0) && x[0] < R(1) && x[1] > R(0) && x[1] < R(1) &&
            !(x[0] >= R(0.5) && x[1] >= R(0.5));
   }
+  // Lower bound on the distance to every face: the square's sides as for the
+  // box, and the notch by the larger of 1/2 - x and 1/2 - y, which bounds the
+  // distance to both notch edges (a segment's distance is at least each of its
+  // coordinate distances); <= 0 outside the open domain.
+  __device__ __forceinline__ static float edge(const float *x) {
+    const float p = x[0] - 0.5f, q = x[1] - 0.5f;
+    return fminf(0.5f - fmaxf(fabsf(p), fabsf(q)), -fminf(p, q));
+  }
+  // The most faces within bridge reach of one step.  A face within reach has
+  // d d' < 9 s^2 (s = sigma sqrt(dt)) and |d - d'| <= 5.77 s (the largest
+  // Box-Muller radius), so both ends lie within 7.06 s of it; below 1/4 that
+  // leaves the two faces of one corner (no two others come closer than 1/2).
+  static int reach(double s) { return 7.06 * s < 0.25 ? 2 : kFaces; }
   template <typename R>
   __device__ __forceinline__ static R face_dist(int j, const R *x) {
     if (j < 4) {

@@ -2,15 +2,12 @@
 //
 // One persistent launch advances every (node, path) of a wave of the global,
 // node-major path index space g = node * n_paths + p.  Each lane owns one
-// path at a time; when its path exits the lane takes the next path from its
-// warp's stash of set-up paths (refilled 32 indices at a time from an atomic
-// cursor), so no lane waits for a long path of another node (lane refill) and
-// the only idle time is at the very end of the wave.
-// Ended paths are parked per warp and scored 32 at a time, and the scores are
-// added at once to exact per-node integer sums (nodefix.cuh), so the per-node
-// mean and standard error do not depend on which lane ran which path and no
-// per-path score is stored (the gradient mode keeps a per-path record for its
-// Jacobian reduction).
+// path at a time and takes the next one from its warp's stash of set-up paths
+// (refilled 32 indices at a time from an atomic cursor), so no lane waits for
+// a long path of another node and the only idle time is at the very end of
+// the wave.  Scores are added at once to exact per-node integer sums
+// (nodefix.cuh), so the per-node mean and standard error do not depend on
+// which lane ran which path and no per-path score is stored.
 //
 // Per step (Eq. 2.8, Dirichlet/elliptic reduction of Sec. 2.2, left-point rule):
 //   X' = X + b(X) dt + sigma sqrt(dt) xi,  Y' = Y e^{c(X) dt},  Z' = Z + f(X) Y dt,
@@ -19,11 +16,21 @@
 // U < P = 1 - prod_j (1 - exp(-2 d_j d'_j / (sigma^2 dt))) over faces with
 // 2 d_j d'_j < 18 sigma^2 dt (exit point = X' projected on the face with the
 // largest term).  P is accumulated without cancellation (bridge_exit) and
-// near-ties of the FP32 path are decided in FP64.  Both tests sit behind one
-// screen: the smallest d d' (> 0 proves X' inside) and a union bound on P
-// above which no crossing is possible, so most steps form neither.
-// Score = g(X_tau) Y' + Z' (Eq. 2.7).
+// near-ties of the FP32 path are decided in FP64.  Score = g(X_tau) Y' + Z'
+// (Eq. 2.7).
+//
+// What bounds it: instruction issue (no contraction, next to no bytes), and
+// with it the lanes that an instruction finds idle.  So the four steps of a
+// unit run without a branch: a lane only notes whether any of them could have
+// been an exit (fast_unit: one bound per step on the distance to the
+// boundary, conservative against every test above).  A unit so noted is not
+// taken: its start is parked, the lane takes another path, and the warp runs
+// 32 parked units together, with the exact tests, all lanes busy
+// (recheck_units).  Paths that exited there are scored at once; false alarms
+// (about one per path) go back to the stash.
 #pragma once
+
+#include <cmath>
 
 #include "common.cuh"
 #include "models.cuh"
@@ -39,6 +46,8 @@ namespace pdd {
 // was 11.4 against 13.0 ms).
 template <typename R>
 constexpr int kPathBlockOf = sizeof(R) == 4 ? 128 : 256;
+
+constexpr int kForwardBlock = 128;  // the forward path kernel, both precisions
 
 struct PathArgs {
   const double *nodes;          // [n_nodes][D]
@@ -61,6 +70,7 @@ struct PathArgs {
   float l2cdt_f;                // c dt log2(e) for constant killing (FP32)
   int32_t max_steps;
   int32_t bridge;
+  float edge_c1, edge_c0;       // fast_unit's bound (see path_step_args)
   float lr_scale;               // sqrt(dt) / sigma (gradient mode)
   ModelConst mc;
 };
@@ -74,6 +84,41 @@ struct PathArgs {
 // log2 of a face count (the union bound's factor), counts 1 .. 6.
 constexpr float kLog2Count[7] = {0.0f, 0.0f, 1.0f, 1.5849625007211562f, 2.0f,
                                  2.321928094887362f, 2.584962500721156f};
+
+// Step constants of a launch from dt, sigma, the killing rate and the bridge
+// flag (host).  kReach: the most faces that can be within bridge reach of one
+// step together.
+//
+// The bound of fast_unit.  With e a lower bound on the distance of a point to
+// every face (Geom::edge; <= 0 outside), every d_j d'_j >= e e', so the step
+// cannot cross while log2 U >= log2 kReach - 2 log2(e) e e' / (sigma^2 dt).
+// log2 U is bounded below by the bits of U read as a fixed-point number
+// (exponent and mantissa: at most 0.086 low), scaled by 2^15 and offset by
+// 2^23: one byte permute.  So the test is
+//   float(2^23 + bits(U) / 2^8) >= edge_c0 + edge_c1 e e',
+// false also for e e' <= 0 (possible exit through the boundary) and for NaN.
+// The margin covers the rounding of the exponents (2^-10 is over four times
+// all of them), the near-tie window of the exact test and the rounding of e
+// (2^-25 absolute, which weighs 2^-25 (e + e') 2.9 / (sigma^2 dt) with e, e'
+// within 12 sigma sqrt(dt) where U can matter: below 2e-6 / (sigma sqrt(dt))).
+// Without the bridge test the slope is -inf: only e e' <= 0 fails.
+inline void path_step_args(PathArgs &a, double sig, double dt, double c_kill, bool bridge,
+                           int kReach) {
+  a.inv_s2dt = 1.0 / (sig * sig * dt);
+  a.dt_d = dt;
+  a.sdt_d = sig * std::sqrt(dt);
+  a.thr_d = 9.0 * sig * sig * dt;
+  a.ecdt_d = std::exp(c_kill * dt);
+  a.dt_f = static_cast<float>(a.dt_d);
+  a.sdt_f = static_cast<float>(a.sdt_d);
+  a.thr_f = static_cast<float>(a.thr_d);
+  a.l2cdt_f = static_cast<float>(c_kill * dt * 1.4426950408889634);
+  a.bridge = bridge ? 1 : 0;
+  const double margin = 0x1p-10 + 4e-6 / a.sdt_d;
+  a.edge_c0 = static_cast<float>(8388608.0 + 32768.0 * (127.0 + std::log2(kReach) + margin));
+  a.edge_c1 = bridge ? static_cast<float>(-2.0 * 1.4426950408889634 * a.inv_s2dt * 32768.0)
+                     : -INFINITY;
+}
 
 template <typename R> struct StepConst;
 template <> struct StepConst<float> {
@@ -101,6 +146,8 @@ template <> struct StepConst<float> {
   __device__ __forceinline__ float kill(float, int32_t n_next) const {
     return ex2_approx(static_cast<float>(n_next) * l2cdt);
   }
+  // the same for a step count held as a float (exact below 2^24)
+  __device__ __forceinline__ float kill_f(float n_next) const { return ex2_approx(n_next * l2cdt); }
   // e^{-a} for a >= 0 (hardware exp2, ~2 ulp; a near-tie decision is redone
   // in FP64 by the caller).
   __device__ __forceinline__ float exp_neg(float a) const {
@@ -263,6 +310,9 @@ static __device__ __noinline__ bool bridge_tie_fp64(float U, float mn, float inv
 // Exit codes of em_step.
 constexpr int kStepContinue = -2;
 constexpr int kStepHardExit = -1;   // >= 0: bridge exit through that face
+// A path stopped by the step cap (set by callers): scored at the projection of
+// its last point on the nearest face.
+constexpr int kStepCapped = -3;
 
 // One Euler-Maruyama step with the exit test.  On kStepContinue, X, Y, Z
 // advance; on an exit, X keeps the start of the step, Xn receives its end,
@@ -486,34 +536,6 @@ __device__ __forceinline__ bool path_unit(const Env &a, const StepConst<R> &k, c
   return true;
 }
 
-// Per-path record of the gradient mode: score, exit point, and the
-// likelihood-ratio sums L_j (already scaled by sqrt(dt)/sigma).
-struct GradRec {
-  float s, x, y, z;
-  float L[kMaxLR];
-};
-
-// Gradient mode: the record's first four words (score and exit point) with
-// the step count, and the likelihood-ratio sums.
-template <int D, typename R>
-__device__ __forceinline__ void write_score(const PathArgs &a, uint64_t slot, R s, int32_t st,
-                                            const R *xe) {
-  float4 *o = reinterpret_cast<float4 *>(static_cast<GradRec *>(a.score) + slot);
-  o[0] = make_float4(static_cast<float>(s), static_cast<float>(xe[0]),
-                     D > 1 ? static_cast<float>(xe[D > 1 ? 1 : 0]) : 0.f,
-                     D > 2 ? static_cast<float>(xe[D > 2 ? 2 : 0]) : 0.f);
-  if (a.steps) a.steps[slot] = st;
-}
-template <typename R>
-__device__ __forceinline__ void write_lr_sums(const PathArgs &a, uint64_t slot, const R *L) {
-  float4 *o = reinterpret_cast<float4 *>(static_cast<GradRec *>(a.score) + slot);
-  const float c = a.lr_scale;
-#pragma unroll
-  for (int q = 0; q < kMaxLR / 4; ++q)
-    o[1 + q] = make_float4(c * static_cast<float>(L[4 * q]), c * static_cast<float>(L[4 * q + 1]),
-                           c * static_cast<float>(L[4 * q + 2]), c * static_cast<float>(L[4 * q + 3]));
-}
-
 // Node of global path index g (32-bit division when the indices fit).
 __device__ __forceinline__ uint64_t path_node(const PathArgs &a, uint64_t g) {
   if (a.end <= 0xffffffffull)
@@ -534,44 +556,125 @@ __device__ __forceinline__ void dump_path(const PathArgs &a, uint64_t slot, R s,
   }
 }
 
-// Per-warp staging in shared memory (one column per lane).  Claiming and
-// setting up a path (atomic, node division, Philox key, FP64 node load) and
-// scoring an ended path (exit point, accurate g) happen once per path, at
-// times that differ from lane to lane: done where they occur, each would run
-// with one lane of the warp active.  Instead a warp claims 32 consecutive
-// paths at once and sets them all up with every lane busy (StartStash), and
-// ended paths are parked (ExitQueue) and scored 32 at a time.  Every path
-// writes its own slot, so the results do not depend on this order.
-template <int D, typename R>
-struct StartStash {
-  unsigned long long slot[32];  // index in the wave
-  uint32_t w0[32], w1[32];      // PhiloxPath words (tag 0)
-  R x[D][32];                   // start point
+// The log2 of fast_unit's bound: 2^23 + (bits of U >> 8) as a float.
+__device__ __forceinline__ float unif_log_bits(float U) {
+  return __uint_as_float(__byte_perm(__float_as_uint(U), 0x4b000000u, 0x7321u));
+}
+
+// Distance bound of a point (binary32 also for binary64 paths: path_step_args'
+// margin covers the rounding).
+template <class Geom, typename R>
+__device__ __forceinline__ float path_edge(const R *X) {
+  float x[Geom::D];
+#pragma unroll
+  for (int d = 0; d < Geom::D; ++d) x[d] = static_cast<float>(X[d]);
+  return Geom::edge(x);
+}
+
+// The four steps of the unit at step n (em_step's arithmetic), without exit
+// tests: returns whether any step may have been an exit (the unit is then not
+// taken).  e: path_edge of X, advanced with it.  n < 2^24 - 4.
+template <class Model, class Geom, typename R>
+__device__ __forceinline__ bool fast_unit(const PathArgs &a, const StepConst<R> &k, const R *z,
+                                          const uint32_t *u, int32_t n, R *X, R &Y, R &Z,
+                                          float &e) {
+  constexpr int D = Model::D;
+  bool maybe = false;
+  const float nf = static_cast<float>(n);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    R b[D], Xn[D];
+    R f = R(0);
+#pragma unroll
+    for (int d = 0; d < D; ++d) b[d] = R(0);
+    if constexpr (Model::kDrift || Model::kSource) Model::coeffs(a.mc, X, b, f);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      if ((Model::kDriftAxes >> d) & 1u)
+        Xn[d] = X[d] + b[d] * k.dt + k.sdt * z[D * j + d];
+      else
+        Xn[d] = X[d] + k.sdt * z[D * j + d];
+    }
+    if constexpr (Model::kSource) Z = Z + f * Y * k.dt;
+    if constexpr (Model::kKill == 1) {
+      if constexpr (sizeof(R) == 4) Y = k.kill_f(nf + static_cast<float>(j + 1));
+      else Y = k.kill(Y, n + j + 1);
+    }
+    const float en = path_edge<Geom, R>(Xn);
+    maybe |= !(unif_log_bits(unif_f(u[j])) >= fmaf(a.edge_c1, e * en, a.edge_c0));
+    e = en;
+#pragma unroll
+    for (int d = 0; d < D; ++d) X[d] = Xn[d];
+  }
+  return maybe;
+}
+
+// The unit at step n again, a step at a time with the exact tests (em_step)
+// and the step cap; the random numbers are shifted down by static indices so
+// that one copy of the step serves all four.
+template <class Model, class Geom, typename R>
+__device__ __forceinline__ int exact_unit(const PathArgs &a, const StepConst<R> &k,
+                                          const PhiloxPath &pp, R *X, R &Y, R &Z, int32_t &n,
+                                          R *Xn) {
+  constexpr int D = Model::D;
+  R z[4 * D];
+  uint32_t u[4];
+  unit_randoms<D, R>(n, pp, a.rk, z, u);
+  int code = kStepContinue;
+#pragma unroll 1
+  for (int j = 0; j < 4; ++j) {
+    code = em_step<Model, Geom, R, false>(a, k, X, Y, Z, z, u[0], n, Xn, static_cast<R *>(nullptr));
+    ++n;
+    if (code != kStepContinue || n >= a.max_steps) break;
+#pragma unroll
+    for (int i = 0; i < 3 * D; ++i) z[i] = z[i + D];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = u[i + 1];
+  }
+  return code;
+}
+
+// Paths at the start of a unit, N of them, in shared memory.  A path's
+// killing weight Y is a function of n in binary32 (and 1 without killing):
+// only binary64 paths with killing keep it.
+template <int D, typename R, bool kY, int N>
+struct PathStash {
+  unsigned long long slot[N];   // index in the wave
+  uint32_t w0[N], w1[N];        // PhiloxPath words (tag 0)
+  int32_t n[N];                 // steps taken
+  R x[D][N], z[N];
+  R y[kY ? N : 1];
 };
-template <int D, typename R>
-struct ExitQueue {
-  unsigned long long slot[32];
-  int32_t st[32], code[32];     // step count (or -max_steps) and exit code
-  R x[D][32], xn[D][32], y[32], z[32];
-};
-template <int D, typename R>
-struct PathStage {
-  StartStash<D, R> start;
-  ExitQueue<D, R> exit;
+// Per warp: the paths to take (a stack) and the units to recheck (a ring).
+// The ring holds at most 31 + 32 units (32 are taken out whenever there are as
+// many).  New paths come in 32 at a time, only into an empty stack, beside at
+// most 31 busy lanes and 31 parked units: so a warp never holds more than 94
+// paths, and the stack never more than that.
+constexpr int kStashCap = 96, kCheckCap = 64;
+template <int D, typename R, bool kY>
+struct ForwardStage {
+  PathStash<D, R, kY, kStashCap> start;
+  PathStash<D, R, kY, kCheckCap> check;
 };
 
-// Exit code of a path stopped by the step cap: scored at the projection of
-// its last point on the nearest face.
-constexpr int kStepCapped = -3;
+template <class Model, typename R>
+constexpr bool kKeepY = Model::kKill == 1 && sizeof(R) == 8;
 
-// Called by all 32 lanes: claim the next 32 indices of the wave, set each up,
-// score at once the ones that start on the boundary (tau = 0, u = g, Eq. 2.1)
-// or outside the closed domain (invalid input: NaN, counted), and stage the
-// interior ones.  Returns how many were staged (warp-uniform).
-template <class Model, class Geom, typename R, bool kLR>
-__device__ __forceinline__ int stage_starts(const PathArgs &a, StartStash<Model::D, R> &st,
-                                            unsigned long long span, bool &exhausted,
-                                            unsigned long long &my_bad) {
+// Y of a path that has taken n steps.
+template <class Model, typename R>
+__device__ __forceinline__ R path_weight(const StepConst<R> &k, int32_t n, R kept) {
+  if constexpr (kKeepY<Model, R>) return kept;
+  else if constexpr (Model::kKill == 1) return k.kill(R(1), n);  // e^0 = 1 exactly
+  else return R(1);
+}
+
+// Called by all 32 lanes with an empty stash: claim the next 32 indices of the
+// wave, set each up, score at once the ones that start on the boundary (tau =
+// 0, u = g, Eq. 2.1) or outside the closed domain (invalid input: NaN,
+// counted), and stash the interior ones.  Returns how many (warp-uniform).
+template <class Model, class Geom, typename R, class Stash>
+__device__ __forceinline__ int stash_starts(const PathArgs &a, Stash &st, unsigned long long span,
+                                            bool &exhausted, unsigned long long &my_bad) {
   constexpr int D = Model::D;
   const unsigned lane = threadIdx.x & 31u;
   __syncwarp();  // earlier reads of the stash are done
@@ -600,30 +703,22 @@ __device__ __forceinline__ int stage_starts(const PathArgs &a, StartStash<Model:
         s0 = R(NAN);
         ++my_bad;
       }
-      if constexpr (kLR) {
-        R L0[kMaxLR];
-#pragma unroll
-        for (int j = 0; j < kMaxLR; ++j) L0[j] = R(0);
-        write_score<D, R>(a, q, s0, 0, x);
-        write_lr_sums<R>(a, q, L0);
-      } else {
-        dump_path<D, R>(a, q, s0, 0, x);
-      }
+      dump_path<D, R>(a, q, s0, 0, x);
     }
   }
-  if constexpr (!kLR) {
-    // starts on the boundary (u = g, tau = 0) or outside the closed domain
-    // (NaN) go straight into the node's sums
-    const bool at_bnd = q < span && !interior;
-    if (__any_sync(kFull, at_bnd))
-      fix_commit<R>(a.fix, at_bnd, node, s0, false, true);
-  }
+  // starts on the boundary (u = g, tau = 0) or outside the closed domain (NaN)
+  // go straight into the node's sums
+  const bool at_bnd = q < span && !interior;
+  if (__any_sync(kFull, at_bnd)) fix_commit<R>(a.fix, at_bnd, node, s0, false, true);
   const unsigned im = __ballot_sync(kFull, interior);
   if (interior) {
     const int e = __popc(im & ((1u << lane) - 1u));
     st.slot[e] = q;
     st.w0[e] = pp.r0_w0;
     st.w1[e] = pp.r0_w1;
+    st.n[e] = 0;
+    st.z[e] = R(0);
+    if constexpr (kKeepY<Model, R>) st.y[e] = R(1);
 #pragma unroll
     for (int d = 0; d < D; ++d) st.x[d][e] = x[d];
   }
@@ -631,75 +726,105 @@ __device__ __forceinline__ int stage_starts(const PathArgs &a, StartStash<Model:
   return __popc(im);
 }
 
-// Called by all 32 lanes: score the first cnt parked paths, one per lane, and
-// add the scores to their nodes' sums (gradient mode: write the record's score
-// and exit point; the likelihood-ratio sums were written when the path ended).
-template <class Model, class Geom, typename R, bool kLR>
-__device__ __forceinline__ void flush_exits(const PathArgs &a, ExitQueue<Model::D, R> &q, int cnt) {
+// Called by all 32 lanes: the cnt (<= 32) oldest parked units (from ring
+// position head) run with the exact tests, one per lane.  Paths that end are
+// scored and added to their nodes' sums; the others are pushed on the stash
+// (n_start of it filled).
+template <class Model, class Geom, typename R, class Stage>
+__device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst<R> &k, Stage &st,
+                                              int head, int cnt, int &n_start,
+                                              unsigned long long &my_steps,
+                                              unsigned long long &my_capped) {
   constexpr int D = Model::D;
   const int lane = static_cast<int>(threadIdx.x & 31u);
   __syncwarp();
-  R s = R(0);
+  const bool has = lane < cnt;
+  bool ends = false, capped = false;
+  R s = R(0), X[D], Xn[D], Y = R(1), Z = R(0);
+  PhiloxPath pp{0, 0, 0};
+  unsigned long long slot = 0;
   uint64_t node = 0;
-  bool capped = false;
-  if (lane < cnt) {
-    R X[D], Xn[D], xe[D];
+  int32_t n = 0;
+  if (has) {
+    const int e = (head + lane) & (kCheckCap - 1);
+    slot = st.check.slot[e];
+    pp.r0_w0 = st.check.w0[e];
+    pp.r0_w1 = st.check.w1[e];
+    n = st.check.n[e];
+    Z = st.check.z[e];
+    R y = R(1);
+    if constexpr (kKeepY<Model, R>) y = st.check.y[e];
+    Y = path_weight<Model, R>(k, n, y);
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      X[d] = q.x[d][lane];
-      Xn[d] = q.xn[d][lane];
-    }
-    const int code = q.code[lane];
-    capped = code == kStepCapped;
-    if (capped) {
+    for (int d = 0; d < D; ++d) X[d] = st.check.x[d][e];
+    const int code = exact_unit<Model, Geom, R>(a, k, pp, X, Y, Z, n, Xn);
+    capped = code == kStepContinue && n >= a.max_steps;
+    ends = capped || code != kStepContinue;
+    if (ends) {
+      R xe[D];
+      if (capped) {  // scored at the projection of its last point on the nearest face
 #pragma unroll
-      for (int d = 0; d < D; ++d) xe[d] = X[d];
-      Geom::project(Geom::nearest_face(X), xe);
-      s = Model::g(a.mc, xe) * q.y[lane] + q.z[lane];
-    } else {
-      s = exit_score<Model, Geom, R>(a.mc, code, X, Xn, q.y[lane], q.z[lane], xe);
-    }
-    if constexpr (kLR) {
-      write_score<D, R>(a, q.slot[lane], s, q.st[lane], xe);
-    } else {
-      node = path_node(a, a.begin + q.slot[lane]);
-      dump_path<D, R>(a, q.slot[lane], s, q.st[lane], xe);
+        for (int d = 0; d < D; ++d) xe[d] = X[d];
+        Geom::project(Geom::nearest_face(X), xe);
+        s = Model::g(a.mc, xe) * Y + Z;
+        ++my_capped;
+      } else {
+        s = exit_score<Model, Geom, R>(a.mc, code, X, Xn, Y, Z, xe);
+      }
+      my_steps += static_cast<unsigned long long>(n);
+      node = path_node(a, a.begin + slot);
+      dump_path<D, R>(a, slot, s, capped ? -a.max_steps : n, xe);
     }
   }
-  if constexpr (!kLR) fix_commit<R>(a.fix, lane < cnt, node, s, capped, false);
+  const unsigned back = __ballot_sync(kFull, has && !ends);
+  if (has && !ends) {
+    const int e = n_start + __popc(back & ((1u << lane) - 1u));
+    st.start.slot[e] = slot;
+    st.start.w0[e] = pp.r0_w0;
+    st.start.w1[e] = pp.r0_w1;
+    st.start.n[e] = n;
+    st.start.z[e] = Z;
+    if constexpr (kKeepY<Model, R>) st.start.y[e] = Y;
+#pragma unroll
+    for (int d = 0; d < D; ++d) st.start.x[d][e] = X[d];
+  }
+  n_start += __popc(back);
+  fix_commit<R>(a.fix, ends, node, s, capped, false);
   __syncwarp();
 }
 
-template <class Model, class Geom, typename R, bool kLR = false>
-__global__ void __launch_bounds__(kPathBlockOf<R>)
-path_kernel(const __grid_constant__ PathArgs a) {
+template <class Model, class Geom, typename R>
+__global__ void __launch_bounds__(kForwardBlock) path_kernel(const __grid_constant__ PathArgs a) {
   constexpr int D = Model::D;
-  constexpr int NL = kLR ? kMaxLR : 1;
-  __shared__ PathStage<D, R> stage_all[kPathBlockOf<R> / 32];
-  PathStage<D, R> &stage = stage_all[threadIdx.x >> 5];
-  R L[NL];
+  using Stage = ForwardStage<D, R, kKeepY<Model, R>>;
+  __shared__ Stage stage_all[kForwardBlock / 32];
+  Stage &stage = stage_all[threadIdx.x >> 5];
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;
   const StepConst<R> k(a);
   const unsigned long long span = a.end - a.begin;
-  R X[D], Xn[D];
-  R Y = R(1), Z = R(0);
+  // the last unit start that cannot reach the step cap (nor a step count that
+  // binary32 does not hold)
+  const int32_t last_fast = (a.max_steps < (1 << 24) ? a.max_steps : 1 << 24) - 4;
+  R X[D], Y = R(1), Z = R(0);
+  float e = 0.0f;
   PhiloxPath pp{0, 0, 0};
   unsigned long long slot = 0;
   int32_t n = 0;
   bool active = false;
-  int n_start = 0, n_exit = 0;  // stash / queue fill (warp-uniform)
+  int n_start = 0;              // stash fill; parked units and the oldest (warp-uniform)
+  int n_check = 0, head = 0;
   bool exhausted = false;       // the wave's indices are all claimed (warp-uniform)
   unsigned long long my_steps = 0, my_capped = 0, my_bad = 0;
 
   for (;;) {
-    // ---- idle lanes take staged paths; the stash is refilled when empty
-    unsigned needmask = __ballot_sync(kFull, !active);
-    if (needmask) {
+    // ---- idle lanes take stashed paths; the stash is refilled when empty
+    // (not while 32 units wait for their recheck)
+    unsigned needmask = n_check < 32 ? __ballot_sync(kFull, !active) : 0u;
     while (needmask) {
       if (n_start == 0) {
         if (exhausted) break;
-        n_start = stage_starts<Model, Geom, R, kLR>(a, stage.start, span, exhausted, my_bad);
+        n_start = stash_starts<Model, Geom, R>(a, stage.start, span, exhausted, my_bad);
         continue;
       }
       const int cnt = __popc(needmask);
@@ -707,71 +832,67 @@ path_kernel(const __grid_constant__ PathArgs a) {
       if (!active) {
         const int r = __popc(needmask & lt_mask);
         if (r < take) {
-          const int e = n_start - 1 - r;
-          slot = stage.start.slot[e];
-          pp.r0_w0 = stage.start.w0[e];
-          pp.r0_w1 = stage.start.w1[e];
+          const int i = n_start - 1 - r;
+          slot = stage.start.slot[i];
+          pp.r0_w0 = stage.start.w0[i];
+          pp.r0_w1 = stage.start.w1[i];
           pp.tag = 0u;
+          n = stage.start.n[i];
+          Z = stage.start.z[i];
+          R y = R(1);
+          if constexpr (kKeepY<Model, R>) y = stage.start.y[i];
+          Y = path_weight<Model, R>(k, n, y);
 #pragma unroll
-          for (int d = 0; d < D; ++d) X[d] = stage.start.x[d][e];
-          Y = R(1);
-          Z = R(0);
-          n = 0;
-#pragma unroll
-          for (int j = 0; j < NL; ++j) L[j] = R(0);
+          for (int d = 0; d < D; ++d) X[d] = stage.start.x[d][i];
+          e = path_edge<Geom, R>(X);
           active = true;
         }
       }
       n_start -= take;
       needmask = __ballot_sync(kFull, !active);
     }
-    if (!__any_sync(kFull, active)) break;
-    }
 
-    // ---- advance the lane's path by one unit
-    int code = kStepContinue;
-    bool done = false;
-    if (active) {
-      code = path_unit_code<Model, Geom, R, kLR, true>(a, k, pp, a.rk, a.max_steps, X, Y, Z, n, Xn, L);
-      done = code != kStepContinue || n >= a.max_steps;
-      if (done) {
-        my_steps += static_cast<unsigned long long>(n);
-        if (code == kStepContinue) {
-          code = kStepCapped;
-          ++my_capped;
-        }
-      }
+    // ---- parked units: 32 together, or what there is when lanes would idle
+    // without them (the wave's end)
+    if (n_check >= 32 || (needmask && n_check > 0)) {
+      const int cnt = n_check < 32 ? n_check : 32;
+      recheck_units<Model, Geom, R>(a, k, stage, head, cnt, n_start, my_steps, my_capped);
+      head = (head + cnt) & (kCheckCap - 1);
+      n_check -= cnt;
+      continue;
     }
+    if (needmask == kFull) break;
 
-    // ---- ended paths: parked, and scored 32 at a time (gradient mode writes
-    // the likelihood-ratio sums at once)
-    const unsigned dm = __ballot_sync(kFull, done);
-    if (dm) {
-      const int nd = __popc(dm);
-      if (n_exit + nd > 32) {
-        flush_exits<Model, Geom, R, kLR>(a, stage.exit, n_exit);
-        n_exit = 0;
-      }
-      if (done) {
-        if constexpr (kLR) write_lr_sums<R>(a, slot, L);
-        const int e = n_exit + __popc(dm & lt_mask);
-        ExitQueue<D, R> &q = stage.exit;
-        q.slot[e] = slot;
-        q.st[e] = code == kStepCapped ? -a.max_steps : n;
-        q.code[e] = code;
+    // ---- one unit of the lane's path; a unit that may hold an exit, or reach
+    // the step cap, is parked as it started
+    bool park = false;
+    R X0[D], Z0 = Z, Y0 = Y;
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-          q.x[d][e] = X[d];
-          q.xn[d][e] = Xn[d];
-        }
-        q.y[e] = Y;
-        q.z[e] = Z;
+    for (int d = 0; d < D; ++d) X0[d] = X[d];
+    if (active) {
+      R z[4 * D];
+      uint32_t u[4];
+      unit_randoms<D, R>(n, pp, a.rk, z, u);
+      park = fast_unit<Model, Geom, R>(a, k, z, u, n, X, Y, Z, e) || n > last_fast;
+      n += 4;
+    }
+    const unsigned pm = __ballot_sync(kFull, park);
+    if (pm) {
+      if (park) {
+        const int i = (head + n_check + __popc(pm & lt_mask)) & (kCheckCap - 1);
+        stage.check.slot[i] = slot;
+        stage.check.w0[i] = pp.r0_w0;
+        stage.check.w1[i] = pp.r0_w1;
+        stage.check.n[i] = n - 4;
+        stage.check.z[i] = Z0;
+        if constexpr (kKeepY<Model, R>) stage.check.y[i] = Y0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) stage.check.x[d][i] = X0[d];
         active = false;
       }
-      n_exit += nd;
+      n_check += __popc(pm);
     }
   }
-  if (n_exit > 0) flush_exits<Model, Geom, R, kLR>(a, stage.exit, n_exit);
 
   // ---- per-warp totals
 #pragma unroll

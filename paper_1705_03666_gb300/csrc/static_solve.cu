@@ -115,17 +115,8 @@ pdd_status run_static(char *base, int device, cudaStream_t stream, const pdd_pro
   a.rk = make_round_keys(mc->seed);
   const double sig = prob->sigma, dt = mc->dt;
   const double c_kill = constant_kill(prob->kind);
-  a.inv_s2dt = 1.0 / (sig * sig * dt);
-  a.dt_d = dt;
-  a.sdt_d = sig * std::sqrt(dt);
-  a.thr_d = 9.0 * sig * sig * dt;
-  a.ecdt_d = std::exp(c_kill * dt);
-  a.dt_f = static_cast<float>(a.dt_d);
-  a.sdt_f = static_cast<float>(a.sdt_d);
-  a.thr_f = static_cast<float>(a.thr_d);
-  a.l2cdt_f = static_cast<float>(c_kill * dt * 1.4426950408889634);
+  path_step_args(a, sig, dt, c_kill, mc->bridge != 0, Geom::reach(sig * std::sqrt(dt)));
   a.max_steps = static_cast<int32_t>(mc->max_steps);
-  a.bridge = mc->bridge ? 1 : 0;
   a.mc.n_params = prob->n_params;
   for (int i = 0; i < prob->n_params; ++i) {
     a.mc.prm[i] = prob->params[i];
@@ -134,12 +125,12 @@ pdd_status run_static(char *base, int device, cudaStream_t stream, const pdd_pro
 
   auto kern = path_kernel<Model, Geom, R>;
   int bps = 0, num_sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPathBlockOf<R>, 0) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kForwardBlock, 0) != cudaSuccess ||
       cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
     return PDD_ECUDA;
   uint64_t grid = static_cast<uint64_t>(std::max(bps, 1)) * static_cast<uint64_t>(num_sms);
-  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kPathBlockOf<R> - 1) / kPathBlockOf<R>));
-  kern<<<static_cast<unsigned>(grid), kPathBlockOf<R>, 0, stream>>>(a);
+  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kForwardBlock - 1) / kForwardBlock));
+  kern<<<static_cast<unsigned>(grid), kForwardBlock, 0, stream>>>(a);
   fix_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
       fix, n, d_mean, d_se, d_npaths, nullptr);
   return cudaGetLastError() == cudaSuccess ? PDD_OK : PDD_ECUDA;
