@@ -656,6 +656,26 @@ struct ForwardStage {
   PathStash<D, R, kY, kStashCap> start;
   PathStash<D, R, kY, kCheckCap> check;
 };
+// At the wave's end lanes idle, and what is left is the longest paths' chain.
+// Parked units are then rerun once they are as many as the busy lanes: neither
+// are the others held up at every unit nor the parked ones for long (16 x 2000
+// paths of the square: 153 us, 190 us when any parked unit is rerun at once,
+// 191 us when they wait until no lane is busy).
+// Binary64 paths are bound by the FP64 pipe to the end, so a warp with at most
+// kDonate of them left leaves them (in its own stash, `given` of them) to the
+// block's other warps and ends: fewer, fuller warps (16 x 10^4 FP64 paths: 11.4
+// -> 6.2 ms with both rules).  Binary32 paths are bound by latency there, and
+// fuller warps only hold each other up (153 -> 190 us on the square).  A warp
+// that leaves publishes its paths before it lowers `alive`; the warp that
+// brings `alive` to zero looks for published paths once more before it ends,
+// so none is lost.
+constexpr int kDonate = 24;
+template <typename R>
+constexpr bool kCompact = sizeof(R) == 8;
+struct DonorBoard {
+  int given[kForwardBlock / 32], taken[kForwardBlock / 32];
+  int alive;
+};
 
 template <class Model, typename R>
 constexpr bool kKeepY = Model::kKill == 1 && sizeof(R) == 8;
@@ -794,7 +814,7 @@ __device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst
 }
 
 template <class Model, class Geom, typename R>
-__global__ void __launch_bounds__(kForwardBlock) path_kernel(const __grid_constant__ PathArgs a) {
+__global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_kernel(const __grid_constant__ PathArgs a) {
   constexpr int D = Model::D;
   using Stage = ForwardStage<D, R, kKeepY<Model, R>>;
   __shared__ Stage stage_all[kForwardBlock / 32];
@@ -815,56 +835,71 @@ __global__ void __launch_bounds__(kForwardBlock) path_kernel(const __grid_consta
   int n_start = 0;              // stash fill; parked units and the oldest (warp-uniform)
   int n_check = 0, head = 0;
   bool exhausted = false;       // the wave's indices are all claimed (warp-uniform)
+  bool last = false;            // the block's last warp (warp-uniform)
   unsigned long long my_steps = 0, my_capped = 0, my_bad = 0;
+  constexpr int kWarps = kForwardBlock / 32;
+  __shared__ DonorBoard board;
+  if (threadIdx.x < kWarps) board.given[threadIdx.x] = board.taken[threadIdx.x] = 0;
+  if (threadIdx.x == 0) board.alive = kWarps;
+  __syncthreads();
 
-  for (;;) {
-    // ---- idle lanes take stashed paths; the stash is refilled when empty
-    // (not while 32 units wait for their recheck)
-    unsigned needmask = n_check < 32 ? __ballot_sync(kFull, !active) : 0u;
-    while (needmask) {
-      if (n_start == 0) {
-        if (exhausted) break;
-        n_start = stash_starts<Model, Geom, R>(a, stage.start, span, exhausted, my_bad);
-        continue;
-      }
-      const int cnt = __popc(needmask);
-      const int take = cnt < n_start ? cnt : n_start;
-      if (!active) {
-        const int r = __popc(needmask & lt_mask);
-        if (r < take) {
-          const int i = n_start - 1 - r;
-          slot = stage.start.slot[i];
-          pp.r0_w0 = stage.start.w0[i];
-          pp.r0_w1 = stage.start.w1[i];
-          pp.tag = 0u;
-          n = stage.start.n[i];
-          Z = stage.start.z[i];
-          R y = R(1);
-          if constexpr (kKeepY<Model, R>) y = stage.start.y[i];
-          Y = path_weight<Model, R>(k, n, y);
+  // entry i of a stash becomes the lane's path
+  auto load = [&](const auto &st, int i) {
+    slot = st.slot[i];
+    pp.r0_w0 = st.w0[i];
+    pp.r0_w1 = st.w1[i];
+    pp.tag = 0u;
+    n = st.n[i];
+    Z = st.z[i];
+    R y = R(1);
+    if constexpr (kKeepY<Model, R>) y = st.y[i];
+    Y = path_weight<Model, R>(k, n, y);
 #pragma unroll
-          for (int d = 0; d < D; ++d) X[d] = stage.start.x[d][i];
-          e = path_edge<Geom, R>(X);
-          active = true;
-        }
-      }
-      n_start -= take;
-      needmask = __ballot_sync(kFull, !active);
+    for (int d = 0; d < D; ++d) X[d] = st.x[d][i];
+    e = path_edge<Geom, R>(X);
+    active = true;
+  };
+  // entry i of a stash from the start of the lane's unit
+  auto store = [&](auto &st, int i, int32_t n0, const R *X0, R Y0, R Z0) {
+    st.slot[i] = slot;
+    st.w0[i] = pp.r0_w0;
+    st.w1[i] = pp.r0_w1;
+    st.n[i] = n0;
+    st.z[i] = Z0;
+    if constexpr (kKeepY<Model, R>) st.y[i] = Y0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) st.x[d][i] = X0[d];
+    active = false;
+  };
+  // idle lanes take published paths, this warp's own first (the last warp's);
+  // returns the lanes still idle
+  auto adopt = [&](unsigned need) -> unsigned {
+    volatile DonorBoard &vb = board;
+    const unsigned from = __ballot_sync(kFull, lane < kWarps && vb.taken[lane % kWarps] < vb.given[lane % kWarps]);
+    if (!from) return need;
+    for (int q = 0; need && q < kWarps; ++q) {
+      const int w = (static_cast<int>(threadIdx.x >> 5) + q) % kWarps;
+      if (!((from >> w) & 1u)) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&board.taken[w], __popc(need));
+      at = __shfl_sync(kFull, at, 0);
+      __threadfence_block();
+      const int i = at + __popc(need & lt_mask);
+      if (!active && i < vb.given[w]) load(stage_all[w].start, i);
+      need = __ballot_sync(kFull, !active);
     }
+    return need;
+  };
 
-    // ---- parked units: 32 together, or what there is when lanes would idle
-    // without them (the wave's end)
-    if (n_check >= 32 || (needmask && n_check > 0)) {
-      const int cnt = n_check < 32 ? n_check : 32;
-      recheck_units<Model, Geom, R>(a, k, stage, head, cnt, n_start, my_steps, my_capped);
-      head = (head + cnt) & (kCheckCap - 1);
-      n_check -= cnt;
-      continue;
-    }
-    if (needmask == kFull) break;
-
-    // ---- one unit of the lane's path; a unit that may hold an exit, or reach
-    // the step cap, is parked as it started
+  // the oldest cnt parked units
+  auto recheck = [&](int cnt) {
+    recheck_units<Model, Geom, R>(a, k, stage, head, cnt, n_start, my_steps, my_capped);
+    head = (head + cnt) & (kCheckCap - 1);
+    n_check -= cnt;
+  };
+  // one unit of the lane's path; a unit that may hold an exit, or reach the
+  // step cap, is parked as it started
+  auto advance = [&]() {
     bool park = false;
     R X0[D], Z0 = Z, Y0 = Y;
 #pragma unroll
@@ -878,20 +913,83 @@ __global__ void __launch_bounds__(kForwardBlock) path_kernel(const __grid_consta
     }
     const unsigned pm = __ballot_sync(kFull, park);
     if (pm) {
-      if (park) {
-        const int i = (head + n_check + __popc(pm & lt_mask)) & (kCheckCap - 1);
-        stage.check.slot[i] = slot;
-        stage.check.w0[i] = pp.r0_w0;
-        stage.check.w1[i] = pp.r0_w1;
-        stage.check.n[i] = n - 4;
-        stage.check.z[i] = Z0;
-        if constexpr (kKeepY<Model, R>) stage.check.y[i] = Y0;
-#pragma unroll
-        for (int d = 0; d < D; ++d) stage.check.x[d][i] = X0[d];
-        active = false;
-      }
+      if (park) store(stage.check, (head + n_check + __popc(pm & lt_mask)) & (kCheckCap - 1), n - 4, X0, Y0, Z0);
       n_check += __popc(pm);
     }
+  };
+
+  // ---- while the wave has paths: every lane busy, parked units 32 together
+  for (;;) {
+    if (n_check >= 32) recheck(32);
+    unsigned need = __ballot_sync(kFull, !active);
+    while (need) {  // idle lanes take stashed paths; an empty stash is refilled
+      if (n_start == 0) {
+        if (exhausted) break;
+        n_start = stash_starts<Model, Geom, R>(a, stage.start, span, exhausted, my_bad);
+        continue;
+      }
+      const int r = __popc(need & lt_mask), cnt = __popc(need);
+      const int take = cnt < n_start ? cnt : n_start;
+      if (!active && r < take) load(stage.start, n_start - 1 - r);
+      n_start -= take;
+      need = __ballot_sync(kFull, !active);
+    }
+    if (need) break;
+    advance();
+  }
+
+  // ---- the wave's end: lanes idle (see DonorBoard)
+#pragma unroll 1
+  for (;;) {
+    unsigned need = __ballot_sync(kFull, !active);
+    if (need && n_start > 0) {
+      const int r = __popc(need & lt_mask), cnt = __popc(need);
+      const int take = cnt < n_start ? cnt : n_start;
+      if (!active && r < take) load(stage.start, n_start - 1 - r);
+      n_start -= take;
+      need = __ballot_sync(kFull, !active);
+    }
+    if (n_check > 0 && (n_check >= 32 || n_check >= 32 - __popc(need))) {
+      recheck(n_check < 32 ? n_check : 32);
+      continue;
+    }
+    if (need) {
+      if constexpr (kCompact<R>) {
+        need = adopt(need);
+        const int left = 32 - __popc(need), all = left + n_check;
+        if (all <= kDonate && !last) {
+          if (active) store(stage.start, __popc(~need & lt_mask), n, X, Y, Z);
+          if (static_cast<int>(lane) < n_check) {  // parked units are paths at a unit's start
+            const int i = (head + static_cast<int>(lane)) & (kCheckCap - 1), o = left + static_cast<int>(lane);
+            stage.start.slot[o] = stage.check.slot[i];
+            stage.start.w0[o] = stage.check.w0[i];
+            stage.start.w1[o] = stage.check.w1[i];
+            stage.start.n[o] = stage.check.n[i];
+            stage.start.z[o] = stage.check.z[i];
+            if constexpr (kKeepY<Model, R>) stage.start.y[o] = stage.check.y[i];
+#pragma unroll
+            for (int d = 0; d < D; ++d) stage.start.x[d][o] = stage.check.x[d][i];
+          }
+          n_check = 0;
+          __threadfence_block();
+          __syncwarp();
+          int before = 0;
+          if (lane == 0) {
+            volatile DonorBoard &vb = board;
+            vb.given[threadIdx.x >> 5] = all;
+            __threadfence_block();
+            before = atomicSub(&board.alive, 1);
+            if (before == 1) board.alive = 1;  // the last warp stays while there are paths
+          }
+          before = __shfl_sync(kFull, before, 0);
+          if (before > 1) break;
+          last = true;
+          need = adopt(kFull);
+        }
+      }
+      if (need == kFull) break;
+    }
+    advance();
   }
 
   // ---- per-warp totals
