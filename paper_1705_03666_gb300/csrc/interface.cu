@@ -60,6 +60,7 @@ pdd_status philox_stream_impl(pdd_ctx *ctx, uint64_t seed, uint32_t j0, uint32_t
 // Scratch layout for one interface solve (offsets in bytes):
 //   [0, 256)          counters (4 x u64) and the queue cursor
 //   [256, +n*112)     per-node exact sums (NodeFix)
+//   then, FP64 paths  the normals' tables (115 KB)
 // No per-path score is stored: the path kernel adds every score to its node's
 // integer sums when the path ends, in one launch over all paths.
 constexpr size_t kFixOff = 256;
@@ -71,7 +72,7 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   const uint64_t N = static_cast<uint64_t>(mc->n_paths);
   const uint64_t total = static_cast<uint64_t>(n) * N;
   const size_t bytes = align_up(kFixOff + static_cast<size_t>(n) * sizeof(NodeFix), 256);
-  pdd_status st = ensure_scratch(ctx, bytes);
+  pdd_status st = ensure_scratch(ctx, bytes + (sizeof(R) == 8 ? kNormalBytes : 0));
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
   auto *counters = reinterpret_cast<unsigned long long *>(base);
@@ -100,6 +101,13 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
     a.dump_score = diag->d_path_score;
     a.steps = diag->d_path_steps;
     a.dump_exit = diag->d_path_exit;
+  }
+
+  if constexpr (sizeof(R) == 8) {
+    auto *tables = reinterpret_cast<double2 *>(base + bytes);
+    launch_normal_tables(tables, ctx->stream);
+    PDD_CUDA_TRY(ctx, cudaGetLastError());
+    a.normal_tables = tables;
   }
 
   auto kern = path_kernel<Model, Geom, R>;

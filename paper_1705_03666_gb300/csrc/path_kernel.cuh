@@ -35,6 +35,7 @@
 #include "common.cuh"
 #include "models.cuh"
 #include "nodefix.cuh"
+#include "normal_tables.cuh"
 
 namespace pdd {
 
@@ -71,6 +72,7 @@ struct PathArgs {
   int32_t max_steps;
   int32_t bridge;
   float edge_c1, edge_c0;       // fast_unit's bound (see path_step_args)
+  const double2 *normal_tables; // FP64 paths: NormalTables
   float lr_scale;               // sqrt(dt) / sigma (gradient mode)
   ModelConst mc;
 };
@@ -435,20 +437,21 @@ __device__ __forceinline__ uint32_t low_bytes_word(uint32_t a, uint32_t b, uint3
 // (w10,w11), step 4q + j takes z[3j..3j+2] and low_bytes_word(w[3j],
 // w[3j+1], w[3j+2]).  Either way 0.75 blocks per step, the least that holds
 // the step's normals and a 23-bit uniform.
-template <int D, typename R>
+// bm(a, b, z0, z1) is the Box-Muller map.
+template <int D, typename R, class BM>
 __device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, const RoundKeys &rk,
-                                             R *z, uint32_t *u) {
+                                             R *z, uint32_t *u, BM bm) {
   if constexpr (D == 3) {
     const uint32_t q3 = 3u * (static_cast<uint32_t>(n) >> 2);
     const uint4 A = philox10_path(q3, pp, rk);
     const uint4 B = philox10_path(q3 + 1u, pp, rk);
     const uint4 C = philox10_path(q3 + 2u, pp, rk);
-    box_muller<R>(A.x, A.y, z[0], z[1]);
-    box_muller<R>(A.z, A.w, z[2], z[3]);
-    box_muller<R>(B.x, B.y, z[4], z[5]);
-    box_muller<R>(B.z, B.w, z[6], z[7]);
-    box_muller<R>(C.x, C.y, z[8], z[9]);
-    box_muller<R>(C.z, C.w, z[10], z[11]);
+    bm(A.x, A.y, z[0], z[1]);
+    bm(A.z, A.w, z[2], z[3]);
+    bm(B.x, B.y, z[4], z[5]);
+    bm(B.z, B.w, z[6], z[7]);
+    bm(C.x, C.y, z[8], z[9]);
+    bm(C.z, C.w, z[10], z[11]);
     u[0] = low_bytes_word(A.x, A.y, A.z);
     u[1] = low_bytes_word(A.w, B.x, B.y);
     u[2] = low_bytes_word(B.z, B.w, C.x);
@@ -462,13 +465,32 @@ __device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, co
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       R z1;
-      box_muller<R>(w[2 * j], w[2 * j + 1], z[D * j], z1);
+      bm(w[2 * j], w[2 * j + 1], z[D * j], z1);
       if constexpr (D == 2) z[D * j + 1] = z1;
     }
     u[0] = C.x;
     u[1] = C.y;
     u[2] = C.z;
     u[3] = C.w;
+  }
+}
+template <int D, typename R>
+__device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, const RoundKeys &rk,
+                                             R *z, uint32_t *u) {
+  unit_randoms<D, R>(n, pp, rk, z, u,
+                     [](uint32_t a, uint32_t b, R &z0, R &z1) { box_muller<R>(a, b, z0, z1); });
+}
+// The forward path kernel's: binary64 normals from the launch's tables.
+template <int D, typename R>
+__device__ __forceinline__ void path_randoms(const PathArgs &a, int32_t n, const PhiloxPath &pp,
+                                             R *z, uint32_t *u) {
+  if constexpr (sizeof(R) == 8) {
+    const NormalTables t(a.normal_tables);
+    unit_randoms<D, R>(n, pp, a.rk, z, u, [&](uint32_t wa, uint32_t wb, R &z0, R &z1) {
+      box_muller_tables(t, wa, wb, z0, z1);
+    });
+  } else {
+    unit_randoms<D, R>(n, pp, a.rk, z, u);
   }
 }
 
@@ -619,7 +641,7 @@ __device__ __forceinline__ int exact_unit(const PathArgs &a, const StepConst<R> 
   constexpr int D = Model::D;
   R z[4 * D];
   uint32_t u[4];
-  unit_randoms<D, R>(n, pp, a.rk, z, u);
+  path_randoms<D, R>(a, n, pp, z, u);
   int code = kStepContinue;
 #pragma unroll 1
   for (int j = 0; j < 4; ++j) {
@@ -907,7 +929,7 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
     if (active) {
       R z[4 * D];
       uint32_t u[4];
-      unit_randoms<D, R>(n, pp, a.rk, z, u);
+      path_randoms<D, R>(a, n, pp, z, u);
       park = fast_unit<Model, Geom, R>(a, k, z, u, n, X, Y, Z, e) || n > last_fast;
       n += 4;
     }

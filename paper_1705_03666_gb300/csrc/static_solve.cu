@@ -20,11 +20,13 @@ namespace pdd {
 namespace {
 
 // 8 MiB on every GPU that loads the library, held until process exit:
-// 256 bytes of counters and 112 bytes of exact sums per node.
+// 256 bytes of counters, 112 bytes of exact sums per node, and at its end the
+// tables of the FP64 paths' normals.
 constexpr size_t kStaticScratchBytes = size_t(8) << 20;
 constexpr int64_t kStaticMaxNodes = 65536;
 constexpr size_t kStaticFixOff = 256;
-static_assert(kStaticFixOff + kStaticMaxNodes * sizeof(NodeFix) <= kStaticScratchBytes,
+constexpr size_t kStaticTableOff = (kStaticScratchBytes - kNormalBytes) & ~size_t(255);
+static_assert(kStaticFixOff + kStaticMaxNodes * sizeof(NodeFix) <= kStaticTableOff,
               "static scratch too small for its node limit");
 
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
@@ -44,6 +46,7 @@ cudaError_t load_kernels() {
       reinterpret_cast<const void *>(path_kernel<EllipticManufactured, Box<3>, double>),
       reinterpret_cast<const void *>(path_kernel<PoissonFourier, Box<2>, float>),
       reinterpret_cast<const void *>(path_kernel<PoissonFourier, Box<2>, double>),
+      reinterpret_cast<const void *>(normal_tables_kernel),
       reinterpret_cast<const void *>(fix_finalize_kernel)};
   for (const void *k : kernels) {
     const cudaError_t e = cudaFuncGetAttributes(&fa, k);
@@ -121,6 +124,12 @@ pdd_status run_static(char *base, int device, cudaStream_t stream, const pdd_pro
   for (int i = 0; i < prob->n_params; ++i) {
     a.mc.prm[i] = prob->params[i];
     a.mc.prmf[i] = static_cast<float>(prob->params[i]);
+  }
+
+  if constexpr (sizeof(R) == 8) {
+    auto *tables = reinterpret_cast<double2 *>(base + kStaticTableOff);
+    launch_normal_tables(tables, stream);
+    a.normal_tables = tables;
   }
 
   auto kern = path_kernel<Model, Geom, R>;
