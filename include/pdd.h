@@ -232,8 +232,8 @@ PDD_API pdd_status pdd_set_params(pdd_ctx *ctx, const double *params,
  * (counter = (block, p, i, 0)), and the sums are the same, so with
  * n_min = n_max = N the results equal pdd_interface_solve's bit for bit.
  * The work list of the second pass is built
- * on the device, and one persistent launch consumes it (lanes take chunks of
- * `chunk` consecutive paths of one node), so the call has no host round trip.
+ * on the device, and one persistent launch consumes it (warps claim
+ * `chunk` consecutive paths of that list at a time), so the call has no host round trip.
  * With use_graph != 0 the whole sequence is captured once into a CUDA graph
  * (rebuilt when any argument or the scratch changes) and replayed; this
  * needs a non-default stream.  Writes d_mean[n], d_se[n] and, if non-NULL,
@@ -255,7 +255,7 @@ typedef struct {
   int64_t n_min, n_max;      /* clamp of the adaptive path count */
   double target_se;          /* standard error aimed for (> 0) */
   int64_t max_steps;         /* per-path step cap */
-  int32_t chunk;             /* paths per lane-chunk (0 = tuned default) */
+  int32_t chunk;             /* paths per claim, in multiples of 32 (0 = tuned default) */
   int32_t bridge;            /* Brownian-bridge exit test on/off */
 } pdd_batch_params;
 
@@ -580,7 +580,7 @@ PDD_API pdd_status pdd_autotune(pdd_ctx *ctx, const double *d_nodes, int64_t n,
                                 int32_t repeats, int32_t *best_blocks_per_sm,
                                 double *best_ms);
 
-/* Same for pdd_batch_solve's lane-chunk size (32 .. 1024 paths). */
+/* Same for pdd_batch_solve's claim size (32 .. 1024 paths). */
 PDD_API pdd_status pdd_autotune_batch(pdd_ctx *ctx, const pdd_problem *problems,
                                       int32_t n_problems,
                                       const pdd_batch_nodes *nodes,

@@ -3,12 +3,13 @@
 // captured once in a CUDA graph and replayed.
 //
 //   0. the nodes are grouped by domain/family (stable partition on the
-//      device); chunk lists follow that order, one kernel per family;
-//   1. pilot: n_pilot paths per node (lane-chunk queue, batch_kernel), their
-//      scores added to the node's exact sums (nodefix.cuh);
+//      device); the path lists follow that order, one kernel per family; the
+//      node table (step constants, start points) is formed;
+//   1. pilot: n_pilot paths per node (batch_kernel), their scores added to the
+//      node's exact sums (nodefix.cuh);
 //   2. per node: pilot mean and variance s^2 from those sums, path count
 //      N_i = clamp(ceil(s^2 / SE*^2), max(n_min, n_pilot), n_max);
-//   3. exclusive scan of the per-node chunk counts of paths [n_pilot, N_i);
+//   3. exclusive scan of the per-node counts of paths [n_pilot, N_i);
 //   4. main pass over that device-built work list (same persistent kernel),
 //      adding to the same sums;
 //   5. per node: mean, standard error and count from the sums.
@@ -78,35 +79,49 @@ batch_partition(int64_t n, const int32_t *prob, int32_t n_probs, int4 combo_of_p
 }
 
 // Pilot work list: every node gets paths [0, n_pilot).
-__global__ void batch_pilot_setup(int64_t n, int64_t n_pilot, int32_t K, int64_t *chunk_off,
-                                  int64_t *first, int64_t *end) {
-  const int64_t cpn = (n_pilot + K - 1) / K;
+__global__ void batch_pilot_setup(int64_t n, int64_t n_pilot, int64_t *off) {
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i <= n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    chunk_off[i] = i * cpn;
-    if (i < n) {
-      first[i] = 0;
-      end[i] = n_pilot;
-    }
-  }
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    off[i] = i * n_pilot;
+}
+
+// The node table.
+struct BatchProblems {
+  BatchProblem p[kMaxBatchProblems];
+};
+__global__ void batch_table(int64_t n, const double *nodes, const int32_t *prob, const double *dt,
+                            int32_t n_probs, const __grid_constant__ BatchProblems P,
+                            BatchNode *table) {
+  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (i >= n) return;
+  const int32_t pi = prob[i];
+  if (pi < 0 || pi >= n_probs) return;  // in no family's range
+  const BatchProblem &B = P.p[pi];
+  BatchNode t;
+  t.k = B.combo == kComboLShapeLaplace
+            ? make_step_const<LShape>(dt[i], B.sigma, B.c_kill, B.bridge != 0)
+        : B.combo == kComboCubeElliptic
+            ? make_step_const<Box<3>>(dt[i], B.sigma, B.c_kill, B.bridge != 0)
+            : make_step_const<Box<2>>(dt[i], B.sigma, B.c_kill, B.bridge != 0);
+  for (int d = 0; d < 3; ++d) t.x[d] = static_cast<float>(nodes[i * 3 + d]);
+  t.prob = pi;
+  table[i] = t;
 }
 
 // Per node, from the exact sums of its pilot paths: the sample variance,
-// N_i and the main work list's per-node entries.  K: paths per main-pass
-// chunk.  Runs over positions j (node i = perm[j]); count2 is written by
-// position (the main scan's order) and the other outputs by node.  Positions
-// of invalid nodes (problem index out of range) get no chunks and are marked
-// invalid in the sums, so that they finish with NaN and a count of 0.
-__global__ void batch_pilot_stats(int64_t n, int64_t n_pilot, int32_t K, const int32_t *perm,
+// N_i and the number of its paths in the main work list.  Runs over positions
+// j (node i = perm[j]); count2 is written by position (the main scan's
+// order).  Positions of invalid nodes (problem index out of range) get no
+// paths and are marked invalid in the sums, so that they finish with NaN and a
+// count of 0.
+__global__ void batch_pilot_stats(int64_t n, int64_t n_pilot, const int32_t *perm,
                                   const int64_t *cstart, NodeFix *fix, double inv_se2,
-                                  int64_t n_min, int64_t n_max, int64_t *first2, int64_t *end2,
-                                  int64_t *count2) {
+                                  int64_t n_min, int64_t n_max, int64_t *count2) {
   const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (j >= n) return;
   const int64_t i = perm[j];
   if (j >= cstart[4]) {
     fix[i].bad = 1;
-    first2[i] = end2[i] = n_pilot;
     count2[j] = 0;
     return;
   }
@@ -120,9 +135,7 @@ __global__ void batch_pilot_stats(int64_t n, int64_t n_pilot, int32_t K, const i
   int64_t Ni = want >= static_cast<double>(n_max) ? n_max : static_cast<int64_t>(want);
   Ni = max(lo, min(n_max, Ni));
   if (isnan(var)) Ni = lo;
-  first2[i] = n_pilot;
-  end2[i] = Ni;
-  count2[j] = (Ni - n_pilot + K - 1) / K;
+  count2[j] = Ni - n_pilot;
 }
 
 // Exclusive scan of count[0..n) into off[0..n] (single block, fixed order).
@@ -181,8 +194,7 @@ int combo_of(const pdd_problem &p) {
 }
 
 struct BatchLayout {
-  size_t off_first, off_end, off_chunk, off_first2, off_end2, off_cnt2, off_chunk2, off_fix,
-      off_perm, off_cstart, total;
+  size_t off_list, off_cnt2, off_list2, off_fix, off_perm, off_cstart, off_table, total;
 };
 
 BatchLayout batch_layout(int64_t n) {
@@ -194,16 +206,13 @@ BatchLayout batch_layout(int64_t n) {
     return at;
   };
   const size_t nn = static_cast<size_t>(n);
-  L.off_first = take(nn * 8);
-  L.off_end = take(nn * 8);
-  L.off_chunk = take((nn + 1) * 8);
-  L.off_first2 = take(nn * 8);
-  L.off_end2 = take(nn * 8);
+  L.off_list = take((nn + 1) * 8);
   L.off_cnt2 = take(nn * 8);
-  L.off_chunk2 = take((nn + 1) * 8);
+  L.off_list2 = take((nn + 1) * 8);
   L.off_fix = take(nn * sizeof(NodeFix));
   L.off_perm = take(nn * sizeof(int32_t));
   L.off_cstart = take(8 * sizeof(int64_t));
+  L.off_table = take(nn * sizeof(BatchNode));
   L.total = o;
   return L;
 }
@@ -214,7 +223,7 @@ BatchLayout batch_layout(int64_t n) {
 // first family runs on the context's stream, the others on side streams
 // forked from it and joined back (event record / wait, which stream capture
 // records as graph dependencies), so the families' kernels overlap and the
-// tail of one (lanes idle while its last chunks finish) is filled by another.
+// tail of one (lanes idle while its last paths finish) is filled by another.
 static pdd_status launch_families(pdd_ctx *ctx, const BatchArgs &a, const unsigned *grid) {
   int launched = 0;
   for (int c = 0; c < 4; ++c) {
@@ -227,16 +236,16 @@ static pdd_status launch_families(pdd_ctx *ctx, const BatchArgs &a, const unsign
     }
     switch (c) {
       case kComboSquareLaplace:
-        batch_kernel<kComboSquareLaplace><<<grid[c], kBatchBlock, 0, s>>>(a);
+        batch_kernel<kComboSquareLaplace><<<grid[c], kForwardBlock, 0, s>>>(a);
         break;
       case kComboLShapeLaplace:
-        batch_kernel<kComboLShapeLaplace><<<grid[c], kBatchBlock, 0, s>>>(a);
+        batch_kernel<kComboLShapeLaplace><<<grid[c], kForwardBlock, 0, s>>>(a);
         break;
       case kComboCubeElliptic:
-        batch_kernel<kComboCubeElliptic><<<grid[c], kBatchBlock, 0, s>>>(a);
+        batch_kernel<kComboCubeElliptic><<<grid[c], kForwardBlock, 0, s>>>(a);
         break;
       default:
-        batch_kernel<kComboSquarePoisson><<<grid[c], kBatchBlock, 0, s>>>(a);
+        batch_kernel<kComboSquarePoisson><<<grid[c], kForwardBlock, 0, s>>>(a);
         break;
     }
     PDD_CUDA_TRY(ctx, cudaGetLastError());
@@ -262,21 +271,17 @@ static pdd_status ensure_side_streams(pdd_ctx *ctx) {
 
 static pdd_status enqueue_batch(pdd_ctx *ctx, const BatchArgs &proto, const BatchLayout &Lay,
                                 const pdd_batch_nodes *nodes, const pdd_batch_params *bp,
-                                int32_t K, int32_t Kp, const unsigned *grid, int4 combo_of_prob,
-                                int32_t n_probs, double *d_mean, double *d_se,
-                                int64_t *d_npaths) {
+                                const unsigned *grid, int4 combo_of_prob, int32_t n_probs,
+                                double *d_mean, double *d_se, int64_t *d_npaths) {
   char *base = static_cast<char *>(ctx->scratch);
   auto *counters = reinterpret_cast<unsigned long long *>(base);
-  auto *first = reinterpret_cast<int64_t *>(base + Lay.off_first);
-  auto *end = reinterpret_cast<int64_t *>(base + Lay.off_end);
-  auto *chunk = reinterpret_cast<int64_t *>(base + Lay.off_chunk);
-  auto *first2 = reinterpret_cast<int64_t *>(base + Lay.off_first2);
-  auto *end2 = reinterpret_cast<int64_t *>(base + Lay.off_end2);
+  auto *list = reinterpret_cast<int64_t *>(base + Lay.off_list);
   auto *cnt2 = reinterpret_cast<int64_t *>(base + Lay.off_cnt2);
-  auto *chunk2 = reinterpret_cast<int64_t *>(base + Lay.off_chunk2);
+  auto *list2 = reinterpret_cast<int64_t *>(base + Lay.off_list2);
   auto *fix = reinterpret_cast<NodeFix *>(base + Lay.off_fix);
   auto *perm = reinterpret_cast<int32_t *>(base + Lay.off_perm);
   auto *cstart = reinterpret_cast<int64_t *>(base + Lay.off_cstart);
+  auto *table = reinterpret_cast<BatchNode *>(base + Lay.off_table);
   auto *cursors = counters + 8;  // one per family
   const int64_t n = nodes->n;
   const unsigned nb = static_cast<unsigned>((n + 255) / 256);
@@ -285,28 +290,29 @@ static pdd_status enqueue_batch(pdd_ctx *ctx, const BatchArgs &proto, const Batc
   PDD_CUDA_TRY(ctx, cudaMemsetAsync(fix, 0, static_cast<size_t>(n) * sizeof(NodeFix), ctx->stream));
   batch_partition<<<1, kScanBlock, 0, ctx->stream>>>(n, nodes->d_problem, n_probs, combo_of_prob,
                                                      perm, cstart, counters + 2);
-  batch_pilot_setup<<<nb + 1, 256, 0, ctx->stream>>>(n, bp->n_pilot, Kp, chunk, first, end);
+  batch_pilot_setup<<<nb + 1, 256, 0, ctx->stream>>>(n, bp->n_pilot, list);
+  BatchProblems P;
+  std::memcpy(P.p, proto.probs, sizeof P.p);
+  batch_table<<<nb, 256, 0, ctx->stream>>>(n, nodes->d_nodes, nodes->d_problem, nodes->d_dt, n_probs,
+                                           P, table);
   BatchArgs a = proto;
   a.perm = perm;
   a.cstart = cstart;
-  a.K = Kp;
-  a.chunk_off = chunk;
-  a.first = first;
-  a.end = end;
+  a.off = list;
+  a.first = 0;
+  a.table = table;
   a.cursor = cursors;
   a.counters = counters;
   a.fix = fix;
   pdd_status st = launch_families(ctx, a, grid);
   if (st != PDD_OK) return st;
-  batch_pilot_stats<<<nb, 256, 0, ctx->stream>>>(n, bp->n_pilot, K, perm, cstart, fix,
+  batch_pilot_stats<<<nb, 256, 0, ctx->stream>>>(n, bp->n_pilot, perm, cstart, fix,
                                                  1.0 / (bp->target_se * bp->target_se),
-                                                 bp->n_min, bp->n_max, first2, end2, cnt2);
-  batch_scan<<<1, kScanBlock, 0, ctx->stream>>>(n, cnt2, chunk2);
+                                                 bp->n_min, bp->n_max, cnt2);
+  batch_scan<<<1, kScanBlock, 0, ctx->stream>>>(n, cnt2, list2);
   PDD_CUDA_TRY(ctx, cudaMemsetAsync(cursors, 0, 4 * sizeof(unsigned long long), ctx->stream));
-  a.K = K;
-  a.chunk_off = chunk2;
-  a.first = first2;
-  a.end = end2;
+  a.off = list2;
+  a.first = bp->n_pilot;
   const auto ev = prof_slot(ctx);
   if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, ctx->stream));
   st = launch_families(ctx, a, grid);
@@ -360,14 +366,14 @@ pdd_status batch_solve_impl(pdd_ctx *ctx, const pdd_problem *problems, int32_t n
     }
   }
   proto.n_probs = n_problems;
-  proto.nodes = nodes->d_nodes;
-  proto.prob = nodes->d_problem;
-  proto.dt = nodes->d_dt;
   proto.n = nodes->n;
   proto.rk = make_round_keys(bp->seed);
   proto.max_steps = static_cast<int32_t>(bp->max_steps);
-  const int32_t K = bp->chunk > 0 ? bp->chunk : (ctx->batch_chunk > 0 ? ctx->batch_chunk : 256);
-  proto.K = K;
+  // paths a warp claims at a time: the caller's chunk, or the tuner's, in whole
+  // stash fills (the cursor sees one atomic per claim; 32 measures as fast as
+  // longer claims and leaves the least at the end)
+  const int32_t K = bp->chunk > 0 ? bp->chunk : (ctx->batch_chunk > 0 ? ctx->batch_chunk : 32);
+  proto.claim = std::max(32, K / 32 * 32);
   if (diag) {
     diag->path_steps = 0;
     diag->capped = 0;
@@ -387,19 +393,12 @@ pdd_status batch_solve_impl(pdd_ctx *ctx, const pdd_problem *problems, int32_t n
                    : c == kComboLShapeLaplace ? reinterpret_cast<const void *>(batch_kernel<kComboLShapeLaplace>)
                    : c == kComboCubeElliptic  ? reinterpret_cast<const void *>(batch_kernel<kComboCubeElliptic>)
                                               : reinterpret_cast<const void *>(batch_kernel<kComboSquarePoisson>);
-    PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, kBatchBlock, 0));
+    PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, kForwardBlock, 0));
     if (bps < 1) bps = 1;
     if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
     grid[c] = static_cast<unsigned>(bps * ctx->num_sms);
   }
   const int4 combo_of_prob = make_int4(cp[0], cp[1], cp[2], cp[3]);
-  unsigned max_grid = 0;
-  for (int c = 0; c < 4; ++c) max_grid = std::max(max_grid, grid[c]);
-  // pilot chunks: the pilot is small (n_pilot paths per node), and chunks of
-  // K paths could leave lanes without work; aim at >= 8 chunks per lane
-  const double pilot_paths = static_cast<double>(nodes->n) * static_cast<double>(bp->n_pilot);
-  const double per_lane = pilot_paths / (8.0 * max_grid * kBatchBlock);
-  const int32_t Kp = static_cast<int32_t>(std::max(1.0, std::min<double>(K, std::floor(per_lane))));
   const BatchLayout Lay = batch_layout(nodes->n);
   pdd_status st = ensure_scratch(ctx, Lay.total);
   if (st != PDD_OK) return st;
@@ -407,7 +406,7 @@ pdd_status batch_solve_impl(pdd_ctx *ctx, const pdd_problem *problems, int32_t n
   if (st != PDD_OK) return st;
 
   if (!use_graph) {
-    st = enqueue_batch(ctx, proto, Lay, nodes, bp, K, Kp, grid, combo_of_prob, n_problems,
+    st = enqueue_batch(ctx, proto, Lay, nodes, bp, grid, combo_of_prob, n_problems,
                        d_mean, d_se, d_npaths);
     if (st != PDD_OK) return st;
   } else {
@@ -434,7 +433,7 @@ pdd_status batch_solve_impl(pdd_ctx *ctx, const pdd_problem *problems, int32_t n
       const bool prof = ctx->profiling;
       ctx->profiling = false;  // no event records inside the capture
       PDD_CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-      st = enqueue_batch(ctx, proto, Lay, nodes, bp, K, Kp, grid, combo_of_prob, n_problems,
+      st = enqueue_batch(ctx, proto, Lay, nodes, bp, grid, combo_of_prob, n_problems,
                        d_mean, d_se, d_npaths);
       cudaGraph_t g = nullptr;
       const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);

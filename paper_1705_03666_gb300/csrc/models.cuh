@@ -223,7 +223,7 @@ struct Box {
   }
   // The most faces within bridge reach of one step (opposite ones cannot both
   // be while sigma^2 dt <= 1/36).
-  static int reach(double) { return D; }
+  __host__ __device__ static int reach(double) { return D; }
   // Distance to the plane of face j, positive on the domain side.
   template <typename R>
   __device__ __forceinline__ static R face_dist(int j, const R *x) {
@@ -357,7 +357,7 @@ struct LShape {
   // d d' < 9 s^2 (s = sigma sqrt(dt)) and |d - d'| <= 5.77 s (the largest
   // Box-Muller radius), so both ends lie within 7.06 s of it; below 1/4 that
   // leaves the two faces of one corner (no two others come closer than 1/2).
-  static int reach(double s) { return 7.06 * s < 0.25 ? 2 : kFaces; }
+  __host__ __device__ static int reach(double s) { return 7.06 * s < 0.25 ? 2 : kFaces; }
   template <typename R>
   __device__ __forceinline__ static R face_dist(int j, const R *x) {
     if (j < 4) {

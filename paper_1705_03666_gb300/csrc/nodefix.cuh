@@ -142,28 +142,6 @@ __device__ __forceinline__ void fix_commit(NodeFix *fix, bool has, uint64_t node
   }
 }
 
-// One lane adds `count` paths of node `node` that all score s (a node on the
-// boundary: tau = 0 for every path, so u = g there), or, for NaN s (a node
-// outside the closed domain), counts them as invalid.  Per-lane atomics:
-// such nodes are rare, and count * digit stays far below 2^63.
-template <typename R>
-__device__ __forceinline__ void fix_add_repeated(NodeFix *fix, uint64_t node, R s,
-                                                 long long count) {
-  unsigned long long *w = reinterpret_cast<unsigned long long *>(fix + node);
-  if (!(fabs(s) < R(0x1p30))) {
-    atomicAdd(w + kFixBad, static_cast<unsigned long long>(count));
-    return;
-  }
-  int32_t d[2 * kFixDigits];
-  fix_limbs(s, d, d + kFixDigits);
-  atomicAdd(w, static_cast<unsigned long long>(count));
-#pragma unroll
-  for (int k = 0; k < 2 * kFixDigits; ++k)
-    if (d[k] != 0)
-      atomicAdd(w + 1 + k, static_cast<unsigned long long>(count * static_cast<long long>(d[k])));
-  atomicAdd(w + kFixBoundary, static_cast<unsigned long long>(count));
-}
-
 // Double-double helpers for the finalisation (Dekker/Knuth error-free
 // transformations with FMA).
 struct DD {

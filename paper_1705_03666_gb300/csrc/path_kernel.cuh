@@ -91,7 +91,7 @@ constexpr float kLog2Count[7] = {0.0f, 0.0f, 1.0f, 1.5849625007211562f, 2.0f,
 // flag (host).  kReach: the most faces that can be within bridge reach of one
 // step together.
 //
-// The bound of fast_unit.  With e a lower bound on the distance of a point to
+// The bound of fast_unit (edge_bound).  With e a lower bound on the distance of a point to
 // every face (Geom::edge; <= 0 outside), every d_j d'_j >= e e', so the step
 // cannot cross while log2 U >= log2 kReach - 2 log2(e) e e' / (sigma^2 dt).
 // log2 U is bounded below by the bits of U read as a fixed-point number
@@ -104,6 +104,11 @@ constexpr float kLog2Count[7] = {0.0f, 0.0f, 1.0f, 1.5849625007211562f, 2.0f,
 // (2^-25 absolute, which weighs 2^-25 (e + e') 2.9 / (sigma^2 dt) with e, e'
 // within 12 sigma sqrt(dt) where U can matter: below 2e-6 / (sigma sqrt(dt))).
 // Without the bridge test the slope is -inf: only e e' <= 0 fails.
+__host__ __device__ inline void edge_bound(double s, bool bridge, int kReach, float *c0, float *c1) {
+  const double margin = 0x1p-10 + 4e-6 / s;  // s = sigma sqrt(dt)
+  *c0 = static_cast<float>(8388608.0 + 32768.0 * (127.0 + log2(static_cast<double>(kReach)) + margin));
+  *c1 = bridge ? static_cast<float>(-2.0 * 1.4426950408889634 * 32768.0 / (s * s)) : -INFINITY;
+}
 inline void path_step_args(PathArgs &a, double sig, double dt, double c_kill, bool bridge,
                            int kReach) {
   a.inv_s2dt = 1.0 / (sig * sig * dt);
@@ -116,10 +121,7 @@ inline void path_step_args(PathArgs &a, double sig, double dt, double c_kill, bo
   a.thr_f = static_cast<float>(a.thr_d);
   a.l2cdt_f = static_cast<float>(c_kill * dt * 1.4426950408889634);
   a.bridge = bridge ? 1 : 0;
-  const double margin = 0x1p-10 + 4e-6 / a.sdt_d;
-  a.edge_c0 = static_cast<float>(8388608.0 + 32768.0 * (127.0 + std::log2(kReach) + margin));
-  a.edge_c1 = bridge ? static_cast<float>(-2.0 * 1.4426950408889634 * a.inv_s2dt * 32768.0)
-                     : -INFINITY;
+  edge_bound(a.sdt_d, bridge, kReach, &a.edge_c0, &a.edge_c1);
 }
 
 template <typename R> struct StepConst;
@@ -127,12 +129,13 @@ template <> struct StepConst<float> {
   float dt, sdt, thr, l2cdt, inv_s2dt;
   float b2;    // -2 log2(e) / (sigma^2 dt): exp(-2 m / (sigma^2 dt)) = 2^(b2 m)
   float boff;  // 0 with the bridge test, -inf without (every bound below is 0)
+  float edge_c0, edge_c1;  // fast_unit's bound (edge_bound)
   StepConst() = default;
   __device__ __forceinline__ StepConst(const PathArgs &a)
       : dt(a.dt_f), sdt(a.sdt_f), thr(a.thr_f), l2cdt(a.l2cdt_f),
         inv_s2dt(static_cast<float>(a.inv_s2dt)),
         b2(static_cast<float>(-2.0 * 1.4426950408889634 * a.inv_s2dt)),
-        boff(a.bridge ? 0.0f : -INFINITY) {}
+        boff(a.bridge ? 0.0f : -INFINITY), edge_c0(a.edge_c0), edge_c1(a.edge_c1) {}
   // half-space crossing probability for a step with d d' = m
   __device__ __forceinline__ float cross_p(float m) const { return ex2_approx(b2 * m); }
   // Bound on every crossing probability of a step whose smallest d d' over
@@ -159,9 +162,10 @@ template <> struct StepConst<float> {
 template <> struct StepConst<double> {
   double dt, sdt, thr, e, inv_s2dt;
   double boff;  // 0 with the bridge test, -inf without
+  float edge_c0, edge_c1;
   __device__ __forceinline__ StepConst(const PathArgs &a)
       : dt(a.dt_d), sdt(a.sdt_d), thr(a.thr_d), e(a.ecdt_d), inv_s2dt(a.inv_s2dt),
-        boff(a.bridge ? 0.0 : -INFINITY) {}
+        boff(a.bridge ? 0.0 : -INFINITY), edge_c0(a.edge_c0), edge_c1(a.edge_c1) {}
   __device__ __forceinline__ double kill(double y, int32_t) const { return y * e; }
   __device__ __forceinline__ double exp_neg(double a) const { return exp(-a); }
   __device__ __forceinline__ double cross_p(double m) const { return exp(-2.0 * m * inv_s2dt); }
@@ -173,6 +177,7 @@ template <> struct StepConst<double> {
 // FP32 step constants for time step dt, generator (1/2) sigma^2 Lap, a
 // constant killing rate c and the bridge test on or off, rounded from the
 // same FP64 expressions the host uses for PathArgs.
+template <class Geom>
 __device__ __forceinline__ StepConst<float> make_step_const(double dt, double sigma, double c,
                                                             bool bridge) {
   StepConst<float> k;
@@ -183,6 +188,8 @@ __device__ __forceinline__ StepConst<float> make_step_const(double dt, double si
   k.inv_s2dt = static_cast<float>(1.0 / (sigma * sigma * dt));
   k.b2 = static_cast<float>(-2.0 * 1.4426950408889634 / (sigma * sigma * dt));
   k.boff = bridge ? 0.0f : -INFINITY;
+  const double s = sigma * sqrt(dt);
+  edge_bound(s, bridge, Geom::reach(s), &k.edge_c0, &k.edge_c1);
   return k;
 }
 
@@ -482,15 +489,15 @@ __device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, co
 }
 // The forward path kernel's: binary64 normals from the launch's tables.
 template <int D, typename R>
-__device__ __forceinline__ void path_randoms(const PathArgs &a, int32_t n, const PhiloxPath &pp,
-                                             R *z, uint32_t *u) {
+__device__ __forceinline__ void path_randoms(const RoundKeys &rk, const double2 *tables, int32_t n,
+                                             const PhiloxPath &pp, R *z, uint32_t *u) {
   if constexpr (sizeof(R) == 8) {
-    const NormalTables t(a.normal_tables);
-    unit_randoms<D, R>(n, pp, a.rk, z, u, [&](uint32_t wa, uint32_t wb, R &z0, R &z1) {
+    const NormalTables t(tables);
+    unit_randoms<D, R>(n, pp, rk, z, u, [&](uint32_t wa, uint32_t wb, R &z0, R &z1) {
       box_muller_tables(t, wa, wb, z0, z1);
     });
   } else {
-    unit_randoms<D, R>(n, pp, a.rk, z, u);
+    unit_randoms<D, R>(n, pp, rk, z, u);
   }
 }
 
@@ -595,9 +602,9 @@ __device__ __forceinline__ float path_edge(const R *X) {
 
 // The four steps of the unit at step n (em_step's arithmetic), without exit
 // tests: returns whether any step may have been an exit (the unit is then not
-// taken).  e: path_edge of X, advanced with it.  n < 2^24 - 4.
+// taken).  e: path_edge of X, advanced with it.  n < 2^24 - 4
 template <class Model, class Geom, typename R>
-__device__ __forceinline__ bool fast_unit(const PathArgs &a, const StepConst<R> &k, const R *z,
+__device__ __forceinline__ bool fast_unit(const ModelConst &mc, const StepConst<R> &k, const R *z,
                                           const uint32_t *u, int32_t n, R *X, R &Y, R &Z,
                                           float &e) {
   constexpr int D = Model::D;
@@ -609,7 +616,7 @@ __device__ __forceinline__ bool fast_unit(const PathArgs &a, const StepConst<R> 
     R f = R(0);
 #pragma unroll
     for (int d = 0; d < D; ++d) b[d] = R(0);
-    if constexpr (Model::kDrift || Model::kSource) Model::coeffs(a.mc, X, b, f);
+    if constexpr (Model::kDrift || Model::kSource) Model::coeffs(mc, X, b, f);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       if ((Model::kDriftAxes >> d) & 1u)
@@ -623,7 +630,7 @@ __device__ __forceinline__ bool fast_unit(const PathArgs &a, const StepConst<R> 
       else Y = k.kill(Y, n + j + 1);
     }
     const float en = path_edge<Geom, R>(Xn);
-    maybe |= !(unif_log_bits(unif_f(u[j])) >= fmaf(a.edge_c1, e * en, a.edge_c0));
+    maybe |= !(unif_log_bits(unif_f(u[j])) >= fmaf(k.edge_c1, e * en, k.edge_c0));
     e = en;
 #pragma unroll
     for (int d = 0; d < D; ++d) X[d] = Xn[d];
@@ -634,18 +641,18 @@ __device__ __forceinline__ bool fast_unit(const PathArgs &a, const StepConst<R> 
 // The unit at step n again, a step at a time with the exact tests (em_step)
 // and the step cap; the random numbers are shifted down by static indices so
 // that one copy of the step serves all four.
-template <class Model, class Geom, typename R>
-__device__ __forceinline__ int exact_unit(const PathArgs &a, const StepConst<R> &k,
-                                          const PhiloxPath &pp, R *X, R &Y, R &Z, int32_t &n,
-                                          R *Xn) {
+template <class Model, class Geom, typename R, class Work>
+__device__ __forceinline__ int exact_unit(const Work &a, const typename Work::Env &env,
+                                          const StepConst<R> &k, const PhiloxPath &pp, R *X, R &Y,
+                                          R &Z, int32_t &n, R *Xn) {
   constexpr int D = Model::D;
   R z[4 * D];
   uint32_t u[4];
-  path_randoms<D, R>(a, n, pp, z, u);
+  path_randoms<D, R>(a.rk, a.normal_tables, n, pp, z, u);
   int code = kStepContinue;
 #pragma unroll 1
   for (int j = 0; j < 4; ++j) {
-    code = em_step<Model, Geom, R, false>(a, k, X, Y, Z, z, u[0], n, Xn, static_cast<R *>(nullptr));
+    code = em_step<Model, Geom, R, false>(env, k, X, Y, Z, z, u[0], n, Xn, static_cast<R *>(nullptr));
     ++n;
     if (code != kStepContinue || n >= a.max_steps) break;
 #pragma unroll
@@ -661,7 +668,7 @@ __device__ __forceinline__ int exact_unit(const PathArgs &a, const StepConst<R> 
 // only binary64 paths with killing keep it.
 template <int D, typename R, bool kY, int N>
 struct PathStash {
-  unsigned long long slot[N];   // index in the wave
+  unsigned long long id[N];     // the path (Work)
   uint32_t w0[N], w1[N];        // PhiloxPath words (tag 0)
   int32_t n[N];                 // steps taken
   R x[D][N], z[N];
@@ -710,52 +717,95 @@ __device__ __forceinline__ R path_weight(const StepConst<R> &k, int32_t n, R kep
   else return R(1);
 }
 
-// Called by all 32 lanes with an empty stash: claim the next 32 indices of the
-// wave, set each up, score at once the ones that start on the boundary (tau =
-// 0, u = g, Eq. 2.1) or outside the closed domain (invalid input: NaN,
-// counted), and stash the interior ones.  Returns how many (warp-uniform).
-template <class Model, class Geom, typename R, class Stash>
-__device__ __forceinline__ int stash_starts(const PathArgs &a, Stash &st, unsigned long long span,
-                                            bool &exhausted, unsigned long long &my_bad) {
-  constexpr int D = Model::D;
-  const unsigned lane = threadIdx.x & 31u;
-  __syncwarp();  // earlier reads of the stash are done
-  unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(a.cursor, 32ull);
-  base = __shfl_sync(kFull, base, 0);
-  if (base + 32 >= span) exhausted = true;
-  const unsigned long long q = base + lane;
-  bool interior = false;
-  R x[D];
-  PhiloxPath pp{0, 0, 0};
-  uint64_t node = 0;
-  R s0 = R(0);
-  if (q < span) {
-    const unsigned long long g = a.begin + q;
+// What a launch's warps work through.  A Work type gives the streams and sums
+// (rk, normal_tables, max_steps, fix, counters), claims paths 32 at a time
+// (claim: lane's path id, node, Philox words and start point; false when the
+// lane has none), and per path id its node, model constants (env) and step
+// constants.  PathWork: every node with the same number of paths and the same
+// constants; the id is the index in the wave.
+struct PathEnv {
+  const ModelConst &mc;
+  int32_t bridge;
+};
+template <int D, typename R>
+struct PathWork {
+  using Env = PathEnv;
+  static constexpr bool kOwnConsts = false;  // step constants per path
+  const PathArgs &a;
+  const RoundKeys &rk;
+  const double2 *normal_tables;
+  NodeFix *fix;
+  unsigned long long *counters;
+  int32_t max_steps;
+  unsigned long long span;
+  __device__ __forceinline__ explicit PathWork(const PathArgs &p)
+      : a(p), rk(p.rk), normal_tables(p.normal_tables), fix(p.fix), counters(p.counters),
+        max_steps(p.max_steps), span(p.end - p.begin) {}
+  __device__ __forceinline__ Env env(unsigned long long) const { return Env{a.mc, a.bridge}; }
+  __device__ __forceinline__ StepConst<R> consts(unsigned long long) const { return StepConst<R>(a); }
+  __device__ __forceinline__ uint64_t node(unsigned long long id) const {
+    return path_node(a, a.begin + id);
+  }
+  __device__ __forceinline__ bool first(unsigned long long) const { return true; }
+  __device__ __forceinline__ bool claim(bool &exhausted, unsigned long long &id, uint64_t &node,
+                                        PhiloxPath &pp, R *x) const {
+    const unsigned lane = threadIdx.x & 31u;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(a.cursor, 32ull);
+    base = __shfl_sync(kFull, base, 0);
+    if (base + 32 >= span) exhausted = true;
+    id = base + lane;
+    if (id >= span) return false;
+    const unsigned long long g = a.begin + id;
     node = path_node(a, g);
     const uint64_t path = g - node * a.n_paths + a.path_offset;
     pp = philox_path(static_cast<uint32_t>(path), static_cast<uint32_t>(node) + a.node_offset, 0u,
                      a.rk);
 #pragma unroll
     for (int d = 0; d < D; ++d) x[d] = static_cast<R>(a.nodes[node * D + d]);
+    return true;
+  }
+  __device__ __forceinline__ void dump(unsigned long long id, R s, int32_t st, const R *xe) const {
+    dump_path<D, R>(a, id, s, st, xe);
+  }
+};
+
+// Called by all 32 lanes with an empty stash: claim up to 32 paths, score at
+// once the ones that start on the boundary (tau = 0, u = g, Eq. 2.1) or
+// outside the closed domain (invalid input: NaN, counted), and stash the
+// interior ones.  Returns how many (warp-uniform).
+template <class Model, class Geom, typename R, class Work, class Stash>
+__device__ __forceinline__ int stash_starts(const Work &a, Stash &st, bool &exhausted,
+                                            unsigned long long &my_bad) {
+  constexpr int D = Model::D;
+  const unsigned lane = threadIdx.x & 31u;
+  __syncwarp();  // earlier reads of the stash are done
+  bool interior = false;
+  R x[D];
+  PhiloxPath pp{0, 0, 0};
+  unsigned long long id = 0;
+  uint64_t node = 0;
+  R s0 = R(0);
+  const bool has = a.claim(exhausted, id, node, pp, x);
+  if (has) {
     interior = Geom::inside_open(x);
     if (!interior) {
-      s0 = Model::g(a.mc, x);
+      s0 = Model::g(a.env(id).mc, x);
       if (!Geom::inside_closed(x)) {
         s0 = R(NAN);
-        ++my_bad;
+        if (a.first(id)) ++my_bad;
       }
-      dump_path<D, R>(a, q, s0, 0, x);
+      a.dump(id, s0, 0, x);
     }
   }
   // starts on the boundary (u = g, tau = 0) or outside the closed domain (NaN)
   // go straight into the node's sums
-  const bool at_bnd = q < span && !interior;
+  const bool at_bnd = has && !interior;
   if (__any_sync(kFull, at_bnd)) fix_commit<R>(a.fix, at_bnd, node, s0, false, true);
   const unsigned im = __ballot_sync(kFull, interior);
   if (interior) {
     const int e = __popc(im & ((1u << lane) - 1u));
-    st.slot[e] = q;
+    st.id[e] = id;
     st.w0[e] = pp.r0_w0;
     st.w1[e] = pp.r0_w1;
     st.n[e] = 0;
@@ -772,9 +822,8 @@ __device__ __forceinline__ int stash_starts(const PathArgs &a, Stash &st, unsign
 // position head) run with the exact tests, one per lane.  Paths that end are
 // scored and added to their nodes' sums; the others are pushed on the stash
 // (n_start of it filled).
-template <class Model, class Geom, typename R, class Stage>
-__device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst<R> &k, Stage &st,
-                                              int head, int cnt, int &n_start,
+template <class Model, class Geom, typename R, class Work, class Stage>
+__device__ __forceinline__ void recheck_units(const Work &a, Stage &st, int head, int cnt, int &n_start,
                                               unsigned long long &my_steps,
                                               unsigned long long &my_capped) {
   constexpr int D = Model::D;
@@ -784,22 +833,24 @@ __device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst
   bool ends = false, capped = false;
   R s = R(0), X[D], Xn[D], Y = R(1), Z = R(0);
   PhiloxPath pp{0, 0, 0};
-  unsigned long long slot = 0;
+  unsigned long long id = 0;
   uint64_t node = 0;
   int32_t n = 0;
   if (has) {
     const int e = (head + lane) & (kCheckCap - 1);
-    slot = st.check.slot[e];
+    id = st.check.id[e];
     pp.r0_w0 = st.check.w0[e];
     pp.r0_w1 = st.check.w1[e];
     n = st.check.n[e];
     Z = st.check.z[e];
+    const StepConst<R> k = a.consts(id);
+    const typename Work::Env env = a.env(id);
     R y = R(1);
     if constexpr (kKeepY<Model, R>) y = st.check.y[e];
     Y = path_weight<Model, R>(k, n, y);
 #pragma unroll
     for (int d = 0; d < D; ++d) X[d] = st.check.x[d][e];
-    const int code = exact_unit<Model, Geom, R>(a, k, pp, X, Y, Z, n, Xn);
+    const int code = exact_unit<Model, Geom, R>(a, env, k, pp, X, Y, Z, n, Xn);
     capped = code == kStepContinue && n >= a.max_steps;
     ends = capped || code != kStepContinue;
     if (ends) {
@@ -808,20 +859,20 @@ __device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst
 #pragma unroll
         for (int d = 0; d < D; ++d) xe[d] = X[d];
         Geom::project(Geom::nearest_face(X), xe);
-        s = Model::g(a.mc, xe) * Y + Z;
+        s = Model::g(env.mc, xe) * Y + Z;
         ++my_capped;
       } else {
-        s = exit_score<Model, Geom, R>(a.mc, code, X, Xn, Y, Z, xe);
+        s = exit_score<Model, Geom, R>(env.mc, code, X, Xn, Y, Z, xe);
       }
       my_steps += static_cast<unsigned long long>(n);
-      node = path_node(a, a.begin + slot);
-      dump_path<D, R>(a, slot, s, capped ? -a.max_steps : n, xe);
+      node = a.node(id);
+      a.dump(id, s, capped ? -a.max_steps : n, xe);
     }
   }
   const unsigned back = __ballot_sync(kFull, has && !ends);
   if (has && !ends) {
     const int e = n_start + __popc(back & ((1u << lane) - 1u));
-    st.start.slot[e] = slot;
+    st.start.id[e] = id;
     st.start.w0[e] = pp.r0_w0;
     st.start.w1[e] = pp.r0_w1;
     st.start.n[e] = n;
@@ -835,23 +886,23 @@ __device__ __forceinline__ void recheck_units(const PathArgs &a, const StepConst
   __syncwarp();
 }
 
-template <class Model, class Geom, typename R>
-__global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_kernel(const __grid_constant__ PathArgs a) {
+// The block's paths, from a Work.
+template <class Model, class Geom, typename R, class Work>
+__device__ __forceinline__ void forward_paths(const Work &a) {
   constexpr int D = Model::D;
   using Stage = ForwardStage<D, R, kKeepY<Model, R>>;
   __shared__ Stage stage_all[kForwardBlock / 32];
   Stage &stage = stage_all[threadIdx.x >> 5];
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt_mask = (1u << lane) - 1u;
-  const StepConst<R> k(a);
-  const unsigned long long span = a.end - a.begin;
-  // the last unit start that cannot reach the step cap (nor a step count that
-  // binary32 does not hold)
-  const int32_t last_fast = (a.max_steps < (1 << 24) ? a.max_steps : 1 << 24) - 4;
+  StepConst<R> k = a.consts(0);
+  // the last unit start that ends below the step cap (and below the step counts
+  // that binary32 does not hold)
+  const int32_t last_fast = (a.max_steps < (1 << 24) ? a.max_steps : 1 << 24) - 5;
   R X[D], Y = R(1), Z = R(0);
   float e = 0.0f;
   PhiloxPath pp{0, 0, 0};
-  unsigned long long slot = 0;
+  unsigned long long id = 0;
   int32_t n = 0;
   bool active = false;
   int n_start = 0;              // stash fill; parked units and the oldest (warp-uniform)
@@ -867,7 +918,8 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
 
   // entry i of a stash becomes the lane's path
   auto load = [&](const auto &st, int i) {
-    slot = st.slot[i];
+    id = st.id[i];
+    if constexpr (Work::kOwnConsts) k = a.consts(id);
     pp.r0_w0 = st.w0[i];
     pp.r0_w1 = st.w1[i];
     pp.tag = 0u;
@@ -883,7 +935,7 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
   };
   // entry i of a stash from the start of the lane's unit
   auto store = [&](auto &st, int i, int32_t n0, const R *X0, R Y0, R Z0) {
-    st.slot[i] = slot;
+    st.id[i] = id;
     st.w0[i] = pp.r0_w0;
     st.w1[i] = pp.r0_w1;
     st.n[i] = n0;
@@ -915,7 +967,7 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
 
   // the oldest cnt parked units
   auto recheck = [&](int cnt) {
-    recheck_units<Model, Geom, R>(a, k, stage, head, cnt, n_start, my_steps, my_capped);
+    recheck_units<Model, Geom, R>(a, stage, head, cnt, n_start, my_steps, my_capped);
     head = (head + cnt) & (kCheckCap - 1);
     n_check -= cnt;
   };
@@ -929,8 +981,8 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
     if (active) {
       R z[4 * D];
       uint32_t u[4];
-      path_randoms<D, R>(a, n, pp, z, u);
-      park = fast_unit<Model, Geom, R>(a, k, z, u, n, X, Y, Z, e) || n > last_fast;
+      path_randoms<D, R>(a.rk, a.normal_tables, n, pp, z, u);
+      park = fast_unit<Model, Geom, R>(a.env(id).mc, k, z, u, n, X, Y, Z, e) || n > last_fast;
       n += 4;
     }
     const unsigned pm = __ballot_sync(kFull, park);
@@ -947,7 +999,7 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
     while (need) {  // idle lanes take stashed paths; an empty stash is refilled
       if (n_start == 0) {
         if (exhausted) break;
-        n_start = stash_starts<Model, Geom, R>(a, stage.start, span, exhausted, my_bad);
+        n_start = stash_starts<Model, Geom, R>(a, stage.start, exhausted, my_bad);
         continue;
       }
       const int r = __popc(need & lt_mask), cnt = __popc(need);
@@ -983,7 +1035,7 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
           if (active) store(stage.start, __popc(~need & lt_mask), n, X, Y, Z);
           if (static_cast<int>(lane) < n_check) {  // parked units are paths at a unit's start
             const int i = (head + static_cast<int>(lane)) & (kCheckCap - 1), o = left + static_cast<int>(lane);
-            stage.start.slot[o] = stage.check.slot[i];
+            stage.start.id[o] = stage.check.id[i];
             stage.start.w0[o] = stage.check.w0[i];
             stage.start.w1[o] = stage.check.w1[i];
             stage.start.n[o] = stage.check.n[i];
@@ -1026,6 +1078,18 @@ __global__ void __launch_bounds__(kForwardBlock, sizeof(R) == 4 ? 7 : 4) path_ke
     if (my_capped) atomicAdd(&a.counters[1], my_capped);
     if (my_bad) atomicAdd(&a.counters[2], my_bad);
   }
+}
+
+// Blocks per SM the registers are held to: 72 registers for binary32 (seven
+// blocks: the 3-D solve 762 ms, 773 at 78 registers and six), 128 and 168 for
+// binary64 without and with drift (spills below).
+template <class Model, typename R>
+constexpr int kForwardBlocks = sizeof(R) == 4 ? 7 : (Model::kDrift ? 3 : 4);
+
+template <class Model, class Geom, typename R>
+__global__ void __launch_bounds__(kForwardBlock, kForwardBlocks<Model, R>)
+path_kernel(const __grid_constant__ PathArgs a) {
+  forward_paths<Model, Geom, R>(PathWork<Model::D, R>(a));
 }
 
 }  // namespace pdd
