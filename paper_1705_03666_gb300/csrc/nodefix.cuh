@@ -142,6 +142,51 @@ __device__ __forceinline__ void fix_commit(NodeFix *fix, bool has, uint64_t node
   }
 }
 
+// Per-warp running sums of one node, for work units so short that an atomic per
+// digit and flush would contend (10^6 walks of a dozen jumps per node): lane l
+// holds word l of the node's sums (the count, then the digits), added to the
+// node with one atomic per word when the warp moves to another node.
+struct FixAccum {
+  long long v = 0;
+  uint64_t node = ~0ull;
+  __device__ __forceinline__ void flush(NodeFix *fix) {
+    const unsigned lane = threadIdx.x & 31u;
+    if (node != ~0ull && lane <= 2u * kFixDigits && v != 0)
+      atomicAdd(reinterpret_cast<unsigned long long *>(fix + node) + lane,
+                static_cast<unsigned long long>(v));
+    v = 0;
+  }
+  // As fix_commit (no boundary starts).
+  template <typename R>
+  __device__ __forceinline__ void add(NodeFix *fix, bool has, uint64_t nd, R s, bool capped) {
+    const unsigned lane = threadIdx.x & 31u;
+    const bool valid = has && fabs(s) < R(0x1p30);  // false for NaN
+    if (has && (!valid || capped))
+      atomicAdd(reinterpret_cast<unsigned long long *>(fix + nd) + (valid ? kFixCapped : kFixBad), 1ull);
+    int32_t d[2 * kFixDigits];
+#pragma unroll
+    for (int k = 0; k < 2 * kFixDigits; ++k) d[k] = 0;
+    if (valid) fix_limbs(s, d, d + kFixDigits);
+    unsigned pending = __ballot_sync(kFull, valid);
+    while (pending) {
+      const uint64_t ln = __shfl_sync(kFull, nd, __ffs(pending) - 1);
+      const bool mem = valid && nd == ln;
+      const unsigned members = __ballot_sync(kFull, mem);
+      if (ln != node) {
+        flush(fix);
+        node = ln;
+      }
+      if (lane == 0) v += __popc(members);
+#pragma unroll
+      for (int k = 0; k < 2 * kFixDigits; ++k) {
+        const int32_t r = __reduce_add_sync(kFull, mem ? d[k] : 0);
+        if (lane == static_cast<unsigned>(k + 1)) v += r;
+      }
+      pending &= ~members;
+    }
+  }
+};
+
 // Double-double helpers for the finalisation (Dekker/Knuth error-free
 // transformations with FMA).
 struct DD {

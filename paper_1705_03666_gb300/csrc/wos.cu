@@ -3,32 +3,45 @@
 // walk jumps to a uniform point on the largest circle inside the domain
 // (radius d(x) = distance to the nearest face) and stops when d(x) <= eps,
 // scoring g at the projection on that face.  No time step; the bias is
-// O(eps) and a path takes O(log 1/eps) jumps.  Same persistent lane-refill
-// layout and per-path score slots as the path kernel, one Philox block per
-// four jumps (block n/4 of stream tag 2), the per-node reduction of reduce.cuh.
+// O(eps) and a path takes O(log 1/eps) jumps.
+//
+// What bounds it: instruction issue, and the lanes that an instruction finds
+// idle (a walk lasts about a dozen jumps).  So a lane runs four jumps, one
+// Philox block (block n/4 of stream tag 2), between looks at its warp; starts
+// are set up 32 at a time into a per-warp stash, and stopped walks are parked
+// and scored 32 at a time straight into the exact per-node sums (nodefix.cuh):
+// no score is stored and no reduction follows.  16 nodes x 10^6 walks at
+// eps = 10^-4: 1.41 ms with a jump per loop trip (a Philox block for a quarter
+// of the lanes at every trip, 17 of 32 lanes busy) and a reduction of 16
+// blocks (0.19 ms); 0.63 ms now (28.5 of 32 lanes).
 #include <cmath>
 #include <cstring>
 
+#include "branch_kernel.cuh"
 #include "ctx.hpp"
-#include "path_kernel.cuh"
-#include "reduce.cuh"
-#include "warp_queue.cuh"
+#include "nodefix.cuh"
 
 namespace pdd {
 
-constexpr unsigned kWosChunk = 256;  // walks claimed per warp-level atomic
+constexpr int kWosBlock = 128;
+constexpr uint64_t kWosClaim = 256;  // most walks claimed per atomic
 
 struct WosArgs {
   const double *nodes;
-  uint64_t n_paths, path_offset, begin, end;
+  uint64_t n_paths, path_offset, total;
   unsigned long long *cursor;
   unsigned long long *counters;  // [0] jumps, [1] capped, [2] bad nodes
-  void *score;
-  int32_t *steps;
-  double *exit;                  // [end - begin][2] stopping points (projected), or null
+  NodeFix *fix;                  // [n] exact per-node sums
+  double *dump_score;            // [total] or null
+  int32_t *steps;                // [total] or null
+  double *exit;                  // [total][2] stopping points (projected), or null
   RoundKeys rk;
   double eps;
   int32_t max_steps;
+  uint32_t claim;                // walks claimed per atomic (a multiple of 32)
+  // x / n_paths for 32-bit x by one multiply-high and shifts
+  uint32_t nt_m;
+  int32_t nt_s1, nt_s2;
   ModelConst mc;
 };
 
@@ -42,20 +55,12 @@ __device__ __forceinline__ void wos_dir(double U, double &cx, double &sy) {
   sincospi(2.0 * U, &sy, &cx);
 }
 
-// Distance to the nearest face and its index, with every face index a
-// compile-time constant so the position stays in registers.
+// Distance to the nearest face; its index only where a walk stops.
 template <class Geom, typename R>
-__device__ __forceinline__ R wos_nearest(const R *x, int &jb) {
+__device__ __forceinline__ R wos_dist(const R *x) {
   R db = Geom::template face_dist<R>(0, x);
-  jb = 0;
 #pragma unroll
-  for (int j = 1; j < Geom::kFaces; ++j) {
-    const R d = Geom::template face_dist<R>(j, x);
-    if (d < db) {
-      db = d;
-      jb = j;
-    }
-  }
+  for (int j = 1; j < Geom::kFaces; ++j) db = fmin(db, Geom::template face_dist<R>(j, x));
   return db;
 }
 template <class Geom, typename R>
@@ -65,84 +70,184 @@ __device__ __forceinline__ void wos_project(int jb, R *x) {
     if (j == jb) Geom::template project<R>(j, x);
 }
 
+template <typename R>
+struct WosStage {
+  // starts (a stack of at most 32)
+  unsigned long long id[32];
+  uint32_t w0[32], w1[32];
+  R x[2][32];
+  // stopped walks (at most 63)
+  unsigned long long eid[64];
+  int32_t en[64];   // jumps
+  R ex[2][64];
+};
+
+// Node of global walk index g.
+__device__ __forceinline__ uint64_t wos_node(const WosArgs &a, uint64_t g) {
+  if (a.total <= 0xffffffffull) {
+    const uint32_t x = static_cast<uint32_t>(g), t = __umulhi(a.nt_m, x);
+    return (t + ((x - t) >> a.nt_s1)) >> a.nt_s2;
+  }
+  return g / a.n_paths;
+}
+
+// Called by all 32 lanes: score the first cnt stopped walks, one per lane.
 template <class Geom, typename R>
-__global__ void __launch_bounds__(kPathBlockOf<R>) wos_kernel(const __grid_constant__ WosArgs a) {
-  const unsigned lane = threadIdx.x & 31u;
+__device__ __forceinline__ void wos_flush(const WosArgs &a, WosStage<R> &st, int first, int cnt,
+                                          FixAccum &acc, unsigned long long &my_steps,
+                                          unsigned long long &my_capped) {
+  const int lane = static_cast<int>(threadIdx.x & 31u);
+  __syncwarp();
+  const bool has = lane < cnt;
+  R s = R(0);
+  uint64_t node = 0;
+  bool capped = false;
+  if (has) {
+    const int e = first + lane;
+    R x[2] = {st.ex[0][e], st.ex[1][e]};
+    const unsigned long long id = st.eid[e];
+    const int32_t n = st.en[e];
+    const int jb = Geom::template nearest_face<R>(x);
+    capped = n >= a.max_steps && wos_dist<Geom, R>(x) > static_cast<R>(a.eps);
+    my_capped += capped ? 1u : 0u;
+    my_steps += static_cast<unsigned long long>(n);
+    wos_project<Geom, R>(jb, x);
+    s = LaplaceExpCos::g<R>(a.mc, x);
+    node = wos_node(a, id);
+    if (a.dump_score) a.dump_score[id] = static_cast<double>(s);
+    if (a.steps) a.steps[id] = n;
+    if (a.exit) {
+      a.exit[2 * id] = static_cast<double>(x[0]);
+      a.exit[2 * id + 1] = static_cast<double>(x[1]);
+    }
+  }
+  acc.add<R>(a.fix, has, node, s, capped);
+  __syncwarp();
+}
+
+template <class Geom, typename R>
+__global__ void __launch_bounds__(kWosBlock) wos_kernel(const __grid_constant__ WosArgs a) {
+  __shared__ WosStage<R> stage_all[kWosBlock / 32];
+  WosStage<R> &st = stage_all[threadIdx.x >> 5];
+  const unsigned lane = threadIdx.x & 31u, lt_mask = (1u << lane) - 1u;
   const R eps = static_cast<R>(a.eps);
-  R X[2] = {R(0), R(0)};
-  PhiloxPath pp{0, 0, 0};
-  uint4 blk = make_uint4(0, 0, 0, 0);
-  uint64_t slot = 0;
+  R X[2] = {R(0), R(0)}, d = R(0);
+  PhiloxPath pp{0, 0, 2u};
+  unsigned long long id = 0;
   int32_t n = 0;
-  bool active = false, need = true;
+  bool active = false, exhausted = false;
+  int n_start = 0, n_stop = 0;                 // warp-uniform
+  unsigned long long next = 0, claimed = 0;    // the warp's claimed range
+  FixAccum acc;
   unsigned long long my_steps = 0, my_capped = 0, my_bad = 0;
-  R *score = static_cast<R *>(a.score);
-  WarpQueue wq;
-  NodeCache<R, 2> nc;
-  const unsigned long long total = a.end - a.begin;
-  bool pending = false;  // stopped walk whose score is written at the next claim
   for (;;) {
-    if (claim_time(active)) {
-      if (pending) {
-        score[slot] = LaplaceExpCos::g<R>(a.mc, X);
-        if (a.steps) a.steps[slot] = n;
-        if (a.exit) {
-          a.exit[2 * slot] = static_cast<double>(X[0]);
-          a.exit[2 * slot + 1] = static_cast<double>(X[1]);
+    // ---- idle lanes take starts; the stash is refilled when empty
+    unsigned need = __ballot_sync(kFull, !active);
+    while (need) {
+      if (n_start == 0) {
+        if (exhausted) break;
+        __syncwarp();
+        if (next >= claimed) {
+          unsigned long long base = 0;
+          if (lane == 0) base = atomicAdd(a.cursor, static_cast<unsigned long long>(a.claim));
+          next = __shfl_sync(kFull, base, 0);
+          claimed = next + a.claim;
         }
-        my_steps += static_cast<unsigned long long>(n);
-        pending = false;
-      }
-      need = !active;
-      while (__any_sync(kFull, need)) {
-        unsigned long long q = 0;
-        if (warp_claim<kWosChunk>(wq, a.cursor, total, need, q)) {
-          slot = q;
-          const unsigned long long g = a.begin + q;
-          nc.locate(g, a.n_paths, a.end, a.nodes);
-          const uint64_t path = g - nc.lo + a.path_offset;
-          pp = philox_path(static_cast<uint32_t>(path), static_cast<uint32_t>(nc.node), 2u, a.rk);
-          X[0] = nc.x[0];
-          X[1] = nc.x[1];
-          n = 0;
-          if (!Geom::inside_closed(X)) {
-            score[slot] = R(NAN);
-            if (a.steps) a.steps[slot] = 0;
-            if (a.exit) {
-              a.exit[2 * slot] = static_cast<double>(X[0]);
-              a.exit[2 * slot + 1] = static_cast<double>(X[1]);
-            }
+        const unsigned long long q = next + lane;
+        next += 32;
+        if (next >= a.total) exhausted = true;
+        bool in = false;
+        R x[2] = {R(0), R(0)};
+        uint64_t node = 0;
+        PhiloxPath p{0, 0, 0};
+        const bool has = q < a.total;
+        if (has) {
+          node = wos_node(a, q);
+          p = philox_path(static_cast<uint32_t>(q - node * a.n_paths + a.path_offset),
+                          static_cast<uint32_t>(node), 2u, a.rk);
+          x[0] = static_cast<R>(a.nodes[2 * node]);
+          x[1] = static_cast<R>(a.nodes[2 * node + 1]);
+          in = Geom::inside_closed(x);
+          if (!in) {
             ++my_bad;
-            need = true;
-          } else {
-            active = true;
+            if (a.dump_score) a.dump_score[q] = static_cast<double>(NAN);
+            if (a.steps) a.steps[q] = 0;
+            if (a.exit) {
+              a.exit[2 * q] = static_cast<double>(x[0]);
+              a.exit[2 * q + 1] = static_cast<double>(x[1]);
+            }
           }
         }
+        if (__any_sync(kFull, has && !in)) fix_commit<R>(a.fix, has && !in, node, R(NAN), false, false);
+        const unsigned im = __ballot_sync(kFull, in);
+        if (in) {
+          const int e = __popc(im & lt_mask);
+          st.id[e] = q;
+          st.w0[e] = p.r0_w0;
+          st.w1[e] = p.r0_w1;
+          st.x[0][e] = x[0];
+          st.x[1][e] = x[1];
+        }
+        __syncwarp();
+        n_start = __popc(im);
+        continue;
       }
-      if (!__any_sync(kFull, active)) break;
+      const int cnt = __popc(need), take = cnt < n_start ? cnt : n_start;
+      const int r = __popc(need & lt_mask);
+      if (!active && r < take) {
+        const int e = n_start - 1 - r;
+        id = st.id[e];
+        pp.r0_w0 = st.w0[e];
+        pp.r0_w1 = st.w1[e];
+        X[0] = st.x[0][e];
+        X[1] = st.x[1][e];
+        d = wos_dist<Geom, R>(X);
+        n = 0;
+        active = true;
+      }
+      n_start -= take;
+      need = __ballot_sync(kFull, !active);
     }
-    if (!active) continue;
-    int jb;
-    const R d = wos_nearest<Geom, R>(X, jb);
-    if (d <= eps || n >= a.max_steps) {
-      if (n >= a.max_steps && d > eps) ++my_capped;
-      wos_project<Geom, R>(jb, X);
-      active = false;
-      pending = true;
-      continue;
+    if (need == kFull) break;
+    // ---- up to four jumps
+    bool go = active && !(d <= eps) && n < a.max_steps;
+    {
+      const uint4 w = philox10_path(static_cast<uint32_t>(n >> 2), pp, a.rk);
+      const uint32_t wj[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (go) {
+          R cx, sy;
+          wos_dir(unif<R>(wj[j]), cx, sy);
+          X[0] += d * cx;
+          X[1] += d * sy;
+          ++n;
+          d = wos_dist<Geom, R>(X);
+          go = !(d <= eps) && n < a.max_steps;
+        }
+      }
     }
-    if ((n & 3) == 0) blk = philox10_path(static_cast<uint32_t>(n >> 2), pp, a.rk);
-    // word n mod 4 of the block: take the front word and rotate
-    const uint32_t w = blk.x;
-    blk.x = blk.y;
-    blk.y = blk.z;
-    blk.z = blk.w;
-    R cx, sy;
-    wos_dir(unif<R>(w), cx, sy);
-    X[0] += d * cx;
-    X[1] += d * sy;
-    ++n;
+    // ---- stopped walks
+    const bool stop = active && !go;
+    const unsigned sm = __ballot_sync(kFull, stop);
+    if (sm) {
+      if (stop) {
+        const int e = n_stop + __popc(sm & lt_mask);
+        st.eid[e] = id;
+        st.en[e] = n;
+        st.ex[0][e] = X[0];
+        st.ex[1][e] = X[1];
+        active = false;
+      }
+      n_stop += __popc(sm);
+      if (n_stop >= 32) {
+        n_stop -= 32;
+        wos_flush<Geom, R>(a, st, n_stop, 32, acc, my_steps, my_capped);
+      }
+    }
   }
+  if (n_stop > 0) wos_flush<Geom, R>(a, st, 0, n_stop, acc, my_steps, my_capped);
+  acc.flush(a.fix);
 #pragma unroll
   for (int m = 16; m > 0; m >>= 1) {
     my_steps += __shfl_xor_sync(kFull, my_steps, m);
@@ -156,65 +261,70 @@ __global__ void __launch_bounds__(kPathBlockOf<R>) wos_kernel(const __grid_const
   }
 }
 
+// Mean and standard error from the exact sums; the count is of all walks, also
+// of a node outside the closed domain (whose mean and error are NaN).
+__global__ void wos_finalize_kernel(const NodeFix *fix, int64_t n, double *mean, double *se,
+                                    int64_t *cnt) {
+  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (i >= n) return;
+  const NodeFix F = fix[i];
+  double m, M2;
+  fix_moments(F, &m, &M2);
+  const double nn = static_cast<double>(F.n);
+  mean[i] = m;
+  se[i] = F.n > 1 ? sqrt(M2 / (nn - 1.0) / nn) : M2;
+  if (cnt) cnt[i] = F.n + F.bad;
+}
+
 template <class Geom, typename R>
 static pdd_status run_wos(pdd_ctx *ctx, const double *d_nodes, int64_t n, const pdd_wos_params *wp,
                           double *d_mean, double *d_se, int64_t *d_npaths, pdd_diag *diag) {
   const uint64_t N = static_cast<uint64_t>(wp->n_paths);
   const uint64_t total = static_cast<uint64_t>(n) * N;
-  const uint64_t wave = std::min<uint64_t>(total, ctx->wave_max_paths);
-  const size_t acc_off = 256;
-  const size_t score_off = align_up(acc_off + static_cast<size_t>(n) * sizeof(NodeAcc), 256);
-  pdd_status st = ensure_scratch(ctx, align_up(score_off + wave * sizeof(R), 256));
+  const size_t fix_off = 256;
+  const size_t bytes = align_up(fix_off + static_cast<size_t>(n) * sizeof(NodeFix), 256);
+  pdd_status st = ensure_scratch(ctx, bytes);
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
   auto *counters = reinterpret_cast<unsigned long long *>(base);
-  auto *acc = reinterpret_cast<NodeAcc *>(base + acc_off);
-  R *score = reinterpret_cast<R *>(base + score_off);
-  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, score_off, ctx->stream));
+  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, bytes, ctx->stream));
   WosArgs a;
   std::memset(&a, 0, sizeof a);
   a.nodes = d_nodes;
   a.n_paths = N;
   a.path_offset = static_cast<uint64_t>(wp->path_offset);
+  a.total = total;
   a.cursor = counters + 4;
   a.counters = counters;
-  a.score = score;
+  a.fix = reinterpret_cast<NodeFix *>(base + fix_off);
   a.rk = make_round_keys(wp->seed);
   a.eps = wp->eps;
   a.max_steps = static_cast<int32_t>(wp->max_steps);
+  branch_divisor(N < (uint64_t(1) << 32) ? static_cast<uint32_t>(N) : 0xffffffffu, &a.nt_m, &a.nt_s1,
+                 &a.nt_s2);
   a.mc = ctx->mc;
+  if (diag) {
+    a.dump_score = diag->d_path_score;
+    a.steps = diag->d_path_steps;
+    a.exit = diag->d_path_exit;
+  }
   auto kern = wos_kernel<Geom, R>;
   int bps = 0;
-  PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPathBlockOf<R>, 0));
+  PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kWosBlock, 0));
   if (bps < 1) bps = 1;
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
-  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (wave + kPathBlockOf<R> - 1) / kPathBlockOf<R>));
-  for (uint64_t b0 = 0; b0 < total; b0 += wave) {
-    const uint64_t b1 = std::min(total, b0 + wave);
-    if (b0 > 0) PDD_CUDA_TRY(ctx, cudaMemsetAsync(a.cursor, 0, sizeof(unsigned long long), ctx->stream));
-    a.begin = b0;
-    a.end = b1;
-    a.steps = (diag && diag->d_path_steps) ? diag->d_path_steps + b0 : nullptr;
-    a.exit = (diag && diag->d_path_exit) ? diag->d_path_exit + 2 * b0 : nullptr;
-    const auto ev = prof_slot(ctx);
-    if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, ctx->stream));
-    kern<<<static_cast<unsigned>(grid), kPathBlockOf<R>, 0, ctx->stream>>>(a);
-    PDD_CUDA_TRY(ctx, cudaGetLastError());
-    if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
-    const uint64_t node_lo = b0 / N, node_hi = (b1 - 1) / N;
-    reduce_wave_kernel<R><<<static_cast<unsigned>(node_hi - node_lo + 1), kReduceBlock, 0,
-                            ctx->stream>>>(score, b0, b1, N, node_lo, acc);
-    PDD_CUDA_TRY(ctx, cudaGetLastError());
-    if (diag && diag->d_path_score) {
-      const uint64_t cnt = b1 - b0;
-      const unsigned g = static_cast<unsigned>(std::min<uint64_t>((cnt + 255) / 256, 8192));
-      widen_scores_kernel<R><<<g, 256, 0, ctx->stream>>>(score, diag->d_path_score + b0, cnt);
-      PDD_CUDA_TRY(ctx, cudaGetLastError());
-    }
-  }
-  finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(acc, n, d_mean,
-                                                                                d_se, d_npaths);
+  grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kWosBlock - 1) / kWosBlock));
+  // a quarter of a warp's share at a time, so that a small call reaches every warp
+  const uint64_t share = total / (grid * (kWosBlock / 32) * 4) / 32 * 32;
+  a.claim = static_cast<uint32_t>(std::max<uint64_t>(32, std::min<uint64_t>(kWosClaim, share)));
+  const auto ev = prof_slot(ctx);
+  if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, ctx->stream));
+  kern<<<static_cast<unsigned>(grid), kWosBlock, 0, ctx->stream>>>(a);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
+  if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
+  wos_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(
+      a.fix, n, d_mean, d_se, d_npaths);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (diag) {
     unsigned long long h[4] = {0, 0, 0, 0};
