@@ -258,17 +258,6 @@ static pdd_status launch_families(pdd_ctx *ctx, const BatchArgs &a, const unsign
   return PDD_OK;
 }
 
-// Side streams and events for launch_families (created once per context).
-static pdd_status ensure_side_streams(pdd_ctx *ctx) {
-  if (ctx->batch_fork) return PDD_OK;
-  for (int k = 0; k < 3; ++k) {
-    PDD_CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ctx->batch_side[k], cudaStreamNonBlocking));
-    PDD_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->batch_join[k], cudaEventDisableTiming));
-  }
-  PDD_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->batch_fork, cudaEventDisableTiming));
-  return PDD_OK;
-}
-
 static pdd_status enqueue_batch(pdd_ctx *ctx, const BatchArgs &proto, const BatchLayout &Lay,
                                 const pdd_batch_nodes *nodes, const pdd_batch_params *bp,
                                 const unsigned *grid, int4 combo_of_prob, int32_t n_probs,

@@ -47,9 +47,9 @@ struct pdd_ctx {
   int batch_chunk = 0;
   cudaGraphExec_t batch_graph = nullptr;
   BatchGraphKey batch_key{};
-  // batch solve: side streams and events that run the per-family kernels
-  // concurrently (forked from and joined back into `stream`); created on
-  // first use
+  // side streams and events that run launches concurrently (the batch's
+  // per-family kernels, the multilevel levels; forked from and joined back into
+  // `stream`); created on first use
   cudaStream_t batch_side[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t batch_fork = nullptr;
   cudaEvent_t batch_join[3] = {nullptr, nullptr, nullptr};
@@ -143,6 +143,18 @@ inline pdd_status ensure_aux(pdd_ctx *ctx, size_t bytes) {
     return fail(ctx, PDD_ENOMEM, "cudaMalloc(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
   }
   ctx->aux_bytes = bytes;
+  return PDD_OK;
+}
+
+// Side streams and events for launches that overlap (the batch's families, the
+// multilevel levels); created once per context.
+inline pdd_status ensure_side_streams(pdd_ctx *ctx) {
+  if (ctx->batch_fork) return PDD_OK;
+  for (int k = 0; k < 3; ++k) {
+    PDD_CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ctx->batch_side[k], cudaStreamNonBlocking));
+    PDD_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->batch_join[k], cudaEventDisableTiming));
+  }
+  PDD_CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->batch_fork, cudaEventDisableTiming));
   return PDD_OK;
 }
 
