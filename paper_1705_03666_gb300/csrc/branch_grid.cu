@@ -26,8 +26,17 @@
 // ids and pruning as for the free-space trees (branch_kernel.cuh).
 //
 // Lane layout: one lane owns one tree and walks it depth-first (pending
-// particles on a per-lane stack in local memory), one step per loop trip;
-// warps claim trees in chunks (warp_queue.cuh).  The estimate of tree g for
+// particles on a per-lane stack in local memory); warps claim trees in chunks
+// (warp_queue.cuh).  What bounds it is instruction issue, and the rare work
+// was most of it: exit tests with their four exponentials, the boundary data
+// of an exit at every later time, branching, popping and storing scores ran
+// with one or a few lanes of 32.  So the step loop carries only the steps, screened
+// by the path kernel's distance bound (edge_bound; a shorter step's bound lies
+// below a full one's); a lane whose step may exit, or whose particle or tree
+// is over, waits until a dozen do, and they are served together, the exits'
+// boundary data and the scores one (lane, time) pair per lane.  48 nodes of the
+// square x 10^5 trees x 16 times: 13.9 -> 6.7 ms (13.7 -> 20 of 32 lanes); 64
+// nodes in free space x 5 x 10^4 x 16 times 1.46 -> 1.34 ms.  The estimate of tree g for
 // time k goes to score[k * wave + slot] (FP32); one NaN-skipping FP64
 // reduction per time plane gives (count, mean, M2) per (time, node).
 #include <cmath>
@@ -36,6 +45,7 @@
 #include "branch_kernel.cuh"
 #include "ctx.hpp"
 #include "models.cuh"
+#include "path_kernel.cuh"
 #include "reduce.cuh"
 #include "warp_queue.cuh"
 
@@ -43,6 +53,12 @@ namespace pdd {
 
 constexpr int kGridMaxTimes = 32;
 constexpr unsigned kGridChunk = 64;  // trees claimed per warp-level atomic
+// Blocks per SM (a fourth, at 64 registers, measured no faster), and the lanes
+// that wait before they are served together (bounded domain; free space): 4, 8,
+// 12 and 16 measured 7.9, 7.1, 7.1 and 7.3 ms on 48 nodes of the square with 16
+// times; free space with 16 times 1.83, 1.76, 1.46 and 1.34 ms for 1, 4, 8 and 16.
+constexpr int kGridBlocks = 3;
+constexpr int kGridBatch = 12, kFreeBatch = 16;
 
 struct FreeSpace {};
 
@@ -71,6 +87,8 @@ struct GridArgs {
   int32_t K, m;
   uint32_t dt_ticks;
   int32_t bridge;
+  float edge_c0, edge_c1;         // screening bound of a full step (edge_bound)
+  int32_t m_log2;                 // smallest power of two >= m
   float cum[kMaxOffspring + 1];    // cumulative q (rounded from FP64 sums)
   float ratio[kMaxOffspring + 1];  // alpha_k / q_k
   uint32_t T[kGridMaxTimes];
@@ -101,7 +119,7 @@ __device__ __forceinline__ float grid_g(const GridArgs &a, const float *x, float
     case 0: return a.psi_prm / (a.psi_prm + (1.0f - a.psi_prm) * expf(a.beta_f * s));
     case 1: return grid_psi<D>(a, x);
     case 2: {
-      const float e = 1.0f + expf(a.psi_prm * x[0] - (5.0f / 6.0f) * a.beta_f * s);
+      const float e = 1.0f + expf(fmaf(-(5.0f / 6.0f) * a.beta_f, s, a.psi_prm * x[0]));
       return 1.0f - __fdividef(1.0f, e * e);
     }
     default: return 0.0f;
@@ -142,121 +160,133 @@ __device__ __forceinline__ bool grid_exit(const GridArgs &a, const float *x0, co
   return true;
 }
 
+// A step of at most dt towards the tick lim from (X, t) with the block v.
+// Advances X, t and e (Geom::edge of X), or, where the step may exit, returns
+// true and leaves it in (Xn, nxt).
+template <class Geom, int D>
+__device__ __forceinline__ bool grid_step(const GridArgs &a, const uint4 &v, uint32_t lim, float sh_full,
+                                          float *X, uint32_t &t, float &e, float *Xn, uint32_t &nxt) {
+  constexpr bool kBounded = GeomTraits<Geom>::kBounded;
+  const uint32_t left = lim - t;
+  const bool last = left <= a.dt_ticks;  // at a grid time or the lifetime's end
+  float sh = sh_full;
+  if (!kBounded || last) sh = sqrt_approx(static_cast<float>(left) * a.inv_tps);
+  nxt = last ? lim : t + a.dt_ticks;
+  float z0, z1;
+  box_muller<float>(v.x, v.y, z0, z1);
+  Xn[0] = X[0] + sh * z0;
+  Xn[1] = D > 1 ? X[1] + sh * z1 : 0.f;
+  if constexpr (kBounded) {
+    // (a full step's bound: also above a shorter one's)
+    const float en = Geom::edge(Xn);
+    if (!(unif_log_bits(unif_f(v.z)) >= fmaf(a.edge_c1, e * en, a.edge_c0))) return true;
+    e = en;
+  }
+  X[0] = Xn[0];
+  X[1] = Xn[1];
+  t = nxt;
+  return false;
+}
+
+// States of a lane.
+enum GridMode : int {
+  kGridIdle,   // no tree, none left
+  kGridRun,    // walking
+  kGridClaim,  // waits for a tree
+  kGridStep,   // holds a step that may exit
+  kGridEnd     // the particle's lifetime is over
+};
+
 // kBinary: two children with probability one and the classical weight (the
 // KPP law), so the offspring count and the mark are constants.
 template <class Geom, int D, bool kBinary>
-__global__ void __launch_bounds__(kBranchBlock) branch_grid_kernel(const __grid_constant__ GridArgs a) {
+__global__ void __launch_bounds__(kBranchBlock, kGridBlocks) branch_grid_kernel(const __grid_constant__ GridArgs a) {
   constexpr bool kBounded = GeomTraits<Geom>::kBounded;
   const unsigned lane = threadIdx.x & 31u;
   const uint32_t Tm = a.T[a.m - 1];
   float4 stk[kBranchMaxDepth];  // pending particles: (x1, x2, birth tick, id | ti << 16)
-  // per-time products in shared memory (bank = lane): a local array indexed
-  // by the running time index lives in local memory, whose footprint over the
-  // grid exceeds L2 and went to DRAM
-  __shared__ float sprod[kGridMaxTimes][kBranchBlock];
-  float *prod_col = &sprod[0][threadIdx.x];
-#define PROD(k) prod_col[(k) * kBranchBlock]
+  // per-time products in shared memory: a local array indexed by the running
+  // time index lives in local memory, whose footprint over the grid exceeds L2
+  // and went to DRAM.  One column per lane, padded so that a column's times
+  // also lie in different banks.
+  constexpr int kCol = kBranchBlock + 1;
+  __shared__ float sprod[kGridMaxTimes * kCol];
+  __shared__ unsigned char exits[kBranchBlock];
+  float *prod_col = &sprod[threadIdx.x];
+#define PROD(k) prod_col[(k) * kCol]
   int sp = 0;
-  float X[2] = {0.f, 0.f};
-  uint32_t id = 0, t = 0, tend = 0, j = 0, u_off = 0;
+  float X[2] = {0.f, 0.f}, Xn[2] = {0.f, 0.f};
+  float e = 0.f;                  // Geom::edge of X
+  uint32_t id = 0, t = 0, tend = 0, lim = 0, nxt = 0, j = 0, u_off = 0, wu = 0;
   int ti = 0;
-  bool start = false;
   PhiloxPath pp{0, 0, 3u};  // the (tree, node, tag 3) half of Philox round one
   uint32_t next_id = 0;
-  int64_t particles = 0;
-  int32_t nsteps = 0;
+  int32_t particles = 0, nsteps = 0;
   uint64_t slot = 0;
-  bool active = false, need = true;
+  int mode = kGridClaim;
   unsigned long long my_steps = 0, my_disc = 0, my_bad = 0;
   WarpQueue wq;
   NodeCache<float, D> nc;
   const unsigned long long total = a.end - a.begin;
+  const float h_full = static_cast<float>(a.dt_ticks) * a.inv_tps;
+  const float sh_full = sqrt_approx(h_full);
 
   for (;;) {
-    if (claim_time(active)) {
-      need = !active;
-      while (__any_sync(kFull, need)) {
-        unsigned long long q = 0;
-        if (warp_claim<kGridChunk>(wq, a.cursor, total, need, q)) {
-          slot = q;
-          const unsigned long long g = a.begin + q;
-          nc.locate(g, a.n_trees, a.end, a.nodes);
-          pp = philox_path(static_cast<uint32_t>(g - nc.lo + a.tree_offset),
-                           static_cast<uint32_t>(nc.node), 3u, a.rk);
-          X[0] = nc.x[0];
-          X[1] = D > 1 ? nc.x[D > 1 ? 1 : 0] : 0.f;
-          for (int k = 0; k < a.m; ++k) PROD(k) = 1.0f;
-          t = 0;
-          ti = 0;  // T_1 > 0
-          id = 0;
-          next_id = 1;
-          sp = 0;
-          particles = 1;
-          nsteps = 0;
-          start = true;
-          bool done = false;
-          if constexpr (kBounded) {
-            if (!Geom::template inside_closed<float>(X)) {
-              for (int k = 0; k < a.m; ++k) a.score[k * a.wave + slot] = NAN;
-              if (a.steps) a.steps[slot] = 0;
-              ++my_bad;
-              done = true;
-            } else if (!Geom::template inside_open<float>(X)) {
-              // on the boundary: absorbed at time 0
-              for (int k = 0; k < a.m; ++k)
-                a.score[k * a.wave + slot] = grid_g<D>(a, X, static_cast<float>(a.T[k]) * a.inv_tps);
-              if (a.steps) a.steps[slot] = 0;
-              done = true;
-            }
+    // ---- steps of the running lanes, until enough lanes wait
+    for (;;) {
+      const int running = __popc(__ballot_sync(kFull, mode == kGridRun));
+      const int waiting = __popc(__ballot_sync(kFull, mode > kGridRun));
+      if (running == 0 || waiting >= min(kBounded ? kGridBatch : kFreeBatch, running)) break;
+      if (mode == kGridRun) {
+        // a step, or a particle's lifetime; in a bounded domain then another
+        // step, unless this one ended at a grid time, at the lifetime's end or
+        // in a step that may exit (free-space steps all end so)
+        const uint32_t cb = (id << 20) | j;
+        const uint4 v0 = philox10_path(cb, pp, a.rk);
+        const uint4 v1 = kBounded ? philox10_path(cb + 1u, pp, a.rk) : v0;
+        const bool born = j == 0;
+        if (born) {
+          // block 0 of the particle's stream: lifetime and offspring count
+          const float ltk = 0.5f * neg2log(unif_f(v0.x)) * a.inv_beta * a.tps;
+          const uint64_t lt = ltk >= 4294967040.0f ? 4294967295ull : static_cast<uint64_t>(__float2uint_rz(ltk));
+          const uint64_t te = static_cast<uint64_t>(t) + lt;
+          tend = te < Tm ? static_cast<uint32_t>(te) : Tm;
+          lim = min(lim, tend);
+          u_off = v0.w;
+        }
+        bool held = false;
+        if (!born) held = grid_step<Geom, D>(a, v0, lim, sh_full, X, t, e, Xn, nxt);
+        wu = v0.z;
+        j += 1;
+        int taken = born ? 0 : 1;
+        if (kBounded && !held && t < lim) {
+          held = grid_step<Geom, D>(a, v1, lim, sh_full, X, t, e, Xn, nxt);
+          wu = v1.z;
+          ++j;
+          ++taken;
+        }
+        nsteps += taken;
+        if (held) {
+          mode = kGridStep;
+        } else if (t == lim) {
+          if (ti < a.m && t == a.T[ti]) {
+            PROD(ti) *= grid_psi<D>(a, X);
+            ++ti;
           }
-          if (done) need = true;
-          else active = true;
+          lim = ti < a.m ? min(a.T[ti], tend) : tend;
+          if (t == tend) mode = kGridEnd;
         }
       }
-      if (!__any_sync(kFull, active)) break;
     }
-    if (!active) continue;
+    if (!__any_sync(kFull, mode != kGridIdle)) break;
 
-    // one Philox block per trip: on the trip that starts a particle, block 0
-    // of its stream (lifetime and offspring count), else the block of its
-    // next step (Philox((id << 20 | j, tree, node, 3)))
-    const bool starting = start;
-    const uint4 v = philox10_path(starting ? id << 20 : (id << 20) | j, pp, a.rk);
-    if (starting) {
-      const float ltk = 0.5f * neg2log(unif_f(v.x)) * a.inv_beta * a.tps;
-      const uint64_t e = ltk >= 4294967040.0f ? 4294967295ull : static_cast<uint64_t>(__float2uint_rz(ltk));
-      const uint64_t te = static_cast<uint64_t>(t) + e;
-      tend = te < Tm ? static_cast<uint32_t>(te) : Tm;
-      u_off = v.w;
-      // ti (first grid time after t) is carried: a child starts where its
-      // parent's walk ended, after the parent scored any grid time equal to t
-      j = 1;
-      start = false;
-    }
-
-    // one step of the current particle (none on its starting trip, and none
-    // at all when its lifetime is under a tick)
-    bool pdone = false;
-    if (!starting && t < tend) {
-      uint32_t nxt = tend;
-      if (ti < a.m && a.T[ti] < nxt) nxt = a.T[ti];
-      if (kBounded && nxt - t > a.dt_ticks) nxt = t + a.dt_ticks;
-      const float h = static_cast<float>(nxt - t) * a.inv_tps;
-      ++j;
-      ++nsteps;
-      float z0, z1;
-      box_muller<float>(v.x, v.y, z0, z1);
-      const float sh = sqrt_approx(h);
-      float Xn[2] = {X[0] + sh * z0, D > 1 ? X[1] + sh * z1 : 0.f};
-      if constexpr (kBounded) {
-        float xe[2] = {0.f, 0.f};
-        if (grid_exit<Geom, D>(a, X, Xn, h, v.z, xe)) {
-          for (int k = ti; k < a.m; ++k)
-            PROD(k) *= grid_g<D>(a, xe, static_cast<float>(a.T[k] - nxt) * a.inv_tps);
-          pdone = true;
-        }
-      }
-      if (!pdone) {
+    // ---- the waiting lanes together
+    bool out = false;  // left the domain
+    float xe[2] = {0.f, 0.f};
+    if (mode == kGridStep) {
+      if constexpr (kBounded)
+        out = grid_exit<Geom, D>(a, X, Xn, static_cast<float>(nxt - t) * a.inv_tps, wu, xe);
+      if (!out) {
         X[0] = Xn[0];
         X[1] = Xn[1];
         t = nxt;
@@ -266,8 +296,31 @@ __global__ void __launch_bounds__(kBranchBlock) branch_grid_kernel(const __grid_
         }
       }
     }
-    bool tree_done = false, bad = false;
-    if (!pdone && t == tend) {
+    if constexpr (kBounded) {
+      // g of every exit at every later grid time: one (exit, time) pair per lane
+      const unsigned om = __ballot_sync(kFull, out);
+      if (om) {
+        unsigned char *const list = &exits[threadIdx.x & ~31u];
+        if (out) list[__popc(om & ((1u << lane) - 1u))] = static_cast<unsigned char>(lane);
+        __syncwarp();
+        const int n_out = __popc(om), per = 32 >> a.m_log2;
+        const int k = static_cast<int>(lane) & ((1 << a.m_log2) - 1);
+        for (int r0 = 0; r0 < n_out; r0 += per) {
+          const int r = r0 + (static_cast<int>(lane) >> a.m_log2);
+          const int el = r < n_out ? list[r] : 0;
+          const float ex[2] = {__shfl_sync(kFull, xe[0], el), __shfl_sync(kFull, xe[1], el)};
+          const uint32_t et = __shfl_sync(kFull, nxt, el);
+          const int ei = __shfl_sync(kFull, ti, el);
+          if (r < n_out && k >= ei && k < a.m) {
+            float *const p = &sprod[k * kCol + (threadIdx.x & ~31u) + el];
+            *p *= grid_g<D>(a, ex, static_cast<float>(a.T[k] - et) * a.inv_tps);
+          }
+        }
+        __syncwarp();
+      }
+    }
+    bool pdone = out, tree_done = false, bad = false, begin = false;
+    if (mode > kGridClaim && !out && t == tend) {
       if (tend == Tm) {
         pdone = true;
       } else {
@@ -292,19 +345,15 @@ __global__ void __launch_bounds__(kBranchBlock) branch_grid_kernel(const __grid_
           tree_done = true;
         } else if (k == 0) {
           pdone = true;
-        } else if constexpr (kBinary) {
-          stk[sp++] = make_float4(X[0], X[1], __uint_as_float(tend),
-                                  __uint_as_float((next_id + 1) | (static_cast<uint32_t>(ti) << 16)));
-          id = next_id;
-          next_id += 2;
-          start = true;  // continue with the first child from (X, tend)
         } else {
+          // ti (first grid time after t) is carried: a child starts where its
+          // parent's walk ended, after the parent scored any grid time equal to t
           for (int c = k - 1; c >= 1; --c)
             stk[sp++] = make_float4(X[0], X[1], __uint_as_float(tend),
                                     __uint_as_float((next_id + c) | (static_cast<uint32_t>(ti) << 16)));
           id = next_id;
           next_id += k;
-          start = true;  // continue with the first child from (X, tend)
+          begin = true;  // continue with the first child from (X, tend)
         }
       }
     }
@@ -318,17 +367,82 @@ __global__ void __launch_bounds__(kBranchBlock) branch_grid_kernel(const __grid_
         t = __float_as_uint(p.z);
         id = __float_as_uint(p.w) & 0xffffu;
         ti = static_cast<int>(__float_as_uint(p.w) >> 16);
-        start = true;
+        begin = true;
       }
     }
-    if (tree_done) {
-      for (int k = 0; k < a.m; ++k)
-        a.score[k * a.wave + slot] = bad ? NAN : PROD(k);
-      if (a.steps) a.steps[slot] = bad ? -nsteps : nsteps;
-      my_steps += static_cast<unsigned long long>(nsteps);
-      if (bad) ++my_disc;
-      active = false;
-      need = true;
+    const unsigned dm = __ballot_sync(kFull, tree_done);
+    if (dm) {
+      // scores: one (tree, time) pair per lane
+      unsigned char *const list = &exits[threadIdx.x & ~31u];
+      if (tree_done) list[__popc(dm & ((1u << lane) - 1u))] = static_cast<unsigned char>(lane);
+      __syncwarp();
+      const int n_done = __popc(dm), per = 32 >> a.m_log2;
+      const unsigned bm = __ballot_sync(kFull, bad);
+      const int k = static_cast<int>(lane) & ((1 << a.m_log2) - 1);
+      for (int r0 = 0; r0 < n_done; r0 += per) {
+        const int r = r0 + (static_cast<int>(lane) >> a.m_log2);
+        const int el = r < n_done ? list[r] : 0;
+        const uint64_t es = __shfl_sync(kFull, slot, el);
+        if (r < n_done && k < a.m)
+          a.score[k * a.wave + es] = (bm >> el) & 1u ? NAN : sprod[k * kCol + (threadIdx.x & ~31u) + el];
+      }
+      __syncwarp();
+      if (tree_done) {
+        if (a.steps) a.steps[slot] = bad ? -nsteps : nsteps;
+        my_steps += static_cast<unsigned long long>(nsteps);
+        if (bad) ++my_disc;
+        mode = kGridClaim;
+      }
+    }
+    bool need = mode == kGridClaim;
+    if (need) mode = kGridIdle;
+    while (__any_sync(kFull, need)) {
+      unsigned long long q = 0;
+      if (warp_claim<kGridChunk>(wq, a.cursor, total, need, q)) {
+        slot = q;
+        const unsigned long long g = a.begin + q;
+        nc.locate(g, a.n_trees, a.end, a.nodes);
+        pp = philox_path(static_cast<uint32_t>(g - nc.lo + a.tree_offset),
+                         static_cast<uint32_t>(nc.node), 3u, a.rk);
+        X[0] = nc.x[0];
+        X[1] = D > 1 ? nc.x[D > 1 ? 1 : 0] : 0.f;
+        t = 0;
+        ti = 0;  // T_1 > 0
+        id = 0;
+        next_id = 1;
+        sp = 0;
+        particles = 1;
+        nsteps = 0;
+        begin = true;
+        if constexpr (kBounded) {
+          if (!Geom::template inside_closed<float>(X)) {
+            for (int k = 0; k < a.m; ++k) a.score[k * a.wave + slot] = NAN;
+            if (a.steps) a.steps[slot] = 0;
+            ++my_bad;
+            begin = false;
+          } else if (!Geom::template inside_open<float>(X)) {
+            // on the boundary: absorbed at time 0
+            for (int k = 0; k < a.m; ++k)
+              a.score[k * a.wave + slot] = grid_g<D>(a, X, static_cast<float>(a.T[k]) * a.inv_tps);
+            if (a.steps) a.steps[slot] = 0;
+            begin = false;
+          }
+        }
+        if (begin)
+          for (int k = 0; k < a.m; ++k) PROD(k) = 1.0f;
+        need = !begin;
+      }
+    }
+    if (begin) {
+      // the particle's first trip draws its lifetime
+      j = 0;
+      tend = Tm;
+    }
+    if (begin || mode > kGridClaim) {
+      mode = kGridRun;
+      lim = tend;
+      if (ti < a.m && a.T[ti] < lim) lim = a.T[ti];
+      if constexpr (kBounded) e = Geom::edge(X);
     }
   }
 #pragma unroll
@@ -412,6 +526,14 @@ static pdd_status run_grid(pdd_ctx *ctx, const double *d_nodes, int64_t n, const
   a.m = m;
   a.dt_ticks = dt_ticks;
   a.bridge = bp->bridge ? 1 : 0;
+  if constexpr (GeomTraits<Geom>::kBounded) {
+    // a full step's standard deviation, with slack for its binary32 rounding; a
+    // face within reach has both ends of the step within 7.06 s of it
+    const double sd = std::sqrt(dt_ticks / tps) * (1.0 + 0x1p-20);
+    edge_bound(sd, bp->bridge != 0, 14.2 * sd < 1.0 ? Geom::reach(sd) : Geom::kFaces, &a.edge_c0,
+               &a.edge_c1);
+  }
+  while ((1 << a.m_log2) < m) ++a.m_log2;
   double cum = 0.0;
   for (int k = 0; k <= a.K; ++k) {
     const double q = prm[4 + k], al = prm[5 + a.K + k];
