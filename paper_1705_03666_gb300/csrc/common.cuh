@@ -74,10 +74,9 @@ __device__ __forceinline__ PhiloxPath philox_path(uint32_t path, uint32_t node,
   return pp;
 }
 
-// Same value as philox10(j, path, node, tag, rk).
-__device__ __forceinline__ uint4 philox10_path(uint32_t j, const PhiloxPath &pp,
-                                               const RoundKeys &rk) {
-  const uint64_t p0 = static_cast<uint64_t>(kPhiloxM0) * j;
+// Same value as philox10(j, path, node, tag, rk), from p0 = M0 j.
+__device__ __forceinline__ uint4 philox10_product(uint64_t p0, const PhiloxPath &pp,
+                                                  const RoundKeys &rk) {
   uint32_t c0 = pp.r0_w0;
   uint32_t c1 = pp.r0_w1;
   uint32_t c2 = static_cast<uint32_t>(p0 >> 32) ^ pp.tag ^ rk.k[1];
@@ -94,6 +93,11 @@ __device__ __forceinline__ uint4 philox10_path(uint32_t j, const PhiloxPath &pp,
     c2 = n2;
   }
   return make_uint4(c0, c1, c2, c3);
+}
+
+__device__ __forceinline__ uint4 philox10_path(uint32_t j, const PhiloxPath &pp,
+                                               const RoundKeys &rk) {
+  return philox10_product(static_cast<uint64_t>(kPhiloxM0) * j, pp, rk);
 }
 
 // ---------------------------------------------------------------------------

@@ -449,10 +449,10 @@ template <int D, typename R, class BM>
 __device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, const RoundKeys &rk,
                                              R *z, uint32_t *u, BM bm) {
   if constexpr (D == 3) {
-    const uint32_t q3 = 3u * (static_cast<uint32_t>(n) >> 2);
-    const uint4 A = philox10_path(q3, pp, rk);
-    const uint4 B = philox10_path(q3 + 1u, pp, rk);
-    const uint4 C = philox10_path(q3 + 2u, pp, rk);
+    const uint64_t p = static_cast<uint64_t>(kPhiloxM0) * (3u * (static_cast<uint32_t>(n) >> 2));
+    const uint4 A = philox10_product(p, pp, rk);
+    const uint4 B = philox10_product(p + kPhiloxM0, pp, rk);
+    const uint4 C = philox10_product(p + 2ull * kPhiloxM0, pp, rk);
     bm(A.x, A.y, z[0], z[1]);
     bm(A.z, A.w, z[2], z[3]);
     bm(B.x, B.y, z[4], z[5]);
@@ -464,10 +464,10 @@ __device__ __forceinline__ void unit_randoms(int32_t n, const PhiloxPath &pp, co
     u[2] = low_bytes_word(B.z, B.w, C.x);
     u[3] = low_bytes_word(C.y, C.z, C.w);
   } else {
-    const uint32_t q3 = 3u * (static_cast<uint32_t>(n) >> 2);
-    const uint4 A = philox10_path(q3, pp, rk);
-    const uint4 B = philox10_path(q3 + 1u, pp, rk);
-    const uint4 C = philox10_path(q3 + 2u, pp, rk);
+    const uint64_t p = static_cast<uint64_t>(kPhiloxM0) * (3u * (static_cast<uint32_t>(n) >> 2));
+    const uint4 A = philox10_product(p, pp, rk);
+    const uint4 B = philox10_product(p + kPhiloxM0, pp, rk);
+    const uint4 C = philox10_product(p + 2ull * kPhiloxM0, pp, rk);
     const uint32_t w[8] = {A.x, A.y, A.z, A.w, B.x, B.y, B.z, B.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
