@@ -639,28 +639,36 @@ __device__ __forceinline__ bool fast_unit(const ModelConst &mc, const StepConst<
 }
 
 // The unit at step n again, a step at a time with the exact tests (em_step)
-// and the step cap; the random numbers are shifted down by static indices so
+// and the step cap; its random numbers are shifted down by static indices so
 // that one copy of the step serves all four.
-template <class Model, class Geom, typename R, class Work>
-__device__ __forceinline__ int exact_unit(const Work &a, const typename Work::Env &env,
-                                          const StepConst<R> &k, const PhiloxPath &pp, R *X, R &Y,
-                                          R &Z, int32_t &n, R *Xn) {
+template <class Model, class Geom, typename R, class Env>
+__device__ __forceinline__ int exact_steps(const Env &env, const StepConst<R> &k, int32_t max_steps,
+                                           R *z, uint32_t *u, R *X, R &Y, R &Z, int32_t &n, R *Xn) {
   constexpr int D = Model::D;
-  R z[4 * D];
-  uint32_t u[4];
-  path_randoms<D, R>(a.rk, a.normal_tables, n, pp, z, u);
   int code = kStepContinue;
 #pragma unroll 1
   for (int j = 0; j < 4; ++j) {
     code = em_step<Model, Geom, R, false>(env, k, X, Y, Z, z, u[0], n, Xn, static_cast<R *>(nullptr));
     ++n;
-    if (code != kStepContinue || n >= a.max_steps) break;
+    if (code != kStepContinue || n >= max_steps) break;
 #pragma unroll
     for (int i = 0; i < 3 * D; ++i) z[i] = z[i + D];
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i] = u[i + 1];
   }
   return code;
+}
+
+// Score (s, exit point xe) of a path that left with the code, or was capped:
+// then at the projection of its last point on the nearest face.
+template <class Model, class Geom, typename R>
+__device__ __forceinline__ R end_score(const ModelConst &mc, int code, bool capped, const R *X,
+                                       const R *Xn, R Y, R Z, R *xe) {
+  if (!capped) return exit_score<Model, Geom, R>(mc, code, X, Xn, Y, Z, xe);
+#pragma unroll
+  for (int d = 0; d < Model::D; ++d) xe[d] = X[d];
+  Geom::project(Geom::nearest_face(X), xe);
+  return Model::g(mc, xe) * Y + Z;
 }
 
 // Paths at the start of a unit, N of them, in shared memory.  A path's
@@ -685,17 +693,16 @@ struct ForwardStage {
   PathStash<D, R, kY, kStashCap> start;
   PathStash<D, R, kY, kCheckCap> check;
 };
-// At the wave's end lanes idle, and what is left is the longest paths' chain.
-// Parked units are then rerun once they are as many as the busy lanes: neither
-// are the others held up at every unit nor the parked ones for long (16 x 2000
-// paths of the square: 153 us, 190 us when any parked unit is rerun at once,
-// 191 us when they wait until no lane is busy).
+// At the wave's end lanes idle, and what is left is the longest paths' chain: a
+// warp's last paths are finished with several lanes to each (finish_together).
+// Before, parked units are rerun once they are as many as the busy lanes: neither
+// are the others held up at every unit nor the parked ones for long.
 // Binary64 paths are bound by the FP64 pipe to the end, so a warp with at most
 // kDonate of them left leaves them (in its own stash, `given` of them) to the
-// block's other warps and ends: fewer, fuller warps (16 x 10^4 FP64 paths: 11.4
-// -> 6.2 ms with both rules).  Binary32 paths are bound by latency there, and
-// fuller warps only hold each other up (153 -> 190 us on the square).  A warp
-// that leaves publishes its paths before it lowers `alive`; the warp that
+// block's other warps and ends: fewer, fuller warps, the last of which finishes
+// its paths as above (16 x 10^4 FP64 paths: 2.06 ms, 2.37 without).  Binary32
+// paths are bound by latency there, and fuller warps only hold each other up.  A
+// warp that leaves publishes its paths before it lowers `alive`; the warp that
 // brings `alive` to zero looks for published paths once more before it ends,
 // so none is lost.
 constexpr int kDonate = 24;
@@ -850,20 +857,16 @@ __device__ __forceinline__ void recheck_units(const Work &a, Stage &st, int head
     Y = path_weight<Model, R>(k, n, y);
 #pragma unroll
     for (int d = 0; d < D; ++d) X[d] = st.check.x[d][e];
-    const int code = exact_unit<Model, Geom, R>(a, env, k, pp, X, Y, Z, n, Xn);
+    R z[4 * D];
+    uint32_t u[4];
+    path_randoms<D, R>(a.rk, a.normal_tables, n, pp, z, u);
+    const int code = exact_steps<Model, Geom, R>(env, k, a.max_steps, z, u, X, Y, Z, n, Xn);
     capped = code == kStepContinue && n >= a.max_steps;
     ends = capped || code != kStepContinue;
     if (ends) {
       R xe[D];
-      if (capped) {  // scored at the projection of its last point on the nearest face
-#pragma unroll
-        for (int d = 0; d < D; ++d) xe[d] = X[d];
-        Geom::project(Geom::nearest_face(X), xe);
-        s = Model::g(env.mc, xe) * Y + Z;
-        ++my_capped;
-      } else {
-        s = exit_score<Model, Geom, R>(env.mc, code, X, Xn, Y, Z, xe);
-      }
+      s = end_score<Model, Geom, R>(env.mc, code, capped, X, Xn, Y, Z, xe);
+      if (capped) ++my_capped;
       my_steps += static_cast<unsigned long long>(n);
       node = a.node(id);
       a.dump(id, s, capped ? -a.max_steps : n, xe);
@@ -884,6 +887,114 @@ __device__ __forceinline__ void recheck_units(const Work &a, Stage &st, int head
   n_start += __popc(back);
   fix_commit<R>(a.fix, ends, node, s, capped, false);
   __syncwarp();
+}
+
+// Called by all 32 lanes with cnt <= kTogether paths at a unit's start in the
+// stash: runs them to their ends, G = 32 / (the next power of two) lanes to a
+// path.  Random numbers are most of a unit's work (about three quarters) and do
+// not depend on the path, so each of a path's lanes forms those of another of
+// its next G units; then all of them take the units together, the random
+// numbers handed round by shuffles, and a unit that may hold an exit at once with
+// the exact tests.  Kept out of line: the main loop's registers are its own.
+// With at most 16 paths to a warp (8: the L-shape 2 % slower): 16 x 2000 paths
+// of the square 141 -> 102 us, 16 x 10^4 FP64 paths with both stages 3.00 ->
+// 2.06 ms.
+constexpr int kTogether = 16;
+struct PathCounts {
+  unsigned long long steps, capped;
+};
+template <class Model, class Geom, typename R, class Work, class Stage>
+__device__ __noinline__ PathCounts finish_together(const Work a, Stage &st, int cnt, int32_t last_fast) {
+  constexpr int D = Model::D;
+  const unsigned lane = threadIdx.x & 31u;
+  StepConst<R> k = a.consts(0);
+  PathCounts mine{0, 0};
+  while (cnt > 0) {
+    int lg = 5;  // log2 G
+    while (lg > 0 && (32 >> lg) < cnt) --lg;
+    const unsigned g = lane & ((1u << lg) - 1u), p = lane >> lg;
+    __syncwarp();
+    bool alive = static_cast<int>(p) < cnt;
+    const int i = alive ? static_cast<int>(p) : 0;
+    const unsigned long long id = st.start.id[i];
+    if constexpr (Work::kOwnConsts) k = a.consts(id);
+    const PhiloxPath pp{st.start.w0[i], st.start.w1[i], 0u};
+    int32_t n = st.start.n[i];
+    R X[D], Xn[D], Z = st.start.z[i], y = R(1);
+    if constexpr (kKeepY<Model, R>) y = st.start.y[i];
+    R Y = path_weight<Model, R>(k, n, y);
+#pragma unroll
+    for (int d = 0; d < D; ++d) X[d] = st.start.x[d][i];
+    float e = path_edge<Geom, R>(X);
+    const typename Work::Env env = a.env(id);
+    __syncwarp();
+    int left = cnt;
+    do {
+      R zg[4 * D];
+      uint32_t ug[4];
+      path_randoms<D, R>(a.rk, a.normal_tables,
+                         static_cast<int32_t>(static_cast<uint32_t>(n) + 4u * g), pp, zg, ug);
+      bool ends = false, capped = false;
+      R s = R(0);
+#pragma unroll 1
+      for (int q = 0; q < (1 << lg); ++q) {
+        const int from = static_cast<int>(lane - g) + q;
+        R z[4 * D];
+        uint32_t u[4];
+#pragma unroll
+        for (int j = 0; j < 4 * D; ++j) z[j] = __shfl_sync(kFull, zg[j], from);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) u[j] = __shfl_sync(kFull, ug[j], from);
+        if (!alive) continue;
+        R X0[D], Y0 = Y, Z0 = Z;
+#pragma unroll
+        for (int d = 0; d < D; ++d) X0[d] = X[d];
+        const bool maybe = fast_unit<Model, Geom, R>(env.mc, k, z, u, n, X, Y, Z, e);
+        if (!maybe && n <= last_fast) {
+          n += 4;
+          continue;
+        }
+#pragma unroll
+        for (int d = 0; d < D; ++d) X[d] = X0[d];
+        Y = Y0;
+        Z = Z0;
+        const int code = exact_steps<Model, Geom, R>(env, k, a.max_steps, z, u, X, Y, Z, n, Xn);
+        capped = code == kStepContinue && n >= a.max_steps;
+        ends = capped || code != kStepContinue;
+        if (ends) {
+          R xe[D];
+          s = end_score<Model, Geom, R>(env.mc, code, capped, X, Xn, Y, Z, xe);
+          if (g == 0) {
+            a.dump(id, s, capped ? -a.max_steps : n, xe);
+            mine.steps += static_cast<unsigned long long>(n);
+            mine.capped += capped ? 1u : 0u;
+          }
+          alive = false;
+        } else {
+          e = path_edge<Geom, R>(X);
+        }
+      }
+      const bool has = ends && g == 0;
+      if (__any_sync(kFull, has)) fix_commit<R>(a.fix, has, has ? a.node(id) : 0, s, capped, false);
+      left = __popc(__ballot_sync(kFull, alive && g == 0));
+    } while (left > 0 && (left > 32 >> (lg + 1) || lg == 5));
+    // fewer paths than half the groups: more lanes to each
+    const unsigned am = __ballot_sync(kFull, alive && g == 0);
+    if (alive && g == 0) {
+      const int o = __popc(am & ((1u << lane) - 1u));
+      st.start.id[o] = id;
+      st.start.w0[o] = pp.r0_w0;
+      st.start.w1[o] = pp.r0_w1;
+      st.start.n[o] = n;
+      st.start.z[o] = Z;
+      if constexpr (kKeepY<Model, R>) st.start.y[o] = Y;
+#pragma unroll
+      for (int d = 0; d < D; ++d) st.start.x[d][o] = X[d];
+    }
+    cnt = left;
+  }
+  __syncwarp();
+  return mine;
 }
 
 // The block's paths, from a Work.
@@ -965,6 +1076,26 @@ __device__ __forceinline__ void forward_paths(const Work &a) {
     return need;
   };
 
+  // every path that the warp holds into its stash (empty before); returns how many
+  auto gather = [&](unsigned need) -> int {
+    const int busy = 32 - __popc(need);
+    if (active) store(stage.start, __popc(~need & lt_mask), n, X, Y, Z);
+    if (static_cast<int>(lane) < n_check) {  // parked units are paths at a unit's start
+      const int i = (head + static_cast<int>(lane)) & (kCheckCap - 1), o = busy + static_cast<int>(lane);
+      stage.start.id[o] = stage.check.id[i];
+      stage.start.w0[o] = stage.check.w0[i];
+      stage.start.w1[o] = stage.check.w1[i];
+      stage.start.n[o] = stage.check.n[i];
+      stage.start.z[o] = stage.check.z[i];
+      if constexpr (kKeepY<Model, R>) stage.start.y[o] = stage.check.y[i];
+#pragma unroll
+      for (int d = 0; d < D; ++d) stage.start.x[d][o] = stage.check.x[d][i];
+    }
+    const int all = busy + n_check;
+    n_check = 0;
+    __syncwarp();
+    return all;
+  };
   // the oldest cnt parked units
   auto recheck = [&](int cnt) {
     recheck_units<Model, Geom, R>(a, stage, head, cnt, n_start, my_steps, my_capped);
@@ -1023,6 +1154,15 @@ __device__ __forceinline__ void forward_paths(const Work &a) {
       n_start -= take;
       need = __ballot_sync(kFull, !active);
     }
+    if (need && 32 - __popc(need) + n_check <= kTogether && (!kCompact<R> || last)) {
+      if constexpr (kCompact<R>) need = adopt(need);
+      if (32 - __popc(need) + n_check <= kTogether) {
+        const PathCounts c = finish_together<Model, Geom, R>(a, stage, gather(need), last_fast);
+        my_steps += c.steps;
+        my_capped += c.capped;
+        break;
+      }
+    }
     if (n_check > 0 && (n_check >= 32 || n_check >= 32 - __popc(need))) {
       recheck(n_check < 32 ? n_check : 32);
       continue;
@@ -1032,19 +1172,7 @@ __device__ __forceinline__ void forward_paths(const Work &a) {
         need = adopt(need);
         const int left = 32 - __popc(need), all = left + n_check;
         if (all <= kDonate && !last) {
-          if (active) store(stage.start, __popc(~need & lt_mask), n, X, Y, Z);
-          if (static_cast<int>(lane) < n_check) {  // parked units are paths at a unit's start
-            const int i = (head + static_cast<int>(lane)) & (kCheckCap - 1), o = left + static_cast<int>(lane);
-            stage.start.id[o] = stage.check.id[i];
-            stage.start.w0[o] = stage.check.w0[i];
-            stage.start.w1[o] = stage.check.w1[i];
-            stage.start.n[o] = stage.check.n[i];
-            stage.start.z[o] = stage.check.z[i];
-            if constexpr (kKeepY<Model, R>) stage.start.y[o] = stage.check.y[i];
-#pragma unroll
-            for (int d = 0; d < D; ++d) stage.start.x[d][o] = stage.check.x[d][i];
-          }
-          n_check = 0;
+          gather(need);
           __threadfence_block();
           __syncwarp();
           int before = 0;
