@@ -307,7 +307,8 @@ static pdd_status enqueue_batch(pdd_ctx *ctx, const BatchArgs &proto, const Batc
   st = launch_families(ctx, a, grid);
   if (st != PDD_OK) return st;
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
-  fix_finalize_kernel<<<nb, 256, 0, ctx->stream>>>(fix, n, d_mean, d_se, d_npaths, nullptr);
+  fix_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0,
+                        ctx->stream>>>(fix, n, d_mean, d_se, d_npaths, nullptr);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   return PDD_OK;
 }

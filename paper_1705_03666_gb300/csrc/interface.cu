@@ -123,7 +123,7 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   kern<<<static_cast<unsigned>(grid), kForwardBlock, 0, ctx->stream>>>(a);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
-  fix_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(
+  fix_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, ctx->stream>>>(
       fix, n, d_mean, d_se, d_npaths, diag ? diag->d_node_flags : nullptr);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
 

@@ -651,7 +651,7 @@ static pdd_status run_mlmc(pdd_ctx *ctx, cudaStream_t stream, char *base, const 
   kern<<<static_cast<unsigned>(grid), kMlmcBlock<R>, 0, stream>>>(a);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, stream));
-  mlmc_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
+  mlmc_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, stream>>>(
       a.fix, n, mp->level, d_mean, d_var, d_fine, d_coarse);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   return PDD_OK;

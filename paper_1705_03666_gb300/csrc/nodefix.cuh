@@ -19,6 +19,8 @@
 // absolute value, far below the rounding of the score itself.
 #pragma once
 
+#include <cstring>
+
 #include "common.cuh"
 
 namespace pdd {
@@ -187,73 +189,103 @@ struct FixAccum {
   }
 };
 
-// Double-double helpers for the finalisation (Dekker/Knuth error-free
-// transformations with FMA).
-struct DD {
-  double hi, lo;
-};
-__device__ __forceinline__ DD dd_two_sum(double a, double b) {
-  const double s = a + b;
-  const double bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
+// 2^e, a normal number.
+__host__ __device__ __forceinline__ double fix_pow2(int e) {
+  const long long b = static_cast<long long>(e + 1023) << 52;
+  double d;
+  memcpy(&d, &b, sizeof d);
+  return d;
 }
-__device__ __forceinline__ DD dd_norm(double hi, double lo) {
-  const double s = hi + lo;
-  return {s, lo - (s - hi)};
-}
-__device__ __forceinline__ DD dd_add(DD a, DD b) {
-  const DD s = dd_two_sum(a.hi, b.hi);
-  return dd_norm(s.hi, s.lo + a.lo + b.lo);
-}
-__device__ __forceinline__ DD dd_mul(DD a, DD b) {
-  const double p = a.hi * b.hi;
-  const double e = fma(a.hi, b.hi, -p);
-  return dd_norm(p, e + a.hi * b.lo + a.lo * b.hi);
-}
-__device__ __forceinline__ DD dd_div(DD a, double d) {
-  const double q1 = a.hi / d;
-  const double p = q1 * d;
-  const double e = fma(q1, d, -p);
-  const double r = ((a.hi - p) - e) + a.lo;
-  return dd_norm(q1, r / d);
-}
-// The exact digit total sum_k l[k] 2^(24k - 60) as a double-double.
-__device__ __forceinline__ DD fix_total(const long long *l) {
-  DD t{0.0, 0.0};
-#pragma unroll
-  for (int k = 0; k < kFixDigits; ++k) {
-    const double sc = ldexp(1.0, 24 * k - 60);
-    const double hi = static_cast<double>(l[k]);
-    const double lo = static_cast<double>(l[k] - static_cast<long long>(hi));
-    t = dd_add(t, DD{hi * sc, lo * sc});
-  }
-  return t;
+// The 63 leading bits m of a (256 bits, w[3] the highest word, not zero) and
+// their weight: a = m 2^e but for what is below m.
+__host__ __device__ __forceinline__ unsigned long long fix_top(const unsigned long long *w, int *e) {
+  int h = 3;
+  while (h > 0 && w[h] == 0) --h;
+  int lz = 0;
+  for (int s = 32; s > 0; s >>= 1)
+    if ((w[h] << lz) >> (64 - s) == 0) lz += s;
+  const unsigned long long below = h > 0 ? w[h - 1] : 0;
+  const unsigned long long top = lz ? (w[h] << lz) | (below >> (64 - lz)) : w[h];
+  *e = 64 * h - lz + 1;
+  return top >> 1;
 }
 
-// Mean and the sum of squared deviations M2 of a node's scores from its
-// exact sums: mean = S1/n, M2 = S2 - S1^2/n in double-double (M2 = 0 when
-// every path started on the boundary, or with one path).  Both NaN when a
-// path was invalid or nothing was scored.
-__device__ __forceinline__ void fix_moments(const NodeFix &F, double *mean, double *m2) {
-  const double nn = static_cast<double>(F.n);
+// Mean and the sum of squared deviations M2 of a node's scores from its exact
+// sums: mean = S1 / n and M2 = (n S2 - S1^2) / n, the numerator in exact
+// integers (256 bits) and rounded once, so that FP64, a 1/64-rate pipe on this
+// part, only has to divide: one warp took 10.4 us for both in double-doubles
+// (some 350 dependent instructions) after every small solve.  M2 = 0 when every
+// path started on the boundary, or with one path; both NaN when a path was
+// invalid or nothing was scored.
+__host__ __device__ __forceinline__ void fix_moments(const NodeFix &F, double *mean, double *m2) {
+  using u64 = unsigned long long;
+  using u128 = unsigned __int128;
   *mean = static_cast<double>(NAN);
   *m2 = static_cast<double>(NAN);
   if (F.bad != 0 || F.n <= 0) return;
-  const DD S1 = fix_total(F.s1), S2 = fix_total(F.s2);
-  const DD mu = dd_div(S1, nn);
-  *mean = mu.hi + mu.lo;
-  *m2 = 0.0;
-  if (F.boundary != F.n && F.n > 1) {
-    const DD q = dd_mul(S1, mu);
-    const DD d = dd_add(S2, DD{-q.hi, -q.lo});
-    *m2 = fmax(0.0, d.hi + d.lo);
+  const u64 n = static_cast<u64>(F.n);
+  const double nn = static_cast<double>(F.n), rn = 1.0 / nn;
+  // S1 2^60: below n 2^90 <= 2^122 in magnitude, so sums mod 2^128 hold it
+  u128 t = 0;
+#pragma unroll
+  for (int k = 0; k < kFixDigits; ++k)
+    t += static_cast<u128>(static_cast<__int128>(F.s1[k])) << (24 * k);
+  const bool neg = (t >> 127) != 0;
+  if (neg) t = 0 - t;
+  const u64 a0 = static_cast<u64>(t), a1 = static_cast<u64>(t >> 64);
+  if (t == 0) {
+    *mean = 0.0;
+  } else {
+    const u64 w[4] = {a0, a1, 0, 0};
+    int e;
+    const u64 m = fix_top(w, &e);
+    const double hi = static_cast<double>(m);
+    const double lo = static_cast<double>(static_cast<long long>(m) - static_cast<long long>(hi));
+    const double q = hi * rn;
+    const double r = (fma(-q, nn, hi) + lo) * rn;
+    *mean = (neg ? -(q + r) : q + r) * fix_pow2(e - 60);
   }
+  *m2 = 0.0;
+  if (F.boundary == F.n || F.n <= 1) return;
+  // n S2 2^120 (S2's digits are not negative)
+  const u128 lo = static_cast<u128>(static_cast<u64>(F.s2[0])) +
+                  (static_cast<u128>(static_cast<u64>(F.s2[1])) << 24) +
+                  (static_cast<u128>(static_cast<u64>(F.s2[2])) << 48);
+  const u128 hi = static_cast<u128>(static_cast<u64>(F.s2[3])) +
+                  (static_cast<u128>(static_cast<u64>(F.s2[4])) << 24);  // weight 2^72
+  const u128 mid = (lo >> 64) + (hi << 8);
+  const u128 p0 = static_cast<u128>(static_cast<u64>(lo)) * n;
+  const u128 p1 = static_cast<u128>(static_cast<u64>(mid)) * n + (p0 >> 64);
+  const u64 n0 = static_cast<u64>(p0), n1 = static_cast<u64>(p1);
+  const u64 n2 = static_cast<u64>(mid >> 64) * n + static_cast<u64>(p1 >> 64);
+  u64 d[4] = {n0 << 60, (n0 >> 4) | (n1 << 60), (n1 >> 4) | (n2 << 60), n2 >> 4};
+  // minus (S1 2^60)^2
+  const u128 q00 = static_cast<u128>(a0) * a0, q01 = static_cast<u128>(a0) * a1 << 1,
+             q11 = static_cast<u128>(a1) * a1;
+  const u128 c1 = (q00 >> 64) + static_cast<u64>(q01);
+  const u128 c2 = (c1 >> 64) + (q01 >> 64) + static_cast<u64>(q11);
+  const u64 sq[4] = {static_cast<u64>(q00), static_cast<u64>(c1), static_cast<u64>(c2),
+                     static_cast<u64>(c2 >> 64) + static_cast<u64>(q11 >> 64)};
+  u64 borrow = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const u128 v = static_cast<u128>(d[k]) - sq[k] - borrow;
+    d[k] = static_cast<u64>(v);
+    borrow = (v >> 127) != 0 ? 1 : 0;
+  }
+  // (the truncation of the scores can leave it negative where they are all alike)
+  if (borrow || (d[0] | d[1] | d[2] | d[3]) == 0) return;
+  int e;
+  const u64 m = fix_top(d, &e);
+  *m2 = static_cast<double>(m) * rn * fix_pow2(e - 120);
 }
 
 // Mean, standard error of the mean, path count and flags per node from the
 // exact sums: se = sqrt(M2 / (n - 1) / n), 0 when every path started on the
 // boundary (tau = 0, the estimate is exact) or with one path; NaN when a
-// path was invalid or nothing was scored.
+// path was invalid or nothing was scored.  32 threads to a block: the warps'
+// FP64 divisions and square roots run on an SM each.
+constexpr int kFinalizeBlock = 32;
 static __global__ void fix_finalize_kernel(const NodeFix *fix, int64_t n_nodes, double *mean,
                                            double *se, int64_t *npaths, int32_t *flags) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -262,7 +294,7 @@ static __global__ void fix_finalize_kernel(const NodeFix *fix, int64_t n_nodes, 
   const double nn = static_cast<double>(F.n);
   double m, M2;
   fix_moments(F, &m, &M2);
-  const double e = F.n > 1 ? sqrt(M2 / (nn - 1.0) / nn) : M2;  // M2 is 0 or NaN for n <= 1
+  const double e = F.n > 1 ? sqrt(M2 / ((nn - 1.0) * nn)) : M2;  // M2 is 0 or NaN for n <= 1
   mean[i] = m;
   se[i] = e;
   if (npaths) npaths[i] = F.n;

@@ -140,7 +140,7 @@ pdd_status run_static(char *base, int device, cudaStream_t stream, const pdd_pro
   uint64_t grid = static_cast<uint64_t>(std::max(bps, 1)) * static_cast<uint64_t>(num_sms);
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kForwardBlock - 1) / kForwardBlock));
   kern<<<static_cast<unsigned>(grid), kForwardBlock, 0, stream>>>(a);
-  fix_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(
+  fix_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, stream>>>(
       fix, n, d_mean, d_se, d_npaths, nullptr);
   return cudaGetLastError() == cudaSuccess ? PDD_OK : PDD_ECUDA;
 }

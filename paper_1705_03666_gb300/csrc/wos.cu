@@ -272,7 +272,7 @@ __global__ void wos_finalize_kernel(const NodeFix *fix, int64_t n, double *mean,
   fix_moments(F, &m, &M2);
   const double nn = static_cast<double>(F.n);
   mean[i] = m;
-  se[i] = F.n > 1 ? sqrt(M2 / (nn - 1.0) / nn) : M2;
+  se[i] = F.n > 1 ? sqrt(M2 / ((nn - 1.0) * nn)) : M2;
   if (cnt) cnt[i] = F.n + F.bad;
 }
 
@@ -323,7 +323,7 @@ static pdd_status run_wos(pdd_ctx *ctx, const double *d_nodes, int64_t n, const 
   kern<<<static_cast<unsigned>(grid), kWosBlock, 0, ctx->stream>>>(a);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
-  wos_finalize_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(
+  wos_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, ctx->stream>>>(
       a.fix, n, d_mean, d_se, d_npaths);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (diag) {
