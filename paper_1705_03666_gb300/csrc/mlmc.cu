@@ -771,7 +771,8 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   // its side streams in turn, so that the end of one level's launch (lanes idle
   // while its last pairs finish) is filled by the next (four levels of 16 nodes:
   // 5.9 ms one after another, 5.45 ms so; a share of the blocks for each level
-  // measured 10 ms)
+  // measured 10 ms); the finest, with the longest walks, first (five levels of 4
+  // nodes and 20000 pairs: 0.88 -> 0.83 ms)
   pdd_mlmc_params lps[13];
   LevelCounts N{};
   for (int l = 0; l < n_levels; ++l) {
@@ -793,8 +794,9 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   for (int k = 0; k < side; ++k)
     PDD_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->batch_side[k], ctx->batch_fork, 0));
   pdd_status launched = PDD_OK;
-  for (int l = 0; l < n_levels && launched == PDD_OK; ++l) {
-    cudaStream_t s = l % 4 == 0 ? ctx->stream : ctx->batch_side[l % 4 - 1];
+  for (int q = 0; q < n_levels && launched == PDD_OK; ++q) {
+    const int l = n_levels - 1 - q;
+    cudaStream_t s = q % 4 == 0 ? ctx->stream : ctx->batch_side[q % 4 - 1];
     launched = mlmc_launch(ctx, s, base + per * l, d_nodes, n, &lps[l], lm + static_cast<size_t>(l) * n,
                            lv + static_cast<size_t>(l) * n, nullptr, nullptr, nullptr);
   }

@@ -28,7 +28,11 @@ struct NodeAcc {  // running (count, mean, M2) per node, FP64
 // summed plainly in FP64 (a few thousand terms per thread).  FP64 is a
 // 1/64-rate pipe on this part, so a compensated FP64 sum per score would
 // make the reduction, not the paths, the cost of short-path workloads.
-// Threads are then combined with compensated FP64 sums in a fixed tree.
+// Threads are then combined in a fixed tree in FP64: two-float sums part by
+// part (their high parts, 24 bits each, add up exactly while they are within
+// 2^20 of one another), binary64 sums compensated.  Compensated additions for
+// both, 170 FP64 instructions per warp, took 76 of 125 us for 1024 nodes of 10^5
+// binary32 scores; 93 us in all now.
 struct F2Sum {
   float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float v) {
@@ -38,6 +42,22 @@ struct F2Sum {
     hi = s;
   }
 };
+
+// The two parts of a two-float sum, added separately.
+struct PartSum {
+  double hi = 0.0, lo = 0.0;
+  __device__ __forceinline__ void merge(const PartSum &o) {
+    hi += o.hi;
+    lo += o.lo;
+  }
+  __device__ __forceinline__ double value() const { return hi + lo; }
+};
+__device__ __forceinline__ PartSum shfl_xor(const PartSum &v, int m) {
+  PartSum o;
+  o.hi = __shfl_xor_sync(kFull, v.hi, m);
+  o.lo = __shfl_xor_sync(kFull, v.lo, m);
+  return o;
+}
 
 template <typename R, bool kSkipNaN>
 struct ThreadSums;
@@ -70,11 +90,10 @@ struct ThreadSums<float, kSkipNaN> {
     s2.add(q);
     s2.lo += e + 2.0f * d * dl;
   }
-  __device__ __forceinline__ void out(CSum &c1, CSum &c2) const {
-    c1.add(static_cast<double>(s1.hi));
-    c1.add(static_cast<double>(s1.lo));
-    c2.add(static_cast<double>(s2.hi));
-    c2.add(static_cast<double>(s2.lo));
+  using Total = PartSum;
+  __device__ __forceinline__ void out(PartSum &c1, PartSum &c2) const {
+    c1 = {static_cast<double>(s1.hi), static_cast<double>(s1.lo)};
+    c2 = {static_cast<double>(s2.hi), static_cast<double>(s2.lo)};
   }
 };
 template <bool kSkipNaN>
@@ -88,6 +107,7 @@ struct ThreadSums<double, kSkipNaN> {
     s1 += d;
     s2 = fma(d, d, s2);
   }
+  using Total = CSum;
   __device__ __forceinline__ void out(CSum &c1, CSum &c2) const {
     c1.add(s1);
     c2.add(s2);
@@ -135,7 +155,8 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
   } else {
     for (uint64_t i = threadIdx.x; i < cnt; i += kReduceBlock) ts.add(s[i], Kr);
   }
-  CSum s1, s2;
+  using Total = typename ThreadSums<R, kSkipNaN>::Total;
+  Total s1, s2;
   ts.out(s1, s2);
   unsigned long long kept = ts.kept;
 #pragma unroll
@@ -144,7 +165,7 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
     s2.merge(shfl_xor(s2, m));
     kept += __shfl_xor_sync(kFull, kept, m);
   }
-  __shared__ CSum sh1[kReduceBlock / 32], sh2[kReduceBlock / 32];
+  __shared__ Total sh1[kReduceBlock / 32], sh2[kReduceBlock / 32];
   __shared__ unsigned long long shk[kReduceBlock / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
@@ -154,7 +175,7 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    CSum t1 = sh1[0], t2 = sh2[0];
+    Total t1 = sh1[0], t2 = sh2[0];
     unsigned long long tk = shk[0];
     for (int w = 1; w < kReduceBlock / 32; ++w) {
       t1.merge(sh1[w]);
