@@ -494,8 +494,11 @@ static pdd_status run_grid(pdd_ctx *ctx, const double *d_nodes, int64_t n, const
   const uint64_t total = static_cast<uint64_t>(n) * N;
   const uint64_t wave = std::min<uint64_t>(total, std::max<uint64_t>(1, ctx->wave_max_paths / m));
   const size_t acc_off = 256;
-  const size_t score_off =
+  const uint64_t wave_nodes = std::min<uint64_t>(static_cast<uint64_t>(n), wave / N + 2);
+  const int parts = reduce_parts(N, wave_nodes * m);
+  const size_t part_off =
       align_up(acc_off + static_cast<size_t>(n) * m * sizeof(NodeAcc), 256);
+  const size_t score_off = part_off + reduce_parts_bytes(wave_nodes * m, parts);
   pdd_status st = ensure_scratch(ctx, align_up(score_off + wave * m * sizeof(float), 256));
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
@@ -503,6 +506,7 @@ static pdd_status run_grid(pdd_ctx *ctx, const double *d_nodes, int64_t n, const
   auto *acc = reinterpret_cast<NodeAcc *>(base + acc_off);
   float *score = reinterpret_cast<float *>(base + score_off);
   PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, score_off, ctx->stream));
+  const ReduceParts rp = reduce_parts_at(base + part_off, wave_nodes * m, parts);
 
   const double *prm = ctx->params.data();
   GridArgs a;
@@ -570,8 +574,8 @@ static pdd_status run_grid(pdd_ctx *ctx, const double *d_nodes, int64_t n, const
     const uint64_t node_lo = b0 / N, node_hi = (b1 - 1) / N;
     // the m time planes in one launch (blockIdx.y = plane)
     reduce_wave_kernel<float, true>
-        <<<dim3(static_cast<unsigned>(node_hi - node_lo + 1), static_cast<unsigned>(m)),
-           kReduceBlock, 0, ctx->stream>>>(score, b0, b1, N, node_lo, acc, wave,
+        <<<dim3(static_cast<unsigned>((node_hi - node_lo + 1) * parts), static_cast<unsigned>(m)),
+           kReduceBlock, 0, ctx->stream>>>(score, b0, b1, N, node_lo, acc, rp, wave,
                                            static_cast<uint64_t>(n));
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     if (diag && diag->d_path_score) {

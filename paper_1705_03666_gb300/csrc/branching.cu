@@ -32,7 +32,10 @@ static pdd_status run_branching(pdd_ctx *ctx, const double *d_nodes_xt, int64_t 
                                            uint64_t(1) << 31);
   const size_t acc_off = 256;
   const size_t xt_off = align_up(acc_off + static_cast<size_t>(n) * sizeof(NodeAcc), 256);
-  const size_t score_off = align_up(xt_off + static_cast<size_t>(n) * sizeof(float4), 256);
+  const uint64_t wave_nodes = std::min<uint64_t>(static_cast<uint64_t>(n), wave / N + 2);
+  const int parts = reduce_parts(N, wave_nodes);
+  const size_t part_off = align_up(xt_off + static_cast<size_t>(n) * sizeof(float4), 256);
+  const size_t score_off = part_off + reduce_parts_bytes(wave_nodes, parts);
   const size_t bytes = align_up(score_off + wave * sizeof(float), 256);
   pdd_status st = ensure_scratch(ctx, bytes);
   if (st != PDD_OK) return st;
@@ -42,7 +45,8 @@ static pdd_status run_branching(pdd_ctx *ctx, const double *d_nodes_xt, int64_t 
   auto *acc = reinterpret_cast<NodeAcc *>(base + acc_off);
   auto *xt_f = reinterpret_cast<float4 *>(base + xt_off);
   float *score = reinterpret_cast<float *>(base + score_off);
-  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, xt_off, ctx->stream));
+  PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, score_off, ctx->stream));
+  const ReduceParts rp = reduce_parts_at(base + part_off, wave_nodes, parts);
   node_xt_f32_kernel<<<static_cast<unsigned>(std::min<int64_t>((n + 255) / 256, 4096)), 256, 0,
                        ctx->stream>>>(d_nodes_xt, n, D, xt_f);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
@@ -111,8 +115,8 @@ static pdd_status run_branching(pdd_ctx *ctx, const double *d_nodes_xt, int64_t 
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
     const uint64_t node_lo = b0 / N, node_hi = (b1 - 1) / N;
-    reduce_wave_kernel<float, true><<<static_cast<unsigned>(node_hi - node_lo + 1), kReduceBlock,
-                                       0, ctx->stream>>>(score, b0, b1, N, node_lo, acc);
+    reduce_wave_kernel<float, true><<<static_cast<unsigned>((node_hi - node_lo + 1) * parts), kReduceBlock,
+                                       0, ctx->stream>>>(score, b0, b1, N, node_lo, acc, rp);
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     if (diag && diag->d_path_score) {
       const uint64_t cnt = b1 - b0;

@@ -2,15 +2,19 @@
 // (the Monte Carlo estimator of Sec. 2: the mean over independent
 // realisations, with its statistical error).
 //
-// Each wave of the path index space is reduced by one block per node: the
+// Each wave of the path index space is reduced by `parts` blocks per node: a
 // block sums the shifted scores (s - K, with K the node's first score in the
-// wave) and their squares with compensated FP64 accumulators, combines the
-// threads in a fixed tree (warp shuffles, then shared memory), and merges the
-// wave's (count, mean, M2) into the node's running triple with Chan's formula.
-// Waves are processed in order, so the result is deterministic.
+// wave) and their squares, combines the threads in a fixed tree (warp shuffles,
+// then shared memory), and the node's last block to finish adds the parts in a
+// fixed tree and merges the wave's (count, mean, M2) into the node's running
+// triple with Chan's formula.  Waves are processed in order, so the result is
+// deterministic.
 #pragma once
 
+#include <cstring>
+
 #include "common.cuh"
+#include "ctx.hpp"
 #include "nodefix.cuh"
 
 namespace pdd {
@@ -114,24 +118,58 @@ struct ThreadSums<double, kSkipNaN> {
   }
 };
 
+// The parts of a wave's nodes (rec [planes][nodes][parts], done [planes][nodes]
+// counts the finished ones, zero before and after).
+struct ReducePart {
+  PartSum s1, s2;  // (a CSum's two words for binary64 scores)
+  unsigned long long kept;
+};
+struct ReduceParts {
+  int parts;
+  ReducePart *rec;
+  unsigned *done;
+};
+// Blocks per node: one while the nodes fill the GPU (512 blocks), else up to 32
+// of at least 4096 scores (4 nodes x 10^5 scores: 36 us with one, 9.6 us with
+// 16; 16 x 10^6: 186 -> 16 us).  A function of the sizes alone, so the order of
+// the additions does not depend on the device.
+inline int reduce_parts(uint64_t n_paths, uint64_t blocks) {
+  int p = 1;
+  while (p < 32 && blocks * p < 512 && n_paths / (2 * p) >= 4096) p *= 2;
+  return p;
+}
+inline size_t reduce_parts_bytes(uint64_t blocks, int parts) {
+  return parts > 1 ? align_up(blocks * parts * sizeof(ReducePart), 256) +
+                         align_up(blocks * sizeof(unsigned), 256)
+                   : 0;
+}
+// The layout at `base` (its counters zeroed by the caller).
+inline ReduceParts reduce_parts_at(char *base, uint64_t blocks, int parts) {
+  return {parts, reinterpret_cast<ReducePart *>(base),
+          reinterpret_cast<unsigned *>(base + align_up(blocks * parts * sizeof(ReducePart), 256))};
+}
+
 // kSkipNaN: NaN scores mark discarded samples (pruned trees) and are left
 // out of the count; the shift K is then 0 (scores are bounded weights).
 template <typename R, bool kSkipNaN = false>
 __global__ void __launch_bounds__(kReduceBlock)
 reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
-                   uint64_t n_paths, uint64_t node_lo, NodeAcc *acc,
+                   uint64_t n_paths, uint64_t node_lo, NodeAcc *acc, ReduceParts rp,
                    uint64_t score_plane = 0, uint64_t acc_plane = 0) {
   // blockIdx.y selects a plane (score + y score_plane, acc + y acc_plane):
   // several score planes of one wave reduced by one launch
   score += blockIdx.y * score_plane;
   acc += blockIdx.y * acc_plane;
-  const uint64_t node = node_lo + blockIdx.x;
-  const uint64_t lo = max(begin, node * n_paths);
-  const uint64_t hi = min(end, (node + 1) * n_paths);
-  if (lo >= hi) return;
+  const uint64_t node = node_lo + blockIdx.x / rp.parts;
+  const unsigned part = blockIdx.x % rp.parts;
+  const uint64_t nlo = max(begin, node * n_paths);
+  const uint64_t nhi = min(end, (node + 1) * n_paths);
+  if (nlo >= nhi) return;
+  const uint64_t lo = nlo + (nhi - nlo) * part / rp.parts;
+  const uint64_t hi = nlo + (nhi - nlo) * (part + 1) / rp.parts;
   const R *s = score + (lo - begin);
   const uint64_t cnt = hi - lo;
-  const R Kr = kSkipNaN ? R(0) : s[0];
+  const R Kr = kSkipNaN ? R(0) : score[nlo - begin];
   const double K = static_cast<double>(Kr);
   ThreadSums<R, kSkipNaN> ts;
   if constexpr (sizeof(R) == 4) {
@@ -174,14 +212,48 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
     shk[warp] = kept;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Total t1 = sh1[0], t2 = sh2[0];
-    unsigned long long tk = shk[0];
-    for (int w = 1; w < kReduceBlock / 32; ++w) {
-      t1.merge(sh1[w]);
-      t2.merge(sh2[w]);
-      tk += shk[w];
+  if (threadIdx.x >= 32) return;
+  Total t1 = sh1[0], t2 = sh2[0];
+  unsigned long long tk = shk[0];
+  for (int w = 1; w < kReduceBlock / 32; ++w) {
+    t1.merge(sh1[w]);
+    t2.merge(sh2[w]);
+    tk += shk[w];
+  }
+  if (rp.parts > 1) {
+    static_assert(sizeof(Total) == sizeof(PartSum), "a part's record");
+    const uint64_t q = blockIdx.y * (gridDim.x / rp.parts) + blockIdx.x / rp.parts;
+    ReducePart *const rec = rp.rec + q * rp.parts;
+    unsigned before = 0;
+    if (lane == 0) {
+      ReducePart o;
+      memcpy(&o.s1, &t1, sizeof t1);
+      memcpy(&o.s2, &t2, sizeof t2);
+      o.kept = tk;
+      rec[part] = o;
+      __threadfence();
+      before = atomicAdd(rp.done + q, 1u);
     }
+    if (__shfl_sync(kFull, before, 0) != static_cast<unsigned>(rp.parts - 1)) return;
+    __threadfence();
+    t1 = t2 = Total{};
+    tk = 0;
+    if (lane < rp.parts) {
+      const volatile ReducePart *const v = rec + lane;
+      const double a[5] = {v->s1.hi, v->s1.lo, v->s2.hi, v->s2.lo, 0.0};
+      memcpy(&t1, a, sizeof t1);
+      memcpy(&t2, a + 2, sizeof t2);
+      tk = v->kept;
+    }
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      t1.merge(shfl_xor(t1, m));
+      t2.merge(shfl_xor(t2, m));
+      tk += __shfl_xor_sync(kFull, tk, m);
+    }
+    if (lane == 0) rp.done[q] = 0;
+  }
+  if (threadIdx.x == 0) {
     if (tk == 0) return;
     const double nb = static_cast<double>(tk);
     const double S1 = t1.value(), S2 = t2.value();

@@ -695,7 +695,10 @@ static pdd_status run_reflect(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   const uint64_t total = static_cast<uint64_t>(n) * N;
   const uint64_t wave = std::min<uint64_t>(total, ctx->wave_max_paths);
   const size_t acc_off = 256;
-  const size_t score_off = align_up(acc_off + static_cast<size_t>(n) * sizeof(NodeAcc), 256);
+  const uint64_t wave_nodes = std::min<uint64_t>(static_cast<uint64_t>(n), wave / N + 2);
+  const int parts = reduce_parts(N, wave_nodes);
+  const size_t part_off = align_up(acc_off + static_cast<size_t>(n) * sizeof(NodeAcc), 256);
+  const size_t score_off = part_off + reduce_parts_bytes(wave_nodes, parts);
   const size_t table_off = align_up(score_off + wave * sizeof(R), 256);
   pdd_status st = ensure_scratch(ctx, table_off + (sizeof(R) == 8 ? kNormalEntries * sizeof(double2) : 0));
   if (st != PDD_OK) return st;
@@ -704,6 +707,7 @@ static pdd_status run_reflect(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   auto *acc = reinterpret_cast<NodeAcc *>(base + acc_off);
   R *score = reinterpret_cast<R *>(base + score_off);
   PDD_CUDA_TRY(ctx, cudaMemsetAsync(base, 0, score_off, ctx->stream));
+  const ReduceParts rp = reduce_parts_at(base + part_off, wave_nodes, parts);
   int32_t *flags = diag ? diag->d_node_flags : nullptr;
   if (flags) PDD_CUDA_TRY(ctx, cudaMemsetAsync(flags, 0, static_cast<size_t>(n) * 4, ctx->stream));
   ReflectArgs a;
@@ -778,8 +782,8 @@ static pdd_status run_reflect(pdd_ctx *ctx, const double *d_nodes, int64_t n,
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
     const uint64_t node_lo = b0 / N, node_hi = (b1 - 1) / N;
-    reduce_wave_kernel<R><<<static_cast<unsigned>(node_hi - node_lo + 1), kReduceBlock, 0,
-                            ctx->stream>>>(score, b0, b1, N, node_lo, acc);
+    reduce_wave_kernel<R><<<static_cast<unsigned>((node_hi - node_lo + 1) * parts), kReduceBlock, 0,
+                            ctx->stream>>>(score, b0, b1, N, node_lo, acc, rp);
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     if (diag && diag->d_path_score) {
       const uint64_t cnt = b1 - b0;
