@@ -3,8 +3,8 @@
 //
 // 1. spline_kernel: a cubic spline with not-a-knot end conditions through the
 //    interface end points (values of g, which they lie on) and the Monte Carlo
-//    node values (one thread; tridiagonal after eliminating the not-a-knot
-//    rows).
+//    node values (tridiagonal after eliminating the not-a-knot rows; parallel
+//    cyclic reduction by one block).
 // 2. fill_kernel: Dirichlet data on the grid boundary -- g on the physical
 //    sides, the spline on the interface side -- and a zero interior.
 // 3. cg_kernel / cg_mixed_kernel / jacobi_kernel: the 5-point system
@@ -15,6 +15,7 @@
 //    transforms (dst.cu).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -34,43 +35,86 @@ constexpr int kStencilBlock = 1024;
 // Interior rows: h_{i-1} M_{i-1} + 2 (h_{i-1} + h_i) M_i + h_i M_{i+1}
 //                = 6 ((y_{i+1} - y_i)/h_i - (y_i - y_{i-1})/h_{i-1}),
 // not-a-knot:    h_1 M_0 - (h_0 + h_1) M_1 + h_0 M_2 = 0 and the mirror row,
-// which are used to eliminate M_0 and M_K; Thomas algorithm on M_1..M_{K-1}.
-__global__ void spline_kernel(const double *s, const double *y, int K, double *M, double *work) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double *a = work, *b = work + (K + 1), *c = work + 2 * (K + 1), *d = work + 3 * (K + 1);
-  for (int i = 1; i < K; ++i) {
-    const double h0 = s[i] - s[i - 1], h1 = s[i + 1] - s[i];
-    a[i] = h0;
-    b[i] = 2.0 * (h0 + h1);
-    c[i] = h1;
-    d[i] = 6.0 * ((y[i + 1] - y[i]) / h1 - (y[i] - y[i - 1]) / h0);
+// which are used to eliminate M_0 and M_K.  M_1..M_{K-1} by parallel cyclic
+// reduction (Hockney): ceil(log2(K - 1)) rounds, each row with one division a
+// round, against a chain of two divisions a row on one thread (the rows are
+// diagonally dominant by a factor of two): 17 intervals 32 + 5 us with the
+// knots' own launch, 12.5 us now; 4000 intervals 6.6 -> 0.2 ms.  The knots first: s[0] and s[K] are the interface
+// end points, where the data are g (Eq. 1.1), s[1..K-1] the nodes' coordinates
+// along the interface.  work: kSplineWork arrays of K + 1.
+constexpr int kSplineWork = 10;
+__global__ void __launch_bounds__(1024)
+spline_kernel(const double *node_s, const double *vals, double s_lo, double s_hi, double fixed,
+              int along_axis, double *s, double *y, int K, double *M, double *work) {
+  const int T = static_cast<int>(blockDim.x), t0 = static_cast<int>(threadIdx.x);
+  for (int i = t0; i <= K; i += T) {
+    if (i == 0 || i == K) {
+      const double t = i == 0 ? s_lo : s_hi;
+      const double x = along_axis == 1 ? fixed : t, yy = along_axis == 1 ? t : fixed;
+      s[i] = t;
+      y[i] = exp(x) * cos(yy);
+    } else {
+      s[i] = node_s[i - 1];
+      y[i] = vals[i - 1];
+    }
   }
+  __syncthreads();
+  const size_t L = static_cast<size_t>(K) + 1;
   const double h0 = s[1] - s[0], h1 = s[2] - s[1];
   const double hl = s[K] - s[K - 1], hm = s[K - 1] - s[K - 2];
-  if (K == 3) {
-    // rows 1 and 2 only; M0 = ((h0+h1) M1 - h0 M2)/h1, M3 = ((hm+hl) M2 - hl M1)/hm
-    const double b1 = b[1] + a[1] * (h0 + h1) / h1, c1 = c[1] - a[1] * h0 / h1;
-    const double a2 = a[2] - c[2] * hl / hm, b2 = b[2] + c[2] * (hm + hl) / hm;
-    const double det = b1 * b2 - c1 * a2;
-    M[1] = (d[1] * b2 - c1 * d[2]) / det;
-    M[2] = (b1 * d[2] - a2 * d[1]) / det;
-  } else {
-    b[1] += a[1] * (h0 + h1) / h1;
-    c[1] -= a[1] * h0 / h1;
-    a[1] = 0.0;
-    b[K - 1] += c[K - 1] * (hm + hl) / hm;
-    a[K - 1] -= c[K - 1] * hl / hm;
-    c[K - 1] = 0.0;
-    for (int i = 2; i < K; ++i) {
-      const double w = a[i] / b[i - 1];
-      b[i] -= w * c[i - 1];
-      d[i] -= w * d[i - 1];
+  for (int i = 1 + t0; i < K; i += T) {
+    const double g0 = s[i] - s[i - 1], g1 = s[i + 1] - s[i];
+    double a = g0, b = 2.0 * (g0 + g1), c = g1;
+    const double d = 6.0 * ((y[i + 1] - y[i]) / g1 - (y[i] - y[i - 1]) / g0);
+    const double a0 = a, c0 = c;
+    if (i == 1) {
+      b += a0 * (h0 + h1) / h1;
+      c -= a0 * h0 / h1;
+      a = 0.0;
     }
-    M[K - 1] = d[K - 1] / b[K - 1];
-    for (int i = K - 2; i >= 1; --i) M[i] = (d[i] - c[i] * M[i + 1]) / b[i];
+    if (i == K - 1) {
+      b += c0 * (hm + hl) / hm;
+      a = i == 1 ? 0.0 : a - c0 * hl / hm;
+      c = 0.0;
+    }
+    work[i] = a;
+    work[L + i] = b;
+    work[2 * L + i] = c;
+    work[3 * L + i] = d;
+    work[4 * L + i] = 1.0 / b;
   }
-  M[0] = ((h0 + h1) * M[1] - h0 * M[2]) / h1;
-  M[K] = ((hm + hl) * M[K - 1] - hl * M[K - 2]) / hm;
+  double *from = work, *to = work + 5 * L;
+  for (int st = 1; st < K - 1; st <<= 1) {
+    __syncthreads();
+    for (int i = 1 + t0; i < K; i += T) {
+      double a = from[i], b = from[L + i], c = from[2 * L + i], d = from[3 * L + i];
+      const double al = i - st >= 1 ? -a * from[4 * L + i - st] : 0.0;
+      const double ga = i + st < K ? -c * from[4 * L + i + st] : 0.0;
+      a = c = 0.0;
+      if (i - st >= 1) {
+        a = al * from[i - st];
+        b = fma(al, from[2 * L + i - st], b);
+        d = fma(al, from[3 * L + i - st], d);
+      }
+      if (i + st < K) {
+        c = ga * from[2 * L + i + st];
+        b = fma(ga, from[i + st], b);
+        d = fma(ga, from[3 * L + i + st], d);
+      }
+      to[i] = a;
+      to[L + i] = b;
+      to[2 * L + i] = c;
+      to[3 * L + i] = d;
+      to[4 * L + i] = 1.0 / b;
+    }
+    double *const x = from;
+    from = to;
+    to = x;
+  }
+  for (int i = 1 + t0; i < K; i += T) M[i] = from[3 * L + i] / from[L + i];
+  __syncthreads();
+  if (t0 == 0) M[0] = ((h0 + h1) * M[1] - h0 * M[2]) / h1;
+  if (t0 == T - 1) M[K] = ((hm + hl) * M[K - 1] - hl * M[K - 2]) / hm;
 }
 
 __device__ double spline_eval(const double *s, const double *y, const double *M, int K, double t) {
@@ -83,23 +127,6 @@ __device__ double spline_eval(const double *s, const double *y, const double *M,
   const double A = s[lo + 1] - t, B = t - s[lo];
   return M[lo] * A * A * A / (6.0 * h) + M[lo + 1] * B * B * B / (6.0 * h) +
          (y[lo] / h - M[lo] * h / 6.0) * A + (y[lo + 1] / h - M[lo + 1] * h / 6.0) * B;
-}
-
-// Interface knots: s[0] and s[K] are the interface end points, where the data
-// are g; s[1..K-1] are the node coordinates along the interface.
-__global__ void knots_kernel(const double *node_s, const double *vals, int64_t m, double s_lo,
-                             double s_hi, double fixed, int along_axis, double *s, double *y) {
-  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (i > m + 1) return;
-  if (i == 0 || i == m + 1) {
-    const double t = i == 0 ? s_lo : s_hi;
-    const double x = along_axis == 1 ? fixed : t, yy = along_axis == 1 ? t : fixed;
-    s[i] = t;
-    y[i] = exp(x) * cos(yy);  // g of the Laplace family, Eq. 1.1 data
-  } else {
-    s[i] = node_s[i - 1];
-    y[i] = vals[i - 1];
-  }
 }
 
 // Boundary data and zero interior on an [ny][nx] grid.
@@ -524,9 +551,9 @@ pdd_status subdomain_solve_impl(pdd_ctx *ctx, const pdd_subdomain *sd, const dou
   const int K = static_cast<int>(m) + 1;
   const size_t npts = static_cast<size_t>(nx) * ny;
   const size_t knot_bytes = align_up(static_cast<size_t>(K + 1) * sizeof(double), 256);
-  // scratch: s, y, M, work(4 x), then 3 grid vectors, then 2 result words
+  // scratch: s, y, M, work, then 3 grid vectors, then 2 result words
   const size_t off_s = 0, off_y = knot_bytes, off_M = 2 * knot_bytes, off_w = 3 * knot_bytes;
-  const size_t off_v = off_w + 4 * knot_bytes;
+  const size_t off_v = off_w + kSplineWork * knot_bytes;
   const size_t vec = align_up(npts * sizeof(double), 256);
   const size_t off_out = off_v + 3 * vec;
   const size_t off_dst = off_out + 256;
@@ -544,10 +571,8 @@ pdd_status subdomain_solve_impl(pdd_ctx *ctx, const pdd_subdomain *sd, const dou
 
   const int ax = sd->iface_axis, along = 1 - ax;
   const double fixed = sd->iface_side ? sd->hi[ax] : sd->lo[ax];
-  knots_kernel<<<static_cast<unsigned>((m + 2 + 255) / 256), 256, 0, ctx->stream>>>(
-      d_iface_s, d_iface_vals, m, sd->lo[along], sd->hi[along], fixed, along, s, y);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
-  spline_kernel<<<1, 32, 0, ctx->stream>>>(s, y, K, M, w);
+  spline_kernel<<<1, static_cast<unsigned>(std::min(1024, (K + 31) / 32 * 32)), 0, ctx->stream>>>(
+      d_iface_s, d_iface_vals, sd->lo[along], sd->hi[along], fixed, along, s, y, K, M, w);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   const double hx = (sd->hi[0] - sd->lo[0]) / (nx - 1), hy = (sd->hi[1] - sd->lo[1]) / (ny - 1);
   fill_kernel<<<static_cast<unsigned>((npts + 255) / 256), 256, 0, ctx->stream>>>(
