@@ -9,9 +9,9 @@
 //                      sqrt(dt)/sigma  (likelihood ratio of the Gaussian
 //                      transition of the discrete scheme; the bridge uniform
 //                      and the exit rule do not depend on phi).
-// The path kernel runs in its gradient mode and writes one 80-byte record per
-// path (score, exit point, L); jac_reduce_kernel and jac_merge_kernel form the
-// per-node means of the 80 components with compensated sums in a fixed order;
+// path_lr_kernel (grad_kernel.cuh) writes one 80-byte record per path (score,
+// exit point, L); jac_reduce_kernel and jac_merge_kernel form the per-node means
+// of the 80 components with compensated sums in a fixed order;
 // vjp_kernel contracts them with a cotangent over the nodes.
 #include <cmath>
 #include <cstring>

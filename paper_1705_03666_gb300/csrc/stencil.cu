@@ -39,9 +39,10 @@ constexpr int kStencilBlock = 1024;
 // reduction (Hockney): ceil(log2(K - 1)) rounds, each row with one division a
 // round, against a chain of two divisions a row on one thread (the rows are
 // diagonally dominant by a factor of two): 17 intervals 32 + 5 us with the
-// knots' own launch, 12.5 us now; 4000 intervals 6.6 -> 0.2 ms.  The knots first: s[0] and s[K] are the interface
-// end points, where the data are g (Eq. 1.1), s[1..K-1] the nodes' coordinates
-// along the interface.  work: kSplineWork arrays of K + 1.
+// knots' own launch, 12.5 us now; 4000 intervals 6.6 -> 0.2 ms.  The knots
+// first: s[0] and s[K] are the interface end points, where the data are g (Eq.
+// 1.1), s[1..K-1] the nodes' coordinates along the interface.  work: kSplineWork
+// arrays of K + 1.
 constexpr int kSplineWork = 10;
 __global__ void __launch_bounds__(1024)
 spline_kernel(const double *node_s, const double *vals, double s_lo, double s_hi, double fixed,

@@ -16,19 +16,6 @@ struct WarpQueue {
   bool exhausted = false;                // the global range ran out (warp-uniform)
 };
 
-// Lanes whose unit finished wait until at least this many lanes of the warp
-// are idle (or all are) before the warp claims new units together: the claim
-// and set-up code then runs once for several lanes instead of once per
-// finishing lane.  Units of a few loop trips (small trees) finish on nearly
-// every trip anyway and claim with B = 1.
-constexpr int kClaimBatch = 8;
-
-template <int B = kClaimBatch>
-__device__ __forceinline__ bool claim_time(bool active) {
-  const unsigned idle = __ballot_sync(kFull, !active);
-  return __popc(idle) >= B || idle == kFull;
-}
-
 // Called by all 32 lanes together.  A lane with `need` set receives the next
 // index in [0, total) in `idx` (returns true, need cleared); once the global
 // range is exhausted the remaining lanes get none (need cleared, false).
