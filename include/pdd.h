@@ -591,15 +591,14 @@ PDD_API pdd_status pdd_autotune_batch(pdd_ctx *ctx, const pdd_problem *problems,
 /* Launch-shape and memory knobs of the path kernels (no effect on results,
  * which do not depend on scheduling):
  *   blocks_per_sm    resident blocks per SM for the persistent path kernels
- *                    (128 threads for binary32 paths, 256 for FP64; 0 = the
- *                    occupancy maximum);
+ *                    (0 = chosen by the number of paths, up to the occupancy
+ *                    maximum);
  *   wave_max_paths   paths per wave of the kernels that store one score per
- *                    path in the context's scratch (Walk on Spheres,
- *                    reflecting faces, branching, multilevel, gradient; 4 or
- *                    8 bytes per path), each wave reduced before the next
- *                    starts (0 = default 2^29).  pdd_interface_solve with
- *                    absorbing faces stores no per-path score and runs all
- *                    paths in one launch.                                   */
+ *                    path in the context's scratch (reflecting faces,
+ *                    branching, gradient; 4 or 8 bytes per path, 80 for the
+ *                    gradient), each wave reduced before the next starts (0 =
+ *                    default 2^29).  The others add to exact per-node sums and
+ *                    run all paths in one launch.                           */
 PDD_API pdd_status pdd_set_tuning(pdd_ctx *ctx, int blocks_per_sm,
                                   int64_t wave_max_paths);
 

@@ -296,6 +296,7 @@ pdd_status interface_grad_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kPathBlockOf<float>, 0));
   if (bps < 1) bps = 1;
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
+  else bps = blocks_for_paths(bps, wave, ctx->num_sms, kPathBlockOf<float>);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (wave + kPathBlockOf<float> - 1) / kPathBlockOf<float>));
 

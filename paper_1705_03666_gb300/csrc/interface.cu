@@ -115,6 +115,7 @@ static pdd_status run_paths(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kForwardBlock, 0));
   if (bps < 1) bps = 1;
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
+  else if (sizeof(R) == 4) bps = blocks_for_paths(bps, total, ctx->num_sms, kForwardBlock);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kForwardBlock - 1) / kForwardBlock));
 

@@ -1214,6 +1214,22 @@ __device__ __forceinline__ void forward_paths(const Work &a) {
 template <class Model, typename R>
 constexpr int kForwardBlocks = sizeof(R) == 4 ? 7 : (Model::kDrift ? 3 : 4);
 
+// Of the bps blocks that fit an SM, those that a launch over `paths` paths uses:
+// more warps hide more latency, but the longest paths' chain at the end runs from
+// the moment the paths are all claimed, and the fewer paths a lane gets the larger
+// its share (and the slower each of the chain's steps, beside more warps).  P
+// paths per lane and block of an SM: about sqrt(P) / 1.6 blocks, at least two.
+// Cube, dt = 10^-3, blocks 2 .. 7: 275 275 291 312 343 377 us (P = 13), 523 484 486
+// 493 509 522 us (41), 762 685 666 664 670 683 us (66), 1519 1258 1172 1144 1137 1150
+// us (154), 2852 2319 2122 2028 1993 1986 us (308); the square and the L-shape, the
+// gradient's and the reflecting paths alike.  (Binary64 absorbing paths, bound by
+// the FP64 pipe from two blocks on, are within 2 % at any number.)
+inline int blocks_for_paths(int bps, uint64_t paths, int num_sms, int block) {
+  const double P = static_cast<double>(paths) / (static_cast<double>(num_sms) * block);
+  const double k = std::sqrt(P) / 1.6 + 0.5;
+  return k >= bps ? bps : std::min(bps, std::max(2, static_cast<int>(k)));
+}
+
 template <class Model, class Geom, typename R>
 __global__ void __launch_bounds__(kForwardBlock, kForwardBlocks<Model, R>)
 path_kernel(const __grid_constant__ PathArgs a) {

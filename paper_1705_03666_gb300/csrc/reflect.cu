@@ -767,6 +767,7 @@ static pdd_status run_reflect(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   PDD_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kBlock, 0));
   if (bps < 1) bps = 1;
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
+  else bps = blocks_for_paths(bps, wave, ctx->num_sms, kBlock);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (wave + kBlock - 1) / kBlock));
   for (uint64_t b0 = 0; b0 < total; b0 += wave) {

@@ -137,7 +137,9 @@ pdd_status run_static(char *base, int device, cudaStream_t stream, const pdd_pro
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, kForwardBlock, 0) != cudaSuccess ||
       cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
     return PDD_ECUDA;
-  uint64_t grid = static_cast<uint64_t>(std::max(bps, 1)) * static_cast<uint64_t>(num_sms);
+  bps = std::max(bps, 1);
+  if (sizeof(R) == 4) bps = blocks_for_paths(bps, total, num_sms, kForwardBlock);
+  uint64_t grid = static_cast<uint64_t>(bps) * static_cast<uint64_t>(num_sms);
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kForwardBlock - 1) / kForwardBlock));
   kern<<<static_cast<unsigned>(grid), kForwardBlock, 0, stream>>>(a);
   fix_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, stream>>>(
