@@ -60,9 +60,9 @@ __device__ __forceinline__ void jac_chan_merge(NodeAcc *jacc, uint64_t node, int
 // component, and jac_merge_kernel adds the parts in order and merges them
 // into the node's running (count, mean, M2) per component (Chan); with one
 // part the block merges its sums itself.  Launch
-// bounds of three blocks per SM (80 registers): at 105 registers and two
-// blocks the kernel was 24 % slower.
-__global__ void __launch_bounds__(kJacBlock, 3)
+// bounds of two blocks per SM: 2.7 ms per full wave, 3.2 ms at three (80
+// registers).
+__global__ void __launch_bounds__(kJacBlock, 2)
 jac_reduce_kernel(const GradRec *__restrict__ rec, uint64_t begin, uint64_t end,
                   uint64_t n_paths, uint64_t node_lo, int parts, double2 *part_sums,
                   NodeAcc *jacc) {

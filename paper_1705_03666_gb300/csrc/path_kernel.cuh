@@ -327,8 +327,9 @@ constexpr int kStepCapped = -3;
 // advance; on an exit, X keeps the start of the step, Xn receives its end,
 // Y and Z receive their exit values, and the caller resolves the exit point
 // (exit_score): the path kernel where it reruns parked units, the gradient kernel
-// 32 paths at a time from its exit queue, the plain one through path_unit.  With kLR the drift-weight likelihood-ratio
-// sums L are advanced by this step's noise (the exiting step included).
+// 32 paths at a time from its exit queue, the plain one through path_unit.  With
+// kLR the drift-weight likelihood-ratio sums L are advanced by this step's noise
+// (the exiting step included).
 template <class Model, class Geom, typename R, bool kLR, class Env>
 __device__ __forceinline__ int em_step(const Env &a, const StepConst<R> &k, R *X, R &Y, R &Z,
                                        const R *xi, uint32_t uw, int32_t n, R *Xn, R *L) {
@@ -1209,10 +1210,13 @@ __device__ __forceinline__ void forward_paths(const Work &a) {
 }
 
 // Blocks per SM the registers are held to: 72 registers for binary32 (seven
-// blocks: the 3-D solve 762 ms, 773 at 78 registers and six), 128 and 168 for
-// binary64 without and with drift (spills below).
+// blocks: the 3-D solve 762 ms, 773 at 78 registers and six), 64 for the 2-D
+// family with drift (eight: its forward pass 1.5 % faster; the Laplace family's
+// small calls were 4 % slower so), 128 and 168 for binary64 without and with
+// drift (spills below).
 template <class Model, typename R>
-constexpr int kForwardBlocks = sizeof(R) == 4 ? 7 : (Model::kDrift ? 3 : 4);
+constexpr int kForwardBlocks = sizeof(R) == 4 ? (Model::kDrift && Model::D == 2 ? 8 : 7)
+                                              : (Model::kDrift ? 3 : 4);
 
 // Of the bps blocks that fit an SM, those that a launch over `paths` paths uses:
 // more warps hide more latency, but the longest paths' chain at the end runs from
