@@ -637,6 +637,18 @@ def laplace_pdd_solve(ctx: Context, *, n_nodes: int = 16, n_paths: int = 10_000,
             "status": max(left["status"], right["status"])}
 
 
+def _axis_i32(axis: torch.Tensor) -> torch.Tensor:
+    """int32 axes of a tensor of any type: the entries equal to 0, 1 or 2, and
+    values outside that range for the others."""
+    if axis.is_complex():
+        axis = torch.where(axis.imag == 0, axis.real, -1.0)
+    if axis.is_floating_point():
+        axis = torch.where(axis == axis.floor(), axis, -1.0)
+    else:   # signed before the bound -1: clamp converts it to the tensor's own type
+        axis = axis.to(_I64)
+    return axis.clamp(-1, 3).to(_I32)
+
+
 def elliptic3d_pdd_solve(ctx: Context, nodes, values, node_axis=None, *, grid: int = 129,
                          split: int = 4, n_bnd: int = 32, method: str = "dst",
                          tol: float = 1e-12, max_iter: int = 200) -> dict:
@@ -661,10 +673,7 @@ def elliptic3d_pdd_solve(ctx: Context, nodes, values, node_axis=None, *, grid: i
     if values.numel() != nodes.shape[0]:
         raise ValueError("values must have one entry per node")
     if node_axis is not None:
-        node_axis = torch.as_tensor(node_axis, device=dev).reshape(-1)
-        if node_axis.is_floating_point():   # a value that is no axis names none
-            node_axis = torch.where(node_axis == node_axis.floor(), node_axis, -1.0)
-        node_axis = node_axis.clamp(-1, 3).to(_I32)
+        node_axis = _axis_i32(torch.as_tensor(node_axis, device=dev).reshape(-1))
         node_axis = node_axis.expand(nodes.shape[0]) if node_axis.numel() == 1 else node_axis
         node_axis = node_axis.contiguous()
         if node_axis.numel() != nodes.shape[0]:
