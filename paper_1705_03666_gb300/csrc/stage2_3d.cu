@@ -57,11 +57,14 @@ struct Box3 {
   int P[3];           // interior points per axis
   double w[3], diag;  // (sigma^2 / 2) / h_a^2 and the operator's diagonal
   int mask;           // bit 2a + side: that face carries interface data
+  int next;           // bit 2a + 1: that face's points are written by the next box along a
   int face_ld[6];       // row length of each face's data (its slow axis)
   int64_t face_off[6];  // offset of each face's data in the caller's array
   // the box's grid in the caller's array: point (i, j, k) is at u_off + k u_sz
-  // + j u_sy + i (a box of its own, or a block of one global grid: boxes that
-  // share a face then write the same values on it)
+  // + j u_sy + i (a box of its own, or a block of one global grid: of the boxes
+  // that share a point the last along every axis writes it, as its first: g on
+  // a shared edge of the cube's boundary depends on the last bit of the
+  // coordinate, and lo + h (n - 1) is not always the next box's lo)
   int64_t u_off, u_sz;
   int u_sy;
 };
@@ -125,18 +128,20 @@ box3_setup_kernel(const Box3 *boxes, ModelConst mc, const double *face, double *
       coef[(kTables ? 0 : 3) * np + q] = f;
       continue;
     }
-    bool physical = false;
+    bool physical = false, next = false;
     int fbest = -1;
     for (int fc = 0; fc < 6; ++fc) {
       const int a = fc >> 1, side = fc & 1;
       const bool on = side ? idx[a] == B.n[a] - 1 : idx[a] == 0;
       if (!on) continue;
+      next |= ((B.next >> fc) & 1) != 0;
       if ((B.mask >> fc) & 1) {
         if (fbest < 0) fbest = fc;
       } else {
         physical = true;
       }
     }
+    if (next) continue;
     double v;
     if (physical || fbest < 0) {
       v = Model::g_tab(tab[0][i], tab[1][j], tab[2][0]);
@@ -867,6 +872,7 @@ pdd_status elliptic3d_stage2_impl(pdd_ctx *ctx, const double *d_nodes, const dou
           if (plane == 0 || plane == split) continue;
           const int a1 = a == 0 ? 1 : 0, a2 = a == 2 ? 1 : 2;
           B.mask |= 1 << fc;
+          if (fc & 1) B.next |= 1 << fc;
           B.face_ld[fc] = grid;
           B.face_off[fc] = (a * (split - 1) + plane - 1) * g2 +
                            static_cast<int64_t>(kk[a2] * (m - 1)) * grid + kk[a1] * (m - 1);
