@@ -603,10 +603,12 @@ static pdd_status rbf_launch(pdd_ctx *ctx, const RbfWork &W, int Mmax) {
   auto *first = rbf_step_kernel<NB, kFirst>;
   auto *next = rbf_step_kernel<NB, kNext>;
   auto *rest = rbf_step_kernel<NB, kRest>;
+  // (the limits belong to the kernels on the device, not to this call: constants,
+  // so that a small system lowers nothing under another thread's elimination)
   PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(panel_smem)));
+                                         static_cast<int>(kRbfPanelBytes)));
   PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(std::max(panel_smem, kRbfOwnSm))));
+                                         static_cast<int>(std::max(kRbfPanelBytes, kRbfOwnSm))));
   const int panels = (Mmax + NB - 1) / NB;
   const unsigned np = static_cast<unsigned>(W.n_planes);
   first<<<np, kRbfThreads + 32, panel_smem, ctx->stream>>>(W, 0, 0, 0);
@@ -732,7 +734,7 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
   if (st != PDD_OK) return st;
   const size_t bsm = static_cast<size_t>(Mmax) * sizeof(double);
   PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rbf_backsub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(bsm)));
+                                         static_cast<int>(kRbfMaxSystem * sizeof(double))));
   rbf_backsub_kernel<<<static_cast<unsigned>(n_planes), kRbfThreads, bsm, ctx->stream>>>(W);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   int64_t qmax = 0;

@@ -378,6 +378,9 @@ box3_plane_kernel(const Box3 *boxes, const int32_t *live, const double *scale,
 // The z pass of 32 columns (blockIdx.x), the division by the eigenvalues and
 // the inverse z pass, in place.
 constexpr int kBox3Cols = 32;
+static size_t box3_z_smem(int P2) {
+  return (static_cast<size_t>(P2) * box3_pad(P2) + 2 * static_cast<size_t>(P2) * kBox3Cols) * sizeof(float);
+}
 __global__ void __launch_bounds__(kBox3Block)
 box3_z_kernel(int P0, int P1, int P2, const int32_t *live, const __grid_constant__ Box3Sines T,
               const double *fac, int64_t fac_stride, float *v) {
@@ -625,10 +628,14 @@ static pdd_status solve_boxes(pdd_ctx *ctx, std::vector<Box3> &boxes, int32_t me
                       kBox3Block, 0, ctx->stream>>>(d_boxes, T, s2, c, fac);
     PDD_CUDA_TRY(ctx, cudaGetLastError());
     const size_t smem_p = box3_plane_smem(P0, P1);
-    const size_t smem_z = (static_cast<size_t>(P2) * ld[2] + 2 * static_cast<size_t>(P2) * kBox3Cols) * sizeof(float);
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_p)));
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_p)));
-    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_z)));
+    const size_t smem_z = box3_z_smem(P2);
+    // (the limits belong to the kernels on the device, not to this call: constants,
+    // so that a call with small boxes lowers nothing under another thread's solve)
+    const int lim_p = static_cast<int>(box3_plane_smem(kBox3MaxInterior, kBox3MaxInterior));
+    const int lim_z = static_cast<int>(box3_z_smem(kBox3MaxInterior));
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim_p));
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_plane_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim_p));
+    PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(box3_z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim_z));
     const dim3 gz(static_cast<unsigned>((P0 * P1 + kBox3Cols - 1) / kBox3Cols), nb);
     const int64_t fac_stride = one_h ? 0 : np;
     // The boxes stop themselves.  The host looks at their number one

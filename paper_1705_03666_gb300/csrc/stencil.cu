@@ -603,7 +603,7 @@ pdd_status subdomain_solve_impl(pdd_ctx *ctx, const pdd_subdomain *sd, const dou
     if (smem + 1024 <= static_cast<size_t>(max_smem)) {
       PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(cg_mixed_kernel<true>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem)));
+                                             max_smem - 1024));  // (not this call's: see stage2_3d.cu)
       cg_mixed_kernel<true><<<1, kStencilBlock, smem, ctx->stream>>>(
           d_u, nx, ny, ihx2, ihy2, v0, v1, v2, sd->max_iter, sd->tol, it_d, res_d);
     } else {
