@@ -246,13 +246,11 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
         who = __ballot_sync(kFull, top && pos == mp);
       }
       const int src = __ffs(who) - 1;
-      // NaN in every unused row: no pivot (flagged; the solution is not used)
-      const bool none = (mh | c_lo[sl][src]) == 0u;
-      const int pr = none ? 0 : c_pos[sl][src];
-      const double akk = S[kk * R + pr];
+      // (some row is unused, so some key is not 0; the largest is 1 or 2 when all
+      // their entries are NaN or zero: flagged, the solution is not used)
       if (lane == 0) {
-        if (none || !((__double2hiint(akk) & 0x7fffffff) | __double2loint(akk))) *W.singular = 1;
-        s_piv[kk] = pr;
+        if (mh == 0u && c_lo[sl][src] <= 2u) *W.singular = 1;
+        s_piv[kk] = c_pos[sl][src];
       }
       __syncwarp();
       bar_sync(kBarPivot, kAll);
@@ -265,7 +263,8 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
   }
   bar_sync(kBarWork, kRbfThreads);
   uint32_t used = 0;  // bit i: own position tid + 512 i has been a pivot
-  // candidate of this thread: bits of |entry| plus one (0: none, and for NaN)
+  // candidate of this thread: bits of |entry| plus two (1 for NaN, 0: no unused
+  // row, so that the panel's pivots are distinct rows whatever the entries are)
   // and its position (the list keeps rows in increasing order, so the lowest
   // position is the lowest row)
   unsigned long long key = 0;
@@ -274,7 +273,7 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
     // (integers only: the FP64 pipe is what bounds the panel)
     const unsigned long long m =
         static_cast<unsigned long long>(__double_as_longlong(v)) & 0x7fffffffffffffffull;
-    const unsigned long long b = m <= 0x7ff0000000000000ull ? m + 1 : 0ull;
+    const unsigned long long b = m <= 0x7ff0000000000000ull ? m + 2 : 1ull;
     if (b > key) {
       key = b;
       kpos = pos;
