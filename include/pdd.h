@@ -343,7 +343,10 @@ PDD_API pdd_status pdd_branching_solve(pdd_ctx *ctx, const double *d_nodes_xt,
  * P_0), d_var (its sample variance) and, if non-NULL, the fine and coarse
  * means.  pdd_mlmc_solve runs the levels and combines them.  diag as for
  * pdd_interface_solve (path_steps counts fine steps; d_path_score receives
- * P_l - P_{l-1} per pair).                                                */
+ * P_l - P_{l-1} per pair).  The sums are exact integers of the scores times a
+ * power of two chosen by the problem's data, so that no finite score falls
+ * outside their range; a node outside the closed domain gets a NaN mean (and,
+ * with diag, PDD_EINVAL and their number in the message).                 */
 typedef struct {
   uint64_t seed;
   int64_t n_paths;     /* pairs per node at this level */

@@ -51,6 +51,7 @@ struct MlmcArgs {
   double *aux;                   // [total][8] per-walk records, or null
   RoundKeys rk;
   double dtf, sdtf, s2;          // fine step, sqrt(fine step), sigma^2
+  double scale;                  // of the scores in the sums (mlmc_scale)
   float edge[2][2];              // (c0, c1) of the screening bound: fine, coarse
   int32_t level, refine, max_steps, bridge;
   // x / n_paths for 32-bit x by one multiply-high and shifts
@@ -284,6 +285,7 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
     U = unif<R>(w.z);
   };
   // finished pairs (first cnt of the queue from `from`) into the sums
+  const R scale = static_cast<R>(a.scale);
   auto commit = [&](int from, int cnt) {
     __syncwarp();
     const bool has = static_cast<int>(lane) < cnt;
@@ -303,7 +305,7 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
       acc.v = st.sum[p][lane];
       acc.node = st.sum_node[p];
       __syncwarp();
-      acc.add<R>(a.fix + p * a.n, has, node, p == 0 ? df : (p == 1 ? f : c), false);
+      acc.add<R>(a.fix + p * a.n, has, node, scale * (p == 0 ? df : (p == 1 ? f : c)), false);
       st.sum[p][lane] = acc.v;
       if (lane == 0) st.sum_node[p] = acc.node;
     }
@@ -565,21 +567,44 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
   }
 }
 
-// fix planes: [3][n] (level 0: the fine score alone); var = M2 / (count - 1).
-// A node outside the closed domain has no scores: NaN mean, zero variance and
-// zero walk means.
-static __global__ void mlmc_finalize_kernel(const NodeFix *fix, int64_t n, int level, double *mean,
+// fix planes: [3][n] (level 0: the fine score alone), of scores times 2^e; var =
+// M2 / (count - 1).  A node outside the closed domain has no scores: NaN mean,
+// zero variance and zero walk means.
+static __global__ void mlmc_finalize_kernel(const NodeFix *fix, int64_t n, int level, int e, double *mean,
                                             double *var, double *fine_mean, double *coarse_mean) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   double m[3], m2[3];
 #pragma unroll
-  for (int p = 0; p < 3; ++p) fix_moments(fix[(level ? p : 0) * n + i], &m[p], &m2[p]);
+  for (int p = 0; p < 3; ++p) {
+    fix_moments(fix[(level ? p : 0) * n + i], &m[p], &m2[p]);
+    m[p] = scalbn(m[p], -e);
+  }
   const long long cnt = fix[i].n;
   mean[i] = m[0];
-  var[i] = cnt > 1 ? m2[0] / (static_cast<double>(cnt) - 1.0) : 0.0;
+  var[i] = cnt > 1 ? scalbn(m2[0] / (static_cast<double>(cnt) - 1.0), -2 * e) : 0.0;
   if (fine_mean) fine_mean[i] = cnt > 0 ? m[1] : 0.0;
   if (coarse_mean) coarse_mean[i] = cnt > 0 && level ? m[2] : 0.0;
+}
+
+// The exponent e of the power of two that the scores of a level are multiplied
+// with before they go to the exact sums (which hold |s| < 2^30 in steps of
+// 2^-60), so that the range fits the problem's data: |g| <= e on the square, <=
+// sum |theta| for the Fourier data, whose source (1) adds at most the time of
+// max_steps steps (twice that in rounded additions); a difference is at most two
+// scores; and a factor of two for the rounding of g.  The same sums with e = 0
+// made a node with a score of 2^30 NaN and dropped squares below 2^-60.
+static int mlmc_scale(const pdd_ctx *ctx, const pdd_mlmc_params *mp, double dtf) {
+  double bound = 2.7182818284590452;
+  if (ctx->prob.kind == PDD_PROB_POISSON_FOURIER) {
+    bound = 2.0 * dtf * static_cast<double>(mp->max_steps);
+    for (int i = 0; i < 64; ++i) bound += std::fabs(ctx->params[static_cast<size_t>(i)]);
+  }
+  if (!std::isfinite(bound)) return 0;
+  int e = 0;
+  std::frexp(4.0 * bound, &e);  // 4 bound < 2^e
+  // (binary32 scores end below 2^128, binary64 ones below 2^1024)
+  return std::max(mp->precision == PDD_FP64 ? -1000 : -100, std::min(60, 30 - e));
 }
 
 // The most faces within bridge reach of one step of standard deviation s whose
@@ -620,6 +645,8 @@ static pdd_status run_mlmc(pdd_ctx *ctx, cudaStream_t stream, char *base, const 
   a.dtf = mp->dt0 / std::pow(static_cast<double>(mp->refine), static_cast<double>(mp->level));
   a.sdtf = std::sqrt(a.dtf);
   a.s2 = ctx->prob.sigma * ctx->prob.sigma;
+  const int scale_e = mlmc_scale(ctx, mp, a.dtf);
+  a.scale = std::ldexp(1.0, scale_e);
   a.level = mp->level;
   a.refine = mp->refine;
   a.max_steps = static_cast<int32_t>(mp->max_steps);
@@ -652,7 +679,7 @@ static pdd_status run_mlmc(pdd_ctx *ctx, cudaStream_t stream, char *base, const 
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, stream));
   mlmc_finalize_kernel<<<static_cast<unsigned>((n + kFinalizeBlock - 1) / kFinalizeBlock), kFinalizeBlock, 0, stream>>>(
-      a.fix, n, mp->level, d_mean, d_var, d_fine, d_coarse);
+      a.fix, n, mp->level, scale_e, d_mean, d_var, d_fine, d_coarse);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
   return PDD_OK;
 }
