@@ -609,7 +609,8 @@ PDD_API pdd_status pdd_set_tuning(pdd_ctx *ctx, int blocks_per_sm,
  * the context's stream around every launch of its dominant kernel (the path
  * kernel of pdd_interface_solve).  pdd_profile_read synchronises the stream and
  * returns the summed elapsed milliseconds and the launch count since the last
- * read (or since profiling was switched on), then resets both.            */
+ * read (or since profiling was switched on), then resets both.  The levels of
+ * pdd_mlmc_solve, side by side otherwise, then run one after another.       */
 PDD_API pdd_status pdd_profile(pdd_ctx *ctx, int enable);
 PDD_API pdd_status pdd_profile_read(pdd_ctx *ctx, double *kernel_ms,
                                     int64_t *launches);

@@ -672,8 +672,7 @@ static pdd_status run_mlmc(pdd_ctx *ctx, cudaStream_t stream, char *base, const 
   if (ctx->path_blocks_per_sm > 0) bps = std::min(bps, ctx->path_blocks_per_sm);
   uint64_t grid = static_cast<uint64_t>(bps) * ctx->num_sms;
   grid = std::max<uint64_t>(1, std::min<uint64_t>(grid, (total + kMlmcBlock<R> - 1) / kMlmcBlock<R>));
-  // (the profiler's events sit on the context's stream)
-  const auto ev = stream == ctx->stream ? prof_slot(ctx) : std::pair<cudaEvent_t, cudaEvent_t>{};
+  const auto ev = prof_slot(ctx);
   if (ev.first) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.first, stream));
   kern<<<static_cast<unsigned>(grid), kMlmcBlock<R>, 0, stream>>>(a);
   PDD_CUDA_TRY(ctx, cudaGetLastError());
@@ -816,14 +815,16 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   st = ensure_side_streams(ctx);
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
-  const int side = std::min(n_levels - 1, 3);
+  // (timed launches follow one another on the context's stream: side by side,
+  // each would count the others' time as its own)
+  const int side = ctx->profiling ? 0 : std::min(n_levels - 1, 3);
   PDD_CUDA_TRY(ctx, cudaEventRecord(ctx->batch_fork, ctx->stream));
   for (int k = 0; k < side; ++k)
     PDD_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->batch_side[k], ctx->batch_fork, 0));
   pdd_status launched = PDD_OK;
   for (int q = 0; q < n_levels && launched == PDD_OK; ++q) {
     const int l = n_levels - 1 - q;
-    cudaStream_t s = q % 4 == 0 ? ctx->stream : ctx->batch_side[q % 4 - 1];
+    cudaStream_t s = side == 0 || q % 4 == 0 ? ctx->stream : ctx->batch_side[q % 4 - 1];
     launched = mlmc_launch(ctx, s, base + per * l, d_nodes, n, &lps[l], lm + static_cast<size_t>(l) * n,
                            lv + static_cast<size_t>(l) * n, nullptr, nullptr, nullptr);
   }
