@@ -29,6 +29,7 @@
 
 #include "branch_kernel.cuh"
 #include "ctx.hpp"
+#include "mlmc_pair.cuh"
 #include "models.cuh"
 #include "path_kernel.cuh"
 
@@ -189,7 +190,7 @@ template <typename R, int N>
 struct PairStash {
   unsigned long long id[N];
   uint32_t w0[N], w1[N];
-  int32_t k[N];                // fine steps taken; bits 30, 31: fine / coarse walk done
+  uint32_t state[N];           // PairState
   R fx[2][N], fz[N], cx[2][N], cz[N];  // a walk that is done keeps its score in its z
 };
 template <typename R>
@@ -202,9 +203,6 @@ struct MlmcStage {
   long long sum[3][32];
   uint64_t sum_node[3];
 };
-constexpr int32_t kFineDone = 1 << 30;
-constexpr int32_t kCoarseDone = static_cast<int32_t>(0x80000000u);
-constexpr int32_t kMlmcSteps = (1 << 30) - 1;
 
 __device__ __forceinline__ uint64_t mlmc_node(const MlmcArgs &a, uint64_t g) {
   if (a.total <= 0xffffffffull) {
@@ -230,7 +228,7 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
                                                                 static_cast<R>(a.refine)),
                                             a.s2, Geom::kFaces, a.bridge != 0);
   const int unit = kMode == 1 ? a.refine : 4;
-  const int32_t last_fast = min(a.max_steps, kMlmcSteps) - unit - 1;
+  const int32_t last_fast = a.max_steps - unit - 1;
   MlmcWalk<R> fw{}, cw{};
   float ef = 0.f, ec = 0.f;
   PhiloxPath pp{0, 0, 16u + static_cast<uint32_t>(a.level)};
@@ -248,10 +246,10 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
     id = q.id[i];
     pp.r0_w0 = q.w0[i];
     pp.r0_w1 = q.w1[i];
-    const int32_t kk = q.k[i];
-    k = kk & kMlmcSteps;
-    fw.done = (kk & kFineDone) != 0;
-    cw.done = (kk & kCoarseDone) != 0;
+    const PairState p = pair_unpack(q.state[i], unit);
+    k = p.steps;
+    fw.done = p.fine_done;
+    cw.done = p.coarse_done;
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       fw.X[d] = q.fx[d][i];
@@ -266,7 +264,7 @@ mlmc_kernel(const __grid_constant__ MlmcArgs a) {
     q.id[i] = id;
     q.w0[i] = pp.r0_w0;
     q.w1[i] = pp.r0_w1;
-    q.k[i] = k0 | (f.done ? kFineDone : 0) | (c.done ? kCoarseDone : 0);
+    q.state[i] = pair_pack(k0, unit, f.done, c.done);
 #pragma unroll
     for (int d = 0; d < 2; ++d) {
       q.fx[d][i] = f.X[d];
