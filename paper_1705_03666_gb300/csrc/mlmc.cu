@@ -617,6 +617,7 @@ static int mlmc_reach(double s, double q) {
 
 // Scratch of one level: 256 bytes of counters, then the sums.
 constexpr size_t kMlmcFixOff = 256;
+constexpr size_t kMlmcApart = size_t(1) << 30;  // most scratch for levels side by side
 static size_t mlmc_bytes(int64_t n) {
   return align_up(kMlmcFixOff + 3 * static_cast<size_t>(n) * sizeof(NodeFix), 256);
 }
@@ -807,15 +808,28 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
     const pdd_status st = mlmc_check(ctx, d_nodes, n, &lps[l], lm, lv);
     if (st != PDD_OK) return st;
   }
+  // (more than kMlmcApart bytes for all of them: the levels follow one another on
+  // one level's scratch, or many nodes times many levels would not fit the device)
   const size_t per = mlmc_bytes(n);
-  pdd_status st = ensure_scratch(ctx, per * n_levels);
+  const bool apart = per <= kMlmcApart / static_cast<size_t>(n_levels);
+  pdd_status st = ensure_scratch(ctx, apart ? per * n_levels : per);
   if (st != PDD_OK) return st;
   st = ensure_side_streams(ctx);
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
+  pdd_status worst = PDD_OK;
+  int64_t steps = 0, capped = 0;
+  auto count = [&](int l) -> pdd_status {
+    pdd_diag ld{};
+    const pdd_status s = mlmc_counts(ctx, base + (apart ? per * l : 0), &ld);
+    if (s == PDD_ECAP) worst = PDD_ECAP;
+    steps += ld.path_steps;
+    capped += ld.capped;
+    return s == PDD_ECAP ? PDD_OK : s;
+  };
   // (timed launches follow one another on the context's stream: side by side,
   // each would count the others' time as its own)
-  const int side = ctx->profiling ? 0 : std::min(n_levels - 1, 3);
+  const int side = ctx->profiling || !apart ? 0 : std::min(n_levels - 1, 3);
   PDD_CUDA_TRY(ctx, cudaEventRecord(ctx->batch_fork, ctx->stream));
   for (int k = 0; k < side; ++k)
     PDD_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->batch_side[k], ctx->batch_fork, 0));
@@ -823,8 +837,10 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
   for (int q = 0; q < n_levels && launched == PDD_OK; ++q) {
     const int l = n_levels - 1 - q;
     cudaStream_t s = side == 0 || q % 4 == 0 ? ctx->stream : ctx->batch_side[q % 4 - 1];
-    launched = mlmc_launch(ctx, s, base + per * l, d_nodes, n, &lps[l], lm + static_cast<size_t>(l) * n,
-                           lv + static_cast<size_t>(l) * n, nullptr, nullptr, nullptr);
+    launched = mlmc_launch(ctx, s, base + (apart ? per * l : 0), d_nodes, n, &lps[l],
+                           lm + static_cast<size_t>(l) * n, lv + static_cast<size_t>(l) * n, nullptr,
+                           nullptr, nullptr);
+    if (diag && !apart && launched == PDD_OK) launched = count(l);
   }
   // (joined also after a failed launch: nothing of this call runs on past it)
   for (int k = 0; k < side; ++k) {
@@ -832,15 +848,9 @@ pdd_status mlmc_solve_impl(pdd_ctx *ctx, const double *d_nodes, int64_t n,
     PDD_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->stream, ctx->batch_join[k], 0));
   }
   if (launched != PDD_OK) return launched;
-  pdd_status worst = PDD_OK;
-  int64_t steps = 0, capped = 0;
-  for (int l = 0; diag && l < n_levels; ++l) {
-    pdd_diag ld{};
-    st = mlmc_counts(ctx, base + per * l, &ld);
-    if (st != PDD_OK && st != PDD_ECAP) return st;
-    if (st == PDD_ECAP) worst = PDD_ECAP;
-    steps += ld.path_steps;
-    capped += ld.capped;
+  for (int l = 0; diag && apart && l < n_levels; ++l) {
+    st = count(l);
+    if (st != PDD_OK) return st;
   }
   mlmc_combine_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, ctx->stream>>>(
       lm, lv, n, n_levels, N, d_mean, d_se);
