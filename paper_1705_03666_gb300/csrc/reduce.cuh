@@ -11,8 +11,6 @@
 // deterministic.
 #pragma once
 
-#include <cstring>
-
 #include "common.cuh"
 #include "ctx.hpp"
 #include "nodefix.cuh"
@@ -32,11 +30,10 @@ struct NodeAcc {  // running (count, mean, M2) per node, FP64
 // summed plainly in FP64 (a few thousand terms per thread).  FP64 is a
 // 1/64-rate pipe on this part, so a compensated FP64 sum per score would
 // make the reduction, not the paths, the cost of short-path workloads.
-// Threads are then combined in a fixed tree in FP64: two-float sums part by
-// part (their high parts, 24 bits each, add up exactly while they are within
-// 2^20 of one another), binary64 sums compensated.  Compensated additions for
-// both, 170 FP64 instructions per warp, took 76 of 125 us for 1024 nodes of 10^5
-// binary32 scores; 93 us in all now.
+// Threads are then combined in fixed trees in FP64, a warp's (warp_total) and the
+// warps' compensated.  Compensated additions throughout, 170 FP64 instructions per
+// warp, took 76 of 125 us for 1024 nodes of 10^5 binary32 scores; 93 us in all with
+// the warp's exact ones.
 struct F2Sum {
   float hi = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float v) {
@@ -47,20 +44,46 @@ struct F2Sum {
   }
 };
 
-// The two parts of a two-float sum, added separately.
-struct PartSum {
-  double hi = 0.0, lo = 0.0;
-  __device__ __forceinline__ void merge(const PartSum &o) {
-    hi += o.hi;
-    lo += o.lo;
+// Whether 32 binary32 numbers add up exactly in FP64 in any order: the last bit of
+// the smallest and the top of the sum within 53 bits (finite, exponents within 24).
+__device__ __forceinline__ bool warp_adds_exactly(float v) {
+  const uint32_t b = __float_as_uint(v) & 0x7fffffffu, e = max(b >> 23, 1u);
+  const uint32_t top = __reduce_max_sync(kFull, b ? e : 0u);
+  const uint32_t low = __reduce_max_sync(kFull, b ? 256u - e : 0u);  // 256 less the smallest
+  return top == 0u || (top < 255u && top + low <= 256u + 24u);
+}
+// The warp's total as an unevaluated sum s + c, in every lane.  Two-float sums: the
+// high and the low parts by themselves where each add up exactly, as they do but
+// for sums of very different size (2 FP64 instructions a step of the tree instead
+// of 9); compensated otherwise, and for binary64 sums.
+__device__ __forceinline__ CSum warp_total(CSum t) {
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) t.merge(shfl_xor(t, m));
+  return t;
+}
+__device__ __forceinline__ CSum warp_total(const F2Sum &v) {
+  CSum t;
+  if (warp_adds_exactly(v.hi) && warp_adds_exactly(v.lo)) {
+    t.s = static_cast<double>(v.hi);
+    t.c = static_cast<double>(v.lo);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      t.s += __shfl_xor_sync(kFull, t.s, m);
+      t.c += __shfl_xor_sync(kFull, t.c, m);
+    }
+    return t;
   }
-  __device__ __forceinline__ double value() const { return hi + lo; }
-};
-__device__ __forceinline__ PartSum shfl_xor(const PartSum &v, int m) {
-  PartSum o;
-  o.hi = __shfl_xor_sync(kFull, v.hi, m);
-  o.lo = __shfl_xor_sync(kFull, v.lo, m);
-  return o;
+  t.add(static_cast<double>(v.hi));
+  t.add(static_cast<double>(v.lo));
+  return warp_total(t);
+}
+// The total of n such sums (n a power of two up to 32), one per lane below n.
+__device__ __forceinline__ CSum lanes_total(const CSum &v, int n) {
+  CSum t;
+  t.add(v.s);
+  t.add(v.c);
+  for (int m = n / 2; m > 0; m >>= 1) t.merge(shfl_xor(t, m));
+  return t;
 }
 
 template <typename R, bool kSkipNaN>
@@ -94,11 +117,8 @@ struct ThreadSums<float, kSkipNaN> {
     s2.add(q);
     s2.lo += e + 2.0f * d * dl;
   }
-  using Total = PartSum;
-  __device__ __forceinline__ void out(PartSum &c1, PartSum &c2) const {
-    c1 = {static_cast<double>(s1.hi), static_cast<double>(s1.lo)};
-    c2 = {static_cast<double>(s2.hi), static_cast<double>(s2.lo)};
-  }
+  __device__ __forceinline__ CSum total1() const { return warp_total(s1); }
+  __device__ __forceinline__ CSum total2() const { return warp_total(s2); }
 };
 template <bool kSkipNaN>
 struct ThreadSums<double, kSkipNaN> {
@@ -111,17 +131,14 @@ struct ThreadSums<double, kSkipNaN> {
     s1 += d;
     s2 = fma(d, d, s2);
   }
-  using Total = CSum;
-  __device__ __forceinline__ void out(CSum &c1, CSum &c2) const {
-    c1.add(s1);
-    c2.add(s2);
-  }
+  __device__ __forceinline__ CSum total1() const { return warp_total(CSum{s1, 0.0}); }
+  __device__ __forceinline__ CSum total2() const { return warp_total(CSum{s2, 0.0}); }
 };
 
 // The parts of a wave's nodes (rec [planes][nodes][parts], done [planes][nodes]
 // counts the finished ones, zero before and after).
 struct ReducePart {
-  PartSum s1, s2;  // (a CSum's two words for binary64 scores)
+  CSum s1, s2;
   unsigned long long kept;
 };
 struct ReduceParts {
@@ -193,18 +210,13 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
   } else {
     for (uint64_t i = threadIdx.x; i < cnt; i += kReduceBlock) ts.add(s[i], Kr);
   }
-  using Total = typename ThreadSums<R, kSkipNaN>::Total;
-  Total s1, s2;
-  ts.out(s1, s2);
+  const CSum s1 = ts.total1(), s2 = ts.total2();
   unsigned long long kept = ts.kept;
 #pragma unroll
-  for (int m = 16; m > 0; m >>= 1) {
-    s1.merge(shfl_xor(s1, m));
-    s2.merge(shfl_xor(s2, m));
-    kept += __shfl_xor_sync(kFull, kept, m);
-  }
-  __shared__ Total sh1[kReduceBlock / 32], sh2[kReduceBlock / 32];
-  __shared__ unsigned long long shk[kReduceBlock / 32];
+  for (int m = 16; m > 0; m >>= 1) kept += __shfl_xor_sync(kFull, kept, m);
+  constexpr int kWarps = kReduceBlock / 32;
+  __shared__ CSum sh1[kWarps], sh2[kWarps];
+  __shared__ unsigned long long shk[kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) {
     sh1[warp] = s1;
@@ -213,44 +225,34 @@ reduce_wave_kernel(const R *__restrict__ score, uint64_t begin, uint64_t end,
   }
   __syncthreads();
   if (threadIdx.x >= 32) return;
-  Total t1 = sh1[0], t2 = sh2[0];
-  unsigned long long tk = shk[0];
-  for (int w = 1; w < kReduceBlock / 32; ++w) {
-    t1.merge(sh1[w]);
-    t2.merge(sh2[w]);
-    tk += shk[w];
-  }
+  CSum t1 = lanes_total(sh1[lane % kWarps], kWarps), t2 = lanes_total(sh2[lane % kWarps], kWarps);
+  unsigned long long tk = 0;
+  for (int w = 0; w < kWarps; ++w) tk += shk[w];
   if (rp.parts > 1) {
-    static_assert(sizeof(Total) == sizeof(PartSum), "a part's record");
     const uint64_t q = blockIdx.y * (gridDim.x / rp.parts) + blockIdx.x / rp.parts;
     ReducePart *const rec = rp.rec + q * rp.parts;
     unsigned before = 0;
     if (lane == 0) {
-      ReducePart o;
-      memcpy(&o.s1, &t1, sizeof t1);
-      memcpy(&o.s2, &t2, sizeof t2);
-      o.kept = tk;
-      rec[part] = o;
+      rec[part] = {t1, t2, tk};
       __threadfence();
       before = atomicAdd(rp.done + q, 1u);
     }
     if (__shfl_sync(kFull, before, 0) != static_cast<unsigned>(rp.parts - 1)) return;
     __threadfence();
-    t1 = t2 = Total{};
+    t1 = t2 = CSum{};
     tk = 0;
     if (lane < rp.parts) {
       const volatile ReducePart *const v = rec + lane;
-      const double a[5] = {v->s1.hi, v->s1.lo, v->s2.hi, v->s2.lo, 0.0};
-      memcpy(&t1, a, sizeof t1);
-      memcpy(&t2, a + 2, sizeof t2);
+      t1.s = v->s1.s;
+      t1.c = v->s1.c;
+      t2.s = v->s2.s;
+      t2.c = v->s2.c;
       tk = v->kept;
     }
+    t1 = lanes_total(t1, rp.parts);
+    t2 = lanes_total(t2, rp.parts);
 #pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
-      t1.merge(shfl_xor(t1, m));
-      t2.merge(shfl_xor(t2, m));
-      tk += __shfl_xor_sync(kFull, tk, m);
-    }
+    for (int m = 16; m > 0; m >>= 1) tk += __shfl_xor_sync(kFull, tk, m);
     if (lane == 0) rp.done[q] = 0;
   }
   if (threadIdx.x == 0) {
