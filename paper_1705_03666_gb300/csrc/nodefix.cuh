@@ -210,13 +210,23 @@ __host__ __device__ __forceinline__ unsigned long long fix_top(const unsigned lo
   return top >> 1;
 }
 
+// m / nn for m < 2^63 and an integer nn below 2^53 with rn = 1 / nn: the quotient
+// of m's leading part corrected by its exact remainder and the rest of m, and one
+// rounding.
+__host__ __device__ __forceinline__ double fix_quotient(unsigned long long m, double nn, double rn) {
+  const double hi = static_cast<double>(m);
+  const double lo = static_cast<double>(static_cast<long long>(m - static_cast<unsigned long long>(hi)));
+  const double q = hi * rn;
+  return q + (fma(-q, nn, hi) + lo) * rn;
+}
+
 // Mean and the sum of squared deviations M2 of a node's scores from its exact
-// sums: mean = S1 / n and M2 = (n S2 - S1^2) / n, the numerator in exact
-// integers (256 bits) and rounded once, so that FP64, a 1/64-rate pipe on this
-// part, only has to divide: one warp took 10.4 us for both in double-doubles
-// (some 350 dependent instructions) after every small solve.  M2 = 0 when every
-// path started on the boundary, or with one path; both NaN when a path was
-// invalid or nothing was scored.
+// sums: mean = S1 / n and M2 = (n S2 - S1^2) / n, the numerator in exact integers
+// (256 bits, cut to 63) and the quotient rounded once, so that FP64, a 1/64-rate
+// pipe on this part, only has to divide: one warp took 10.4 us for both in
+// double-doubles (some 350 dependent instructions) after every small solve.  M2 =
+// 0 when every path started on the boundary, or with one path; both NaN when a
+// path was invalid or nothing was scored.
 __host__ __device__ __forceinline__ void fix_moments(const NodeFix &F, double *mean, double *m2) {
   using u64 = unsigned long long;
   using u128 = unsigned __int128;
@@ -239,11 +249,8 @@ __host__ __device__ __forceinline__ void fix_moments(const NodeFix &F, double *m
     const u64 w[4] = {a0, a1, 0, 0};
     int e;
     const u64 m = fix_top(w, &e);
-    const double hi = static_cast<double>(m);
-    const double lo = static_cast<double>(static_cast<long long>(m) - static_cast<long long>(hi));
-    const double q = hi * rn;
-    const double r = (fma(-q, nn, hi) + lo) * rn;
-    *mean = (neg ? -(q + r) : q + r) * fix_pow2(e - 60);
+    const double q = fix_quotient(m, nn, rn);
+    *mean = (neg ? -q : q) * fix_pow2(e - 60);
   }
   *m2 = 0.0;
   if (F.boundary == F.n || F.n <= 1) return;
@@ -277,7 +284,7 @@ __host__ __device__ __forceinline__ void fix_moments(const NodeFix &F, double *m
   if (borrow || (d[0] | d[1] | d[2] | d[3]) == 0) return;
   int e;
   const u64 m = fix_top(d, &e);
-  *m2 = static_cast<double>(m) * rn * fix_pow2(e - 120);
+  *m2 = fix_quotient(m, nn, rn) * fix_pow2(e - 120);
 }
 
 // Mean, standard error of the mean, path count and flags per node from the
