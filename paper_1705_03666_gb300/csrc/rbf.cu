@@ -22,8 +22,10 @@
 // So the serial pivot chain of a panel runs beside the update, which spreads
 // over the whole GPU.  Every matrix element sees the same multiply-adds in
 // the same order as in the plain row-by-row elimination (one FMA per step in
-// step order, l = a / pivot), whatever the panel width.  Factored rows go to U
-// in pivot order.
+// step order, l = a / pivot), whatever the panel width.  A factored row stays where
+// it is in A, with the list of the pivot rows beside (perm); only its entries in the
+// panel after its own go aside: the blocks of launch 1 that update that panel all
+// form them for themselves, so none may overwrite them in A.
 //
 // Measured on the 9 planes (device time): 11.75 ms by one 8-block cluster per
 // plane with a cluster barrier per step (20 us a step); 2.2 ms in panels (step
@@ -43,6 +45,7 @@ constexpr int64_t kRbfMaxSystem = 6144;  // unknowns per plane (weights + 3)
 constexpr int kRbfThreads = 512;
 constexpr int kRbfTileR = 32, kRbfTileC = 32;  // rows and columns of an update tile
 constexpr size_t kRbfOwnSm = 116 * 1024;  // more than half of an SM's shared memory
+constexpr size_t kRbfBackBytes = sizeof(double) + sizeof(int32_t);  // shared memory of a row in the back substitution
 constexpr size_t kRbfPanelBytes = 200 * 1024;  // panel in shared memory (rows x NB doubles)
 
 struct RbfPlane {
@@ -60,7 +63,8 @@ struct RbfWork {
   const RbfPlane *planes;
   int32_t n_planes;
   double *A;             // systems, row-major, M x (M + 1) each
-  double *U;             // factored rows in pivot order, same layout
+  double *side;          // pivot rows' entries in the panel after their own [row0 + step][NB]
+  int32_t *perm;         // pivot rows in step order [row0 + step]
   double *x;             // solutions [row0 + k]
   double *L[2];          // multipliers of the active rows, by panel parity: [row0 + pos][NB]
   int32_t *act[2];       // active rows (not yet a pivot) after a panel, by parity: [row0 + pos]
@@ -216,7 +220,7 @@ enum { kBarCand = 1, kBarPivot = 2, kBarWork = 3 };
 // FP64 reciprocal there would queue behind the workers' updates), the workers
 // update the columns behind.  On return the list
 // of rows still active, their multipliers, the pivot rows and their own
-// multipliers are stored for the update, and U has the panel's columns of the
+// multipliers are stored for the update, and A has the panel's columns of the
 // pivot rows.
 template <int NB>
 __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel, double *smem) {
@@ -227,8 +231,7 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
   const int R = M - k0;  // active rows before this panel
   const int par = panel & 1;
   const int32_t *act = W.act[par ^ 1] + P.row0;
-  const double *A = W.A + P.sys0;
-  double *U = W.U + P.sys0;
+  double *A = W.A + P.sys0;
   double *S = smem;  // S[c * R + pos]
   constexpr int nw = kRbfThreads / 32, kAll = kRbfThreads + 32;
   __shared__ uint32_t c_hi[2][nw], c_lo[2][nw];
@@ -341,15 +344,15 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
     }
   }
   bar_sync(kBarWork, kRbfThreads);
-  // the panel's columns of U, the pivot rows, their multipliers
+  // the panel's columns of the pivot rows in A, the list, their multipliers
   double *L11 = W.L11[par] + (blockIdx.x * NB) * NB;
   for (int e = tid; e < nb * nb; e += kRbfThreads) {
     const int i = e / nb, c = e % nb;
     const double v = S[c * R + s_piv[i]];
-    if (c >= i) U[static_cast<int64_t>(k0 + i) * ld + k0 + c] = v;
+    if (c >= i) A[static_cast<int64_t>(act[s_piv[i]]) * ld + k0 + c] = v;
     else L11[i * NB + c] = v;
   }
-  if (tid < nb) W.piv[par][blockIdx.x * NB + tid] = act[s_piv[tid]];
+  if (tid < nb) W.perm[P.row0 + k0 + tid] = W.piv[par][blockIdx.x * NB + tid] = act[s_piv[tid]];
   // rows still active keep their order: the new position is the old one less
   // the pivots before it
   int32_t *act2 = W.act[par] + P.row0;
@@ -366,17 +369,19 @@ __device__ void rbf_factor_panel(const RbfWork &W, const RbfPlane &P, int panel,
 // The pivot rows' entries of panel `panel` in the TC columns from column c0
 // (below c1): a unit lower triangular solve, a warp per pivot row and a lane
 // per column, so that the triangle spreads over the four schedulers' FP64
-// pipes.  The result is stored in U and left in Us [NB][TC].
-template <int NB, int TC>
+// pipes.  The result is left in Us [NB][TC] and stored: kSide, the columns of the
+// panel after it, aside (by the block that is to, `store`); else in place.
+template <int NB, int TC, bool kSide>
 __device__ void rbf_pivot_rows(const RbfWork &W, const RbfPlane &P, int plane, int panel, int c0,
-                               int c1, double *Us, double *L11) {
+                               int c1, double *Us, double *L11, bool store) {
   const int k0 = panel * NB, ld = P.M + 1;
   const int nb = min(NB, P.M - k0);
   const int par = panel & 1, tid = threadIdx.x;
   const int i = tid >> 5, c = tid & 31;
   const bool on = i < nb && c < TC && c0 + c < c1;
   double ui = 0.0;
-  if (on) ui = W.A[P.sys0 + static_cast<int64_t>(W.piv[par][plane * NB + i]) * ld + c0 + c];
+  double *const at = W.A + P.sys0 + static_cast<int64_t>(on ? W.piv[par][plane * NB + i] : 0) * ld + c0 + c;
+  if (on) ui = *at;
   for (int e = tid; e < NB * NB; e += kRbfThreads) {
     const int row = e / NB, k = e % NB;
     L11[e] = k < row && row < nb ? W.L11[par][plane * NB * NB + e] : 0.0;
@@ -388,16 +393,20 @@ __device__ void rbf_pivot_rows(const RbfWork &W, const RbfPlane &P, int plane, i
     bar_sync(kBarWork, kRbfThreads);
     if (i > k && on) ui = fma(-L11[i * NB + k], Us[k * TC + c], ui);
   }
-  if (on) W.U[P.sys0 + static_cast<int64_t>(k0 + i) * ld + c0 + c] = ui;
+  if (on && store) {
+    if constexpr (kSide) W.side[(P.row0 + k0 + i) * NB + c] = ui;
+    else *at = ui;
+  }
 }
 
 // Update by panel `panel` (already factored, the pivot rows' entries Us
 // [NB][TC]) of a tile of TC columns from column c0 (below c1) and TR active
 // rows from position r0: one FMA per element and pivot, in pivot order.
-// Threads tid of kRbfThreads; Ls: [TR][NB + 1] of shared memory.
-template <int NB, int TC, int TR, class Sync>
+// Threads tid of kRbfThreads; Ls: [TR][NB + 1] of shared memory.  mid() runs once
+// the tile's own loads are under way, sync() before Us and Ls are read.
+template <int NB, int TC, int TR, class Mid, class Sync>
 __device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int panel, int r0, int c0,
-                                int c1, const double *Us, double *Ls, int tid, Sync sync) {
+                                int c1, const double *Us, double *Ls, int tid, Mid mid, Sync sync) {
   const int k0 = panel * NB, ld = P.M + 1;
   const int nb = min(NB, P.M - k0);
   const int R = P.M - k0 - nb;
@@ -417,6 +426,7 @@ __device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int panel, 
     pa[q] = row < rows && j < c1 ? A + static_cast<int64_t>(act[row]) * ld + j : nullptr;
     a[q] = pa[q] ? *pa[q] : 0.0;
   }
+  mid();
   for (int e = tid; e < rows * NB; e += kRbfThreads)
     Ls[(e / NB) * (NB + 1) + e % NB] = e % NB < nb ? L[e] : 0.0;
   sync();
@@ -437,8 +447,8 @@ __device__ void rbf_update_tile(const RbfWork &W, const RbfPlane &P, int panel, 
 
 // kFirst: panel 0 of every plane is factored (blockIdx.x = plane).
 // kNext, blockIdx.y = plane: blocks [0, row_tiles) update the columns of panel
-// + 1 by `panel` (and store their part of U); the others form the pivot rows'
-// entries of 32 columns behind them (U).
+// + 1 by `panel` (the first stores the pivot rows' part); the others form the pivot
+// rows' entries of 32 columns behind them.
 // kRest: blocks [0, n_planes) factor panel + 1; the others update the columns
 // behind it by `panel`, two tiles per block (tile index = (plane, row tile,
 // column tile), column tiles fastest).  Launched with more than half of an
@@ -463,13 +473,13 @@ rbf_step_kernel(const __grid_constant__ RbfWork W, int panel, int row_tiles, int
     if (static_cast<int>(blockIdx.x) < row_tiles) {
       const int r0 = blockIdx.x * kRbfTileR, c0 = k0 + NB, c1 = min(k0 + 2 * NB, P.M);
       if (R <= 0 || r0 >= R) return;  // no next panel, or no such rows
-      rbf_pivot_rows<NB, NB>(W, P, blockIdx.y, panel, c0, c1, Us, L11);
-      rbf_update_tile<NB, NB, kRbfTileR>(W, P, panel, r0, c0, c1, Us, Ls, threadIdx.x,
+      rbf_pivot_rows<NB, NB, true>(W, P, blockIdx.y, panel, c0, c1, Us, L11, blockIdx.x == 0);
+      rbf_update_tile<NB, NB, kRbfTileR>(W, P, panel, r0, c0, c1, Us, Ls, threadIdx.x, [] {},
                                          [] { bar_sync(kBarWork, kRbfThreads); });
     } else {
       const int c0 = min(k0 + 2 * NB, P.M) + (blockIdx.x - row_tiles) * TC;
       if (c0 > P.M) return;
-      rbf_pivot_rows<NB, TC>(W, P, blockIdx.y, panel, c0, P.M + 1, Us, L11);
+      rbf_pivot_rows<NB, TC, false>(W, P, blockIdx.y, panel, c0, P.M + 1, Us, L11, true);
     }
   } else {
     if (static_cast<int>(blockIdx.x) < W.n_planes) {
@@ -489,13 +499,21 @@ rbf_step_kernel(const __grid_constant__ RbfWork W, int panel, int row_tiles, int
     const int r0 = rt * kRbfTileR, c0 = min(k0 + 2 * NB, P.M) + ct * TC;
     if (k0 + NB >= P.M || r0 >= P.M - k0 - NB || c0 > P.M) return;
     double *Us = rbf_smem + half * rbf_tile_doubles(NB), *Ls = Us + NB * TC;
-    for (int e = tid; e < NB * TC; e += kRbfThreads) {
-      const int j = c0 + e % TC;
-      Us[e] = j <= P.M ? W.U[P.sys0 + static_cast<int64_t>(k0 + e / TC) * ld + j] : 0.0;
-    }
+    // the pivot rows' entries, one per thread, loaded beside the tile's rows
+    static_assert(NB * TC <= kRbfThreads, "one entry per thread");
+    const int uj = c0 + tid % TC;
+    const bool has_u = tid < NB * TC && uj <= P.M;
+    const int32_t upiv = has_u ? W.piv[panel & 1][p * NB + tid / TC] : 0;
+    double u = 0.0;
     const int bar = kBarWork + half;
     rbf_update_tile<NB, TC, kRbfTileR>(W, P, panel, r0, c0, P.M + 1, Us, Ls, tid,
-                                       [bar] { bar_sync(bar, kRbfThreads); });
+                                       [&] {
+                                         if (has_u) u = W.A[P.sys0 + static_cast<int64_t>(upiv) * ld + uj];
+                                       },
+                                       [&] {
+                                         if (tid < NB * TC) Us[tid] = u;
+                                         bar_sync(bar, kRbfThreads);
+                                       });
   }
 }
 
@@ -504,21 +522,33 @@ rbf_step_kernel(const __grid_constant__ RbfWork W, int panel, int row_tiles, int
 // formed together, the quotient corrected once by its exact remainder), then
 // every row above
 // subtracts the block's 32 columns, one thread per row.
+template <int NB>
 __global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_constant__ RbfWork W) {
   extern __shared__ __align__(16) double rbf_smem[];
   const RbfPlane P = W.planes[blockIdx.x];
   const int M = P.M, ld = M + 1;
-  const double *U = W.U + P.sys0;
+  const double *A = W.A + P.sys0, *side = W.side + P.row0 * NB;
+  // step k's row of the triangular factor, column j >= k
+  auto u_at = [&](int k, const double *row, int j) {
+    const int s = j - (k / NB + 1) * NB;
+    const double *at = s >= 0 && s < NB ? side + static_cast<int64_t>(k) * NB + s : row + j;
+    return *at;
+  };
   double *y = rbf_smem;        // M
+  int32_t *perm = reinterpret_cast<int32_t *>(y + M);
   __shared__ double T[32][33];
   const int tid = threadIdx.x, lane = tid & 31;
-  for (int k = tid; k < M; k += kRbfThreads) y[k] = U[static_cast<int64_t>(k) * ld + M];
+  for (int k = tid; k < M; k += kRbfThreads) {
+    const int32_t row = W.perm[P.row0 + k];
+    perm[k] = row;
+    y[k] = A[static_cast<int64_t>(row) * ld + M];
+  }
   for (int b1 = M; b1 > 0;) {
     const int b0 = max(0, b1 - 32), nb = b1 - b0;
     __syncthreads();
     for (int e = tid; e < nb * nb; e += kRbfThreads) {
       const int i = e / nb, c = e % nb;
-      T[i][c] = U[static_cast<int64_t>(b0 + i) * ld + b0 + c];
+      if (c >= i) T[i][c] = u_at(b0 + i, A + static_cast<int64_t>(perm[b0 + i]) * ld, b0 + c);
     }
     __syncthreads();
     if (tid < 32) {
@@ -536,10 +566,10 @@ __global__ void __launch_bounds__(kRbfThreads) rbf_backsub_kernel(const __grid_c
     }
     __syncthreads();
     for (int k = tid; k < b0; k += kRbfThreads) {
-      const double *row = U + static_cast<int64_t>(k) * ld + b0;
+      const double *row = A + static_cast<int64_t>(perm[k]) * ld;
       double v = y[k];
 #pragma unroll 8
-      for (int c = 0; c < nb; ++c) v = fma(-row[c], y[b0 + c], v);
+      for (int c = 0; c < nb; ++c) v = fma(-u_at(k, row, b0 + c), y[b0 + c], v);
       y[k] = v;
     }
     b1 = b0;
@@ -600,7 +630,7 @@ rbf_eval_kernel(const __grid_constant__ RbfWork W, const double *__restrict__ pt
   }
 }
 
-// The launches of the elimination for panel width NB.
+// The launches of the elimination and the back substitution for panel width NB.
 template <int NB>
 static pdd_status rbf_launch(pdd_ctx *ctx, const RbfWork &W, int Mmax) {
   const size_t panel_smem = static_cast<size_t>(Mmax) * NB * sizeof(double);
@@ -631,6 +661,10 @@ static pdd_status rbf_launch(pdd_ctx *ctx, const RbfWork &W, int Mmax) {
     }
     PDD_CUDA_TRY(ctx, cudaGetLastError());
   }
+  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rbf_backsub_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kRbfMaxSystem * kRbfBackBytes)));
+  rbf_backsub_kernel<NB><<<np, kRbfThreads, static_cast<size_t>(Mmax) * kRbfBackBytes, ctx->stream>>>(W);
+  PDD_CUDA_TRY(ctx, cudaGetLastError());
   return PDD_OK;
 }
 
@@ -693,7 +727,8 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
   const size_t off_pts = take(static_cast<size_t>(pts0) * 2 * sizeof(double));
   const size_t off_pv = take(static_cast<size_t>(pts0) * sizeof(double));
   const size_t off_A = take(static_cast<size_t>(sys0) * sizeof(double));
-  const size_t off_U = take(static_cast<size_t>(sys0) * sizeof(double));
+  const size_t off_side = take(static_cast<size_t>(row0) * NB * sizeof(double));
+  const size_t off_perm = take(static_cast<size_t>(row0) * sizeof(int32_t));
   const size_t off_x = take(static_cast<size_t>(row0) * sizeof(double));
   size_t off_L[2], off_act[2], off_L11[2], off_piv[2];
   for (int h = 0; h < 2; ++h) {
@@ -712,7 +747,8 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
   W.planes = d_pl;
   W.n_planes = n_planes;
   W.A = reinterpret_cast<double *>(base + off_A);
-  W.U = reinterpret_cast<double *>(base + off_U);
+  W.side = reinterpret_cast<double *>(base + off_side);
+  W.perm = reinterpret_cast<int32_t *>(base + off_perm);
   W.x = reinterpret_cast<double *>(base + off_x);
   for (int h = 0; h < 2; ++h) {
     W.L[h] = reinterpret_cast<double *>(base + off_L[h]);
@@ -737,11 +773,6 @@ pdd_status interface_interp_impl(pdd_ctx *ctx, int32_t n_planes, const int32_t *
      : NB == 8 ? rbf_launch<8>(ctx, W, Mmax)
                : rbf_launch<4>(ctx, W, Mmax);
   if (st != PDD_OK) return st;
-  const size_t bsm = static_cast<size_t>(Mmax) * sizeof(double);
-  PDD_CUDA_TRY(ctx, cudaFuncSetAttribute(rbf_backsub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kRbfMaxSystem * sizeof(double))));
-  rbf_backsub_kernel<<<static_cast<unsigned>(n_planes), kRbfThreads, bsm, ctx->stream>>>(W);
-  PDD_CUDA_TRY(ctx, cudaGetLastError());
   int64_t qmax = 0;
   for (const auto &P : pl) qmax = std::max(qmax, P.q);
   constexpr int64_t kPer = kRbfEvalBlock * kRbfQ;

@@ -456,6 +456,56 @@ box3_jacobi_kernel(const Box3 *boxes, const int32_t *live, double s2, double c, 
   }
 }
 
+// Blocks of a Jacobi sweep over np interior points.
+static int box3_blocks(int64_t np) {
+  return static_cast<int>(std::min<int64_t>((np + kBox3Block - 1) / kBox3Block, 1024));
+}
+// Scratch of a batch of boxes (offsets).
+struct Box3Layout {
+  size_t it, res, state_bytes, rn, inv, r0, live, ticket, nlive, box, coef, drift, part, un, r, fac, v,
+      S[3], cm1[3], total;
+  bool one_h;  // boxes of one mesh size share one table of eigenvalue factors
+};
+static Box3Layout box3_layout(const std::vector<Box3> &boxes, bool jacobi, int64_t u_span) {
+  const Box3 &B0 = boxes[0];
+  const size_t NB = boxes.size();
+  const int64_t np = static_cast<int64_t>(B0.P[0]) * B0.P[1] * B0.P[2];
+  Box3Layout L;
+  L.one_h = true;
+  for (const Box3 &B : boxes)
+    for (int a = 0; a < 3; ++a) L.one_h = L.one_h && B.h[a] == B0.h[a];
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = align_up(o + bytes, 256);
+    return at;
+  };
+  // the boxes' state first: one copy back at the end
+  L.it = take(NB * sizeof(int64_t));
+  L.res = take(NB * sizeof(double));
+  L.state_bytes = o;
+  L.rn = take(NB * sizeof(double));
+  L.inv = take(NB * sizeof(double));
+  L.r0 = take(NB * sizeof(double));
+  L.live = take(NB * sizeof(int32_t));
+  L.ticket = take(NB * sizeof(int32_t));
+  L.nlive = take(sizeof(int32_t));
+  L.box = take(NB * sizeof(Box3));
+  L.coef = take(NB * (jacobi ? 4 : 1) * np * sizeof(double));
+  L.drift = take(NB * 2 * kBox3Axis * sizeof(double));
+  L.part = take(NB * std::max(box3_blocks(np), B0.P[2]) * sizeof(double));
+  L.un = take(jacobi ? u_span * sizeof(double) : 0);
+  L.r = take(jacobi ? 0 : NB * np * sizeof(double));
+  L.fac = take(jacobi ? 0 : (L.one_h ? 1 : NB) * np * sizeof(double));
+  L.v = take(jacobi ? 0 : NB * np * sizeof(float));
+  for (int a = 0; a < 3; ++a) {
+    L.S[a] = take(static_cast<size_t>(B0.P[a]) * box3_pad(B0.P[a]) * sizeof(float));
+    L.cm1[a] = take(static_cast<size_t>(B0.P[a]) * sizeof(double));
+  }
+  L.total = o;
+  return L;
+}
+
 // The boxes' solves (one grid size and method; faces and grids where the boxes
 // say, u_span values of d_u in all).  *iters and *resid (if non-null) get the
 // largest count and relative residual over the boxes; iters_each / resid_each
@@ -475,51 +525,19 @@ static pdd_status solve_boxes(pdd_ctx *ctx, std::vector<Box3> &boxes, int32_t me
   const bool jacobi = method == PDD_STENCIL_JACOBI;
   const int64_t np = static_cast<int64_t>(B0.P[0]) * B0.P[1] * B0.P[2];
   const size_t NB = static_cast<size_t>(nb);
-  const int nblk = static_cast<int>(std::min<int64_t>((np + kBox3Block - 1) / kBox3Block, 1024));
-  const int ld[3] = {box3_pad(B0.P[0]), box3_pad(B0.P[1]), box3_pad(B0.P[2])};
-  // boxes of one mesh size share one table of eigenvalue factors
-  bool one_h = true;
-  for (const Box3 &B : boxes)
-    for (int a = 0; a < 3; ++a) one_h = one_h && B.h[a] == B0.h[a];
-  size_t o = 0;
-  auto take = [&](size_t bytes) {
-    const size_t at = o;
-    o = align_up(o + bytes, 256);
-    return at;
-  };
-  // the boxes' state first: one copy back at the end
-  const size_t off_it = take(NB * sizeof(int64_t));
-  const size_t off_res = take(NB * sizeof(double));
-  const size_t state_bytes = o;
-  const size_t off_rn = take(NB * sizeof(double));
-  const size_t off_inv = take(NB * sizeof(double));
-  const size_t off_r0 = take(NB * sizeof(double));
-  const size_t off_live = take(NB * sizeof(int32_t));
-  const size_t off_ticket = take(NB * sizeof(int32_t));
-  const size_t off_nlive = take(sizeof(int32_t));
-  const size_t off_box = take(NB * sizeof(Box3));
-  const size_t off_coef = take(NB * (jacobi ? 4 : 1) * np * sizeof(double));
-  const size_t off_drift = take(NB * 2 * kBox3Axis * sizeof(double));
-  const size_t off_part = take(NB * std::max(nblk, B0.P[2]) * sizeof(double));
-  const size_t off_un = take(jacobi ? u_span * sizeof(double) : 0);
-  const size_t off_r = take(jacobi ? 0 : NB * np * sizeof(double));
-  const size_t off_fac = take(jacobi ? 0 : (one_h ? 1 : NB) * np * sizeof(double));
-  const size_t off_v = take(jacobi ? 0 : NB * np * sizeof(float));
-  size_t off_S[3], off_cm1[3];
-  for (int a = 0; a < 3; ++a) {
-    off_S[a] = take(static_cast<size_t>(B0.P[a]) * ld[a] * sizeof(float));
-    off_cm1[a] = take(static_cast<size_t>(B0.P[a]) * sizeof(double));
-  }
-  pdd_status st = ensure_scratch(ctx, o);
+  const int nblk = box3_blocks(np);
+  const Box3Layout L = box3_layout(boxes, jacobi, u_span);
+  const bool one_h = L.one_h;
+  pdd_status st = ensure_scratch(ctx, L.total);
   if (st != PDD_OK) return st;
   char *base = static_cast<char *>(ctx->scratch);
-  double *rn = reinterpret_cast<double *>(base + off_rn);  // per box: |r|_2 (Jacobi: largest change)
-  int32_t *live = reinterpret_cast<int32_t *>(base + off_live);
-  Box3 *d_boxes = reinterpret_cast<Box3 *>(base + off_box);
-  double *coef = reinterpret_cast<double *>(base + off_coef);
-  double *drift = reinterpret_cast<double *>(base + off_drift);
-  double *part = reinterpret_cast<double *>(base + off_part);
-  double *un = reinterpret_cast<double *>(base + off_un);
+  double *rn = reinterpret_cast<double *>(base + L.rn);  // per box: |r|_2 (Jacobi: largest change)
+  int32_t *live = reinterpret_cast<int32_t *>(base + L.live);
+  Box3 *d_boxes = reinterpret_cast<Box3 *>(base + L.box);
+  double *coef = reinterpret_cast<double *>(base + L.coef);
+  double *drift = reinterpret_cast<double *>(base + L.drift);
+  double *part = reinterpret_cast<double *>(base + L.part);
+  double *un = reinterpret_cast<double *>(base + L.un);
 
   // host state of the correction loop (copied to and from the device
   // synchronously, so these buffers outlive every copy)
@@ -599,21 +617,21 @@ static pdd_status solve_boxes(pdd_ctx *ctx, std::vector<Box3> &boxes, int32_t me
     if (st != PDD_OK) return st;
     Box3Sines T;
     for (int a = 0; a < 3; ++a) {
-      T.S[a] = reinterpret_cast<float *>(base + off_S[a]);
-      T.cm1[a] = reinterpret_cast<double *>(base + off_cm1[a]);
+      T.S[a] = reinterpret_cast<float *>(base + L.S[a]);
+      T.cm1[a] = reinterpret_cast<double *>(base + L.cm1[a]);
     }
     Box3State S;
     S.rn = rn;
-    S.inv = reinterpret_cast<double *>(base + off_inv);
-    S.r0 = reinterpret_cast<double *>(base + off_r0);
-    S.res = reinterpret_cast<double *>(base + off_res);
-    S.iters = reinterpret_cast<int64_t *>(base + off_it);
+    S.inv = reinterpret_cast<double *>(base + L.inv);
+    S.r0 = reinterpret_cast<double *>(base + L.r0);
+    S.res = reinterpret_cast<double *>(base + L.res);
+    S.iters = reinterpret_cast<int64_t *>(base + L.it);
     S.live = live;
-    S.ticket = reinterpret_cast<int32_t *>(base + off_ticket);
-    S.n_live = reinterpret_cast<int32_t *>(base + off_nlive);
-    double *r = reinterpret_cast<double *>(base + off_r);
-    double *fac = reinterpret_cast<double *>(base + off_fac);
-    float *v = reinterpret_cast<float *>(base + off_v);
+    S.ticket = reinterpret_cast<int32_t *>(base + L.ticket);
+    S.n_live = reinterpret_cast<int32_t *>(base + L.nlive);
+    double *r = reinterpret_cast<double *>(base + L.r);
+    double *fac = reinterpret_cast<double *>(base + L.fac);
+    float *v = reinterpret_cast<float *>(base + L.v);
     PDD_CUDA_TRY(ctx, cudaMemsetAsync(S.ticket, 0, NB * sizeof(int32_t), ctx->stream));
     const int32_t h_nlive = nb;
     PDD_CUDA_TRY(ctx, cudaMemcpyAsync(S.n_live, &h_nlive, sizeof h_nlive, cudaMemcpyHostToDevice,
@@ -657,11 +675,11 @@ static pdd_status solve_boxes(pdd_ctx *ctx, std::vector<Box3> &boxes, int32_t me
       box3_plane_kernel<true><<<gp, kBox3Block, smem_p, ctx->stream>>>(d_boxes, live, rn, T, nullptr, v, d_u);
       PDD_CUDA_TRY(ctx, cudaGetLastError());
     }
-    std::vector<char> h_state(state_bytes);
-    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(h_state.data(), base, state_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    std::vector<char> h_state(L.state_bytes);
+    PDD_CUDA_TRY(ctx, cudaMemcpyAsync(h_state.data(), base, L.state_bytes, cudaMemcpyDeviceToHost, ctx->stream));
     PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-    std::memcpy(h_it.data(), h_state.data() + off_it, NB * sizeof(int64_t));
-    std::memcpy(h_res.data(), h_state.data() + off_res, NB * sizeof(double));
+    std::memcpy(h_it.data(), h_state.data() + L.it, NB * sizeof(int64_t));
+    std::memcpy(h_res.data(), h_state.data() + L.res, NB * sizeof(double));
   }
   if (ev.second) PDD_CUDA_TRY(ctx, cudaEventRecord(ev.second, ctx->stream));
   PDD_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
@@ -859,8 +877,6 @@ pdd_status elliptic3d_stage2_impl(pdd_ctx *ctx, const double *d_nodes, const dou
     h_off[p] = p * cap;
     h_q[p] = g2;
   }
-  st = interface_interp_impl(ctx, np, h_axis, h_pos, h_cnt, pn, pv, sp->n_bnd, h_q, q, d_planes, h_off);
-  if (st != PDD_OK) return st;
   std::vector<Box3> boxes;
   for (int kz = 0; kz < split; ++kz)
     for (int ky = 0; ky < split; ++ky)
@@ -889,6 +905,11 @@ pdd_status elliptic3d_stage2_impl(pdd_ctx *ctx, const double *d_nodes, const dou
         B.u_off = (kz * g2 + static_cast<int64_t>(ky) * grid + kx) * (m - 1);
         boxes.push_back(B);
       }
+  // (scratch for the larger of the two parts at once)
+  st = ensure_scratch(ctx, box3_layout(boxes, sp->method == PDD_STENCIL_JACOBI, g2 * grid).total);
+  if (st != PDD_OK) return st;
+  st = interface_interp_impl(ctx, np, h_axis, h_pos, h_cnt, pn, pv, sp->n_bnd, h_q, q, d_planes, h_off);
+  if (st != PDD_OK) return st;
   return solve_boxes(ctx, boxes, sp->method, sp->max_iter, sp->tol, d_planes, d_u, g2 * grid, iters,
                      resid, nullptr, nullptr);
 }
