@@ -623,15 +623,17 @@ PDD_API pdd_status pdd_profile_read(pdd_ctx *ctx, double *kernel_ms,
  * It computes the same estimate as pdd_interface_solve (same kernels, same
  * streams, same exact per-node sums, no diagnostics) on `device` and
  * `cuda_stream`, without a context, in one path-kernel launch and one
- * finalisation launch.  The caller still provides the inputs and outputs
+ * finalisation launch (FP64 paths: and before them one that forms the tables of
+ * their normals).  The caller still provides the inputs and outputs
  * (device pointers, as for pdd_interface_solve).  Scratch comes from one
  * static 8 MiB device array that every GPU loading this library holds until
- * process exit (256 bytes of counters and 112 bytes per node); n is limited
- * to 65536 nodes and node_offset + n to 2^32 (PDD_EINVAL beyond), the path
- * count is not limited.  The first call on a device loads the kernels; every
- * call looks up the array's device address (no allocation).  All calls share
- * the array and each clears it at the start, so calls that overlap on the GPU
- * (different streams, or different threads) race: serialise them.
+ * process exit (256 bytes of counters, 112 bytes per node and, at its end, 115 KB
+ * for those tables); n is limited to 65536 nodes and node_offset + n to 2^32
+ * (PDD_EINVAL beyond), the path count is not limited.  The first call on a device
+ * loads the kernels; every call looks up the array's device address (no
+ * allocation).  All calls share the array and each clears it at the start, so calls
+ * that overlap on the GPU (different streams, or different threads) race: serialise
+ * them.
  * It calls no cudaMalloc, cudaFree or allocating library routine.          */
 PDD_API pdd_status pdd_interface_solve_static(const pdd_problem *problem,
                                               int device, void *cuda_stream,

@@ -148,12 +148,13 @@ __device__ __forceinline__ void flush_exits(const PathArgs &a, ExitQueue<Model::
   __syncwarp();
 }
 
+constexpr int kGradBlock = 128;
 template <class Model, class Geom, typename R>
-__global__ void __launch_bounds__(kPathBlockOf<R>)
+__global__ void __launch_bounds__(kGradBlock)
 path_lr_kernel(const __grid_constant__ PathArgs a) {
   constexpr int D = Model::D;
   constexpr int NL = kMaxLR;
-  __shared__ PathStage<D, R> stage_all[kPathBlockOf<R> / 32];
+  __shared__ PathStage<D, R> stage_all[kGradBlock / 32];
   PathStage<D, R> &stage = stage_all[threadIdx.x >> 5];
   R L[NL];
   const unsigned lane = threadIdx.x & 31u;

@@ -16,8 +16,8 @@
 // scheme (fine path only).  Left point for Y and Z.  Dimensions 1 and 2.
 //
 // What bounds it: instruction issue.  The kernel works as the path kernel
-// does (path_kernel.cuh): a unit of steps (four fine ones; R for R other than
-// 2 and 4) runs without a branch under one conservative distance bound per
+// does (path_kernel.cuh): a unit of steps (four fine ones at level 0 and for R = 2,
+// else R) runs without a branch under one conservative distance bound per
 // step and walk, and a unit that may hold an exit is parked and rerun with
 // the exact tests, 32 at a time.  Finished pairs are queued and added to the
 // exact sums of the difference, the fine and the coarse score 32 at a time

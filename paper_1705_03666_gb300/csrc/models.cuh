@@ -221,8 +221,9 @@ struct Box {
     if constexpr (D == 3) m = max3_abs(m, x[1] - 0.5f, x[2] - 0.5f);
     return 0.5f - m;
   }
-  // The most faces within bridge reach of one step (opposite ones cannot both
-  // be while sigma^2 dt <= 1/36).
+  // The most faces that can count in one step: the exact test takes one candidate
+  // face per axis, the one with the smaller d d'.  (At sigma^2 dt = 1/36 a step of
+  // 4.8 standard deviations across the box is within reach of both faces.)
   __host__ __device__ static int reach(double) { return D; }
   // Distance to the plane of face j, positive on the domain side.
   template <typename R>
@@ -232,8 +233,8 @@ struct Box {
   }
   // Screening of a step X -> X' (X in the closed box): the smallest
   //   d d' = min over k of min(x_k x'_k, (1 - x_k)(1 - x'_k))
-  // over the face of each axis that can be within bridge reach (the other
-  // one cannot while sigma^2 dt <= 1/36).  A result > 0 puts X' strictly
+  // over the nearer face of each axis (the other one is out of bridge reach but for
+  // a step of several standard deviations across the box).  A result > 0 puts X' strictly
   // inside the box: with x_k in [0, 1], both products of an axis are positive
   // only for x'_k in (0, 1) (a rounded product keeps its sign; an underflow
   // to zero gives 0).

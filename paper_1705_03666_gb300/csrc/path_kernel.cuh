@@ -39,16 +39,11 @@
 
 namespace pdd {
 
-// Threads per block of the persistent path kernels, by path precision.  With
-// 128-thread blocks ptxas gives the binary32 kernels ~70 registers and the
-// SM holds 7 blocks (28 warps); with 256-thread blocks it held them to 64
-// registers for 4 blocks (32 warps), and the 3-D solve ran 840 against
-// 836 ms.  The FP64 kernels keep 256-thread blocks (their 2-D two-stage run
-// was 11.4 against 13.0 ms).
-template <typename R>
-constexpr int kPathBlockOf = sizeof(R) == 4 ? 128 : 256;
-
-constexpr int kForwardBlock = 128;  // the forward path kernel, both precisions
+// Threads per block of the forward path kernel, both precisions.  In binary32 ptxas
+// gives 128-thread blocks 72 registers and the SM holds seven (28 warps); 256-thread
+// blocks are held to 64 registers for four (32 warps): 840 against 836 ms on the 3-D
+// solve when that was measured.
+constexpr int kForwardBlock = 128;
 
 struct PathArgs {
   const double *nodes;          // [n_nodes][D]
