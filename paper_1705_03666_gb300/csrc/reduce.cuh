@@ -52,37 +52,39 @@ __device__ __forceinline__ bool warp_adds_exactly(float v) {
   const uint32_t low = __reduce_max_sync(kFull, b ? 256u - e : 0u);  // 256 less the smallest
   return top == 0u || (top < 255u && top + low <= 256u + 24u);
 }
-// The warp's total as an unevaluated sum s + c, in every lane.  Two-float sums: the
-// high and the low parts by themselves where each add up exactly, as they do but
-// for sums of very different size (2 FP64 instructions a step of the tree instead
-// of 9); compensated otherwise, and for binary64 sums.
-__device__ __forceinline__ CSum warp_total(CSum t) {
+// The total of n unevaluated sums s + c (n a power of two up to 32), one per lane
+// below n: compensated, the larger of two found by their bits (an FP64 comparison
+// occupies its scheduler's pipe for 64 clocks as the additions do, five of them a
+// step of the tree).
+__device__ __forceinline__ CSum lanes_total(CSum t, int n) {
 #pragma unroll
-  for (int m = 16; m > 0; m >>= 1) t.merge(shfl_xor(t, m));
+  for (int m = 16; m > 0; m >>= 1) {
+    if (m >= n) continue;
+    const CSum o = shfl_xor(t, m);
+    constexpr unsigned long long kAbs = 0x7fffffffffffffffull;
+    const bool own = (static_cast<unsigned long long>(__double_as_longlong(t.s)) & kAbs) >=
+                     (static_cast<unsigned long long>(__double_as_longlong(o.s)) & kAbs);
+    const double big = own ? t.s : o.s, small = own ? o.s : t.s, sum = t.s + o.s;
+    t.c = t.c + o.c + ((big - sum) + small);
+    t.s = sum;
+  }
   return t;
 }
+// The warp's total, in every lane.  Two-float sums: the high and the low parts by
+// themselves where the high ones add up exactly, as they do but for sums of very
+// different size (the low ones, below 2^-24 of them, then lose 2^-77, a two-float sum
+// itself 2^-48); compensated otherwise, and for binary64 sums.
+__device__ __forceinline__ CSum warp_total(const CSum &t) { return lanes_total(t, 32); }
 __device__ __forceinline__ CSum warp_total(const F2Sum &v) {
   CSum t;
-  if (warp_adds_exactly(v.hi) && warp_adds_exactly(v.lo)) {
-    t.s = static_cast<double>(v.hi);
-    t.c = static_cast<double>(v.lo);
+  t.s = static_cast<double>(v.hi);
+  t.c = static_cast<double>(v.lo);
+  if (!warp_adds_exactly(v.hi)) return lanes_total(t, 32);
 #pragma unroll
-    for (int m = 16; m > 0; m >>= 1) {
-      t.s += __shfl_xor_sync(kFull, t.s, m);
-      t.c += __shfl_xor_sync(kFull, t.c, m);
-    }
-    return t;
+  for (int m = 16; m > 0; m >>= 1) {
+    t.s += __shfl_xor_sync(kFull, t.s, m);
+    t.c += __shfl_xor_sync(kFull, t.c, m);
   }
-  t.add(static_cast<double>(v.hi));
-  t.add(static_cast<double>(v.lo));
-  return warp_total(t);
-}
-// The total of n such sums (n a power of two up to 32), one per lane below n.
-__device__ __forceinline__ CSum lanes_total(const CSum &v, int n) {
-  CSum t;
-  t.add(v.s);
-  t.add(v.c);
-  for (int m = n / 2; m > 0; m >>= 1) t.merge(shfl_xor(t, m));
   return t;
 }
 
