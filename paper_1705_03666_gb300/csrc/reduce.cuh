@@ -149,8 +149,8 @@ struct ReduceParts {
   unsigned *done;
 };
 // Blocks per node: one while the nodes fill the GPU (512 blocks), else up to 32
-// of at least 4096 scores (4 nodes x 10^5 scores: 36 us with one, 9.6 us with
-// 16; 16 x 10^6: 186 -> 16 us).  A function of the sizes alone, so the order of
+// of at least 4096 scores (4 nodes x 10^5 scores: 36 us with one, 14 us
+// with 16; 16 x 10^6: 186 -> 30 us).  A function of the sizes alone, so the order of
 // the additions does not depend on the device.
 inline int reduce_parts(uint64_t n_paths, uint64_t blocks) {
   int p = 1;
